@@ -490,7 +490,14 @@ int gc_top_closeness(gc_graph *g, int32_t k, const gc_opts *opts_in, int32_t *ou
   GC_CUDA(cudaMemcpyAsync(&g->gctl->best_f, &thr.best_f, sizeof(long long), cudaMemcpyHostToDevice, g->stream));
   GC_TRY(launch_select(g, kSelKey, 0, 0, kTauHost, -T));
   GC_TRY(read_ctl(g));
-  const int32_t n_surv = g->h_sctl->n_sel;
+  int32_t n_surv = g->h_sctl->n_sel;
+  if (opts.round0_lanes >= 0 && ecc <= kShallowLevels && n_surv > 0 && !(opts.flags & GC_OPT_R0_NO_PROBE)) {
+    // as in round 0 of gc_greedy: bounds from the low-degree vertices out of two hops' reach
+    GC_TRY(launch_far_bound(g));
+    GC_TRY(launch_select(g, kSelKey, 0, 0, kTauHost, -T));
+    GC_TRY(read_ctl(g));
+    n_surv = g->h_sctl->n_sel;
+  }
   int r0_w = 0;
   if (n_surv > 0 && opts.round0_lanes >= 0 && ecc <= kShallowLevels) {
     const int want = opts.round0_lanes > 0 ? opts.round0_lanes : (n_surv > 128 ? 256 : n_surv > 64 ? 128 : 64);
@@ -856,6 +863,17 @@ int gc_greedy(gc_graph *g, int32_t k, const gc_opts *opts_in, int32_t *out_group
   // (triangle inequality) are weak there and are skipped.
   const int32_t ecc_a = g->h_bctl->levels;
   int r0_w = 0;
+  // The far-vertex probe starts with counts alone: low-degree vertices that no
+  // path of two hops can reach raise the survivors' bounds (k_far_counts), and
+  // the survivors above the threshold are cut without a search.
+  if (opts.round0_lanes >= 0 && ecc_a <= kShallowLevels && n_surv > 0 && !(opts.flags & GC_OPT_R0_NO_PROBE)) {
+    GC_TRY(launch_far_bound(g));
+    GC_TRY(launch_select(g, kSelKey, 0, 0, kTauDevice, 0));
+    GC_TRY(read_ctl(g));
+    r0_probe[0] = 1;
+    r0_probe[1] = n_surv - g->h_sctl->n_sel;
+    n_surv = g->h_sctl->n_sel;
+  }
   if (opts.round0_lanes >= 0 && ecc_a <= kShallowLevels && n_surv > 0) {
     // automatic: 256 lanes at most (measured on R-MAT scale 24: 512 lanes are no
     // faster, their wider gathers cancel the halved batch count)
@@ -916,8 +934,8 @@ int gc_greedy(gc_graph *g, int32_t k, const gc_opts *opts_in, int32_t *out_group
     r0_bu[1] = (int64_t)r0c.bu_scanned;
     r0_bu[2] = (int64_t)r0c.bu_gathers;
     r0_bu[3] = (int64_t)r0c.dense_clears;
-    r0_probe[0] = (int64_t)r0c.probe_levels;
-    r0_probe[1] = (int64_t)r0c.probe_cut;
+    r0_probe[0] += (int64_t)r0c.probe_levels;
+    r0_probe[1] += (int64_t)r0c.probe_cut;
     r0_probe[2] = (int64_t)r0c.bu_vertices;
     r0_probe[3] = (int64_t)r0c.bu_visreads;
   } else if (n_surv <= kRound0GridMax) {

@@ -397,6 +397,10 @@ int launch_fill_i64(gc_graph *g, long long *p, long long v, int64_t count);
 int launch_sum_dist(gc_graph *g, const int32_t *dist);
 // round-0 lower bound key[v] = -LB(v) (two-level degree bound)
 int launch_round0_keys(gc_graph *g);
+// round 0: key[v] lowered for the selected vertices list[0 .. sctl->n_sel) by
+// counting the low-degree vertices that cannot be within two hops of v (uses
+// lgain as scratch; sctl->tau is the threshold the list was selected with)
+int launch_far_bound(gc_graph *g);
 // validation: returns GC_OK / GC_EINVAL via sctl->err
 int launch_validate(gc_graph *g);
 
