@@ -128,10 +128,11 @@ typedef struct gc_opts {
                               updates d_S on one CTA; 0 or negative = never */
   int32_t lazy_ctas;       /* step_mode 3: CTAs of the persistent kernel (fewer
                               CTAs make its grid barriers cheaper); 0 = one per
-                              SM; clamped to that */
+                              SM; clamped to that.  gc_batch_greedy: CTAs of a
+                              team in the lazy rounds; 0 = automatic */
   int32_t batch_grid_min_n; /* gc_batch_greedy: graphs with at least this many
                               vertices run their lazy rounds grid-wide, one
-                              graph at a time; the others CTA-locally;
+                              graph at a time; the others by teams of CTAs;
                               0 = 2097152, negative = none */
   int32_t round0_lanes;    /* gc_greedy round 0 on shallow graphs (the BFS from
                               the lowest-bound vertex has at most 32 levels):
@@ -476,8 +477,9 @@ int64_t gc_recorded(gc_graph *g);
 
 /* ------------------------------------------------- batched solving ----- */
 /* Many graphs solved together: the batch is held as one block-diagonal union
- * graph on the device and solved by ONE persistent cooperative kernel (round 0,
- * round 1 and every lazy round of every graph, no host round trip), optionally
+ * graph on the device and solved by three persistent cooperative kernels
+ * (rounds 0 and 1, every lazy round of every graph, the farness check; no host
+ * round trip between them), optionally
  * replayed from a captured CUDA graph (opts.flags & GC_OPT_CAPTURE).  Each
  * graph's group equals gc_greedy's on that graph alone. */
 typedef struct gc_batch gc_batch; /* opaque: union CSR + per-graph state */

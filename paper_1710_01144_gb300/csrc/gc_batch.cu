@@ -1,4 +1,5 @@
-// Batched Greedy++ over many graphs in ONE persistent cooperative launch.
+// Batched Greedy++ over many graphs: three persistent cooperative launches, no
+// host round trip between them.
 //
 // The batch is stored as one block-diagonal union CSR (global vertex ids;
 // graph g owns ids [off[g], off[g+1])).  Distances never cross components, so
@@ -7,7 +8,8 @@
 // graph -- round-0 cut thresholds, argmin/argmax, the lazy round state and its
 // acceptance test (Sec. 4.2), the group -- lives in per-graph arrays.
 //
-// Phases (bounded grid barriers between them):
+// Phases (bounded grid barriers between them); P0 to P5 are k_batch_solve, P6
+// k_batch_lazy, P7 k_batch_check:
 //   P0  lower bounds LB(v) and, per graph, the vertex v_a of smallest bound
 //   P1  BFS from all v_a; per-graph farness f_a
 //   P2  every v with LB(v) <= f_a evaluated by the 64-lane BFS in farness
@@ -17,9 +19,13 @@
 //   P4  round 1: every candidate of every graph, graph-aligned 64-lane batches
 //       from a dynamic task counter; per-graph argmax; picks; BFS from picks
 //   P5  per graph (one CTA): active list of the largest bounds
-//   P6  lazy rounds: each CTA runs its graphs' rounds to completion -- fold,
-//       decide, select 64, evaluate them (64-lane BFS), and on acceptance a
-//       CTA-local pruned BFS from the pick -- so no graph waits for another.
+//   P6  lazy rounds: teams of CTAs, each running the rounds of one graph after
+//       another (longest first) to completion -- fold, decide, select 64,
+//       evaluate them by the whole team, update d_S from the pick's claim log --
+//       so no graph waits for another.  A team's steps are those of the
+//       single-graph persistent kernel.  One CTA per graph, as before, left
+//       most of the GPU idle behind the slowest graph: 24 mixed graphs 717 ms
+//       (lazy rounds 634), with teams 207 ms (124); 256 graphs 1468 -> 1109 ms.
 //   P7  check: one BFS from every graph's whole group; each graph's farness
 //       must equal f(s0) minus the sum of its accepted gains.
 #include <limits.h>
@@ -28,6 +34,9 @@
 
 #include <algorithm>
 #include <chrono>
+#include <cmath>
+#include <functional>
+#include <queue>
 #include <string>
 #include <vector>
 
@@ -53,6 +62,18 @@ struct BatchCtl {
   unsigned long long ns_lazy[3];  // lazy rounds, summed over graphs: selection (with list
                                   // rebuilds), gain batches, d_S updates
   int32_t blk_tot[kMaxGridCtas];
+  unsigned long long t_start;  // the solve's start (CTA 0's clock)
+  int32_t stage;               // kernels of the solve that have completed without an error
+  int32_t lazy_next;           // next entry of the lazy rounds' graph order
+};
+
+// One team of the lazy rounds: its barrier, the graph it works on and its
+// grid-batch control block.
+struct TeamCtl {
+  GridBar bar;
+  int32_t g;
+  int32_t pad;
+  GridGainCtl gg;
 };
 
 static __device__ void check_fail(BatchCtl *c, int phase, int g, long long want, long long got) {
@@ -81,7 +102,7 @@ struct BatchArgs {
   unsigned long long *packed;
   long long *fa, *farness, *bestf;
   LazyCtl *lc;
-  int32_t *act, *act_n, *full;
+  int32_t *act, *act_n;
   int32_t A;
   int32_t kmax;
   int32_t *picks;
@@ -91,9 +112,20 @@ struct BatchArgs {
   int32_t *scount, *tstart;  // per-graph survivor counts, task prefix [count+1]
   BatchCtl *ctl;
   GainCtl *gctl;
-  GridGainCtl *gg;    // grid-wide batches of the big graphs' lazy rounds
-  GridSelScratch *gsel;  // their grid-wide selection
-  int32_t *gx;        // their scratch: 3 * max_n
+  // lazy rounds (k_batch_lazy): teams of team_size CTAs, each with its control
+  // block and selection scratch; 3 n_g entries of gx and 2 n_g of the claim log
+  // per graph, at 3 off[g] and 2 off[g]; wide steps: 64 candidates per CTA
+  TeamCtl *teams;
+  GridSelScratch *gsel;
+  int32_t *gx;
+  ClaimRec *clog;
+  int32_t *wsel;
+  long long *wgain;
+  int32_t *depth;     // BFS levels of the deepest round-1 batch, per graph
+  const int32_t *order;  // graphs of the team phase, longest first; order_n of them
+  int32_t order_n;
+  int32_t team_size;
+  int32_t list_cap;   // entries of a shared-memory list (a power of two, at most kCta0SelectMax)
   int32_t grid_min_n; // graphs with at least this many vertices run their lazy rounds grid-wide
   int32_t bounded;    // round 1 with two-hop bounds (batch_round1_bounded) and the refresh after it
   long long *g3;      // [2 * count]: sum of (d - 3)^+ per graph for round 1, then for the refresh
@@ -101,11 +133,8 @@ struct BatchArgs {
 };
 
 constexpr int kBatchThreads = kGainThreads;
-// lazy rounds grid-wide from this many vertices.  On the 256-graph mix
-// (10^4 to 5 x 10^5 vertices per graph) the whole solve took 1.72 s with
-// 65,536, 1.70 s with 262,144 and 1.56 s with every graph CTA-local: one CTA
-// per graph in parallel beats graphs of that size taking the grid in turn, so
-// only much larger graphs go grid-wide
+// lazy rounds grid-wide from this many vertices: graphs of 10^4 to 5 x 10^5
+// vertices finish sooner by teams side by side than by taking the grid in turn
 constexpr int32_t kBatchGridMinN = 1 << 21;
 
 static __device__ __forceinline__ bool bsync(const BatchArgs &a) { return grid_sync(&a.ctl->bar, &a.ctl->err, a.tns); }
@@ -185,107 +214,6 @@ static __device__ bool batch_prune(const BatchArgs &a) {
   return bsync(a);
 }
 
-
-static __device__ bool grid_refresh_graph(const BatchArgs &a, int g);
-static __device__ void cta_build_list(const BatchArgs &a, int g);
-
-// Lazy rounds (Sec. 4.2) of one big graph g by the whole grid: every CTA
-// takes part in each step's decision and selection (grid_lazy_step) over the
-// graph's active list (built in P5), evaluates the 64 selected as one
-// grid-wide 64-lane batch, and each pick updates d_S by the grid relabel BFS,
-// checked against the pick's gain.  When the list cannot certify a pick, the
-// graph's bounds are refreshed and the list rebuilt; a second failure in the
-// same round lists every candidate from then on.  Every CTA runs the same loop.
-static __device__ bool batch_grid_lazy(const BatchArgs &a, int g) {
-  const int tid = threadIdx.x, b = blockIdx.x;
-  LazyCtl *lc = &a.lc[g];
-  const int o = a.off[g], ng = a.ng[g];
-  bool every = false, fold = false;
-  int rebuilt = -1;  // round of the last rebuild
-  unsigned long long t_ph[3] = {0, 0, 0}, t_mark = global_ns();  // CTA 0's phase clocks
-  auto lap = [&](int q) {
-    if (b == 0 && tid == 0) {
-      const unsigned long long now = global_ns();
-      t_ph[q] += now - t_mark;
-      t_mark = now;
-    }
-    __syncwarp();  // reconverge warp 0 before the warp-synchronous code that follows
-  };
-  for (;;) {
-    const int r = *(volatile int32_t *)&lc->round;
-    if (r >= a.kk[g]) break;
-    const int32_t *list = every ? a.iota + o : a.act + (size_t)g * a.A;
-    const int m = every ? ng : *(volatile int32_t *)&a.act_n[g];
-    int dec;
-    if (!grid_lazy_step(list, m, a.ub, a.stamp, nullptr, nullptr, lc, a.gg, fold, lc->sel, lc->selpos,
-                        lc->gsel, kLanes, a.gsel, &a.ctl->bar, &a.ctl->err, a.tns, &dec))
-      return false;
-    if (!bsync(a)) return false;
-    lap(0);
-    if (dec == 2) {
-      if (every) {  // cannot happen with every candidate listed
-        if (b == 0 && tid == 0) check_fail(a.ctl, 6, g, 1, 2);
-        return false;
-      }
-      if (rebuilt == r) {
-        every = true;
-        if (b == 0 && tid == 0) lc->theta = LLONG_MIN;
-      } else {
-        rebuilt = r;
-        if (!grid_refresh_graph(a, g)) return false;
-        if (b == 0) cta_build_list(a, g);
-      }
-      if (!bsync(a)) return false;
-      lap(0);
-      fold = false;
-      continue;
-    }
-    if (dec == 0) {
-      if (!grid_gain_batch<kModeGain>(a.rpf, a.cif, a.N, a.dS, lc->sel, 0, &lc->n_sel, lc->gsel, a.ws, a.gx,
-                                      a.goff, a.gg, a.gctl, &a.ctl->bar, &a.ctl->err, a.tns, a.mx, a.c3, o,
-                                      a.max_n))
-        return false;
-      if (b == 0 && tid == 0 && *(volatile int32_t *)&a.gg->err)
-        atomicExch(&a.ctl->err, *(volatile int32_t *)&a.gg->err);
-      if (!bsync(a)) return false;  // workspace clean, gains visible
-      lap(1);
-      fold = true;
-      continue;
-    }
-    // accept the round's best and update d_S from it
-    fold = false;
-    if (b == 0 && tid == 0) {
-      a.ctl->pk[0] = a.ctl->pk[1] = a.ctl->pk[2] = 0;
-      a.ctl->decrease = 0;
-    }
-    if (!bsync(a)) return false;
-    if (!grid_relabel_bfs(a.rpf, a.cif, a.N, a.dS, &lc->best_id, 1, a.q0, a.q1, a.ctl->pk, nullptr,
-                          &a.ctl->decrease, nullptr, a.goff, a.st1, &a.ctl->bar, &a.ctl->err, a.tns, nullptr,
-                          a.c3))
-      return false;
-    if (!bsync(a)) return false;
-    if (b == 0 && tid == 0) {
-      const int pick = lc->best_id;
-      const long long gain = lc->best_gain;
-      a.ctl->pk[0] = a.ctl->pk[1] = a.ctl->pk[2] = 0;
-      if ((long long)a.ctl->decrease != gain) check_fail(a.ctl, 6, g, gain, (long long)a.ctl->decrease);
-      a.picks[(size_t)g * a.kmax + r] = pick;
-      a.pgain[(size_t)g * a.kmax + r] = gain;
-      a.ub[pick] = -1;
-      lc->last_gain = gain;
-      lc->best_id = -1;
-      lc->best_gain = -1;
-      lc->round = r + 1;
-    }
-    if (!bsync(a)) return false;
-    lap(2);
-  }
-  if (b == 0 && tid == 0) {
-    atomicAdd((unsigned long long *)&a.ctl->iterations, (unsigned long long)lc->steps);
-    for (int q = 0; q < 3; ++q) atomicAdd(&a.ctl->ns_lazy[q], t_ph[q]);
-  }
-  return true;
-}
 
 // per-graph sum of d over all vertices (warp-aggregated when a warp's vertices
 // share a graph); unreached vertices raise GC_EDISCONNECTED
@@ -543,8 +471,10 @@ static __device__ bool batch_round1_bounded(const BatchArgs &a, const GainWs &my
     if (g >= a.count) break;
     const int m = a.scount[g], o = a.off[g];
     if (m == 0) continue;
+    const unsigned long long lev0 = cnt.levels;
     cta_gain_batch<kModeGain, true, true>(a.rpf, a.cif, a.N, a.dS1, a.slist + o, m, s_out, myws, a.gctl, a.mx,
                                           LaneGraphs(), cnt, o, a.c3);
+    if (tid == 0) a.depth[g] = (int)(cnt.levels - lev0);
     if (tid < m) {
       const int v = a.slist[o + tid];
       a.ub[v] = s_out[tid];
@@ -643,39 +573,17 @@ static __device__ bool batch_bound_refresh(const BatchArgs &a) {
 // longer certify a pick (the single-graph path refreshes before each rebuild
 // of its list the same way): c3 for the current d_S into q0, G3 of the graph,
 // then every candidate's bound lowered to the two-hop bound for the current
-// group.  The CTA form runs inside one CTA (P6b); the grid form is spread over
-// every CTA, with three grid barriers (P6a).
-static __device__ void cta_refresh_graph(const BatchArgs &a, int g) {
+// group.  By the CTAs of one team, with three team barriers.
+static __device__ bool team_refresh_graph(const BatchArgs &a, int g, TeamCtl *tc, Team tm) {
   __shared__ long long s_ll[32];
-  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, nw = blockDim.x >> 5;
-  const int o = a.off[g], n = a.ng[g];
-  long long x3 = 0;
-  for (int i = tid; i < n; i += blockDim.x) x3 += max(a.dS[o + i] - 3, 0);
-  for (int u = o + wid; u < o + n; u += nw) {
-    int c = 0;
-    for (int e = a.rpf[u] + lane; e < a.rpf[u + 1]; e += 32) c += a.dS[a.cif[e]] >= 3;
-    c = warp_sum(c);
-    if (lane == 0) a.q0[u] = c;
-  }
-  const long long G3 = block_sum(x3, s_ll);  // its barriers also publish q0
-  for (int v = o + wid; v < o + n; v += nw) {
-    if (a.ub[v] < 0) continue;  // a member (warp-uniform)
-    const long long s = warp_two_hop(a, a.dS, a.q0, v) + G3;
-    if (lane == 0 && s < a.ub[v]) a.ub[v] = s;
-  }
-  cta_sync();
-}
-
-static __device__ bool grid_refresh_graph(const BatchArgs &a, int g) {
-  __shared__ long long s_ll[32];
-  const int tid = threadIdx.x, lane = tid & 31, b = blockIdx.x, G = gridDim.x, T = blockDim.x;
-  const int gw = (b * T + tid) >> 5, nw = (G * T) >> 5;
+  const int tid = threadIdx.x, lane = tid & 31, T = blockDim.x;
+  const int gw = (tm.b * T + tid) >> 5, nw = (tm.G * T) >> 5;
   const int o = a.off[g], n = a.ng[g];
   long long *g3 = a.g3 + a.count + g;
-  if (b == 0 && tid == 0) *g3 = 0;
-  if (!bsync(a)) return false;
+  if (tm.b == 0 && tid == 0) *g3 = 0;
+  if (!grid_sync(&tc->bar, &a.ctl->err, a.tns, tm)) return false;
   long long x3 = 0;
-  for (int i = b * T + tid; i < n; i += G * T) x3 += max(a.dS[o + i] - 3, 0);
+  for (int i = tm.b * T + tid; i < n; i += tm.G * T) x3 += max(a.dS[o + i] - 3, 0);
   x3 = block_sum(x3, s_ll);
   if (tid == 0 && x3) atomicAdd((unsigned long long *)g3, (unsigned long long)x3);
   for (int u = o + gw; u < o + n; u += nw) {
@@ -684,14 +592,231 @@ static __device__ bool grid_refresh_graph(const BatchArgs &a, int g) {
     c = warp_sum(c);
     if (lane == 0) a.q0[u] = c;
   }
-  if (!bsync(a)) return false;
+  if (!grid_sync(&tc->bar, &a.ctl->err, a.tns, tm)) return false;
   const long long G3 = *(volatile long long *)g3;
   for (int v = o + gw; v < o + n; v += nw) {
     if (a.ub[v] < 0) continue;  // a member (warp-uniform)
     const long long s = warp_two_hop(a, a.dS, a.q0, v) + G3;
     if (lane == 0 && s < a.ub[v]) a.ub[v] = s;
   }
-  return bsync(a);
+  return grid_sync(&tc->bar, &a.ctl->err, a.tns, tm);
+}
+
+// Lazy rounds (Sec. 4.2) of graph g by one team of CTAs, from its list built in
+// P5 to its last pick: the loop of the single-graph persistent kernel
+// (gc_lazy.cu) on a part of the grid.  Three forms of a step:
+//   lean  (list of at most list_cap entries): the team's CTA 0 keeps the list in
+//         shared memory with its sorted view, folds, decides, selects and runs
+//         level 0; the team runs the rest of the 64-lane batch, and a pick
+//         updates d_S from the claim log (or the relabel BFS past its capacity);
+//   wide  (deep graphs: more than kWideLevels levels per round-1 batch): one
+//         64-lane batch per CTA of the team, no team barrier inside;
+//   grid  (longer lists): the whole team selects (grid_lazy_step).
+// When the list cannot certify a pick, the graph's bounds are refreshed and the
+// list rebuilt; a second failure in the same round lists every candidate from
+// then on.  Every CTA of the team runs the same loop.
+static __device__ bool team_lazy(const BatchArgs &a, int g, TeamCtl *tc, Team tm, GridSelScratch *gsel,
+                                 GainCounters &cnt, GridCounts &gcnt, unsigned char *s_list) {
+  __shared__ Cta0State s_st;
+  __shared__ int s_nord;
+  __shared__ u64 s_red[32];
+  const int tid = threadIdx.x, b = tm.b;
+  const bool lead = b == 0 && tid == 0;
+  LazyCtl *lc = &a.lc[g];
+  const int o = a.off[g], ng = a.ng[g], k = a.kk[g];
+  const int first = blockIdx.x - b;  // the team's first CTA: its workspace serves the team's batches
+  unsigned char *ws0 = a.ws + a.ws_stride * (size_t)first;
+  const GainWs myws = gain_ws(a.ws, a.ws_stride, a.max_n, blockIdx.x);
+  int32_t *gx = a.gx + 3 * (size_t)o;
+  ClaimRec *clog = a.clog + 2 * (size_t)o;
+  const u64 clog_cap = 2 * (u64)ng;
+  int32_t *wsel = a.wsel + (size_t)first * kLanes;
+  long long *wgain = a.wgain + (size_t)first * kLanes;
+  const bool wide = a.depth[g] > kWideLevels;
+  auto sync = [&]() { return grid_sync(&tc->bar, &a.ctl->err, a.tns, tm); };
+
+  // CTA 0's list: bounds, ids, stamps, and the sorted view of them
+  const int cap = a.list_cap;
+  long long *sk = reinterpret_cast<long long *>(s_list);
+  int32_t *sa = reinterpret_cast<int32_t *>(sk + cap), *ss = sa + cap;
+  SortedView view;
+  view.ord = reinterpret_cast<uint16_t *>(ss + cap);
+  view.tmp = view.ord + cap;
+  view.mark = reinterpret_cast<unsigned char *>(view.tmp + cap);
+  view.nord = &s_nord;
+  bool every = false, fold = false;
+  int rebuilt = -1;  // round of the last rebuild
+  const int32_t *list = nullptr;
+  int m = 0;
+  bool lean = false;
+  // the list of the coming steps (every CTA), and CTA 0's copy of it
+  auto load = [&]() {
+    list = every ? a.iota + o : a.act + (size_t)g * a.A;
+    m = every ? ng : *(volatile int32_t *)&a.act_n[g];
+    lean = !wide && m <= cap;
+    if (!lean || b != 0) return;
+    if (tid == 0) {
+      s_st.bpos = -1;
+      s_st.bid = lc->best_id;
+      s_st.bgain = lc->best_gain;
+      s_st.theta = lc->theta;
+      s_st.log_mark = lc->log_mark;
+      s_st.nsel = 0;
+      s_st.dec = 0;
+    }
+    cta_sync();
+    for (int i = tid; i < m; i += blockDim.x) {
+      const int v = list[i];
+      sa[i] = v;
+      sk[i] = a.ub[v];
+      ss[i] = a.stamp[v];
+      if (v == s_st.bid) {
+        s_st.bpos = i;
+        lc->best_pos = i;
+      }
+    }
+    cta_sync();
+    sv_build(sk, m, view);
+  };
+  unsigned long long t_ph[3] = {0, 0, 0}, t_mark = lead ? global_ns() : 0;  // phase clocks
+  auto lap = [&](int q) {
+    if (lead) {
+      const unsigned long long now = global_ns();
+      t_ph[q] += now - t_mark;
+      t_mark = now;
+    }
+    __syncwarp();  // reconverge warp 0 before the warp-synchronous code that follows
+  };
+  load();
+  int r = *(volatile int32_t *)&lc->round;
+  if (!sync()) return false;
+  while (r < k) {
+    if (lean) {
+      if (b == 0) {
+        lean_step(sa, a.ub, a.stamp, lc, &tc->gg, fold, r, sk, ss, view, s_st);
+        cta_sync();  // s_st.dec, the batch and the reset batch control block
+        const int d = s_st.dec;
+        if (d == 0)
+          grid_gain_batch<kModeGain>(a.rpf, a.cif, a.N, a.dS, s_st.sel, 0, &s_st.nsel, s_st.gout, ws0, gx, a.goff,
+                                     &tc->gg, a.gctl, &tc->bar, &a.ctl->err, a.tns, a.mx, a.c3, o, a.max_n,
+                                     kBatchLevel0, clog, &lc->log_n, clog_cap, nullptr, tm, ng);
+      }
+    } else if (wide) {
+      if (b == 0)
+        lazy_cta0_step(list, m, a.ub, a.stamp, lc, nullptr, fold, nullptr, 0, nullptr, nullptr, wsel, wgain, nullptr,
+                       tm.G * kLanes);
+    } else {
+      int dec_local;
+      if (!grid_lazy_step(list, m, a.ub, a.stamp, nullptr, nullptr, lc, &tc->gg, fold, lc->sel, lc->selpos, lc->gsel,
+                          kLanes, gsel, &tc->bar, &a.ctl->err, a.tns, &dec_local, tm))
+        return false;
+    }
+    if (lead) {  // an accepted pick's update starts from zero
+      lc->pk[0] = lc->pk[1] = lc->pk[2] = 0;
+      lc->decrease = 0;
+    }
+    if (!sync()) return false;
+    const int dec = *(volatile int32_t *)&lc->dec;
+    lap(0);
+    if (dec == 2) {
+      if (every) {  // cannot happen with every candidate listed
+        if (lead) check_fail(a.ctl, 6, g, 1, 2);
+        return false;
+      }
+      if (rebuilt == r) {
+        every = true;
+        if (lead) lc->theta = LLONG_MIN;
+      } else {
+        rebuilt = r;
+        if (!team_refresh_graph(a, g, tc, tm)) return false;
+        if (b == 0) cta_build_list(a, g);
+      }
+      if (!sync()) return false;
+      load();
+      fold = false;
+      lap(0);
+      continue;
+    }
+    if (dec == 0) {
+      if (wide) {
+        const int ns = *(volatile int32_t *)&lc->n_sel, nb = (ns + kLanes - 1) / kLanes;
+        for (int bi = b; bi < nb; bi += tm.G)
+          cta_gain_batch<kModeGain, true, false>(a.rpf, a.cif, a.N, a.dS, wsel + bi * kLanes,
+                                                 min(kLanes, ns - bi * kLanes), wgain + bi * kLanes, myws, a.gctl,
+                                                 a.mx, LaneGraphs(), cnt, o, a.c3);
+        if (!sync()) return false;  // gains visible to CTA 0
+      } else {
+        // CTA 0 keeps a lean batch in shared memory, the others read its copy
+        const bool st0 = lean && b == 0;
+        if (!grid_gain_batch<kModeGain>(a.rpf, a.cif, a.N, a.dS, st0 ? s_st.sel : lc->sel, 0,
+                                        st0 ? &s_st.nsel : &lc->n_sel, st0 ? s_st.gout : lc->gsel, ws0, gx, a.goff,
+                                        &tc->gg, a.gctl, &tc->bar, &a.ctl->err, a.tns, a.mx, a.c3, o, a.max_n,
+                                        lean ? kBatchRest : kBatchAll, clog, &lc->log_n, clog_cap, &gcnt, tm, ng))
+          return false;
+        if (!lean && !sync()) return false;  // a team-wide fold reads the gains CTA 0 wrote
+        if (lead && *(volatile int32_t *)&tc->gg.err) atomicExch(&a.ctl->err, *(volatile int32_t *)&tc->gg.err);
+      }
+      lap(1);
+      fold = true;
+      continue;
+    }
+    // accept the round's best and update d_S from it
+    fold = false;
+    const int blane = *(volatile int32_t *)&lc->best_lane, pick = *(volatile int32_t *)&lc->best_id;
+    const u64 l0 = *(volatile u64 *)&lc->best_seg0, l1 = *(volatile u64 *)&lc->best_seg1;
+    if (!wide && blane >= 0 && blane < kLanes && l0 <= l1 && l1 <= clog_cap) {
+      const u64 bit = 1ull << blane;
+      u64 dec_sum = 0;
+      for (u64 i = l0 + (u64)b * blockDim.x + tid; i < l1; i += (u64)tm.G * blockDim.x) {
+        const int4 e = *reinterpret_cast<const int4 *>(clog + i);
+        if (!(((u64)(unsigned)e.z | ((u64)(unsigned)e.w << 32)) & bit)) continue;
+        const int old = atomicMin(&a.dS[e.x], e.y);
+        if (old > e.y) dec_sum += (u64)(old - e.y);
+      }
+      if (lead) {  // the pick itself (level 0)
+        const int old = atomicMin(&a.dS[pick], 0);
+        if (old > 0) dec_sum += (u64)old;
+      }
+      dec_sum = block_sum(dec_sum, s_red);
+      if (tid == 0 && dec_sum) atomicAdd(&lc->decrease, dec_sum);
+    } else if (!grid_relabel_bfs(a.rpf, a.cif, a.N, a.dS, &lc->best_id, 1, a.q0 + o, a.q1 + o, lc->pk, nullptr,
+                                 &lc->decrease, nullptr, a.goff + o, a.st1 + o, &tc->bar, &a.ctl->err, a.tns, nullptr,
+                                 a.c3, tm)) {
+      return false;
+    }
+    if (!sync()) return false;
+    if (lead) {
+      const long long gain = lean ? s_st.bgain : lc->best_gain;
+      const u64 d = *(volatile u64 *)&lc->decrease;
+      if ((long long)d != gain) check_fail(a.ctl, 6, g, gain, (long long)d);
+      a.picks[(size_t)g * a.kmax + r] = pick;
+      a.pgain[(size_t)g * a.kmax + r] = gain;
+      a.ub[pick] = -1;  // a member: never a candidate again
+      if (lean && s_st.bpos >= 0 && s_st.bpos < m && sa[s_st.bpos] == pick) sk[s_st.bpos] = -1;
+      lc->last_gain = gain;
+      lc->best_id = -1;
+      lc->best_gain = -1;
+      lc->best_lane = -1;
+      lc->log_n = 0;  // the next round's log (its first batch starts after a barrier)
+      lc->log_mark = 0;
+      if (lean) {
+        s_st.bid = -1;
+        s_st.bgain = -1;
+        s_st.bpos = -1;
+        s_st.log_mark = 0;
+      }
+      lc->round = r + 1;
+    }
+    ++r;
+    if (lean) cta_sync();  // only CTA 0 reads the bookkeeping before the next step's barrier
+    else if (!sync()) return false;
+    lap(2);
+  }
+  if (lead) {
+    atomicAdd((unsigned long long *)&a.ctl->iterations, (unsigned long long)lc->steps);
+    for (int q = 0; q < 3; ++q) atomicAdd(&a.ctl->ns_lazy[q], t_ph[q]);
+  }
+  return true;
 }
 
 // Two CTAs per SM (64 registers, no spills): the CTA-local phases are latency
@@ -704,6 +829,7 @@ __global__ void __launch_bounds__(kBatchThreads, 2) k_batch_solve(const BatchArg
   const int tid = threadIdx.x, lane = tid & 31, b = blockIdx.x, G = gridDim.x, T = blockDim.x;
   GainCounters cnt;
   const unsigned long long t_start = global_ns();
+  if (b == 0 && tid == 0) a.ctl->t_start = t_start;
   const GainWs myws = gain_ws(a.ws, a.ws_stride, a.max_n, b);  // this CTA's workspace, sized for the largest graph
   // ---- P0: lower bounds, per-graph argmin ----
   {
@@ -876,8 +1002,10 @@ __global__ void __launch_bounds__(kBatchThreads, 2) k_batch_solve(const BatchArg
     if (a.kk[g] < 2) continue;
     const int o = a.off[g], first = (t - a.bstart[g]) * a.lanes1;
     const int nl = min(a.lanes1, a.ng[g] - first);
+    const unsigned long long lev0 = cnt.levels;
     cta_gain_batch<kModeGain, true, true>(a.rpf, a.cif, a.N, a.dS1, a.iota + o + first, nl, a.ub + o + first, myws,
                                           a.gctl, a.mx, LaneGraphs(), cnt, o, a.c3);
+    if (tid == 0) atomicMax(&a.depth[g], (int)(cnt.levels - lev0));
   }
   if (!bsync(a)) return;
   if (b == 0 && tid == 0) a.ctl->ns_ph[5] = global_ns() - t_start;
@@ -951,93 +1079,81 @@ __global__ void __launch_bounds__(kBatchThreads, 2) k_batch_solve(const BatchArg
   for (int g = b; g < a.count; g += G) {
     if (a.kk[g] <= 2) continue;
     cta_build_list(a, g);
-    if (tid == 0) a.full[g] = 0;
   }
   if (!bsync(a)) return;
-  if (b == 0 && tid == 0) a.ctl->ns_ph[1] = global_ns() - t_start;
-  // ---- P6a: lazy rounds of the big graphs, one graph at a time by the grid ----
-  for (int g = 0; g < a.count; ++g)
-    if (a.ng[g] >= a.grid_min_n && a.kk[g] > 2 && !batch_grid_lazy(a, g)) return;
-  // ---- P6b: the other graphs' lazy rounds; each CTA runs its graphs to
-  // completion (no grid barrier: a graph never waits for another graph's step) ----
-  {
-    __shared__ int s_stop;
-    for (int g = b; g < a.count; g += G) {
-      if (a.ng[g] >= a.grid_min_n) continue;  // done in P6a
-      LazyCtl *lc = &a.lc[g];
-      const int o = a.off[g];
-      unsigned long long t_ph[3] = {0, 0, 0}, t_mark = global_ns();  // thread 0's phase clocks
-      for (;;) {
-        if (tid == 0) s_stop = (lc->round >= a.kk[g]) || (*(volatile int32_t *)&a.ctl->err != 0);
-        cta_sync();
-        if (s_stop) break;
-        const bool full = a.full[g] == 1;  // 0: list, 2 + r: list rebuilt in round r, 1: every candidate
-        const int32_t *act = full ? a.iota + o : a.act + (size_t)g * a.A;
-        const int m = full ? a.ng[g] : a.act_n[g];
-        if (full && tid == 0) lc->theta = LLONG_MIN;
-        cta_sync();
-        lazy_cta0_step(act, m, a.ub, a.stamp, lc, nullptr, lc->pad != 0, nullptr, 0);
-        cta_sync();
-        const int dec = *(volatile int32_t *)&lc->dec;
-        if (tid == 0) {
-          const unsigned long long now = global_ns();
-          t_ph[0] += now - t_mark;
-          t_mark = now;
-        }
-        int ph = 0;  // the rest of the step: 0 list rebuild, 1 gain batch, 2 d_S update
-        if (dec == 0) {  // evaluate the selected batch
-          cta_gain_batch<kModeGain, true, false>(a.rpf, a.cif, a.N, a.dS, lc->sel, lc->n_sel, lc->gsel, myws,
-                                                 a.gctl, a.mx, LaneGraphs(), cnt, o, a.c3);
-          if (tid == 0) lc->pad = 1;  // fold it next step
-          ph = 1;
-        } else if (dec == 1) {  // accept: record, then update d_S from the pick
-          ph = 2;
-          const int pick = lc->best_id;
-          const long long gain = lc->best_gain;
-          const int r = lc->round;
-          cta_sync();
-          const long long decr = cta_relabel_bfs(a.rpf, a.cif, a.dS, pick, myws.qv0, myws.qv1);
-          if (tid == 0) {
-            if (decr != gain) check_fail(a.ctl, 6, g, gain, decr);
-            a.picks[(size_t)g * a.kmax + r] = pick;
-            a.pgain[(size_t)g * a.kmax + r] = gain;
-            a.ub[pick] = -1;
-            lc->last_gain = gain;
-            lc->best_id = -1;
-            lc->best_gain = -1;
-            lc->pad = 0;
-            lc->round = r + 1;
-            lc->steps += 0;
-          }
-        } else {  // the list cannot certify: refresh the bounds and rebuild it
-          const int r = lc->round;
-          const bool again = a.full[g] == 2 + r;
-          cta_sync();
-          if (!again) {
-            cta_refresh_graph(a, g);
-            cta_build_list(a, g);
-          }
-          if (tid == 0) {
-            a.full[g] = again ? 1 : 2 + r;  // a second failure in one round: every candidate
-            lc->pad = 0;
-          }
-        }
-        if (tid == 0) {
-          const unsigned long long now = global_ns();
-          t_ph[ph] += now - t_mark;
-          t_mark = now;
-          if (now - t_start > 6ull * a.tns) atomicExch(&a.ctl->err, GC_ETIMEOUT);
-        }
-        cta_sync();
+  if (b == 0 && tid == 0) {
+    a.ctl->ns_ph[1] = global_ns() - t_start;
+    a.ctl->stage = 1;
+  }
+  // work counters
+  u64 c_scalar = block_sum(cnt.scalar, s_red);
+  u64 c_union = block_sum(cnt.uni, s_red);
+  u64 c_front = block_sum(cnt.front, s_red);
+  u64 c_push = block_sum(cnt.push, s_red);
+  if (tid == 0) {
+    atomicAdd(&a.gctl->edges_scalar, c_scalar);
+    atomicAdd(&a.gctl->edges_union, c_union);
+    atomicAdd(&a.gctl->frontier, c_front);
+    atomicAdd(&a.gctl->pushes, c_push);
+    atomicAdd(&a.gctl->levels, cnt.levels);
+    atomicAdd(&a.gctl->batches, cnt.batches);
+    atomicAdd(&a.gctl->lanes, cnt.lanes);
+  }
+}
+
+// P6: the lazy rounds.  Graphs of at least grid_min_n vertices take the whole
+// grid in turn; the others go to teams of team_size consecutive CTAs, each team
+// taking the next graph of `order` (longest first) and running it to
+// completion, so that no graph waits for another graph's step.  One CTA per SM
+// (128 registers), as in the single-graph kernel.
+__global__ void __launch_bounds__(kBatchThreads, 1) k_batch_lazy(const BatchArgs a) {
+  extern __shared__ __align__(16) unsigned char s_list[];  // list_cap * 21 bytes
+  __shared__ u64 s_red[32];
+  if (*(volatile int32_t *)&a.ctl->stage != 1) return;  // an earlier phase failed
+  const int tid = threadIdx.x, b = blockIdx.x;
+  GainCounters cnt;
+  GridCounts gcnt;
+  bool ok = true;
+  for (int g = 0; g < a.count && ok; ++g)
+    if (a.ng[g] >= a.grid_min_n && a.kk[g] > 2)
+      ok = team_lazy(a, g, &a.teams[0], whole_grid(), a.gsel, cnt, gcnt, s_list);
+  const int S = a.team_size, t = b / S;
+  const Team tm{b - t * S, S};
+  if ((t + 1) * S <= (int)gridDim.x) {  // (a remainder of fewer than S CTAs stays idle)
+    TeamCtl *tc = &a.teams[1 + t];
+    while (ok) {
+      if (tm.b == 0 && tid == 0) {
+        const int i = atomicAdd(&a.ctl->lazy_next, 1);
+        tc->g = i < a.order_n ? a.order[i] : -1;
       }
-      if (tid == 0) {
-        atomicAdd((unsigned long long *)&a.ctl->iterations, (unsigned long long)lc->steps);
-        for (int q = 0; q < 3; ++q) atomicAdd(&a.ctl->ns_lazy[q], t_ph[q]);
-      }
+      ok = grid_sync(&tc->bar, &a.ctl->err, a.tns, tm);
+      if (!ok) break;
+      const int g = *(volatile int32_t *)&tc->g;
+      if (g < 0) break;
+      ok = team_lazy(a, g, tc, tm, a.gsel + 1 + t, cnt, gcnt, s_list) &&
+           grid_sync(&tc->bar, &a.ctl->err, a.tns, tm);  // everyone has read tc->g
     }
   }
-  if (!bsync(a)) return;
-  if (b == 0 && tid == 0) a.ctl->ns_ph[2] = global_ns() - t_start;
+  u64 c_scalar = block_sum(cnt.scalar + gcnt.scalar, s_red);
+  u64 c_union = block_sum(cnt.uni + gcnt.uni, s_red);
+  u64 c_front = block_sum(cnt.front + gcnt.front, s_red);
+  u64 c_push = block_sum(cnt.push + gcnt.push, s_red);
+  if (tid == 0) {
+    atomicAdd(&a.gctl->edges_scalar, c_scalar);
+    atomicAdd(&a.gctl->edges_union, c_union);
+    atomicAdd(&a.gctl->frontier, c_front);
+    atomicAdd(&a.gctl->pushes, c_push);
+    atomicAdd(&a.gctl->levels, cnt.levels);
+    atomicAdd(&a.gctl->batches, cnt.batches);
+    atomicAdd(&a.gctl->lanes, cnt.lanes);
+    atomicMax(&a.ctl->ns_ph[2], global_ns() - a.ctl->t_start);
+  }
+}
+
+// P7: every group's farness by one BFS from all picks of all graphs.
+__global__ void __launch_bounds__(kBatchThreads, 2) k_batch_check(const BatchArgs a) {
+  if (*(volatile int32_t *)&a.ctl->stage != 1 || *(volatile int32_t *)&a.ctl->err != 0) return;  // set before the launch
+  const int tid = threadIdx.x, b = blockIdx.x, G = gridDim.x, T = blockDim.x;
   // ---- P7: check every group's farness with one BFS ----
   for (int v = b * T + tid; v < a.N; v += G * T) a.dS[v] = kInf;
   if (b == 0) {
@@ -1069,21 +1185,7 @@ __global__ void __launch_bounds__(kBatchThreads, 2) k_batch_solve(const BatchArg
   if (!bsync(a)) return;
   for (int g = b * T + tid; g < a.count; g += G * T)
     if (a.farness[g] != a.fa[g]) check_fail(a.ctl, 7, g, a.fa[g], a.farness[g]);
-  if (b == 0 && tid == 0) a.ctl->ns_ph[3] = global_ns() - t_start;
-  // work counters
-  u64 c_scalar = block_sum(cnt.scalar, s_red);
-  u64 c_union = block_sum(cnt.uni, s_red);
-  u64 c_front = block_sum(cnt.front, s_red);
-  u64 c_push = block_sum(cnt.push, s_red);
-  if (tid == 0) {
-    atomicAdd(&a.gctl->edges_scalar, c_scalar);
-    atomicAdd(&a.gctl->edges_union, c_union);
-    atomicAdd(&a.gctl->frontier, c_front);
-    atomicAdd(&a.gctl->pushes, c_push);
-    atomicAdd(&a.gctl->levels, cnt.levels);
-    atomicAdd(&a.gctl->batches, cnt.batches);
-    atomicAdd(&a.gctl->lanes, cnt.lanes);
-  }
+  if (b == 0 && tid == 0) a.ctl->ns_ph[3] = global_ns() - a.ctl->t_start;
 }
 
 __global__ void k_iota(int32_t *p, int32_t n) {
@@ -1132,15 +1234,20 @@ struct gc_batch {
   int32_t *dS = nullptr, *mx = nullptr, *stamp = nullptr, *q0 = nullptr, *q1 = nullptr, *goff = nullptr,
           *st1 = nullptr;
   int32_t *rpf = nullptr, *cif = nullptr, *c3 = nullptr, *gx = nullptr, *dS1 = nullptr;
-  GridGainCtl *gg = nullptr;
   GridSelScratch *gsel = nullptr;
+  TeamCtl *teams = nullptr;     // [1 + lazy_ctas]: the whole grid's, then the teams'
+  ClaimRec *clog = nullptr;
+  int32_t *wsel = nullptr, *depth = nullptr, *order = nullptr;
+  long long *wgain = nullptr;
+  int lazy_ctas = 0;            // CTAs of the lazy rounds (one per SM)
+  std::vector<int64_t> h_nnz;   // adjacency entries per graph
   long long *ub = nullptr, *key = nullptr, *f0 = nullptr;
   unsigned char *ws = nullptr;
   size_t ws_stride = 0;
   unsigned long long *packed = nullptr;
   long long *fa = nullptr, *farness = nullptr, *bestf = nullptr, *g3 = nullptr;
   LazyCtl *lc = nullptr;
-  int32_t *act = nullptr, *act_n = nullptr, *full = nullptr, *kk = nullptr, *bstart = nullptr;
+  int32_t *act = nullptr, *act_n = nullptr, *kk = nullptr, *bstart = nullptr;
   int32_t A = 0, act_cap = 0;
   int32_t kcap = 0;
   int32_t *picks = nullptr;
@@ -1155,13 +1262,13 @@ struct gc_batch {
   cudaGraph_t graph = nullptr;
   cudaStream_t cap_stream = nullptr;  // private stream the sequence is captured on
   std::vector<int32_t> cap_k;
-  int32_t cap_A = 0, cap_lanes = 0, cap_grid_min_n = 0;
+  int32_t cap_A = 0, cap_lanes = 0, cap_grid_min_n = 0, cap_lazy_ctas = 0;
   uint32_t cap_flags = 0;
   std::vector<int32_t> h_picks;
   std::vector<long long> h_pgain, h_far;
   int32_t *h_picks_pinned = nullptr;
   long long *h_far_pinned = nullptr;
-  int32_t *h_k_pinned = nullptr, *h_bstart_pinned = nullptr;  // sources of the captured copies
+  int32_t *h_k_pinned = nullptr, *h_bstart_pinned = nullptr, *h_order_pinned = nullptr;  // sources of the captured copies
 };
 
 static void batch_release(gc_batch *b) {
@@ -1171,8 +1278,9 @@ static void batch_release(gc_batch *b) {
   if (b->cap_stream) cudaStreamDestroy(b->cap_stream);
   void *dev[] = {b->rp, b->ci, b->gid, b->off, b->ng, b->iota, b->dS, b->mx, b->stamp, b->q0, b->q1, b->goff, b->st1,
                  b->ub, b->key, b->f0, b->ws, b->packed, b->fa, b->farness, b->bestf, b->lc, b->act, b->act_n,
-                 b->full, b->kk, b->bstart, b->picks, b->pgain, b->seeds, b->ctl, b->gctl, b->slist,
-                 b->scount, b->tstart, b->rpf, b->cif, b->c3, b->gx, b->gg, b->gsel, b->dS1, b->g3};
+                 b->kk, b->bstart, b->picks, b->pgain, b->seeds, b->ctl, b->gctl, b->slist,
+                 b->scount, b->tstart, b->rpf, b->cif, b->c3, b->gx, b->teams, b->gsel, b->dS1, b->g3, b->clog, b->wsel, b->wgain, b->depth,
+                 b->order};
   for (void *p : dev)
     if (p) cudaFree(p);
   if (b->h_ctl) cudaFreeHost(b->h_ctl);
@@ -1181,6 +1289,7 @@ static void batch_release(gc_batch *b) {
   if (b->h_far_pinned) cudaFreeHost(b->h_far_pinned);
   if (b->h_k_pinned) cudaFreeHost(b->h_k_pinned);
   if (b->h_bstart_pinned) cudaFreeHost(b->h_bstart_pinned);
+  if (b->h_order_pinned) cudaFreeHost(b->h_order_pinned);
   delete b;
 }
 
@@ -1193,6 +1302,44 @@ static bool balloc(T **p, size_t count) {
     return false;
   }
   return true;
+}
+
+// The lazy rounds' plan: sorts the graphs by estimated time (longest first)
+// and returns the CTAs of a team: the power of two with the shortest list
+// schedule.  `ctas` > 0 asks for that size.  The estimate of a round in
+// microseconds is fitted to team sizes 1 to 76 on 24 graphs of 10^4 to 3 x 10^4
+// and of 10^4 to 5 x 10^5 vertices: a step's barriers, selection and dependent
+// loads do not shrink with the team, its edges and the bound refreshes do.
+static int plan_teams(const gc_batch *b, const int32_t *ks, std::vector<int32_t> &order, int32_t ctas) {
+  auto est = [&](int32_t g, int s) {
+    const double e = (double)b->h_nnz[g];
+    return (double)(ks[g] - 2) * (45.0 + (0.22 * std::sqrt(e) + 1.1e-4 * e) / s);
+  };
+  std::sort(order.begin(), order.end(), [&](int32_t x, int32_t y) {
+    const double a = est(x, 1), c = est(y, 1);
+    return a > c || (a == c && x < y);
+  });
+  const int G = b->lazy_ctas;
+  if (ctas > 0) return std::min<int>(ctas, G);
+  int best = 1;
+  double best_t = 0;
+  for (int s = 1; s <= G; s *= 2) {
+    // list scheduling in that order: the next graph goes to the team that is free first
+    std::priority_queue<double, std::vector<double>, std::greater<double>> load(
+        std::greater<double>(), std::vector<double>((size_t)(G / s), 0.0));
+    double t = 0;
+    for (int32_t g : order) {
+      const double end = load.top() + est(g, s);
+      load.pop();
+      load.push(end);
+      t = std::max(t, end);
+    }
+    if (s == 1 || t < best_t) {
+      best = s;
+      best_t = t;
+    }
+  }
+  return best;
 }
 
 // The union CSR of `count` graphs.  Host arrays (nnzs == nullptr: the entry
@@ -1213,6 +1360,7 @@ static int batch_load_impl(int32_t count, const int32_t *const *row_ptrs, const 
   b->h_n.assign(ns, ns + count);
   std::vector<int64_t> eoff(count + 1);
   int64_t N = 0, E = 0;
+  b->h_nnz.resize(count);
   for (int32_t g = 0; g < count; ++g) {
     const int64_t e = nnzs ? nnzs[g] : (ns[g] >= 1 && row_ptrs[g] ? row_ptrs[g][ns[g]] : -1);
     if (ns[g] < 1 || !row_ptrs[g] || e < 0 || (!nnzs && row_ptrs[g][0] != 0) || (e > 0 && !col_idxs[g])) {
@@ -1222,6 +1370,7 @@ static int batch_load_impl(int32_t count, const int32_t *const *row_ptrs, const 
     }
     b->h_off[g] = (int32_t)N;
     eoff[g] = E;
+    b->h_nnz[g] = e;
     N += ns[g];
     E += e;
     b->max_n = std::max(b->max_n, ns[g]);
@@ -1245,6 +1394,15 @@ static int batch_load_impl(int32_t count, const int32_t *const *row_ptrs, const 
     return GC_ECUDA;
   }
   b->ctas = std::min(kMaxGridCtas, occ * b->num_sms);
+  if (cudaFuncSetAttribute(k_batch_lazy, cudaFuncAttributeMaxDynamicSharedMemorySize, kLazyListSmem) != cudaSuccess ||
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_batch_lazy, kBatchThreads, kLazyListSmem) != cudaSuccess ||
+      occ < 1 ||
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_batch_check, kBatchThreads, 0) != cudaSuccess || occ < 1) {
+    batch_release(b);
+    set_error("gc_batch_load: the batch kernels cannot be resident");
+    return GC_ECUDA;
+  }
+  b->lazy_ctas = std::min(b->ctas, std::min(kMaxGridCtas, b->num_sms));
   const size_t Nn = (size_t)N;
   bool ok = balloc(&b->rp, Nn + 1) && balloc(&b->ci, (size_t)E) && balloc(&b->gid, Nn) &&
             balloc(&b->off, (size_t)count + 1) && balloc(&b->ng, (size_t)count) && balloc(&b->iota, Nn) &&
@@ -1252,12 +1410,15 @@ static int batch_load_impl(int32_t count, const int32_t *const *row_ptrs, const 
             balloc(&b->q1, Nn) && balloc(&b->goff, Nn + 1) && balloc(&b->st1, Nn) && balloc(&b->ub, Nn) && balloc(&b->key, Nn) &&
             balloc(&b->f0, Nn) && balloc(&b->packed, (size_t)count) && balloc(&b->fa, (size_t)count) &&
             balloc(&b->farness, (size_t)count) && balloc(&b->bestf, (size_t)count) &&
-            balloc(&b->lc, (size_t)count) && balloc(&b->act_n, (size_t)count) && balloc(&b->full, (size_t)count) &&
+            balloc(&b->lc, (size_t)count) && balloc(&b->act_n, (size_t)count) &&
             balloc(&b->kk, (size_t)count) && balloc(&b->bstart, (size_t)count + 1) && balloc(&b->ctl, 1) &&
             balloc(&b->slist, Nn) && balloc(&b->scount, (size_t)count) && balloc(&b->tstart, (size_t)count + 1) &&
             balloc(&b->rpf, Nn + 1) && balloc(&b->cif, std::max<size_t>(1, (size_t)E)) && balloc(&b->c3, Nn) &&
             balloc(&b->dS1, Nn) && balloc(&b->g3, 2 * (size_t)count) &&
-            balloc(&b->gx, 3 * (size_t)std::max<int32_t>(1, b->max_n)) && balloc(&b->gg, 1) && balloc(&b->gsel, 1) &&
+            balloc(&b->gx, 3 * Nn) && balloc(&b->clog, 2 * Nn) && balloc(&b->teams, (size_t)b->lazy_ctas + 1) &&
+            balloc(&b->gsel, (size_t)b->lazy_ctas + 1) && balloc(&b->wsel, (size_t)b->lazy_ctas * kLanes) &&
+            balloc(&b->wgain, (size_t)b->lazy_ctas * kLanes) && balloc(&b->depth, (size_t)count) &&
+            balloc(&b->order, (size_t)count) &&
             balloc(&b->gctl, 1) && cudaMallocHost((void **)&b->h_ctl, sizeof(BatchCtl)) == cudaSuccess &&
             cudaMallocHost((void **)&b->h_gctl, sizeof(GainCtl)) == cudaSuccess;
   int64_t *d_eoff = nullptr;
@@ -1389,6 +1550,8 @@ int gc_batch_greedy(gc_batch *b, const int32_t *ks, const gc_opts *opts_in, int3
   }
   if (!b->h_k_pinned && (cudaMallocHost((void **)&b->h_k_pinned, (size_t)b->count * sizeof(int32_t)) != cudaSuccess ||
                          cudaMallocHost((void **)&b->h_bstart_pinned, ((size_t)b->count + 1) * sizeof(int32_t)) !=
+                             cudaSuccess ||
+                         cudaMallocHost((void **)&b->h_order_pinned, (size_t)b->count * sizeof(int32_t)) !=
                              cudaSuccess)) {
     set_error("gc_batch_greedy: pinned allocation failed");
     return GC_ENOMEM;
@@ -1396,7 +1559,7 @@ int gc_batch_greedy(gc_batch *b, const int32_t *ks, const gc_opts *opts_in, int3
   std::vector<int32_t> bstart(b->count + 1, 0);
   for (int32_t g = 0; g < b->count; ++g) bstart[g + 1] = bstart[g] + (b->h_n[g] + lanes1 - 1) / lanes1;
   const bool same = b->exec && !resized && b->cap_k == std::vector<int32_t>(ks, ks + b->count) && b->cap_A == A && b->cap_grid_min_n == opts.batch_grid_min_n && b->cap_flags == opts.flags &&
-                    b->cap_lanes == lanes1;
+                    b->cap_lanes == lanes1 && b->cap_lazy_ctas == opts.lazy_ctas;
   BatchArgs a;
   a.rp = b->rp;
   a.ci = b->ci;
@@ -1421,13 +1584,27 @@ int gc_batch_greedy(gc_batch *b, const int32_t *ks, const gc_opts *opts_in, int3
   a.cif = b->cif;
   a.c3 = b->c3;
   a.dS1 = b->dS1;
-  a.gg = b->gg;
+  a.teams = b->teams;
   a.gsel = b->gsel;
   a.gx = b->gx;
+  a.clog = b->clog;
+  a.wsel = b->wsel;
+  a.wgain = b->wgain;
+  a.depth = b->depth;
+  a.order = b->order;
   a.bounded = (opts.flags & GC_OPT_NO_ROUND1_BOUND) ? 0 : 1;
   a.g3 = b->g3;
   a.grid_min_n = opts.batch_grid_min_n == 0 ? kBatchGridMinN
                  : (opts.batch_grid_min_n < 0 ? INT32_MAX : opts.batch_grid_min_n);
+  // the lazy rounds' plan: the graphs left to teams, longest first, and the
+  // size of a team
+  std::vector<int32_t> order;
+  for (int32_t g = 0; g < b->count; ++g)
+    if (ks[g] > 2 && b->h_n[g] < a.grid_min_n) order.push_back(g);
+  a.order_n = (int32_t)order.size();
+  a.team_size = plan_teams(b, ks, order, opts.lazy_ctas);
+  a.list_cap = kLanes;
+  while (a.list_cap < A && a.list_cap < kCta0SelectMax) a.list_cap *= 2;
   a.ub = b->ub;
   a.key = b->key;
   a.f0 = b->f0;
@@ -1440,7 +1617,6 @@ int gc_batch_greedy(gc_batch *b, const int32_t *ks, const gc_opts *opts_in, int3
   a.lc = b->lc;
   a.act = b->act;
   a.act_n = b->act_n;
-  a.full = b->full;
   a.A = A;
   a.kmax = kmax;
   a.picks = b->picks;
@@ -1466,10 +1642,22 @@ int gc_batch_greedy(gc_batch *b, const int32_t *ks, const gc_opts *opts_in, int3
     if ((e = cudaMemsetAsync(b->lc, 0, (size_t)b->count * sizeof(LazyCtl), st))) return e;
     if ((e = cudaMemsetAsync(b->ctl, 0, sizeof(BatchCtl), st))) return e;
     if ((e = cudaMemsetAsync(b->gctl, 0, sizeof(GainCtl), st))) return e;
-    if ((e = cudaMemsetAsync(b->gg, 0, sizeof(GridGainCtl), st))) return e;
-    if ((e = cudaMemsetAsync(b->gsel, 0, sizeof(GridSelScratch), st))) return e;
+    if ((e = cudaMemcpyAsync(b->order, b->h_order_pinned, (size_t)b->count * sizeof(int32_t), cudaMemcpyHostToDevice,
+                             st)))
+      return e;
+    const size_t teams = 1 + (size_t)(b->lazy_ctas / a.team_size);
+    if ((e = cudaMemsetAsync(b->teams, 0, teams * sizeof(TeamCtl), st))) return e;
+    if ((e = cudaMemsetAsync(b->gsel, 0, teams * sizeof(GridSelScratch), st))) return e;
+    if ((e = cudaMemsetAsync(b->depth, 0, (size_t)b->count * sizeof(int32_t), st))) return e;
     void *args[] = {(void *)&a};
     if ((e = cudaLaunchCooperativeKernel((const void *)k_batch_solve, dim3(b->ctas), dim3(kBatchThreads), args, 0,
+                                         st)))
+      return e;
+    if (kmax > 2 &&
+        (e = cudaLaunchCooperativeKernel((const void *)k_batch_lazy, dim3(b->lazy_ctas), dim3(kBatchThreads), args,
+                                         (size_t)a.list_cap * 21, st)))
+      return e;
+    if ((e = cudaLaunchCooperativeKernel((const void *)k_batch_check, dim3(b->ctas), dim3(kBatchThreads), args, 0,
                                          st)))
       return e;
     if ((e = cudaMemcpyAsync(b->h_picks_pinned, b->picks, (size_t)b->count * kmax * sizeof(int32_t),
@@ -1484,8 +1672,10 @@ int gc_batch_greedy(gc_batch *b, const int32_t *ks, const gc_opts *opts_in, int3
   bool used_graph = false;
   if (!(capture && same)) {  // a replay reads the pinned buffers it was captured from (same contents)
     cudaStreamSynchronize(st);  // no earlier copy may still read them
+    b->cap_k.clear();           // an earlier captured sequence reads the same buffers: record it again
     memcpy(b->h_k_pinned, ks, (size_t)b->count * sizeof(int32_t));
     memcpy(b->h_bstart_pinned, bstart.data(), bstart.size() * sizeof(int32_t));
+    std::copy(order.begin(), order.end(), b->h_order_pinned);
   }
   if (capture && same) {
     if (cudaGraphLaunch(b->exec, st) != cudaSuccess) return cuda_fail(cudaGetLastError(), "cudaGraphLaunch");
@@ -1501,6 +1691,7 @@ int gc_batch_greedy(gc_batch *b, const int32_t *ks, const gc_opts *opts_in, int3
     b->cap_A = A;
     b->cap_lanes = lanes1;
     b->cap_grid_min_n = opts.batch_grid_min_n;
+    b->cap_lazy_ctas = opts.lazy_ctas;
     b->cap_flags = opts.flags;
     // capture on a private non-blocking stream (the legacy default stream
     // cannot be captured); the graph is then launched on the caller's stream
@@ -1560,13 +1751,13 @@ int gc_batch_greedy(gc_batch *b, const int32_t *ks, const gc_opts *opts_in, int3
     stats->frontier = (int64_t)b->h_gctl->frontier;
     stats->pushes = (int64_t)b->h_gctl->pushes;
     stats->lanes = (int64_t)b->h_gctl->lanes;
-    stats->kernel_launches = 1;
+    stats->kernel_launches = kmax > 2 ? 3 : 2;
     stats->graph_replay = used_graph ? 1 : 0;
     // phases of the solve (CTA 0's clock): rounds 0, 1, the lazy rounds, the check
     const unsigned long long *ph = b->h_ctl->ns_ph;
     stats->ms_round0 = ph[0] * 1e-6;
     stats->ms_round1 = (ph[1] - ph[0]) * 1e-6;
-    stats->ms_lazy_kernel = (ph[2] - ph[1]) * 1e-6;  // the lazy rounds of every graph (P6)
+    stats->ms_lazy_kernel = ph[2] > ph[1] ? (ph[2] - ph[1]) * 1e-6 : 0.0;  // the lazy rounds of every graph (P6)
     stats->ms_lazy_select = b->h_ctl->ns_lazy[0] * 1e-6;  // their phases, summed over graphs
     stats->ms_lazy_gain = b->h_ctl->ns_lazy[1] * 1e-6;
     stats->ms_lazy_update = b->h_ctl->ns_lazy[2] * 1e-6;

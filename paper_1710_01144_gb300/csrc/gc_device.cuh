@@ -26,9 +26,17 @@ __device__ __forceinline__ void cta_sync() {
   __syncthreads();
 }
 
-// Grid barrier for cooperative launches (all CTAs co-resident).  One 32-bit
-// word per barrier: in every episode CTA 0 adds 2^31 - (G - 1) and each other
-// CTA adds 1 (G = gridDim.x), so the episode adds exactly 2^31: bit 31 of the
+// The CTAs that work together on a grid-wide function: CTA b of G.  The whole
+// grid, or a team of consecutive CTAs of it (the batched solver); every team
+// has barriers and scratch of its own.
+struct Team {
+  int b, G;
+};
+__device__ __forceinline__ Team whole_grid() { return Team{(int)blockIdx.x, (int)gridDim.x}; }
+
+// Grid barrier for cooperative launches (all CTAs co-resident) among the CTAs
+// of one team.  One 32-bit word per barrier: in every episode CTA 0 of the team
+// adds 2^31 - (G - 1) and each other CTA adds 1 (G = the team's size), so the episode adds exactly 2^31: bit 31 of the
 // word flips at the last arrival and the low 31 bits come back to zero, ready
 // for the next episode (of any grid size).  Arrival is a release atomic by
 // thread 0, the wait an acquire poll of bit 31; the CTA barriers on both sides
@@ -38,12 +46,12 @@ __device__ __forceinline__ void cta_sync() {
 // leaves its kernel.  Returns false as well when *err is already set.  A word
 // left mid-episode by such an exit must be zeroed before its next launch.
 __device__ __forceinline__ bool grid_sync(GridBar *bar, int32_t *err,
-                                          unsigned long long timeout_ns) {
+                                          unsigned long long timeout_ns, Team tm) {
   __shared__ int s_ok;
   cta_sync();
   if (threadIdx.x == 0) {
     int ok = 1;
-    const unsigned int add = blockIdx.x == 0 ? 0x80000000u - (gridDim.x - 1u) : 1u;
+    const unsigned int add = tm.b == 0 ? 0x80000000u - ((unsigned)tm.G - 1u) : 1u;
     unsigned int old;
     asm volatile("atom.add.release.gpu.u32 %0, [%1], %2;" : "=r"(old) : "l"(&bar->count), "r"(add) : "memory");
     const unsigned long long t0 = global_ns();
@@ -63,6 +71,10 @@ __device__ __forceinline__ bool grid_sync(GridBar *bar, int32_t *err,
   }
   cta_sync();
   return s_ok != 0;
+}
+
+__device__ __forceinline__ bool grid_sync(GridBar *bar, int32_t *err, unsigned long long timeout_ns) {
+  return grid_sync(bar, err, timeout_ns, whole_grid());
 }
 
 // A load through the read-only data path when RO (the data must not change

@@ -81,6 +81,9 @@ static __device__ __forceinline__ int warp_find_start(const int32_t *start, int 
 // With `acc`, each thread adds its work counts (scalar and union adjacency
 // entries, frontier entries, pushes) to *acc instead of the batch summing them
 // over the CTA and into gctl (a persistent caller sums them once at its end).
+// With `tm`, the CTAs of one team run the batch (bar, ctl, ws_base and gx are
+// the team's own); gx_n, if given, is the stride of gx's three parts (at least
+// the vertices of the graph, where ws_n is the workspace's layout).
 constexpr int kBatchAll = 0, kBatchLevel0 = 1, kBatchRest = 2;
 struct GridCounts {
   u64 scalar = 0, uni = 0, front = 0, push = 0;
@@ -94,7 +97,7 @@ static __device__ __forceinline__ bool grid_gain_batch(const int32_t *__restrict
                                 const int32_t *__restrict__ c3 = nullptr, int voff = 0, int ws_n = -1,
                                 int phase = kBatchAll, ClaimRec *log = nullptr,
                                 unsigned long long *log_n = nullptr, unsigned long long log_cap = 0,
-                                GridCounts *acc = nullptr) {
+                                GridCounts *acc = nullptr, Team tm = whole_grid(), int gx_n = -1) {
   constexpr int T = kGridGainThreads;
   __shared__ u64 s_gain[kLanes];
   __shared__ unsigned int s_cnt[kLanes];
@@ -110,15 +113,16 @@ static __device__ __forceinline__ bool grid_gain_batch(const int32_t *__restrict
   (void)goff;
 
   const int tid = threadIdx.x, lane = tid & 31;
-  const int G = gridDim.x, b = blockIdx.x;
+  const int G = tm.G, b = tm.b;
   const int nl = nl_dev ? min(kLanes, *(volatile const int32_t *)nl_dev) : nl_arg;
   if (ws_n < 0) ws_n = n;
+  if (gx_n < 0) gx_n = ws_n;
   const GainWs ws = gain_ws(ws_base, 0, ws_n, 0);
   // frontier lists by level mod 3 and range starts by level parity (selected,
   // not indexed, so that nothing lands in local memory)
-  int32_t *const list2 = gx + 2 * (size_t)ws_n;
+  int32_t *const list2 = gx + 2 * (size_t)gx_n;
   auto list_of = [&](int r) -> int32_t * { return r == 0 ? ws.qv0 : (r == 1 ? ws.qv1 : list2); };
-  auto starts_of = [&](int p) -> int32_t * { return p ? gx + (size_t)ws_n : gx; };
+  auto starts_of = [&](int p) -> int32_t * { return p ? gx + (size_t)gx_n : gx; };
   auto words_of = [&](int r) -> LaneWords { return r == 0 ? ws.nx[0] : (r == 1 ? ws.nx[1] : ws.nx[2]); };
   u64 c_scalar = 0, c_union = 0, c_front = 0, c_push = 0;
   if (tid < kLanes) {
@@ -189,7 +193,7 @@ static __device__ __forceinline__ bool grid_gain_batch(const int32_t *__restrict
   if (phase == kBatchLevel0) return true;
   bool ok = true;
   if (phase == kBatchRest) cta_sync();  // s_gain and s_cnt are zero
-  else ok = grid_sync(bar, err, timeout_ns);
+  else ok = grid_sync(bar, err, timeout_ns, tm);
   // invalid candidate ids leave their lanes empty
   if (ok && MODE == kModeFarness) {
     if (tid < kLanes) {
@@ -396,7 +400,7 @@ static __device__ __forceinline__ bool grid_gain_batch(const int32_t *__restrict
       }
     }
     F_prev = F;
-    ok = grid_sync(bar, err, timeout_ns);
+    ok = grid_sync(bar, err, timeout_ns, tm);
     if (!ok) break;
     if (MODE == kModeFarness) {
       // the same BFScut test in every CTA: all vertices within L+1 are
@@ -466,7 +470,7 @@ static __device__ __forceinline__ bool grid_gain_batch(const int32_t *__restrict
       atomicAdd(&gctl->lanes, (u64)nl);
     }
   }
-  const bool ok2 = grid_sync(bar, err, timeout_ns);
+  const bool ok2 = grid_sync(bar, err, timeout_ns, tm);
   if (b == 0 && tid < nl) {
     const int c = cand[tid];
     long long r;
@@ -510,14 +514,14 @@ static __device__ __forceinline__ bool grid_relabel_bfs(
     const int32_t *seeds, int32_t n_seeds, int32_t *q0, int32_t *q1, unsigned long long *pk, int32_t *levels_out,
     unsigned long long *decrease, unsigned long long *relabelled, int32_t *st0, int32_t *st1,
     GridBar *bar, int32_t *err, unsigned long long timeout_ns, unsigned long long *work = nullptr,
-    const int32_t *__restrict__ c3 = nullptr) {
+    const int32_t *__restrict__ c3 = nullptr, Team tm = whole_grid()) {
   constexpr int kT = 1024;  // staging capacity (blockDim.x <= 1024)
   __shared__ unsigned long long sh_bfs[32];
   __shared__ int s_go[kT + 1];
   __shared__ int s_rs[kT];
   __shared__ int s_x0;
   const int tid = threadIdx.x, lane = tid & 31, T = blockDim.x;
-  const int G = gridDim.x, b = blockIdx.x;
+  const int G = tm.G, b = tm.b;
   unsigned long long dec = 0, rel = 0;
 
   // queue w for level lev: warp-aggregated slot and range start (whole warp)
@@ -562,7 +566,7 @@ static __device__ __forceinline__ bool grid_relabel_bfs(
     }
     enqueue(q, s, 0, q ? row_len(rp, c3, s, 0) : 0);
   }
-  bool ok = grid_sync(bar, err, timeout_ns);
+  bool ok = grid_sync(bar, err, timeout_ns, tm);
   for (int L = 0; ok; ++L) {
     const unsigned long long pkl = *(volatile unsigned long long *)&pk[L % 3];
     const int F = (int)(pkl >> 32);
@@ -625,7 +629,7 @@ static __device__ __forceinline__ bool grid_relabel_bfs(
         x += cntx;
       }
     }
-    ok = grid_sync(bar, err, timeout_ns);
+    ok = grid_sync(bar, err, timeout_ns, tm);
     if (ok && b == 0 && tid == 0 && levels_out) *levels_out = L + 1;
   }
   dec = block_sum(dec, sh_bfs);

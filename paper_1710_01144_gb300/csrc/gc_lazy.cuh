@@ -687,7 +687,7 @@ static __device__ bool grid_lazy_step(const int32_t *act, int32_t m, long long *
                                       long long *akey, int32_t *ast, LazyCtl *lc, GridGainCtl *gg, bool fold,
                                       int32_t *sel, int32_t *selpos, const long long *gsel, int cap,
                                       GridSelScratch *sc, GridBar *bar, int32_t *err, unsigned long long tns,
-                                      int *dec_out) {
+                                      int *dec_out, Team tm = whole_grid()) {
   __shared__ long long s_v[32];
   __shared__ int s_id[32];
   __shared__ long long s_ll[32];
@@ -695,7 +695,7 @@ static __device__ bool grid_lazy_step(const int32_t *act, int32_t m, long long *
   __shared__ int s_scan[33];
   __shared__ int s_b, s_lane;
   __shared__ long long s_ab;
-  const int tid = threadIdx.x, T = blockDim.x, G = gridDim.x, b = blockIdx.x;
+  const int tid = threadIdx.x, T = blockDim.x, G = tm.G, b = tm.b;
   const int r = *(volatile int32_t *)&lc->round;
   const int P = (m + G - 1) / G;
   const int lo = min(m, b * P), hi = min(m, lo + P);
@@ -786,7 +786,7 @@ static __device__ bool grid_lazy_step(const int32_t *act, int32_t m, long long *
     sc->umin[b] = umin;
     sc->cnt[b] = cnt;
   }
-  if (!grid_sync(bar, err, tns)) return false;
+  if (!grid_sync(bar, err, tns, tm)) return false;
   // ---- 3. decision (every CTA the same) ----
   umax = LLONG_MIN;
   vmax = -1;
@@ -841,7 +841,7 @@ static __device__ bool grid_lazy_step(const int32_t *act, int32_t m, long long *
       cta_sync();
       for (int i = tid; i < kSelBins; i += T)
         if (s_hist[i]) atomicAdd(&gh[i], s_hist[i]);
-      if (!grid_sync(bar, err, tns)) return false;
+      if (!grid_sync(bar, err, tns, tm)) return false;
       last_hist = hb;
       // walk down from the top bin: thread t owns bins 1023-2t and 1022-2t
       const int b0 = kSelBins - 1 - 2 * tid, b1 = b0 - 1;
@@ -893,7 +893,7 @@ static __device__ bool grid_lazy_step(const int32_t *act, int32_t m, long long *
     sc->gt[b] = n_gt;
     sc->eq[b] = n_eq;
   }
-  if (!grid_sync(bar, err, tns)) return false;
+  if (!grid_sync(bar, err, tns, tm)) return false;
   if (b == 0 && last_hist >= 0)  // every histogram has been read: all three zero for the next step
     for (int i = tid; i < 3 * kSelBins; i += T) (&sc->hist[0][0])[i] = 0;
   long long gt_off = 0, eq_off = 0, gt_tot = 0;
