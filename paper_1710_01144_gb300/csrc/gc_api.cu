@@ -33,6 +33,15 @@ static int fail(int code, const std::string &msg) {
 constexpr int32_t kRound0GridMax = 256;  // round-0 survivors handled by grid-wide batches
 constexpr int kRound0Pivots = 8;         // round 0: at most this many pivot bounds
 constexpr int32_t kShallowLevels = 32;   // round 0: wide bottom-up batches up to this BFS depth
+// gc_greedy, lists that cannot certify a pick: from this many candidates whose
+// bounds reach the best gain (64 grid-wide steps) a sweep in CTA batches runs.
+// On a sparse R-MAT graph (89,928 vertices, average degree 9, k = 28) round 3
+// must evaluate nearly every candidate: 1,420 steps, 64.5 ms; with the sweep 80
+// steps and 5.7 ms for the whole call.
+constexpr int32_t kSweepMin = 1024;
+// list rebuilds at one length before it grows (R-MAT scale 21, edge factor 3, k = 50:
+// 13.3 ms growing at once, 9.4 ms so; scale 24: 65.1 ms either way)
+constexpr int kSameLenRebuilds = 6;
 constexpr int32_t kR1Propose = 1024;     // round 1: candidates the proposal chooses the first batch from
 
 #define GC_TRY(expr)              \
@@ -1028,10 +1037,39 @@ int gc_greedy(gc_graph *g, int32_t k, const gc_opts *opts_in, int32_t *out_group
       // cost), at least two wide steps for wide ones
       int32_t target = opts.active_target > 0 ? opts.active_target
                                               : (step_form == 2 ? std::max<int32_t>(4096, 2 * g->wcap) : 2048);
+      int same_len = 0;
       for (;;) {
         // two-hop bounds for the current group, before every (re)launch: the
         // candidates round 1 skipped would otherwise keep their round-1 bounds
         if (round1_bound) GC_TRY(launch_bound_refresh(g));
+        bool swept = false;
+        if (lazy_launches > 0 && step_form == 1 && g->h_lctl->best_id >= 0) {
+          // The list could not certify a pick.  If many candidates' bounds
+          // still reach the round's best exact gain, evaluate them all now,
+          // one 64-lane batch per CTA (as in round 1), instead of 64 per
+          // grid-wide step: after that no unevaluated bound reaches the best
+          GC_TRY(launch_round_begin(g));
+          GC_TRY(launch_select(g, kSelLazy, g->h_lctl->round, 0, kTauHost, g->h_lctl->best_gain));
+          GC_TRY(read_ctl(g));
+          if (g->h_sctl->n_sel > kSweepMin) {
+            GC_TRY(gains_timed(kModeGain, g->list, 0, &g->sctl->n_sel, kLanes));
+            GC_TRY(launch_after_eval(g, g->h_lctl->round, 0));
+            GC_TRY(read_ctl(g));
+            GC_TRY(device_errors(g));
+            // the sweep keeps no claim log: its best, if it leads the round, goes
+            // through one more step, whose log then gives the d_S update
+            const long long sg = g->h_sctl->best_gain;
+            const int32_t sv = g->h_sctl->best_id;
+            if (sv >= 0 && (sg > g->h_lctl->best_gain || (sg == g->h_lctl->best_gain && sv < g->h_lctl->best_id)))
+              GC_TRY(launch_fill_i32(g, g->stamp + sv, 0, 1));
+            swept = true;
+          }
+        }
+        // a longer list next time, unless the round was swept or few bounds
+        // reach its best: lists up to kCta0SelectMax are selected from by one CTA
+        // without grid barriers, so the same length again is cheaper at first
+        if (lazy_launches > 0 && !swept && (step_form != 1 || ++same_len > kSameLenRebuilds))
+          target = target > (1 << 28) ? g->n : target * 4;
         GC_TRY(launch_select(g, kSelActive, 0, target, kTauHistogramTheta, 0));
         cudaEvent_t le0 = nullptr, le1 = nullptr;
         GC_TRY(gain_event(g, ev_used, &le0));
@@ -1053,7 +1091,6 @@ int gc_greedy(gc_graph *g, int32_t k, const gc_opts *opts_in, int32_t *out_group
         }
         if (g->h_lctl->round >= k) break;
         if (g->h_lctl->dec != 2) return fail(GC_EINTERNAL, "persistent lazy kernel stopped early");
-        target = target > (1 << 28) ? g->n : target * 4;
       }
       lazy1 = *g->h_gctl;
       lazy_steps = g->h_lctl->steps;
