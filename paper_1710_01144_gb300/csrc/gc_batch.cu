@@ -13,8 +13,11 @@
 //   P0  lower bounds LB(v) and, per graph, the vertex v_a of smallest bound
 //   P1  BFS from all v_a; per-graph farness f_a
 //   P2  every v with LB(v) <= f_a evaluated by the 64-lane BFS in farness
-//       mode with per-graph cuts (graph-aligned batches from a dynamic task
-//       counter over all CTAs); per graph s0 = argmin (f, id)
+//       mode with per-graph cuts (graph-aligned batches, by teams of CTAs on
+//       graphs with few survivors), after the far counts have raised the
+//       bounds; per graph s0 = argmin (f, id).  Measured with round 1's
+//       batches by teams too: rounds 0 and 1 of 24 mixed graphs 45 + 32 -> 17
+//       + 12 ms, of 256 graphs 623 + 190 -> 493 + 167 ms
 //   P3  BFS from all s0 (d_S), per-graph farness, neighbour bound mx
 //   P4  round 1: every candidate of every graph, graph-aligned 64-lane batches
 //       from a dynamic task counter; per-graph argmax; picks; BFS from picks
@@ -25,7 +28,7 @@
 //       so no graph waits for another.  A team's steps are those of the
 //       single-graph persistent kernel.  One CTA per graph, as before, left
 //       most of the GPU idle behind the slowest graph: 24 mixed graphs 717 ms
-//       (lazy rounds 634), with teams 207 ms (124); 256 graphs 1468 -> 1109 ms.
+//       (lazy rounds 634), with teams and sweeps 102 ms; 256 graphs 1468 -> 976 ms.
 //   P7  check: one BFS from every graph's whole group; each graph's farness
 //       must equal f(s0) minus the sum of its accepted gains.
 #include <limits.h>
@@ -74,6 +77,7 @@ struct TeamCtl {
   int32_t g;
   int32_t sweep_n, sweep_next;  // sweep: candidates listed, next one to take
   int32_t pad;
+  long long best;                 // round 0: the cut threshold of the current task
   unsigned long long sweep_best;  // its best exact gain: gain << 32 | ~(id in the graph)
   GridGainCtl gg;
 };
@@ -124,6 +128,7 @@ struct BatchArgs {
   int32_t *wsel;
   long long *wgain;
   int32_t *depth;     // BFS levels of the deepest round-1 batch, per graph
+  unsigned long long *cls;  // [2 count]: members of the two degree classes of each graph (far counts)
   const int32_t *order;  // graphs of the team phase, longest first; order_n of them
   int32_t order_n;
   int32_t team_size;
@@ -437,6 +442,227 @@ static __device__ void seg_sum_excess3(const BatchArgs &a, const int32_t *d, lon
   }
 }
 
+// Graphs with at most this many listed vertices run their tasks by teams.
+constexpr int kTeamListMax = 4 * kLanes;
+
+// tstart[g] = tasks (64 listed vertices each) of the graphs before g, of the
+// graphs with short lists or of the others; the task counter starts again.
+// One thread.
+static __device__ void task_prefix(const BatchArgs &a, bool short_lists) {
+  int acc = 0;
+  for (int g = 0; g < a.count; ++g) {
+    a.tstart[g] = acc;
+    const int m = a.scount[g];
+    if ((m <= kTeamListMax) == short_lists) acc += (m + kLanes - 1) / kLanes;
+  }
+  a.tstart[a.count] = acc;
+  a.ctl->task = 0;
+}
+
+// the graph with tstart[g] <= task < tstart[g + 1]
+static __device__ int task_graph(const BatchArgs &a, int task) {
+  int lo = 0, hi = a.count - 1;
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (a.tstart[mid] <= task) lo = mid;
+    else hi = mid - 1;
+  }
+  return lo;
+}
+
+// CTAs of a team for n_tasks tasks of short lists on G CTAs.  Such lists are
+// the vertices whose searches reach everything (round-0 survivors of a graph
+// with few, the 64 largest bounds of round 1): one CTA takes 38 ms for a 64-lane
+// batch on the largest graph of a mix (10.7M entries), the grid 1 ms, so few
+// tasks leave most of the GPU idle behind the longest one.  Up to four tasks
+// per CTA go to teams.  Long lists (graphs whose every vertex survives the
+// bounds; searches that are cut early) keep one CTA per batch.
+static __device__ __forceinline__ int task_team(int n_tasks, int G) {
+  return max(1, min(G, 4 * G / max(1, n_tasks)));
+}
+
+// One 64-lane batch of graph g by a team (its own control block, its first
+// CTA's workspace, the queues of its second CTA's workspace as scratch).
+// Results in s_out of the team's CTA 0.  Not inlined: the CTA-local phases keep
+// their registers.
+template <int MODE>
+static __device__ __noinline__ bool team_batch(const BatchArgs &a, int g, const int32_t *cand, int nl, TeamCtl *tc,
+                                               Team tm, long long *s_out) {
+  const int first = blockIdx.x - tm.b, o = a.off[g];
+  unsigned char *ws0 = a.ws + a.ws_stride * (size_t)first;
+  int32_t *gx = gain_ws(a.ws, a.ws_stride, a.max_n, first + 1).qv0;
+  const int gx_n = (int)(ws_align((size_t)a.max_n * sizeof(int32_t)) / sizeof(int32_t));
+  const bool gain = MODE == kModeGain;
+  return grid_gain_batch<MODE>(gain ? a.rpf : a.rp, gain ? a.cif : a.ci, a.N, gain ? a.dS1 : a.dS, cand, nl, nullptr,
+                               s_out, ws0, gx, a.goff, &tc->gg, a.gctl, &tc->bar, &a.ctl->err, a.tns,
+                               gain ? a.mx : nullptr, gain ? a.c3 : nullptr, o, a.max_n, kBatchAll, nullptr, nullptr,
+                               0, nullptr, tm, gx_n, gain ? nullptr : &tc->best, a.ng[g]);
+}
+
+// The tasks of the lists in slist (scount entries per graph) that tstart counts,
+// by teams of S CTAs:
+// kModeFarness  f0[v] <- f({v}) or -1, cut by the graph's best (round 0);
+// kModeGain     ub[v] <- Delta(v | {s0}), stamp[v] <- 1, bestf[g] <- the best gain.
+// Ends without a grid barrier.
+template <int MODE>
+static __device__ bool run_tasks(const BatchArgs &a, const GainWs &myws, GainCounters &cnt, long long *s_out,
+                                 const int S) {
+  __shared__ int s_task;
+  __shared__ long long s_ll[32];
+  const int tid = threadIdx.x;
+  const int n_tasks = a.tstart[a.count];
+  const int t = blockIdx.x / S;
+  const Team tm{(int)blockIdx.x - t * S, S};
+  if ((t + 1) * S > (int)gridDim.x) return true;  // a remainder of fewer than S CTAs
+  TeamCtl *tc = &a.teams[1 + t];
+  const LaneGraphs lg = MODE == kModeFarness ? LaneGraphs{a.gid, a.ng, a.bestf} : LaneGraphs();
+  for (;;) {
+    if (S == 1) {
+      if (tid == 0) s_task = atomicAdd(&a.ctl->task, 1);
+      cta_sync();
+    } else {
+      if (tm.b == 0) {  // the next task and a fresh control block for its batch
+        unsigned int *w = reinterpret_cast<unsigned int *>(&tc->gg);
+        for (int i = tid; i < (int)(sizeof(GridGainCtl) / 4); i += blockDim.x) w[i] = 0;
+        if (tid == 0) {
+          const int next = atomicAdd(&a.ctl->task, 1);
+          tc->g = next;
+          // one threshold for the whole team: other teams may lower the graph's
+          // best while this batch runs, and every CTA must cut the same lanes
+          if (MODE == kModeFarness && next < n_tasks)
+            tc->best = *(volatile long long *)&a.bestf[task_graph(a, next)];
+        }
+      }
+      if (!grid_sync(&tc->bar, &a.ctl->err, a.tns, tm)) return false;
+      if (tid == 0) s_task = *(volatile int32_t *)&tc->g;
+      cta_sync();
+    }
+    const int task = s_task;
+    cta_sync();
+    if (task >= n_tasks) return true;
+    const int g = task_graph(a, task), o = a.off[g], first = (task - a.tstart[g]) * kLanes;
+    const int nl = min(kLanes, a.scount[g] - first);
+    const int32_t *cand = a.slist + o + first;
+    int levels = 0;
+    if (S > 1) {
+      if (!team_batch<MODE>(a, g, cand, nl, tc, tm, s_out)) return false;
+      if (tm.b != 0) continue;
+      cta_sync();  // s_out
+      if (tid == 0) levels = tc->gg.levels;
+    } else if (MODE == kModeFarness) {
+      cta_gain_batch<MODE, true, false>(a.rp, a.ci, a.N, a.dS, cand, nl, s_out, myws, a.gctl, nullptr, lg, cnt, o);
+    } else {
+      const unsigned long long lev0 = cnt.levels;
+      cta_gain_batch<MODE, true, true>(a.rpf, a.cif, a.N, a.dS1, cand, nl, s_out, myws, a.gctl, a.mx, lg, cnt, o,
+                                       a.c3);
+      levels = (int)(cnt.levels - lev0);
+    }
+    if (MODE == kModeFarness) {
+      if (tid < nl) {
+        a.f0[cand[tid]] = s_out[tid];
+        if (S > 1 && s_out[tid] >= 0) atomicMin(&a.bestf[g], s_out[tid]);
+      }
+    } else {
+      if (tid < nl) {
+        a.ub[cand[tid]] = s_out[tid];
+        a.stamp[cand[tid]] = 1;
+      }
+      const long long best = block_max_ll(tid < nl ? s_out[tid] : -1ll, s_ll);
+      if (tid == 0) {
+        atomicMax(&a.bestf[g], best);
+        atomicMax(&a.depth[g], levels);
+      }
+    }
+    cta_sync();
+  }
+}
+
+// Every task of the lists: short lists by teams, then long ones by CTAs.  Called
+// after a grid barrier (the lists are complete), ends with one.
+template <int MODE>
+static __device__ bool batch_tasks(const BatchArgs &a, const GainWs &myws, GainCounters &cnt, long long *s_out) {
+  for (int pass = 0; pass < 2; ++pass) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) task_prefix(a, pass == 0);
+    if (!bsync(a)) return false;
+    const int n_tasks = a.tstart[a.count];
+    if (n_tasks && !run_tasks<MODE>(a, myws, cnt, s_out, pass == 0 ? task_team(n_tasks, gridDim.x) : 1)) return false;
+    if (!bsync(a)) return false;
+  }
+  return true;
+}
+
+// Round 0: the far counts of the single-graph path (k_far_counts, k_far_bound in
+// gc_bfs.cu) over the union: per vertex the neighbours of degree 1 to kFarDeg in
+// two classes (packed in ub, zero so far), per graph the members of each class,
+// then a tighter key for every survivor.  One thread per counted row, a warp
+// per survivor's row.
+static __device__ bool batch_far_bounds(const BatchArgs &a) {
+  const int tid = threadIdx.x, lane = tid & 31, T = blockDim.x, G = gridDim.x;
+  unsigned long long *cnt = reinterpret_cast<unsigned long long *>(a.ub);
+  for (int base = (blockIdx.x * T + tid) & ~31; base < a.N; base += G * T) {
+    const int u = base + lane;
+    int g = -1, beg = 0, end = 0;
+    if (u < a.N) {
+      g = a.gid[u];
+      beg = a.rp[u];
+      end = a.rp[u + 1];
+    }
+    const unsigned long long c = far_class(end - beg);
+    if (c)
+      for (int e = beg; e < end; ++e) atomicAdd(&cnt[a.ci[e]], c);
+    const int g0 = __shfl_sync(0xffffffffu, g, 0);
+    if (__all_sync(0xffffffffu, g == g0 || g < 0)) {
+      const unsigned lo = __ballot_sync(0xffffffffu, c == 1ull), hi = __ballot_sync(0xffffffffu, c > 1ull);
+      if (lane == 0 && lo) atomicAdd(&a.cls[2 * g0], (unsigned long long)__popc(lo));
+      if (lane == 0 && hi) atomicAdd(&a.cls[2 * g0 + 1], (unsigned long long)__popc(hi));
+    } else if (c) {
+      atomicAdd(&a.cls[2 * g + (c == 1ull ? 0 : 1)], 1ull);
+    }
+  }
+  if (!bsync(a)) return false;
+  for (int base = (blockIdx.x * T + tid) & ~31; base < a.N; base += G * T) {
+    const int v = base + lane;
+    int g = -1, deg = 0, beg = 0;
+    long long k = LLONG_MIN, fa = 0;
+    if (v < a.N) {
+      g = a.gid[v];
+      fa = a.fa[g];
+      k = a.key[v];
+      beg = a.rp[v];
+      deg = a.rp[v + 1] - beg;
+    }
+    unsigned todo = __ballot_sync(0xffffffffu, v < a.N && -k <= fa);
+    long long near0 = 0, near1 = 0;
+    for (unsigned m = todo; m; m &= m - 1) {
+      const int q = __ffs(m) - 1;
+      const int rb = __shfl_sync(0xffffffffu, beg, q), rd = __shfl_sync(0xffffffffu, deg, q);
+      long long x0 = 0, x1 = 0;
+#pragma unroll 4
+      for (int e = rb + lane; e < rb + rd; e += 32) {
+        const unsigned long long x = cnt[a.ci[e]];
+        x0 += (long long)(x & 0xffffffffull);
+        x1 += (long long)(x >> 32);
+      }
+      x0 = warp_sum(x0);
+      x1 = warp_sum(x1);
+      if (lane == q) {
+        near0 = x0;
+        near1 = x1;
+      }
+    }
+    if ((todo >> lane) & 1u) {
+      const unsigned long long c = far_class(deg), own = cnt[v];
+      const long long rest = max(0ll, (long long)a.ng[g] - 1 - deg);
+      const long long f0 = (long long)a.cls[2 * g] - (c == 1ull) - near0 - (long long)(own & 0xffffffffull);
+      const long long f1 = (long long)a.cls[2 * g + 1] - (c > 1ull) - near1 - (long long)(own >> 32);
+      const long long far = min(rest, max(0ll, f0) + max(0ll, f1));
+      const long long c2 = min((long long)deg + 3 * rest + k, rest - far);  // the degree bound's c2 from its key
+      a.key[v] = -((long long)deg + 2 * c2 + 3 * (rest - c2));
+    }
+  }
+  return bsync(a);
+}
+
 // Round 1 with two-hop bounds (the single-graph path's round 1, per graph):
 // every candidate gets the bound for S = {s0}; the 64 largest bounds of each
 // graph are evaluated as one CTA batch, then every candidate whose bound
@@ -466,32 +692,14 @@ static __device__ bool batch_round1_bounded(const BatchArgs &a, const GainWs &my
   // the first batch of each graph: its 64 largest bounds
   for (int g = b; g < a.count; g += G) {
     const int m = a.kk[g] >= 2 ? cta_top_bounds(a.ub, a.off[g], a.ng[g], kLanes, a.slist + a.off[g]) : 0;
-    if (tid == 0) a.scount[g] = m;
-    cta_sync();
-  }
-  if (!bsync(a)) return false;
-  for (;;) {
-    if (tid == 0) s_task = atomicAdd(&a.ctl->task, 1);
-    cta_sync();
-    const int g = s_task;
-    cta_sync();
-    if (g >= a.count) break;
-    const int m = a.scount[g], o = a.off[g];
-    if (m == 0) continue;
-    const unsigned long long lev0 = cnt.levels;
-    cta_gain_batch<kModeGain, true, true>(a.rpf, a.cif, a.N, a.dS1, a.slist + o, m, s_out, myws, a.gctl, a.mx,
-                                          LaneGraphs(), cnt, o, a.c3);
-    if (tid == 0) a.depth[g] = (int)(cnt.levels - lev0);
-    if (tid < m) {
-      const int v = a.slist[o + tid];
-      a.ub[v] = s_out[tid];
-      a.stamp[v] = 1;
+    if (tid == 0) {
+      a.scount[g] = m;
+      a.bestf[g] = -1;  // the best exact gain of round 1 so far
     }
-    const long long best = block_max_ll(tid < m ? s_out[tid] : -1ll, s_ll);
-    if (tid == 0) a.bestf[g] = best;
     cta_sync();
   }
   if (!bsync(a)) return false;
+  if (!batch_tasks<kModeGain>(a, myws, cnt, s_out)) return false;
   // every other candidate whose bound reaches the first batch's best
   for (int g = b; g < a.count; g += G) {
     const int o = a.off[g], n = a.ng[g];
@@ -515,41 +723,7 @@ static __device__ bool batch_round1_bounded(const BatchArgs &a, const GainWs &my
     cta_sync();
   }
   if (!bsync(a)) return false;
-  if (b == 0 && tid == 0) {
-    int acc = 0;
-    for (int g = 0; g < a.count; ++g) {
-      a.tstart[g] = acc;
-      acc += (a.scount[g] + kLanes - 1) / kLanes;
-    }
-    a.tstart[a.count] = acc;
-    a.ctl->task = 0;
-  }
-  if (!bsync(a)) return false;
-  const int n_tasks = a.tstart[a.count];
-  for (;;) {
-    if (tid == 0) s_task = atomicAdd(&a.ctl->task, 1);
-    cta_sync();
-    const int t = s_task;
-    cta_sync();
-    if (t >= n_tasks) break;
-    int lo = 0, hi = a.count - 1;  // graph with tstart[g] <= t < tstart[g+1] (non-empty)
-    while (lo < hi) {
-      const int mid = (lo + hi + 1) >> 1;
-      if (a.tstart[mid] <= t) lo = mid;
-      else hi = mid - 1;
-    }
-    const int g = lo, o = a.off[g], first = (t - a.tstart[g]) * kLanes;
-    const int nl = min(kLanes, a.scount[g] - first);
-    cta_gain_batch<kModeGain, true, true>(a.rpf, a.cif, a.N, a.dS1, a.slist + o + first, nl, s_out, myws, a.gctl,
-                                          a.mx, LaneGraphs(), cnt, o, a.c3);
-    if (tid < nl) {
-      const int v = a.slist[o + first + tid];
-      a.ub[v] = s_out[tid];
-      a.stamp[v] = 1;
-    }
-    cta_sync();
-  }
-  return bsync(a);
+  return batch_tasks<kModeGain>(a, myws, cnt, s_out);
 }
 
 // Bound refresh before the lazy rounds: the two-hop bound for the group after
@@ -924,7 +1098,7 @@ __global__ void __launch_bounds__(kBatchThreads, 2) k_batch_solve(const BatchArg
         a.f0[v] = -1;
         a.dS[v] = kInf;
         a.stamp[v] = 0;
-        a.ub[v] = LLONG_MAX;
+        a.ub[v] = 0;  // the far counts of P2 (bounds and gains come in round 1)
         atomicMin(&a.packed[g], ((unsigned long long)lb << 32) | (unsigned long long)(v - a.off[g]));
       }
     }
@@ -942,6 +1116,7 @@ __global__ void __launch_bounds__(kBatchThreads, 2) k_batch_solve(const BatchArg
   if (b == 0 && tid == 0) a.ctl->pk[0] = a.ctl->pk[1] = a.ctl->pk[2] = 0;
   if (!bsync(a)) return;
   // ---- P2: round-0 survivors (every v with LB(v) <= f_a) ----
+  if (!batch_far_bounds(a)) return;
   // P2a, one CTA per graph: compact the graph's survivors into its own region
   // of slist (graph-aligned, so batches never mix graphs)
   for (int g = b; g < a.count; g += G) {
@@ -971,42 +1146,8 @@ __global__ void __launch_bounds__(kBatchThreads, 2) k_batch_solve(const BatchArg
     cta_sync();
   }
   if (!bsync(a)) return;
-  // P2b: task prefix over graphs (64 survivors per task)
-  if (b == 0 && tid == 0) {
-    int acc = 0;
-    for (int g = 0; g < a.count; ++g) {
-      a.tstart[g] = acc;
-      acc += (a.scount[g] + kLanes - 1) / kLanes;
-    }
-    a.tstart[a.count] = acc;
-    a.ctl->task = 0;
-  }
-  if (!bsync(a)) return;
-  // P2c: every CTA takes survivor batches from a dynamic counter
-  {
-    const int n_tasks = a.tstart[a.count];
-    const LaneGraphs lg{a.gid, a.ng, a.bestf};
-    for (;;) {
-      if (tid == 0) s_task = atomicAdd(&a.ctl->task, 1);
-      cta_sync();
-      const int t = s_task;
-      cta_sync();
-      if (t >= n_tasks) break;
-      int lo = 0, hi = a.count - 1;  // graph with tstart[g] <= t < tstart[g+1] (non-empty)
-      while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (a.tstart[mid] <= t) lo = mid;
-        else hi = mid - 1;
-      }
-      const int g = lo, o = a.off[g], first = (t - a.tstart[g]) * kLanes;
-      const int nl = min(kLanes, a.scount[g] - first);
-      cta_gain_batch<kModeFarness, true, false>(a.rp, a.ci, a.N, a.dS, a.slist + o + first, nl, s_out, myws, a.gctl, nullptr,
-                                   lg, cnt, o);
-      if (tid < nl) a.f0[a.slist[o + first + tid]] = s_out[tid];
-      cta_sync();
-    }
-  }
-  if (!bsync(a)) return;
+  // P2b: 64 survivors per task, by teams or CTAs
+  if (!batch_tasks<kModeFarness>(a, myws, cnt, s_out)) return;
   // P2d, one CTA per graph: s0 = argmin (f, id) over the exact farness values
   for (int g = b; g < a.count; g += G) {
     const int s0 = cta_argmin_f0(a, g);
@@ -1306,7 +1447,7 @@ struct gc_batch {
           *st1 = nullptr;
   int32_t *rpf = nullptr, *cif = nullptr, *c3 = nullptr, *gx = nullptr, *dS1 = nullptr;
   GridSelScratch *gsel = nullptr;
-  TeamCtl *teams = nullptr;     // [1 + lazy_ctas]: the whole grid's, then the teams'
+  TeamCtl *teams = nullptr;     // [1 + ctas]: the whole grid's, then the teams'
   ClaimRec *clog = nullptr;
   int32_t *wsel = nullptr, *depth = nullptr, *order = nullptr;
   long long *wgain = nullptr;
@@ -1316,6 +1457,7 @@ struct gc_batch {
   unsigned char *ws = nullptr;
   size_t ws_stride = 0;
   unsigned long long *packed = nullptr;
+  unsigned long long *cls = nullptr;
   long long *fa = nullptr, *farness = nullptr, *bestf = nullptr, *g3 = nullptr;
   LazyCtl *lc = nullptr;
   int32_t *act = nullptr, *act_n = nullptr, *kk = nullptr, *bstart = nullptr;
@@ -1351,7 +1493,7 @@ static void batch_release(gc_batch *b) {
                  b->ub, b->key, b->f0, b->ws, b->packed, b->fa, b->farness, b->bestf, b->lc, b->act, b->act_n,
                  b->kk, b->bstart, b->picks, b->pgain, b->seeds, b->ctl, b->gctl, b->slist,
                  b->scount, b->tstart, b->rpf, b->cif, b->c3, b->gx, b->teams, b->gsel, b->dS1, b->g3, b->clog, b->wsel, b->wgain, b->depth,
-                 b->order};
+                 b->order, b->cls};
   for (void *p : dev)
     if (p) cudaFree(p);
   if (b->h_ctl) cudaFreeHost(b->h_ctl);
@@ -1378,13 +1520,15 @@ static bool balloc(T **p, size_t count) {
 // The lazy rounds' plan: sorts the graphs by estimated time (longest first)
 // and returns the CTAs of a team: the power of two with the shortest list
 // schedule.  `ctas` > 0 asks for that size.  The estimate of a round in
-// microseconds is fitted to team sizes 1 to 76 on 24 graphs of 10^4 to 3 x 10^4
-// and of 10^4 to 5 x 10^5 vertices: a step's barriers, selection and dependent
-// loads do not shrink with the team, its edges and the bound refreshes do.
+// microseconds is fitted to team sizes 1 to 76: a step's barriers, selection and
+// dependent loads do not shrink with the team, its edges and the bound refreshes
+// do.  Lazy rounds in ms at 1, 4, 8, 16, 38 CTAs: 24 graphs of 10^4 to 5 x 10^5
+// vertices 173, 48, 26, 14, 18; 24 of 10^4 to 3 x 10^4: 13.8, 4.8, 3.3, 4.8,
+// 7.6; 256 of 10^4 to 5 x 10^5 (1, 4, 8, 16): 408, 150, 121, 125.
 static int plan_teams(const gc_batch *b, const int32_t *ks, std::vector<int32_t> &order, int32_t ctas) {
   auto est = [&](int32_t g, int s) {
     const double e = (double)b->h_nnz[g];
-    return (double)(ks[g] - 2) * (45.0 + (0.22 * std::sqrt(e) + 1.1e-4 * e) / s);
+    return (double)(ks[g] - 2) * (60.0 + (0.1 * std::sqrt(e) + 6e-4 * e) / s);
   };
   std::sort(order.begin(), order.end(), [&](int32_t x, int32_t y) {
     const double a = est(x, 1), c = est(y, 1);
@@ -1486,10 +1630,10 @@ static int batch_load_impl(int32_t count, const int32_t *const *row_ptrs, const 
             balloc(&b->slist, Nn) && balloc(&b->scount, (size_t)count) && balloc(&b->tstart, (size_t)count + 1) &&
             balloc(&b->rpf, Nn + 1) && balloc(&b->cif, std::max<size_t>(1, (size_t)E)) && balloc(&b->c3, Nn) &&
             balloc(&b->dS1, Nn) && balloc(&b->g3, 2 * (size_t)count) &&
-            balloc(&b->gx, 3 * Nn) && balloc(&b->clog, 2 * Nn) && balloc(&b->teams, (size_t)b->lazy_ctas + 1) &&
+            balloc(&b->gx, 3 * Nn) && balloc(&b->clog, 2 * Nn) && balloc(&b->teams, (size_t)b->ctas + 1) &&
             balloc(&b->gsel, (size_t)b->lazy_ctas + 1) && balloc(&b->wsel, (size_t)b->lazy_ctas * kLanes) &&
             balloc(&b->wgain, (size_t)b->lazy_ctas * kLanes) && balloc(&b->depth, (size_t)count) &&
-            balloc(&b->order, (size_t)count) &&
+            balloc(&b->order, (size_t)count) && balloc(&b->cls, 2 * (size_t)count) &&
             balloc(&b->gctl, 1) && cudaMallocHost((void **)&b->h_ctl, sizeof(BatchCtl)) == cudaSuccess &&
             cudaMallocHost((void **)&b->h_gctl, sizeof(GainCtl)) == cudaSuccess;
   int64_t *d_eoff = nullptr;
@@ -1663,6 +1807,7 @@ int gc_batch_greedy(gc_batch *b, const int32_t *ks, const gc_opts *opts_in, int3
   a.wgain = b->wgain;
   a.depth = b->depth;
   a.order = b->order;
+  a.cls = b->cls;
   a.bounded = (opts.flags & GC_OPT_NO_ROUND1_BOUND) ? 0 : 1;
   a.g3 = b->g3;
   a.grid_min_n = opts.batch_grid_min_n == 0 ? kBatchGridMinN
@@ -1716,9 +1861,10 @@ int gc_batch_greedy(gc_batch *b, const int32_t *ks, const gc_opts *opts_in, int3
     if ((e = cudaMemcpyAsync(b->order, b->h_order_pinned, (size_t)b->count * sizeof(int32_t), cudaMemcpyHostToDevice,
                              st)))
       return e;
-    const size_t teams = 1 + (size_t)(b->lazy_ctas / a.team_size);
-    if ((e = cudaMemsetAsync(b->teams, 0, teams * sizeof(TeamCtl), st))) return e;
-    if ((e = cudaMemsetAsync(b->gsel, 0, teams * sizeof(GridSelScratch), st))) return e;
+    if ((e = cudaMemsetAsync(b->teams, 0, (1 + (size_t)b->ctas) * sizeof(TeamCtl), st))) return e;
+    if ((e = cudaMemsetAsync(b->gsel, 0, (1 + (size_t)(b->lazy_ctas / a.team_size)) * sizeof(GridSelScratch), st)))
+      return e;
+    if ((e = cudaMemsetAsync(b->cls, 0, 2 * (size_t)b->count * sizeof(unsigned long long), st))) return e;
     if ((e = cudaMemsetAsync(b->depth, 0, (size_t)b->count * sizeof(int32_t), st))) return e;
     void *args[] = {(void *)&a};
     if ((e = cudaLaunchCooperativeKernel((const void *)k_batch_solve, dim3(b->ctas), dim3(kBatchThreads), args, 0,

@@ -168,12 +168,6 @@ __global__ void __launch_bounds__(1024) k_round0_keys_heavy(const int32_t *__res
 // top-100 closeness at scale 18: 17.4 -> 3.60 ms (12,848 survivors -> 57); one
 // survivor batch at scale 20: 9.88 -> 9.84 ms, so the counts run whenever any
 // vertex survives on a shallow graph.
-constexpr int kFarDeg = 8;
-
-__device__ __forceinline__ unsigned long long far_class(int deg) {  // the class's unit in a packed pair of counts
-  return deg < 1 || deg > kFarDeg ? 0ull : (deg <= 2 ? 1ull : 1ull << 32);
-}
-
 // cnt[w] += the classes of w's neighbours of degree 1 .. kFarDeg (low half
 // {1, 2}, high half the rest), one thread per such neighbour's row;
 // total[0..1] = members per class.  cnt and total start at zero.

@@ -146,6 +146,13 @@ __device__ __forceinline__ int block_excl_scan(int v, int *sh, int *total) {
   return r;
 }
 
+// Degree classes of the round-0 far counts (k_far_counts in gc_bfs.cu).
+constexpr int kFarDeg = 8;
+
+__device__ __forceinline__ unsigned long long far_class(int deg) {  // the class's unit in a packed pair of counts
+  return deg < 1 || deg > kFarDeg ? 0ull : (deg <= 2 ? 1ull : 1ull << 32);
+}
+
 // (value, id) pairs ordered by larger value, then smaller id.
 __device__ __forceinline__ bool better_max(long long v, int id, long long bv, int bid) {
   return v > bv || (v == bv && (unsigned)id < (unsigned)bid);

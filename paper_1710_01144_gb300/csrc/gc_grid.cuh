@@ -83,7 +83,10 @@ static __device__ __forceinline__ int warp_find_start(const int32_t *start, int 
 // over the CTA and into gctl (a persistent caller sums them once at its end).
 // With `tm`, the CTAs of one team run the batch (bar, ctl, ws_base and gx are
 // the team's own); gx_n, if given, is the stride of gx's three parts (at least
-// the vertices of the graph, where ws_n is the workspace's layout).
+// the vertices of the graph, where ws_n is the workspace's layout).  Farness
+// mode over one graph of a union: n_graph is its vertex count and *best_of the
+// cut threshold, which must not change during the batch (every CTA compares
+// with it by itself, and they must agree).
 constexpr int kBatchAll = 0, kBatchLevel0 = 1, kBatchRest = 2;
 struct GridCounts {
   u64 scalar = 0, uni = 0, front = 0, push = 0;
@@ -97,7 +100,8 @@ static __device__ __forceinline__ bool grid_gain_batch(const int32_t *__restrict
                                 const int32_t *__restrict__ c3 = nullptr, int voff = 0, int ws_n = -1,
                                 int phase = kBatchAll, ClaimRec *log = nullptr,
                                 unsigned long long *log_n = nullptr, unsigned long long log_cap = 0,
-                                GridCounts *acc = nullptr, Team tm = whole_grid(), int gx_n = -1) {
+                                GridCounts *acc = nullptr, Team tm = whole_grid(), int gx_n = -1,
+                                const long long *best_of = nullptr, int n_graph = 0) {
   constexpr int T = kGridGainThreads;
   __shared__ u64 s_gain[kLanes];
   __shared__ unsigned int s_cnt[kLanes];
@@ -117,6 +121,7 @@ static __device__ __forceinline__ bool grid_gain_batch(const int32_t *__restrict
   const int nl = nl_dev ? min(kLanes, *(volatile const int32_t *)nl_dev) : nl_arg;
   if (ws_n < 0) ws_n = n;
   if (gx_n < 0) gx_n = ws_n;
+  const long long n_all = best_of ? n_graph : n;  // farness mode: the vertices a search must reach
   const GainWs ws = gain_ws(ws_base, 0, ws_n, 0);
   // frontier lists by level mod 3 and range starts by level parity (selected,
   // not indexed, so that nothing lands in local memory)
@@ -409,7 +414,7 @@ static __device__ __forceinline__ bool grid_gain_batch(const int32_t *__restrict
       // changes until the next barrier: the cumulative sums would already be
       // growing with the next level in faster CTAs)
       const int Fn = (int)(*(volatile unsigned long long *)&ctl->pk[(L + 1) % 3] >> 32);
-      const long long best = *(volatile long long *)&gctl->best_f;
+      const long long best = *(volatile const long long *)(best_of ? best_of : &gctl->best_f);
       if (tid < nl) {
         s_tg[tid] += ((volatile u64 *)ctl->dgain[(L + 1) % 3])[tid];
         s_tc[tid] += ((volatile u64 *)ctl->dcnt[(L + 1) % 3])[tid];
@@ -419,7 +424,7 @@ static __device__ __forceinline__ bool grid_gain_batch(const int32_t *__restrict
         if (!((alive >> j) & 1ull)) continue;
         const long long s = (long long)s_tg[j];
         const long long c = (long long)s_tc[j];
-        if (Fn > 0 && s + (long long)(L + 2) * ((long long)n - c) > best) alive &= ~(1ull << j);
+        if (Fn > 0 && s + (long long)(L + 2) * (n_all - c) > best) alive &= ~(1ull << j);
       }
       if (alive == 0) {
         // every lane is cut: clear the claim words of this frontier and of the
@@ -465,6 +470,7 @@ static __device__ __forceinline__ bool grid_gain_batch(const int32_t *__restrict
       atomicAdd(&gctl->pushes, c_push);
     }
     if (b == 0) {
+      ctl->levels = L;
       atomicAdd(&gctl->levels, (u64)L);
       atomicAdd(&gctl->batches, 1ull);
       atomicAdd(&gctl->lanes, (u64)nl);
@@ -480,14 +486,14 @@ static __device__ __forceinline__ bool grid_gain_batch(const int32_t *__restrict
       r = (long long)((volatile u64 *)ctl->gain)[tid];
     } else if (!((alive >> tid) & 1ull)) {
       r = -1;
-    } else if ((long long)s_tc[tid] != n) {
+    } else if ((long long)s_tc[tid] != n_all) {
       r = -1;
       gctl->short_vertex = c;
       gctl->short_count = (long long)s_tc[tid];
       atomicExch(&gctl->err, GC_EDISCONNECTED);
     } else {
       r = (long long)s_tg[tid];
-      if (!gctl->fixed_best) atomicMin(&gctl->best_f, r);
+      if (!best_of && !gctl->fixed_best) atomicMin(&gctl->best_f, r);
     }
     out[tid] = r;
   }

@@ -130,7 +130,7 @@ struct GainCtl {
 struct GridGainCtl {
   GridBar bar;
   int32_t err;
-  int32_t F;          // (unused)
+  int32_t levels;     // levels the last batch expanded
   int32_t qn[2];      // (unused)
   int32_t touched;    // vertices with a non-zero visited word
   int32_t pad;
