@@ -110,10 +110,10 @@ static __device__ __forceinline__ bool grid_gain_batch(const int32_t *__restrict
   __shared__ u64 s_sm[T];
   __shared__ int s_x0;
   __shared__ u64 s_red[32];
-  // farness mode: running per-lane distance sums and counts, the same in every
-  // CTA (each adds the same per-level totals), so that every CTA takes the
-  // same BFScut decisions
-  __shared__ u64 s_tg[kLanes], s_tc[kLanes];
+  // farness mode: running per-lane distance sums and counts, and the level's sums
+  // of deg - 1, the same in every CTA (each adds the same per-level totals), so
+  // that every CTA takes the same BFScut decisions
+  __shared__ u64 s_tg[kLanes], s_tc[kLanes], s_td[kLanes];
   (void)goff;
 
   const int tid = threadIdx.x, lane = tid & 31;
@@ -367,7 +367,9 @@ static __device__ __forceinline__ bool grid_gain_batch(const int32_t *__restrict
             // row's entries all carry the lane of the vertex being expanded)
             // are summed over the threads of the warp that won the same lane,
             // and one thread adds the sum; claims of several lanes add each
-            const u64 wt = MODE == kModeGain ? (u64)(dw[k] - nlev) : (u64)nlev;
+            // (farness: deg - 1 of the claimed vertex; the distances follow from
+            // the counts, level by level)
+            const u64 wt = MODE == kModeGain ? (u64)(dw[k] - nlev) : (u64)(lw[k] - 1);
             const bool one = won != 0ull && (won & (won - 1ull)) == 0ull;
             const int j1 = one ? __ffsll((long long)won) - 1 : -1;  // (the -1 group adds nothing here)
             const unsigned grp = __match_any_sync(0xffffffffu, j1);
@@ -416,15 +418,19 @@ static __device__ __forceinline__ bool grid_gain_batch(const int32_t *__restrict
       const int Fn = (int)(*(volatile unsigned long long *)&ctl->pk[(L + 1) % 3] >> 32);
       const long long best = *(volatile const long long *)(best_of ? best_of : &gctl->best_f);
       if (tid < nl) {
-        s_tg[tid] += ((volatile u64 *)ctl->dgain[(L + 1) % 3])[tid];
-        s_tc[tid] += ((volatile u64 *)ctl->dcnt[(L + 1) % 3])[tid];
+        const u64 c1 = ((volatile u64 *)ctl->dcnt[(L + 1) % 3])[tid];
+        s_td[tid] = ((volatile u64 *)ctl->dgain[(L + 1) % 3])[tid];
+        s_tg[tid] += (u64)(L + 1) * c1;
+        s_tc[tid] += c1;
       }
       cta_sync();
       for (int j = 0; j < nl; ++j) {
         if (!((alive >> j) & 1ull)) continue;
-        const long long s = (long long)s_tg[j];
-        const long long c = (long long)s_tc[j];
-        if (Fn > 0 && s + (long long)(L + 2) * (n_all - c) > best) alive &= ~(1ull << j);
+        // at most s_td vertices are at distance L+2 (neighbours of the vertices
+        // claimed in this level, one neighbour of each being nearer)
+        const long long s = (long long)s_tg[j], rest = n_all - (long long)s_tc[j];
+        const long long nx = min(rest, (long long)s_td[j]);
+        if (Fn > 0 && s + (long long)(L + 2) * nx + (long long)(L + 3) * (rest - nx) > best) alive &= ~(1ull << j);
       }
       if (alive == 0) {
         // every lane is cut: clear the claim words of this frontier and of the

@@ -140,7 +140,7 @@ struct GridGainCtl {
   unsigned long long gain[kLanes];  // gain mode: per-lane gain
   unsigned long long cnt[kLanes];   // (unused in farness mode, see dgain/dcnt)
   int32_t blk_tot[kMaxGridCtas];    // per-CTA adjacency totals of the level
-  // farness mode: per-lane distance sums and counts of the vertices claimed at
+  // farness mode: per-lane sums of deg - 1 and counts of the vertices claimed at
   // distance d, in dgain/dcnt[d mod 3] (written during one level, read by every
   // CTA after its barrier, cleared two levels later)
   unsigned long long dgain[3][kLanes];
