@@ -32,6 +32,9 @@ static int fail(int code, const std::string &msg) {
 
 constexpr int32_t kRound0GridMax = 256;  // round-0 survivors handled by grid-wide batches
 constexpr int kRound0Pivots = 8;         // round 0: at most this many pivot bounds
+constexpr int kSoloStages = 12;          // deep graphs: at most this many sampled stages per round
+constexpr int kSoloRegion = 96;          // deep graphs: persistent rounds once n <= this times the round
+constexpr int kSoloDegree = 8;           // graphs up to this average degree may take the one-source searches
 constexpr int32_t kShallowLevels = 32;   // round 0: wide bottom-up batches up to this BFS depth
 // gc_greedy, lists that cannot certify a pick: from this many candidates whose
 // bounds reach the best gain (64 grid-wide steps) a sweep in CTA batches runs.
@@ -75,7 +78,7 @@ static void release(gc_graph *g) {
                  g->ws, g->dec, g->ggctl, g->goff, g->lctl, g->picks, g->pgain, g->pdec, g->mx_buf,
                  g->two_hop, g->score, g->rec_count, g->akey, g->ast, g->gx, g->wsel, g->wpos, g->wgain,
                  g->lev_cnt, g->lev_C, g->lev_M, g->lev_max, g->rpf, g->cif, g->c3, g->gsel, g->heavy, g->n_heavy,
-                 g->g3, g->c3s, g->r0_vis, g->wt, g->w_ws, g->clog, g->x_ws};
+                 g->g3, g->c3s, g->r0_vis, g->wt, g->w_ws, g->clog, g->x_ws, g->solo_q};
   for (void *p : dev)
     if (p) cudaFree(p);
   if (g->h_sctl) cudaFreeHost(g->h_sctl);
@@ -154,6 +157,23 @@ static int distances_from(gc_graph *g, const int32_t *seeds_dev, int32_t n_seeds
                                       std::to_string(g->n) + " vertices unreached");
   if (farness) *farness = g->h_sctl->sum;
   return GC_OK;
+}
+
+// Hops that cover m vertices from `want` sampled ones (about 2 d^2 vertices lie
+// within d hops on a grid-like graph).
+static int cover(int32_t m, int32_t want, int lo, int hi) {
+  return std::min(hi, std::max(lo, (int)(1.5 * std::sqrt((double)m / want)) + 1));
+}
+
+// One sampled stage of round 0 on a deep graph: of the selected vertices
+// list[0..m), a spread sample is searched to the end, and the bounds
+// f({x}) >= f({v}) - d(v, x) (n - 2) go to the neighbourhoods.
+static int solo_stage(gc_graph *g, int32_t m, int stage) {
+  const int32_t want = g->solo_ctas;
+  GC_TRY(launch_sample(g, want, (uint32_t)stage));
+  GC_TRY(launch_solo(g, kModeFarness, g->list, 0, &g->sctl->n_sel, g->lgain, nullptr, 0, true, false));
+  GC_TRY(launch_after_eval(g, 0, 0));
+  return launch_relax(g, true, nullptr, cover(m, want, 2, 64), 0);
 }
 
 static int check_ids(const gc_graph *g, const int32_t *a, int32_t len, const char *what) {
@@ -299,6 +319,12 @@ int gc_load_csr(int32_t n, const int32_t *row_ptr, const int32_t *col_idx, uint3
   g->gain_ctas = want;
   g->ws_count = want;
   if ((rc = dalloc(&g->ws, (size_t)want * g->ws_stride))) return bail(rc);
+  // queues of the one-source searches of deep graphs: at most 1 GB, on sparse
+  // graphs only (roads, grids, trees)
+  if (nnz <= (int64_t)kSoloDegree * n) {
+    if ((rc = solo_plan(n, g->num_sms, std::min<size_t>(free_b / 16, (size_t)1 << 30), &g->solo_ctas))) return bail(rc);
+    if (g->solo_ctas > 0 && (rc = dalloc(&g->solo_q, (size_t)g->solo_ctas * N))) return bail(rc);
+  }
   if (cudaMemsetAsync(g->ws, 0, (size_t)want * g->ws_stride, st) != cudaSuccess ||
       cudaMemsetAsync(g->hist, 0, kHistBins * sizeof(unsigned int), st) != cudaSuccess ||
       cudaMemsetAsync(g->lev_cnt, 0, N * sizeof(unsigned long long), st) != cudaSuccess ||
@@ -342,7 +368,12 @@ static int gains_core(gc_graph *g, const int32_t *S_dev, int32_t s_len, const in
     GC_TRY(launch_fill_i32(g, g->dS, kInf, g->n));
     GC_TRY(launch_bfs_relabel(g, g->dS, S_dev, s_len, timeout_ns(nullptr)));
   }
-  return launch_gains(g, kModeGain, cand_dev, n_cand, nullptr, out_dev, 0);
+  // How deep the graph is is known on the device only: two launches, one of
+  // which does the work (the other ends at once).  Distances to a group of more
+  // than one vertex in 32 are short on any graph.
+  const bool solo = g->solo_ctas > 0 && g->gain_lanes == kLanes && (int64_t)s_len * 32 <= g->n;
+  if (solo) GC_TRY(launch_solo(g, kModeGain, cand_dev, n_cand, nullptr, out_dev, nullptr, 0, false, true));
+  return launch_gains(g, kModeGain, cand_dev, n_cand, nullptr, out_dev, 0, kLanes, false, true, solo);
 }
 
 int gc_marginal_gains(gc_graph *g, const int32_t *S, int32_t s_len, const int32_t *cand,
@@ -357,6 +388,7 @@ int gc_marginal_gains(gc_graph *g, const int32_t *S, int32_t s_len, const int32_
   GC_CUDA(cudaMemcpyAsync(g->io_a, S, (size_t)s_len * sizeof(int32_t), cudaMemcpyHostToDevice, g->stream));
   GC_CUDA(cudaMemsetAsync(g->gctl, 0, sizeof(GainCtl), g->stream));
   GC_TRY(distances_from(g, g->io_a, s_len, timeout_ns(nullptr), nullptr));
+  const bool solo = g->solo_ctas > 0 && g->gain_lanes == kLanes && g->h_bctl->levels > kWideLevels;
   float ms_k = 0.f;
   int64_t launches = 0;
   for (int32_t off = 0; off < n_cand; off += g->n) {
@@ -367,7 +399,8 @@ int gc_marginal_gains(gc_graph *g, const int32_t *S, int32_t s_len, const int32_
     GC_TRY(gain_event(g, 0, &e0));
     GC_TRY(gain_event(g, 1, &e1));
     GC_CUDA(cudaEventRecord(e0, g->stream));
-    GC_TRY(launch_gains(g, kModeGain, g->list, len, nullptr, g->lgain, 0));
+    if (solo) GC_TRY(launch_solo(g, kModeGain, g->list, len, nullptr, g->lgain, nullptr, 0, false, false));
+    else GC_TRY(launch_gains(g, kModeGain, g->list, len, nullptr, g->lgain, 0));
     GC_CUDA(cudaEventRecord(e1, g->stream));
     GC_CUDA(cudaMemcpyAsync(out_gain + off, g->lgain, (size_t)len * sizeof(long long),
                             cudaMemcpyDeviceToHost, g->stream));
@@ -466,6 +499,7 @@ int gc_top_closeness(gc_graph *g, int32_t k, const gc_opts *opts_in, int32_t *ou
   GC_TRY(distances_from(g, &g->sctl->arg_id, 1, tns, nullptr));
   const int32_t ecc = g->h_bctl->levels;
   if (ecc > kShallowLevels) GC_TRY(launch_pivot_bound(g));
+  const bool deep = ecc > kShallowLevels && g->solo_ctas > 0 && opts.round0_lanes == 0 && opts.max_ctas == 0;
   // 2. probes, searched with no cut (threshold +infinity, kept fixed)
   struct {
     long long best_f;
@@ -478,7 +512,9 @@ int gc_top_closeness(gc_graph *g, int32_t k, const gc_opts *opts_in, int32_t *ou
   const int32_t n_probe = std::min<int32_t>(g->h_sctl->n_sel, (k + kLanes - 1) / kLanes * kLanes);
   if (n_probe < k) return fail(GC_EINTERNAL, "top-k closeness: fewer probes than k");
   GC_TRY(launch_clamp_nsel(g, n_probe));
-  if (n_probe <= kRound0GridMax) {
+  if (deep) {
+    GC_TRY(launch_solo(g, kModeFarness, g->list, n_probe, nullptr, g->lgain, nullptr, 0, true, false));
+  } else if (n_probe <= kRound0GridMax) {
     for (int32_t off = 0; off < n_probe; off += kLanes)
       GC_TRY(launch_gains_grid(g, kModeFarness, g->list + off, std::min<int32_t>(kLanes, n_probe - off), nullptr,
                                g->lgain + off, tns, false));
@@ -500,7 +536,7 @@ int gc_top_closeness(gc_graph *g, int32_t k, const gc_opts *opts_in, int32_t *ou
   GC_TRY(launch_select(g, kSelKey, 0, 0, kTauHost, -T));
   GC_TRY(read_ctl(g));
   int32_t n_surv = g->h_sctl->n_sel;
-  if (opts.round0_lanes >= 0 && ecc <= kShallowLevels && n_surv > 0 && !(opts.flags & GC_OPT_R0_NO_PROBE)) {
+  if (opts.round0_lanes >= 0 && ecc <= kShallowLevels && n_surv > kLanes && !(opts.flags & GC_OPT_R0_NO_PROBE)) {
     // as in round 0 of gc_greedy: bounds from the low-degree vertices out of two hops' reach
     GC_TRY(launch_far_bound(g));
     GC_TRY(launch_select(g, kSelKey, 0, 0, kTauHost, -T));
@@ -520,9 +556,22 @@ int gc_top_closeness(gc_graph *g, int32_t k, const gc_opts *opts_in, int32_t *ou
       if ((double)two_hop_sum < passes * (double)g->nnz) r0_w = 0;
     }
   }
+  // deep graphs: sampled stages until few vertices are left, as in round 0 of
+  // gc_greedy
+  int64_t sampled = 0;
+  for (int st = 0; deep && n_surv > 2 * g->solo_ctas && st < kSoloStages; ++st) {
+    GC_TRY(solo_stage(g, n_surv, st));
+    GC_TRY(read_ctl(g));
+    sampled += g->h_sctl->n_sel;
+    GC_TRY(launch_select(g, kSelKey, 0, 0, kTauHost, -T));
+    GC_TRY(read_ctl(g));
+    n_surv = g->h_sctl->n_sel;
+  }
   float ms_wide = 0.f;
   if (n_surv > 0) {
-    if (r0_w > 0) {
+    if (deep) {
+      GC_TRY(launch_solo(g, kModeFarness, g->list, n_surv, nullptr, g->lgain, nullptr, 0, false, false));
+    } else if (r0_w > 0) {
       cudaEvent_t e0 = nullptr, e1 = nullptr;
       GC_TRY(gain_event(g, 0, &e0));
       GC_TRY(gain_event(g, 1, &e1));
@@ -568,7 +617,7 @@ int gc_top_closeness(gc_graph *g, int32_t k, const gc_opts *opts_in, int32_t *ou
   }
   if (stats) {
     memset(stats, 0, sizeof(*stats));
-    stats->round0_evals = (int64_t)n_probe + n_surv;
+    stats->round0_evals = (int64_t)n_probe + sampled + n_surv;
     stats->batches = (int64_t)g->h_gctl->batches;
     stats->edges_union = (int64_t)g->h_gctl->edges_union;
     stats->levels = (int64_t)g->h_gctl->levels;
@@ -874,8 +923,10 @@ int gc_greedy(gc_graph *g, int32_t k, const gc_opts *opts_in, int32_t *out_group
   int r0_w = 0;
   // The far-vertex probe starts with counts alone: low-degree vertices that no
   // path of two hops can reach raise the survivors' bounds (k_far_counts), and
-  // the survivors above the threshold are cut without a search.
-  if (opts.round0_lanes >= 0 && ecc_a <= kShallowLevels && n_surv > 0 && !(opts.flags & GC_OPT_R0_NO_PROBE)) {
+  // the survivors above the threshold are cut without a search.  Up to 64
+  // survivors are one narrow batch, which costs no more than the counts and
+  // their selection (BA 13,573 vertices, m = 6: 1.79 ms without, 1.85 with).
+  if (opts.round0_lanes >= 0 && ecc_a <= kShallowLevels && n_surv > kLanes && !(opts.flags & GC_OPT_R0_NO_PROBE)) {
     GC_TRY(launch_far_bound(g));
     GC_TRY(launch_select(g, kSelKey, 0, 0, kTauDevice, 0));
     GC_TRY(read_ctl(g));
@@ -902,12 +953,46 @@ int gc_greedy(gc_graph *g, int32_t k, const gc_opts *opts_in, int32_t *out_group
       if ((double)two_hop_sum < passes * (double)g->nnz) r0_w = 0;
     }
   }
+  // Deep graphs (roads, grids, trees): searches of one source per CTA, and the
+  // bounds that a search gives its neighbourhood (gc_solo.cu)
+  const bool auto_steps = opts.step_mode == 0 && opts.step_form == 0 && opts.eval_per_step == 0 &&
+                          opts.step_lanes == 0 && opts.max_ctas == 0 && opts.active_target == 0 &&
+                          opts.lazy_ctas == 0 && opts.round1_heavy == 0 && opts.local_update_max_gain == 0;
+  const bool deep = ecc_a > kShallowLevels && g->solo_ctas > 0 && opts.round0_lanes == 0 && auto_steps &&
+                    !opts.use_proposal && !(g->rec_X && g->rec_cap > 0) && g->gain_lanes == kLanes &&
+                    !(opts.flags & (GC_OPT_NO_ROUND1_BOUND | GC_OPT_NO_EXPAND_BOUND | GC_OPT_FULL_ADJACENCY));
+  int64_t solo_upd = 0;  // deep graphs: labels lowered by the d_S updates of rounds >= 2
+  auto solo_timed = [&](int mode, int32_t *region, int32_t slack, bool no_cut) -> int {
+    cudaEvent_t e0 = nullptr, e1 = nullptr;
+    GC_TRY(gain_event(g, ev_used, &e0));
+    GC_TRY(gain_event(g, ev_used + 1, &e1));
+    ev_used += 2;
+    ev_k64.push_back(0);
+    GC_CUDA(cudaEventRecord(e0, g->stream));
+    GC_TRY(launch_solo(g, mode, g->list, 0, &g->sctl->n_sel, g->lgain, region, slack, no_cut, false));
+    GC_CUDA(cudaEventRecord(e1, g->stream));
+    return GC_OK;
+  };
+  bool solo_done = false;
+  if (deep && n_surv > 0) {
+    GC_TRY(launch_pivot_bound(g));
+    for (int st = 0;; ++st) {
+      GC_TRY(launch_select(g, kSelKey, 0, 0, kTauHost, -g->h_gctl->best_f));
+      GC_TRY(read_ctl(g));
+      n_surv = g->h_sctl->n_sel;
+      if (n_surv <= 2 * g->solo_ctas || st >= kSoloStages) break;
+      GC_TRY(solo_stage(g, n_surv, st));
+      GC_TRY(read_ctl(g));
+    }
+    if (n_surv > 0) GC_TRY(solo_timed(kModeFarness, nullptr, 0, false));
+    solo_done = true;
+  }
   // Many survivors (deep graphs, where the degree bound is weak): tighten the
   // bounds with the BFS levels of pivots (triangle inequality, see
   // k_pivot_bound).  The first pivot is the vertex just searched; each further
   // pivot is the undecided vertex of smallest bound, searched exactly, so it
   // may also lower the threshold.
-  for (int piv = 0; r0_w == 0 && n_surv > kRound0GridMax && piv < kRound0Pivots; ++piv) {
+  for (int piv = 0; !solo_done && r0_w == 0 && n_surv > kRound0GridMax && piv < kRound0Pivots; ++piv) {
     if (piv > 0) {
       GC_TRY(launch_argmin_lb(g));
       GC_TRY(distances_from(g, &g->sctl->arg_id, 1, tns, nullptr));
@@ -947,6 +1032,8 @@ int gc_greedy(gc_graph *g, int32_t k, const gc_opts *opts_in, int32_t *out_group
     r0_probe[1] += (int64_t)r0c.probe_cut;
     r0_probe[2] = (int64_t)r0c.bu_vertices;
     r0_probe[3] = (int64_t)r0c.bu_visreads;
+  } else if (solo_done) {
+    // searched above
   } else if (n_surv <= kRound0GridMax) {
     // few survivors (hubs with large searches): one grid-wide batch per 64
     for (int32_t off = 0; off < n_surv; off += kLanes)
@@ -974,7 +1061,7 @@ int gc_greedy(gc_graph *g, int32_t k, const gc_opts *opts_in, int32_t *out_group
     g->mx = g->mx_buf;
   }
   // pruned adjacency: drop the entries no later round can use (d_S[w] <= 1)
-  if (!(opts.flags & GC_OPT_FULL_ADJACENCY)) {
+  if (!(opts.flags & GC_OPT_FULL_ADJACENCY) && !deep) {
     GC_TRY(launch_prune_csr(g));
     pruned = true;
   }
@@ -1016,7 +1103,12 @@ int gc_greedy(gc_graph *g, int32_t k, const gc_opts *opts_in, int32_t *out_group
   std::vector<long long> gains_picked(k, 0), decreases(k, 0);
   gains_picked[0] = f;
   for (int32_t r = 1; r < k; ++r) {
-    if (r >= 2 && persistent) {
+    // Deep graphs keep to host-driven steps of one-source searches until the
+    // regions (about n / r vertices) are so small that a round's 30 launches
+    // outweigh them: per round, persistent against host-driven, 71 and 148 us
+    // at n = 779 (r = 20..75), 145 and 188 (r = 3..20); 169 and 191 at n = 4,091
+    // (r = 20..75), 500 and 330 (r = 3..20); 363 and 245 at n = 9,976
+    if (r >= 2 && persistent && (!deep || (int64_t)g->n <= (int64_t)kSoloRegion * r)) {
       // rounds r..k-1 on the device: persistent kernel over an active list
       LazyCtl init;
       memset(&init, 0, sizeof(init));
@@ -1118,7 +1210,29 @@ int gc_greedy(gc_graph *g, int32_t k, const gc_opts *opts_in, int32_t *out_group
     }
     GC_TRY(launch_round_begin(g));
     for (int step = 0;; ++step) {
-      if (r == 1 && round1_bound) {
+      if (deep) {
+        // The largest stale bounds first (they give the level to reach), then
+        // every candidate whose bound reaches the best gain: all of them if
+        // they fit a few waves of CTAs, else a spread sample with relaxed
+        // pruning, whose bounds cut most of its neighbourhood
+        const int32_t want = g->solo_ctas;
+        int32_t hops = 0;
+        if (step == 0 && r > 1) {
+          GC_TRY(launch_select(g, kSelLazy, r, std::max<int32_t>(kLanes, want / 4), kTauHistogram, 0));
+        } else {
+          const long long best = step == 0 ? 0 : std::max<long long>(0, g->h_sctl->best_gain);
+          GC_TRY(launch_select(g, kSelLazy, r, 0, kTauHost, best));
+          GC_CUDA(cudaMemcpyAsync(g->h_sctl, g->sctl, sizeof(SelCtl), cudaMemcpyDeviceToHost, g->stream));
+          GC_TRY(sync(g));
+          const int32_t m = g->h_sctl->n_sel;
+          if (m > 2 * want && step < kSoloStages) {
+            hops = cover(m, want, 1, 12);
+            GC_TRY(launch_sample(g, want, (uint32_t)(r * 64 + step)));
+          }
+        }
+        GC_TRY(solo_timed(kModeGain, hops ? g->ast : nullptr, hops, false));
+        if (hops) GC_TRY(launch_relax(g, false, g->ast, hops, r));
+      } else if (r == 1 && round1_bound) {
         if (step == 0 && g->rec_X && g->rec_cap > 0) {
           // recording run (training data for the proposal): the 1024 largest
           // bounds, every one evaluated exactly and recorded with the
@@ -1190,9 +1304,10 @@ int gc_greedy(gc_graph *g, int32_t k, const gc_opts *opts_in, int32_t *out_group
     GC_TRY(launch_round_end(g));
     GC_CUDA(cudaMemsetAsync(g->bctl, 0, sizeof(BfsCtl), g->stream));
     GC_TRY(launch_bfs_relabel(g, g->dS, &g->sctl->best_id, 1, tns, pruned));
-    GC_CUDA(cudaMemcpyAsync(&g->h_bctl->decrease, &g->bctl->decrease, sizeof(unsigned long long),
+    GC_CUDA(cudaMemcpyAsync(&g->h_bctl->decrease, &g->bctl->decrease, 2 * sizeof(unsigned long long),
                             cudaMemcpyDeviceToHost, g->stream));
     GC_TRY(sync(g));
+    if (deep && r >= 2) solo_upd += (int64_t)g->h_bctl->relabelled;
     decreases[r] = (long long)g->h_bctl->decrease;
     if (decreases[r] != gains_picked[r])
       return fail(GC_EINTERNAL, "gain of the pick disagrees with the d_S update (round " +
@@ -1252,7 +1367,7 @@ int gc_greedy(gc_graph *g, int32_t k, const gc_opts *opts_in, int32_t *out_group
     stats->lazy_lanes = (int64_t)(lazy1.lanes - lazy0.lanes);
     stats->lazy_upd_frontier = (int64_t)g->h_lctl->upd_work[0];
     stats->lazy_upd_edges = (int64_t)g->h_lctl->upd_work[1];
-    stats->lazy_upd_relabels = (int64_t)g->h_lctl->upd_relabels;
+    stats->lazy_upd_relabels = (int64_t)g->h_lctl->upd_relabels + solo_upd;
     stats->lazy_sel_scanned = (int64_t)g->h_lctl->sel_scanned;
     stats->lazy_log_picks = (int64_t)g->h_lctl->log_picks;
     stats->lazy_upd_log = (int64_t)g->h_lctl->upd_log;

@@ -42,9 +42,11 @@ __global__ void __launch_bounds__(kGainThreads, 2)
               const int32_t *__restrict__ dS, const int32_t *__restrict__ cand, int32_t n_cand_arg,
               const int32_t *__restrict__ n_cand_dev, long long *__restrict__ out,
               unsigned char *ws_base, size_t ws_stride, GainCtl *ctl, int lanes,
-              const int32_t *__restrict__ mx, const LaneGraphs lg, const int32_t *__restrict__ c3) {
+              const int32_t *__restrict__ mx, const LaneGraphs lg, const int32_t *__restrict__ c3,
+              const BfsCtl *shallow_only) {
   __shared__ int s_batch;
   __shared__ u64 s_red[32];
+  if (shallow_only && *(volatile const int32_t *)&shallow_only->levels > kWideLevels) return;
   const int tid = threadIdx.x;
   const GainWs ws = gain_ws(ws_base, ws_stride, n, blockIdx.x);
   const int n_cand = n_cand_dev ? *n_cand_dev : n_cand_arg;
@@ -90,13 +92,14 @@ int gain_kernel_occupancy(int *blocks_per_sm) {
 }
 
 int launch_gains(gc_graph *g, int mode, const int32_t *cand, int32_t n_cand,
-                 const int32_t *n_cand_dev, long long *out, int max_ctas, int lanes, bool pruned) {
+                 const int32_t *n_cand_dev, long long *out, int max_ctas, int lanes, bool pruned,
+                 bool fresh_ctl, bool shallow_only) {
   if (!n_cand_dev && n_cand <= 0) return GC_OK;
   if (lanes < 1 || lanes > kLanes) lanes = kLanes;
   // full batches of gains at the handle's width above 64: the wide kernel
   if (mode == kModeGain && lanes == kLanes && g->gain_lanes > kLanes)
     return launch_gains_wide(g, cand, n_cand, n_cand_dev, out, max_ctas, pruned);
-  GC_CUDA(cudaMemsetAsync(&g->gctl->batch_next, 0, sizeof(unsigned int), g->stream));
+  if (!fresh_ctl) GC_CUDA(cudaMemsetAsync(&g->gctl->batch_next, 0, sizeof(unsigned int), g->stream));
   int ctas = g->gain_ctas;
   if (max_ctas > 0 && max_ctas < ctas) ctas = max_ctas;
   if (!n_cand_dev) {
@@ -109,11 +112,11 @@ int launch_gains(gc_graph *g, int mode, const int32_t *cand, int32_t n_cand,
   if (mode == kModeGain)
     k_gains64<kModeGain><<<ctas, kGainThreads, 0, g->stream>>>(
         rp, ci, g->n, g->dS, cand, n_cand, n_cand_dev, out, g->ws, g->ws_stride, g->gctl, lanes, g->mx,
-        LaneGraphs(), c3);
+        LaneGraphs(), c3, shallow_only ? g->bctl : nullptr);
   else
     k_gains64<kModeFarness><<<ctas, kGainThreads, 0, g->stream>>>(
         g->rp, g->ci, g->n, g->dS, cand, n_cand, n_cand_dev, out, g->ws, g->ws_stride, g->gctl, lanes, nullptr,
-        g->lane_graphs, nullptr);
+        g->lane_graphs, nullptr, nullptr);
   GC_CUDA(cudaGetLastError());
   return GC_OK;
 }

@@ -350,6 +350,10 @@ struct gc_graph {
   unsigned char *ws = nullptr;
   size_t ws_stride = 0;
   int ws_count = 0;
+  // one-source-per-CTA searches of deep graphs (gc_solo.cu): a queue of n
+  // vertices per CTA; 0 CTAs: dense graph, or too large for the bitmap
+  int32_t *solo_q = nullptr;
+  int solo_ctas = 0;
   int gain_ctas = 0;       // resident CTAs of the gain kernel
   int bfs_ctas = 0;        // resident CTAs of the cooperative BFS
   int grid_ctas = 0;       // resident CTAs of the grid-wide gain kernel
@@ -411,10 +415,26 @@ enum GainMode { kModeGain = 0, kModeFarness = 1 };
 // lanes: candidates per batch (1..64); fewer lanes spread one step's work
 // over more CTAs.
 // pruned (gain mode only): the pruned adjacency, as for launch_bfs_relabel.
+// fresh_ctl: *gctl has just been zeroed (so batch_next need not be).
+// shallow_only: does nothing if the BFS that filled d_S had more than
+// kWideLevels levels (launch_solo beside it does the work).
 int launch_gains(gc_graph *g, int mode, const int32_t *cand, int32_t n_cand,
                  const int32_t *n_cand_dev, long long *out, int max_ctas, int lanes = kLanes,
-                 bool pruned = false);
+                 bool pruned = false, bool fresh_ctl = false, bool shallow_only = false);
 size_t gain_ws_stride(int32_t n);
+// One candidate per CTA (deep graphs, gc_solo.cu): gains with the pruning
+// relaxed by `slack` (region[i]: vertices visited), or farness values (no_cut:
+// exact for every candidate).  deep_only: does nothing unless the BFS that
+// filled d_S had more than kWideLevels levels.
+int solo_plan(int32_t n, int num_sms, size_t budget, int *ctas);
+int launch_solo(gc_graph *g, int mode, const int32_t *cand, int32_t n_cand, const int32_t *n_cand_dev, long long *out,
+                int32_t *region, int32_t slack, bool no_cut, bool deep_only);
+// bounds from the searched vertices list[0 .. sctl->n_sel) (results in lgain)
+// to the vertices within `hops` of them: key (farness) or ub of candidates not
+// evaluated in `round`
+int launch_relax(gc_graph *g, bool farness, const int32_t *region, int32_t hops, int32_t round);
+// list[0 .. sctl->n_sel) <- about `want` of its entries, spread by a hash
+int launch_sample(gc_graph *g, int32_t want, uint32_t salt);
 // Gain mode with 128 or 256 candidates per batch (g->gain_lanes), one CTA per
 // batch; the same contract as launch_gains at 64 lanes.
 int launch_gains_wide(gc_graph *g, const int32_t *cand, int32_t n_cand, const int32_t *n_cand_dev,
