@@ -34,6 +34,7 @@ constexpr int32_t kRound0GridMax = 256;  // round-0 survivors handled by grid-wi
 constexpr int kRound0Pivots = 8;         // round 0: at most this many pivot bounds
 constexpr int kSoloStages = 12;          // deep graphs: at most this many sampled stages per round
 constexpr int kSoloRegion = 96;          // deep graphs: persistent rounds once n <= this times the round
+constexpr int32_t kWholeSearchMax = 1024;  // weighted round 0: full searches up to this many vertices (one wave)
 constexpr int kSoloDegree = 8;           // graphs up to this average degree may take the one-source searches
 constexpr int32_t kShallowLevels = 32;   // round 0: wide bottom-up batches up to this BFS depth
 // gc_greedy, lists that cannot certify a pick: from this many candidates whose
@@ -78,7 +79,7 @@ static void release(gc_graph *g) {
                  g->ws, g->dec, g->ggctl, g->goff, g->lctl, g->picks, g->pgain, g->pdec, g->mx_buf,
                  g->two_hop, g->score, g->rec_count, g->akey, g->ast, g->gx, g->wsel, g->wpos, g->wgain,
                  g->lev_cnt, g->lev_C, g->lev_M, g->lev_max, g->rpf, g->cif, g->c3, g->gsel, g->heavy, g->n_heavy,
-                 g->g3, g->c3s, g->r0_vis, g->wt, g->w_ws, g->clog, g->x_ws, g->solo_q};
+                 g->g3, g->c3s, g->r0_vis, g->wt, g->w_ws, g->clog, g->x_ws, g->solo_q, g->ci_w, g->wt_w};
   for (void *p : dev)
     if (p) cudaFree(p);
   if (g->h_sctl) cudaFreeHost(g->h_sctl);
@@ -654,15 +655,24 @@ int gc_set_weights(gc_graph *g, const int32_t *weights, uint32_t flags) {
                                                          : "a weight is below 1");
   if ((int64_t)(g->n - 1) * (int64_t)h[1] >= (int64_t)kInf)
     return fail(GC_ERANGE, "(n - 1) * max weight reaches 2^30: path lengths could overflow");
+  // the rows ordered by weight, for round 0 of gc_greedy_weighted
+  g->w_max = h[1];
+  int rc = GC_OK;
+  if (!g->ci_w && ((rc = dalloc(&g->ci_w, (size_t)g->nnz)) || (rc = dalloc(&g->wt_w, (size_t)g->nnz)))) return rc;
+  int32_t *tmp = nullptr;  // cif (scratch here) holds the ids of a middle pass, tmp its weights
+  if (g->w_max > 255 && (rc = dalloc(&tmp, (size_t)g->nnz))) return rc;
+  rc = launch_wsort(g, g->cif, tmp);
+  if (rc == GC_OK) rc = sync(g);
+  cudaFree(tmp);
+  GC_TRY(rc);
   g->w_ok = true;
   return GC_OK;
 }
 
 // Weighted Greedy: Algorithm 2 with every SSSP a shortest-path search (the
 // paper's weighted case) and the pruning of Sec. 4.1 and the lazy bounds of
-// Sec. 4.2 unchanged.  Round 0 evaluates f({v}) of every vertex by a full
-// search (a label-correcting search has no distance order to cut on);
-// later rounds take host-driven lazy steps, one candidate per CTA; d_S is
+// Sec. 4.2 unchanged.  Round 0 searches every vertex in distance order, cut once
+// its bound passes the best farness (k_wsearch); later rounds take host-driven lazy steps, one candidate per CTA; d_S is
 // updated in place from each pick and its decrease must equal the pick's gain.
 int gc_greedy_weighted(gc_graph *g, int32_t k, const gc_opts *opts_in, int32_t *out_group, int64_t *out_farness,
                        gc_stats *stats) {
@@ -678,7 +688,7 @@ int gc_greedy_weighted(gc_graph *g, int32_t k, const gc_opts *opts_in, int32_t *
   const int32_t n = g->n;
   if (!g->w_ws) {  // per-CTA search workspaces: within 40% of free memory and 16 GB
     int occ = 0;
-    GC_TRY(wsssp_occupancy(&occ));
+    GC_TRY(wsearch_occupancy(g, &occ));
     g->w_stride = wws_stride(n);
     size_t free_b = 0, total_b = 0;
     GC_CUDA(cudaMemGetInfo(&free_b, &total_b));
@@ -693,19 +703,22 @@ int gc_greedy_weighted(gc_graph *g, int32_t k, const gc_opts *opts_in, int32_t *
     }
     g->w_ctas = want;
     g->w_task = (unsigned int *)(g->w_ws + (size_t)want * g->w_stride);
-    // queue flags 0, then every workspace's dist = kInf
-    for (int c = 0; c < want; ++c) {
-      unsigned char *p = g->w_ws + (size_t)c * g->w_stride;
-      GC_CUDA(cudaMemsetAsync(p, 0, g->w_stride, g->stream));
-    }
-    for (int c = 0; c < want; ++c)
-      GC_TRY(launch_fill_i32(g, (int32_t *)(g->w_ws + (size_t)c * g->w_stride), kInf, n));
+    GC_TRY(launch_wfar_init(g));
   }
   GC_CUDA(cudaMemsetAsync(g->sctl, 0, sizeof(SelCtl), g->stream));
-  // ---- round 0: f({v}) of every vertex, s0 = argmin (f, id) ----
-  GC_TRY(launch_iota(g, g->list, n));
-  GC_CUDA(cudaMemcpyAsync(&g->sctl->n_sel, &n, sizeof(int32_t), cudaMemcpyHostToDevice, g->stream));
-  GC_TRY(launch_wsssp(g, kWFarness, g->list, &g->sctl->n_sel, g->f0, g->w_task));
+  // ---- round 0: s0 = argmin (f({v}), id).  The vertices of largest degree are
+  // searched first, in full; their best farness cuts the other searches ----
+  GC_TRY(launch_fill_i64(g, g->f0, -1, n));
+  GC_TRY(launch_fill_i64(g, &g->gctl->best_f, LLONG_MAX, 1));
+  const bool whole = n <= kWholeSearchMax;
+  if (!whole) {
+    GC_TRY(launch_fill_i64(g, g->ub, 0, n));
+    GC_TRY(launch_degree_keys(g));
+    GC_TRY(launch_select(g, kSelKey, 0, kLanes, kTauHistogram, 0));
+    GC_TRY(launch_clamp_nsel(g, 4 * kLanes));
+    GC_TRY(launch_wsearch(g, kWFarness, g->list, &g->sctl->n_sel, 0, g->f0, &g->gctl->best_f, 0));
+  }
+  GC_TRY(launch_wsearch(g, kWFarness, nullptr, nullptr, n, g->f0, &g->gctl->best_f, whole ? kInf : 0));
   GC_TRY(launch_argmin_f0(g));
   GC_TRY(read_ctl(g));
   if (g->h_sctl->err) return fail(g->h_sctl->err, g->h_sctl->err == GC_EDISCONNECTED ? "graph is disconnected"
@@ -716,45 +729,55 @@ int gc_greedy_weighted(gc_graph *g, int32_t k, const gc_opts *opts_in, int32_t *
   // d_S = d(s0, .) by the in-place search from s0; its sum must equal f_s0
   GC_TRY(launch_fill_i32(g, g->dS, kInf, n));
   GC_CUDA(cudaMemcpyAsync(g->io_a, &s0, sizeof(int32_t), cudaMemcpyHostToDevice, g->stream));
-  GC_TRY(launch_wrelabel(g, g->io_a, &g->bctl->decrease));
+  long long *const dec = (long long *)&g->bctl->decrease;
+  GC_TRY(launch_wsearch(g, kWRelabel, g->io_a, nullptr, 1, dec, nullptr, kInf));
   GC_TRY(launch_sum_dist(g, g->dS));
   GC_TRY(read_ctl(g));
   if (g->h_sctl->count != 0 || (long long)g->h_sctl->sum != f_s0)
     return fail(GC_EINTERNAL, "gc_greedy_weighted: farness of s0 disagrees between round 0 and d_S");
   long long f = f_s0;
   out_group[0] = s0;
-  // ---- rounds 1..k-1: host-driven lazy steps, one candidate per CTA ----
+  // ---- rounds 1..k-1: host-driven lazy steps, one candidate per CTA.  Pruned
+  // searches run in one bucket: their regions are small, and R-MAT scale 14 took 26
+  // ms for 49 rounds in buckets of a quarter of the mean distance, 8 in one ----
   GC_TRY(launch_fill_i64(g, g->ub, LLONG_MAX, n));
   GC_TRY(launch_fill_i64(g, g->ub + s0, -1, 1));
   GC_TRY(launch_fill_i32(g, g->stamp, 0, n));
   const int32_t step_want = g->w_ctas;
   int64_t steps = 0, evals = 0;
+  long long gain = 0;  // of the last pick, whose d_S update may still run
+  // the decrease of the last update arrives with the next synchronisation
+  auto update_matches = [&](int32_t r) -> int {
+    if ((long long)g->h_bctl->decrease != gain)
+      return fail(GC_EINTERNAL, "gc_greedy_weighted: gain of the pick disagrees with the d_S update (round " +
+                                    std::to_string(r) + ")");
+    return GC_OK;
+  };
   for (int32_t r = 1; r < k; ++r) {
     GC_TRY(launch_round_begin(g));
-    for (;;) {
+    for (int step = 0;; ++step) {
       GC_TRY(launch_select(g, kSelLazy, r, step_want, kTauHistogram, 0));
-      GC_TRY(launch_wsssp(g, kWGain, g->list, &g->sctl->n_sel, g->lgain, g->w_task));
+      GC_TRY(launch_wsearch(g, kWGain, g->list, &g->sctl->n_sel, 0, g->lgain, nullptr, kInf));
       GC_TRY(launch_after_eval(g, r, 0));
       GC_TRY(launch_unevaluated_best(g, r));
-      GC_TRY(read_ctl(g));
+      GC_CUDA(cudaMemcpyAsync(g->h_sctl, g->sctl, sizeof(SelCtl), cudaMemcpyDeviceToHost, g->stream));
+      GC_TRY(sync(g));
       if (g->h_sctl->err) return fail(g->h_sctl->err, "weighted search failed");
+      if (step == 0 && r > 1) GC_TRY(update_matches(r - 1));
       ++steps;
       evals += g->h_sctl->n_sel;
       if (g->h_sctl->accepted) break;
       if (g->h_sctl->n_sel == 0) return fail(GC_EINTERNAL, "gc_greedy_weighted: lazy step selected no candidate");
     }
-    const int32_t pick = g->h_sctl->best_id;
-    const long long gain = g->h_sctl->best_gain;
-    GC_TRY(launch_round_end(g));
-    GC_CUDA(cudaMemcpyAsync(g->io_a, &pick, sizeof(int32_t), cudaMemcpyHostToDevice, g->stream));
-    GC_TRY(launch_wrelabel(g, g->io_a, &g->bctl->decrease));
-    GC_TRY(read_ctl(g));
-    if ((long long)g->h_bctl->decrease != gain)
-      return fail(GC_EINTERNAL, "gc_greedy_weighted: gain of the pick disagrees with the d_S update (round " +
-                                    std::to_string(r) + ")");
+    gain = g->h_sctl->best_gain;
     f -= gain;
-    out_group[r] = pick;
+    out_group[r] = g->h_sctl->best_id;
+    GC_TRY(launch_round_end(g));
+    GC_TRY(launch_wsearch(g, kWRelabel, &g->sctl->best_id, nullptr, 1, dec, nullptr, kInf));
+    GC_CUDA(cudaMemcpyAsync(&g->h_bctl->decrease, dec, sizeof(long long), cudaMemcpyDeviceToHost, g->stream));
   }
+  GC_TRY(sync(g));
+  if (k > 1) GC_TRY(update_matches(k - 1));
   *out_farness = f;
   if (stats) {
     memset(stats, 0, sizeof(*stats));

@@ -291,6 +291,8 @@ struct gc_graph {
   size_t w_stride = 0;
   int w_ctas = 0;
   unsigned int *w_task = nullptr;
+  int32_t w_max = 0;               // largest weight
+  int32_t *ci_w = nullptr, *wt_w = nullptr;  // the rows ordered by weight (built by gc_set_weights)
   // candidates per batch of the CTA-batched gain kernel (gc_set_gain_lanes):
   // 64, or 128 / 256 for the wide kernel (gc_gain_wide.cu), whose per-CTA
   // workspaces are allocated on first use
@@ -462,17 +464,19 @@ int launch_argmin_lb(gc_graph *g);
 int launch_round0_seed(gc_graph *g);
 // top-k closeness: key <- -f0 for searched vertices; lgain[i] <- f0[list[i]]
 int launch_topk_keys(gc_graph *g);
-// weighted searches (gc_weighted.cu): kWFarness f({v}) of each listed source,
-// kWGain Delta(v|S) of each listed candidate (one CTA per search, out[i] per
-// list entry); kWRelabel d_S <- min(d_S, d(s, .)) in place (one CTA)
+// weighted searches (gc_weighted.cu), one CTA each, of list[0 .. *m_dev or m) or
+// of every vertex 0 .. m - 1 (list == nullptr): kWFarness out[v] <- f({v}) or -1
+// (cut at *best); kWGain out[i] <- Delta(v|S) of list entry i; kWRelabel d_S <-
+// min(d_S, d(list[0], .)) in place, out[0] <- the decrease.  delta: bucket width
+// (0: from *best)
 enum WMode { kWFarness = 0, kWGain = 1, kWRelabel = 2 };
 size_t wws_stride(int32_t n);
-int wsssp_occupancy(int *blocks_per_sm);
-int launch_wsssp(gc_graph *g, int mode, const int32_t *list, const int32_t *m_dev, long long *out,
-                 unsigned int *task);
-int launch_wrelabel(gc_graph *g, const int32_t *src, unsigned long long *decrease);
+int wsearch_occupancy(const gc_graph *g, int *blocks_per_sm);
+int launch_wfar_init(gc_graph *g);
+int launch_wsort(gc_graph *g, int32_t *tmp_ci, int32_t *tmp_wt);
+int launch_wsearch(gc_graph *g, int mode, const int32_t *list, const int32_t *m_dev, int32_t m, long long *out,
+                   long long *best, int32_t delta);
 int launch_wcheck(gc_graph *g, bool mirror, int32_t *bad, int32_t *max_w);
-int launch_iota(gc_graph *g, int32_t *p, int32_t n);
 // bitGreedy++ sweep (gc_bits.cu): mode 0 farness of every vertex, mode 1 gain
 // of every vertex against d_S; B holds 2 n W words and then 2 n bytes (row
 // flags), out n int64; ctl->best

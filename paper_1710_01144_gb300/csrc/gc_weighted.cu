@@ -6,18 +6,11 @@
 // relaxing only into vertices the candidate would bring strictly closer finds
 // the exact distance of every vertex that contributes to the gain.
 //
-// One search per CTA: a frontier-based label-correcting SSSP (parallel
-// Bellman-Ford).  A warp takes a frontier vertex and its row; a relaxation
-// lowers dist[w] with atomicMin and, if it lowered it, puts w into the next
-// frontier once (a queue flag).  A vertex lowered after its warp read it is
-// queued again, so the search ends with exact distances.  Workspace per CTA:
-// dist, two frontier queues, the touched list and the queue flags (20 bytes
-// per vertex); dist is kInf and the flags zero between searches.
-//
-// Modes: kWFarness  f({v}) of each listed source (a full search),
-//        kWGain     Delta(v | S) of each listed candidate against d_S,
-//        kWRelabel  d_S <- min(d_S, d(s, .)) in place from one source (the
-//                   d_S update), the decrease summed for the gain check.
+// One search per CTA (k_wsearch), in distance order.  Modes:
+//   kWFarness  f({v}) of each source, cut by the best farness (round 0);
+//   kWGain     Delta(v | S) of each listed candidate against d_S;
+//   kWRelabel  d_S <- min(d_S, d(s, .)) in place from one source (the d_S
+//              update), the decrease summed for the gain check.
 #include <limits.h>
 
 #include <algorithm>
@@ -27,157 +20,343 @@
 
 namespace gc {
 
-constexpr int kWThreads = 512;
+// Rows ordered by weight (built once per gc_set_weights): one stable counting
+// pass over 8 bits of the weights, a warp per row, 32 entries at a time; equal
+// digits of a tile are ranked by match-any.  LSD passes over all weight bits
+// sort the rows.
+constexpr int kWSortWarps = 8;
 
-struct WWs {
-  int32_t *dist, *q0, *q1, *touched;
-  unsigned int *inq;
-};
-
-__device__ __forceinline__ WWs wws(unsigned char *base, size_t stride, int32_t n, int idx) {
-  unsigned char *p = base + stride * (size_t)idx;
-  const size_t a4 = ws_align((size_t)n * 4);
-  WWs w;
-  w.dist = (int32_t *)p;
-  w.q0 = (int32_t *)(p + a4);
-  w.q1 = (int32_t *)(p + 2 * a4);
-  w.touched = (int32_t *)(p + 3 * a4);
-  w.inq = (unsigned int *)(p + 4 * a4);
-  return w;
-}
-
-size_t wws_stride(int32_t n) { return 5 * ws_align((size_t)n * 4); }
-
-// One search from s by the whole CTA.  d is the distance array the search
-// lowers (the workspace's dist, or d_S itself in kWRelabel); dS (kWGain) the
-// group's distances the search must beat.  Returns, in every thread, the
-// search's sum: farness, gain, or the decrease of d_S.  *reached (thread 0)
-// gets the number of vertices the search lowered from kInf.
-template <int MODE>
-static __device__ long long cta_wsssp(const int32_t *__restrict__ rp, const int32_t *__restrict__ ci,
-                                      const int32_t *__restrict__ wt, int32_t *d, const int32_t *dS,
-                                      const WWs &ws, int s, long long *reached) {
-  __shared__ int s_F, s_nt;
-  __shared__ long long s_red[32];
-  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, nw = blockDim.x >> 5;
-  long long acc = 0;  // kWRelabel: this thread's share of the decrease
-  if (tid == 0) {
-    s_nt = 0;
-    const int old = d[s];
-    d[s] = 0;
-    if (MODE == kWRelabel && old < kInf) acc += old;
-    if (MODE != kWRelabel) ws.touched[s_nt++] = s;
-    ws.q0[0] = s;
-    s_F = 1;
-  }
-  cta_sync();
-  int32_t *cur = ws.q0, *nxt = ws.q1;
-  for (;;) {
-    const int F = s_F;
-    if (F == 0) break;
-    for (int i = tid; i < F; i += blockDim.x) ws.inq[cur[i]] = 0u;  // may be queued again below
-    cta_sync();
-    if (tid == 0) s_F = 0;
-    cta_sync();
-    for (int i = wid; i < F; i += nw) {
-      const int u = cur[i];
-      const int du = __ldcg(&d[u]);  // the latest value (a lower one requeues u)
-      for (int e = rp[u] + lane; e < rp[u + 1]; e += 32) {
-        const int w = ci[e];
-        const int nd = du + wt[e];
-        if (MODE == kWGain && nd >= dS[w]) continue;  // pruned (Sec. 4.1)
-        if (nd >= __ldcg(&d[w])) continue;
-        const int old = atomicMin(&d[w], nd);
-        if (nd < old) {
-          if (MODE == kWRelabel) {
-            if (old < kInf) acc += old - nd;
-          } else if (old == kInf) {
-            ws.touched[atomicAdd(&s_nt, 1)] = w;
-          }
-          if (atomicExch(&ws.inq[w], 1u) == 0u) nxt[atomicAdd(&s_F, 1)] = w;
-        }
+__global__ void __launch_bounds__(32 * kWSortWarps) k_wsort(const int32_t *__restrict__ rp, int32_t n,
+                                                            const int32_t *__restrict__ ci0,
+                                                            const int32_t *__restrict__ wt0, int32_t *ci1,
+                                                            int32_t *wt1, int shift) {
+  __shared__ int s_at[kWSortWarps][256];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  int *at = s_at[wid];
+  for (int v = blockIdx.x * kWSortWarps + wid; v < n; v += gridDim.x * kWSortWarps) {
+    const int e0 = rp[v], e1 = rp[v + 1];
+    for (int i = lane; i < 256; i += 32) at[i] = 0;
+    __syncwarp();
+    for (int e = e0 + lane; e < e1; e += 32) atomicAdd(&at[(wt0[e] >> shift) & 255], 1);
+    __syncwarp();
+    int carry = e0;  // counts -> first slots
+    for (int base = 0; base < 256; base += 32) {
+      const int c = at[base + lane];
+      int incl = c;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += y;
       }
+      at[base + lane] = carry + incl - c;
+      carry += __shfl_sync(0xffffffffu, incl, 31);
     }
-    cta_sync();
-    int32_t *t = cur;
-    cur = nxt;
-    nxt = t;
-  }
-  long long r = 0;
-  if (MODE == kWRelabel) {
-    r = acc;
-  } else {
-    const int nt = s_nt;
-    for (int i = tid; i < nt; i += blockDim.x) {
-      const int w = ws.touched[i];
-      const int dw = __ldcg(&d[w]);
-      r += MODE == kWFarness ? (long long)dw : (long long)(dS[w] - dw);
+    __syncwarp();
+    for (int base = e0; base < e1; base += 32) {
+      const int e = base + lane;
+      const int w = e < e1 ? wt0[e] : 0;
+      const int g = e < e1 ? (w >> shift) & 255 : 256 + lane;  // (idle lanes match nobody)
+      const unsigned same = __match_any_sync(0xffffffffu, g);
+      if (e < e1) {
+        const int slot = at[g] + __popc(same & ((1u << lane) - 1u));
+        ci1[slot] = ci0[e];
+        wt1[slot] = w;
+      }
+      __syncwarp();
+      if (e < e1 && lane == __ffs(same) - 1) at[g] += __popc(same);
+      __syncwarp();
     }
   }
-  r = block_sum(r, s_red);
-  if (tid == 0 && reached) *reached = s_nt;
-  if (MODE != kWRelabel) {  // the workspace back to kInf for the next search
-    const int nt = s_nt;
-    for (int i = tid; i < nt; i += blockDim.x) d[ws.touched[i]] = kInf;
-  }
-  cta_sync();
-  return r;
 }
 
-// Every listed source, one CTA per search, from a task counter.  out[i]: the
-// farness (-1 if the search reached fewer than n vertices: disconnected) or
-// the gain (0 for a member of S).
-template <int MODE>
-__global__ void __launch_bounds__(kWThreads) k_wsssp(const int32_t *__restrict__ rp, const int32_t *__restrict__ ci,
-                                                     const int32_t *__restrict__ wt, int32_t n, const int32_t *dS,
-                                                     const int32_t *list, const int32_t *m_dev, long long *out,
-                                                     unsigned char *ws_base, size_t ws_stride, unsigned int *task,
-                                                     int32_t *err) {
-  __shared__ int s_i;
-  const WWs ws = wws(ws_base, ws_stride, n, blockIdx.x);
-  const int m = *m_dev;
+// A search settles the vertices in buckets [., T): within a bucket it is a
+// label-correcting search that relaxes only the entries with dist[u] + weight <
+// T, a prefix of u's row, since rows are ordered by weight; ptr[u] keeps where
+// the prefix ended, and u stays in the pending list until T has passed its last
+// entry.  At the end of a bucket everything below T is final.  Gains and the d_S
+// update relax only into vertices they bring strictly closer than d_S.
+//
+// Farness, BFScut (Sec. 3.1) on weighted distances: at the end of a bucket every
+// unsettled vertex is at least as far as the nearest pending entry reaches, so
+// with `cnt` settled vertices of distance sum `sum`,
+//   f({v}) >= sum + (nearest pending) (n - cnt),
+// and a search whose bound exceeds the best farness is cut: on R-MAT scale 14
+// with weights in [1, 16] after 11% of the entries on average, where a full
+// search of every vertex reads the whole graph n times over.  Measured, round 0
+// at scale 14 in ms, weights up to 1, 16, 1000: 25, 47, 99 -> 1.7, 11.8, 37; the
+// whole call (k = 50) 34, 60, 119 -> 7.6, 19.5, 47.
+//
+// A search's random accesses are its distances and two flags per vertex.  For
+// 300 to 1,200 searches at a time they do not fit L2 (round 0 at scale 14: 26 ms
+// with them in the workspace, bound by DRAM sectors), so up to kWFarSmemN
+// vertices they live in shared memory (SM: 13 ms; four CTAs of 512 threads per SM
+// at scale 14, one of 1024 beyond 24,000 vertices); the queues and lists in
+// global memory are written and read in order.  Larger graphs keep them in the
+// workspace.
+constexpr int kWFarSmemN = 48000;  // 199 KB, and 13 KB of static arrays at 1024 threads
+constexpr unsigned kWNear = 1u, kWBucket = 2u;  // queued; listed in a bucket (settled at its end)
+
+// per CTA: near queues, pending and bucket lists, ptr, and without SM the
+// distances, the flags and the touched list
+size_t wws_stride(int32_t n) { return 8 * ws_align((size_t)n * 4); }
+static size_t wfar_smem(int32_t n) { return (size_t)n * 4 + 2 * (((size_t)n + 31) / 32) * 4; }
+
+// How a graph is searched: 0 shared memory, 512 threads (two CTAs per SM or
+// more); 1 shared memory, one CTA of 1024 threads per SM; 2 workspace, 512
+// threads.  Between 24,000 and kWFarSmemN vertices, 1 gives up the many CTAs
+// that hide a sparse search's latency and pays off on dense rows only: R-MAT
+// scale 16 (46,693 vertices, 39 entries each) round 0 279 ms by 1, 624 by 2; BA
+// n = 47,000, m = 3, 38 by 1, and n = 49,000 28 by 2.
+static int wform(const gc_graph *g) {
+  if (g->n <= kWFarSmemN / 2) return 0;
+  return g->n <= kWFarSmemN && g->nnz >= 16ll * g->n ? 1 : 2;
+}
+static int wthreads(int mode, int form) { return form == 1 || (form == 0 && mode == kWRelabel) ? 1024 : 512; }
+
+// The workspaces' dist words to kInf and flags to 0.
+__global__ void k_wfar_init(unsigned char *base, size_t stride, int32_t n) {
+  unsigned char *p = base + stride * (size_t)blockIdx.x;
+  const size_t a4 = ws_align((size_t)n * 4);
+  int32_t *d = (int32_t *)(p + 5 * a4);
+  unsigned int *fl = (unsigned int *)(p + 6 * a4);
+  for (int i = threadIdx.x; i < n; i += blockDim.x) {
+    d[i] = kInf;
+    fl[i] = 0u;
+  }
+}
+
+// Sources list[i] (list == nullptr: every vertex i), i < m.  ci, wt: the rows
+// ordered by weight.  delta > 0: the bucket width; 0: from the best farness.
+// kWFarness  out[v]: the farness of source v, -1 if cut; sources whose out[v] is
+//            already >= 0 are skipped.  *best: the smallest farness found so far,
+//            lowered as searches complete.
+// kWGain     out[i]: the gain (0 for a member of S).
+// kWRelabel  out[0]: the decrease of d_S over labels with a finite old value.
+template <int MODE, int TH, bool SM>
+__global__ void __launch_bounds__(TH)
+    k_wsearch(const int32_t *__restrict__ rp, const int32_t *__restrict__ ci, const int32_t *__restrict__ wt,
+              int32_t n, int32_t *dS, const int32_t *list, const int32_t *m_dev, int32_t m_arg, long long *out,
+              unsigned char *ws_base, size_t ws_stride, unsigned int *task, long long *best, int32_t w_max,
+              int32_t delta_arg, int32_t *err) {
+  extern __shared__ __align__(16) int32_t s_dist[];  // SM: distances, then the two flag bitmaps
+  __shared__ int s_i, s_F, s_nt, s_np, s_nb, s_min;
+  __shared__ int s_off[TH], s_e0[TH], s_du[TH];
+  __shared__ int s_scan[33];
+  __shared__ long long s_bst;
+  __shared__ long long s_red[32];
+  const int tid = threadIdx.x, lane = tid & 31;
+  const size_t a4 = ws_align((size_t)n * 4);
+  unsigned char *base_p = ws_base + ws_stride * (size_t)blockIdx.x;
+  auto arr = [&](int k) { return (int32_t *)(base_p + k * a4); };
+  int32_t *q0 = arr(0), *q1 = arr(1), *pend = arr(2), *bucket = arr(3), *ptr = arr(4), *gd = arr(5),
+          *touched = arr(7);
+  unsigned int *fl = (unsigned int *)arr(6);
+  const int nw = (n + 31) / 32;
+  unsigned int *s_near = (unsigned int *)(s_dist + n), *s_buck = s_near + nw;
+  auto dist = [&](int v) -> int { return SM ? *(volatile int32_t *)&s_dist[v] : __ldcg(&gd[v]); };
+  auto lower = [&](int v, int x) -> int { return atomicMin(SM ? &s_dist[v] : &gd[v], x); };
+  // set a flag; true if it was clear
+  auto flag = [&](int v, unsigned f) -> bool {
+    if (SM) return !(atomicOr((f == kWNear ? s_near : s_buck) + (v >> 5), 1u << (v & 31)) & (1u << (v & 31)));
+    return !(atomicOr(&fl[v], f) & f);
+  };
+  auto unqueue = [&](int v) {
+    if (SM) atomicAnd(&s_near[v >> 5], ~(1u << (v & 31)));
+    else atomicAnd(&fl[v], ~kWNear);
+  };
+  const int m = m_dev ? *m_dev : m_arg;
   for (;;) {
-    if (threadIdx.x == 0) s_i = (int)atomicAdd(task, 1u);
+    if (SM) {
+      for (int i = tid; i < n; i += TH) s_dist[i] = kInf;
+      for (int i = tid; i < 2 * nw; i += TH) s_near[i] = 0u;
+    }
+    if (tid == 0) {
+      s_i = (int)atomicAdd(task, 1u);
+      s_bst = MODE == kWFarness ? *(volatile long long *)best : LLONG_MAX;
+    }
     cta_sync();
     const int i = s_i;
+    const long long bst = s_bst;
     cta_sync();
     if (i >= m) break;
-    const int s = list[i];
+    const int s = list ? list[i] : i;
+    if (MODE == kWFarness && out[s] >= 0) continue;  // searched before (uniform)
     if (s < 0 || s >= n) {
-      if (threadIdx.x == 0) {
+      if (tid == 0) {
         out[i] = -1;
         atomicExch(err, GC_EINVAL);
       }
       continue;
     }
     if (MODE == kWGain && dS[s] == 0) {  // a member: no gain
-      if (threadIdx.x == 0) out[i] = 0;
+      if (tid == 0) out[i] = 0;
       continue;
     }
-    long long reached = 0;
-    const long long r = cta_wsssp<MODE>(rp, ci, wt, ws.dist, dS, ws, s, &reached);
-    if (threadIdx.x == 0) {
-      if (MODE == kWFarness && reached != n) {
-        out[i] = -1;
-        atomicExch(err, GC_EDISCONNECTED);
-      } else {
-        out[i] = r;
+    // bucket width: given, or an eighth of the best mean distance
+    const int delta = delta_arg > 0 ? delta_arg
+                      : bst < LLONG_MAX ? (int)max(1ll, bst / (8ll * n)) : max(1, w_max / 4);
+    if (tid == 0) {
+      lower(s, 0);
+      if (!SM) touched[0] = s;
+      flag(s, kWNear);
+      q0[0] = s;
+      s_nt = 1;
+      s_F = 1;
+      s_np = 0;
+    }
+    int T = min(delta, kInf - 1);
+    long long sum = 0, cnt = 0;  // settled: farness, gain or decrease, and vertices (the same in every thread)
+    bool cut = false;
+    int32_t *cur = q0, *nxt = q1;
+    cta_sync();
+    for (;;) {
+      if (tid == 0) s_nb = 0;
+      // ---- one bucket: label-correcting below T ----
+      for (;;) {
+        cta_sync();
+        const int F = s_F;
+        cta_sync();
+        if (F == 0) break;
+        if (tid == 0) s_F = 0;
+        for (int base = 0; base < F; base += TH) {
+          // a thread per queued vertex: its distance (one value for the whole
+          // row; if it is lowered meanwhile the vertex is queued again) and the
+          // part of its row up to T: from the start, or, for a settled vertex
+          // taken up again (queued as ~u), from where the last bucket stopped
+          const int q = base + tid;
+          int du = 0, e0 = 0, len = 0;
+          if (q < F) {
+            const int x = cur[q];
+            const bool again = x < 0;
+            const int u = again ? ~x : x;
+            if (!again) {
+              unqueue(u);
+              if (flag(u, kWBucket)) bucket[atomicAdd(&s_nb, 1)] = u;
+            }
+            du = dist(u);
+            const int e1 = rp[u + 1];
+            e0 = again ? ptr[u] : rp[u];
+            // (one bucket: the whole row)
+            int lo = T == kInf - 1 ? e1 : e0, step = 4;  // galloping: the prefixes are short
+            while (lo + step <= e1 && du + wt[lo + step - 1] < T) {
+              lo += step;
+              step *= 2;
+            }
+            int hi = min(e1, lo + step);
+            while (lo < hi) {
+              const int mid = (lo + hi) >> 1;
+              if (du + wt[mid] < T) lo = mid + 1;
+              else hi = mid;
+            }
+            ptr[u] = lo;
+            len = lo - e0;
+          }
+          int total;
+          const int off = block_excl_scan(len, s_scan, &total);
+          s_off[tid] = off;
+          s_e0[tid] = e0;
+          s_du[tid] = du;
+          cta_sync();
+          // the chunk's entries, spread over the threads
+          for (int e = tid; e < total; e += TH) {
+            int lo = 0, hi = TH - 1;  // largest j with s_off[j] <= e (its row is non-empty)
+            while (lo < hi) {
+              const int mid = (lo + hi + 1) >> 1;
+              if (s_off[mid] <= e) lo = mid;
+              else hi = mid - 1;
+            }
+            const int x = s_e0[lo] + (e - s_off[lo]);
+            const int w = ci[x], nd = s_du[lo] + wt[x];
+            if (MODE != kWFarness && nd >= dS[w]) continue;  // pruned (Sec. 4.1)
+            if (nd >= dist(w)) continue;
+            const int old = lower(w, nd);
+            if (nd >= old) continue;
+            if (!SM && old == kInf) touched[atomicAdd(&s_nt, 1)] = w;
+            if (flag(w, kWNear)) nxt[atomicAdd(&s_F, 1)] = w;
+          }
+          cta_sync();
+        }
+        int32_t *t = cur;
+        cur = nxt;
+        nxt = t;
+      }
+      // ---- everything below T is settled; the pending entries ----
+      const int nb = s_nb, np = s_np;
+      long long x = 0;
+      for (int q = tid; q < nb; q += TH) {
+        const int v = bucket[q], dv = dist(v);
+        if (MODE == kWFarness) {
+          x += dv;
+        } else {
+          const int old = dS[v];
+          if (old < kInf) x += old - dv;
+          if (MODE == kWRelabel) dS[v] = dv;
+        }
+      }
+      x = block_sum(x, s_red);
+      sum += x;
+      cnt += nb;
+      if (MODE == kWFarness && cnt == n) break;  // complete
+      if (tid == 0) {
+        s_np = 0;
+        s_min = kInf;
+      }
+      int mn = kInf;
+      const int all = np + nb;
+      for (int base = 0; base < all; base += TH) {  // in place: reads stay ahead of writes
+        const int q = base + tid;
+        const int u = q < np ? pend[q] : q < all ? bucket[q - np] : -1;
+        bool keep = false;
+        if (u >= 0) {
+          const int e = ptr[u];
+          keep = e < rp[u + 1];
+          if (keep) mn = min(mn, dist(u) + wt[e]);
+        }
+        cta_sync();
+        if (keep) pend[atomicAdd(&s_np, 1)] = u;
+        cta_sync();
+      }
+      mn = __reduce_min_sync(0xffffffffu, mn);
+      if (lane == 0) atomicMin(&s_min, mn);
+      cta_sync();
+      mn = s_min;
+      const int left = s_np;
+      if (left == 0) break;  // nothing more to reach (farness short of n: disconnected)
+      if (MODE == kWFarness && sum + (long long)mn * ((long long)n - cnt) > bst) {
+        cut = true;
+        break;
+      }
+      // ---- the next bucket: rows with an entry below the new T go on ----
+      T = mn > kInf - 1 - delta ? kInf - 1 : mn + delta;
+      for (int q = tid; q < left; q += TH) {
+        const int u = pend[q];
+        if (dist(u) + wt[ptr[u]] < T) cur[atomicAdd(&s_F, 1)] = ~u;
       }
     }
+    cta_sync();
+    if (tid == 0) {
+      if (MODE != kWFarness) {
+        out[i] = sum;
+      } else if (cut) {
+        out[s] = -1;
+      } else if (cnt != n) {
+        out[s] = -1;
+        atomicExch(err, GC_EDISCONNECTED);
+      } else {
+        out[s] = sum;
+        atomicMin(best, sum);
+      }
+    }
+    if (!SM) {  // the workspace back to rest
+      const int nt = s_nt;
+      for (int q = tid; q < nt; q += TH) {
+        const int w = touched[q];
+        gd[w] = kInf;
+        fl[w] = 0u;
+      }
+    }
+    cta_sync();
   }
-}
-
-// d_S update from one source by one CTA, in place; *decrease gets the sum of
-// (old - new) over the lowered labels with a finite old label.
-__global__ void __launch_bounds__(kWThreads) k_wrelabel(const int32_t *__restrict__ rp,
-                                                        const int32_t *__restrict__ ci,
-                                                        const int32_t *__restrict__ wt, int32_t *dS,
-                                                        const int32_t *src, unsigned char *ws_base,
-                                                        size_t ws_stride, int32_t n,
-                                                        unsigned long long *decrease) {
-  const WWs ws = wws(ws_base, ws_stride, n, 0);
-  const long long r = cta_wsssp<kWRelabel>(rp, ci, wt, dS, nullptr, ws, *src, nullptr);
-  if (threadIdx.x == 0) *decrease = (unsigned long long)r;
 }
 
 // weights: w >= 1 everywhere, the same in both rows of an edge (binary search
@@ -214,26 +393,72 @@ __global__ void k_wcheck(const int32_t *__restrict__ rp, const int32_t *__restri
   if (lane == 0 && mx) atomicMax(max_w, mx);
 }
 
-int launch_wsssp(gc_graph *g, int mode, const int32_t *list, const int32_t *m_dev, long long *out,
-                 unsigned int *task) {
-  GC_CUDA(cudaMemsetAsync(task, 0, sizeof(unsigned int), g->stream));
+template <int MODE>
+static const void *wsearch_fn(int form) {
+  return form == 2 ? (const void *)k_wsearch<MODE, 512, false>
+         : wthreads(MODE, form) == 512 ? (const void *)k_wsearch<MODE, 512, true>
+                                       : (const void *)k_wsearch<MODE, 1024, true>;
+}
+
+static const void *wsearch_fn(int mode, int form) {
+  return mode == kWFarness ? wsearch_fn<kWFarness>(form)
+         : mode == kWGain  ? wsearch_fn<kWGain>(form)
+                           : wsearch_fn<kWRelabel>(form);
+}
+
+int launch_wfar_init(gc_graph *g) {
   ++g->launches;
-  const int grid = g->w_ctas;
-  if (mode == kWFarness)
-    k_wsssp<kWFarness><<<grid, kWThreads, 0, g->stream>>>(g->rp, g->ci, g->wt, g->n, g->dS, list, m_dev, out,
-                                                          g->w_ws, g->w_stride, task, &g->sctl->err);
-  else
-    k_wsssp<kWGain><<<grid, kWThreads, 0, g->stream>>>(g->rp, g->ci, g->wt, g->n, g->dS, list, m_dev, out,
-                                                       g->w_ws, g->w_stride, task, &g->sctl->err);
+  k_wfar_init<<<g->w_ctas, 512, 0, g->stream>>>(g->w_ws, g->w_stride, g->n);
   GC_CUDA(cudaGetLastError());
   return GC_OK;
 }
 
-int launch_wrelabel(gc_graph *g, const int32_t *src, unsigned long long *decrease) {
+int launch_wsearch(gc_graph *g, int mode, const int32_t *list, const int32_t *m_dev, int32_t m, long long *out,
+                   long long *best, int32_t delta) {
+  GC_CUDA(cudaMemsetAsync(g->w_task, 0, sizeof(unsigned int), g->stream));
   ++g->launches;
-  k_wrelabel<<<1, kWThreads, 0, g->stream>>>(g->rp, g->ci, g->wt, g->dS, src, g->w_ws, g->w_stride, g->n,
-                                             decrease);
+  const int32_t *rp = g->rp, *ci = g->ci_w, *wt = g->wt_w;
+  int32_t n = g->n, w_max = g->w_max, *err = &g->sctl->err, *dS = g->dS;
+  unsigned char *ws = g->w_ws;
+  size_t stride = g->w_stride;
+  unsigned int *task = g->w_task;
+  void *args[] = {(void *)&rp, (void *)&ci,  (void *)&wt,     (void *)&n,    (void *)&dS,   (void *)&list,
+                  (void *)&m_dev, (void *)&m, (void *)&out, (void *)&ws, (void *)&stride, (void *)&task, (void *)&best,
+                  (void *)&w_max, (void *)&delta, (void *)&err};
+  const int form = wform(g);
+  GC_CUDA(cudaLaunchKernel(wsearch_fn(mode, form), dim3(mode == kWRelabel ? 1 : g->w_ctas), dim3(wthreads(mode, form)),
+                           args, form == 2 ? 0 : wfar_smem(n), g->stream));
+  return GC_OK;
+}
+
+// ci_w, wt_w <- the rows ordered by weight (an LSD pass per 8 bits of w_max;
+// tmp: scratch of nnz entries for ids and weights, used by more than one pass)
+int launch_wsort(gc_graph *g, int32_t *tmp_ci, int32_t *tmp_wt) {
+  int passes = 1;
+  while (passes < 4 && (g->w_max >> (8 * passes)) > 0) ++passes;
+  const int32_t *c0 = g->ci, *w0 = g->wt;
+  for (int p = 0; p < passes; ++p) {
+    const bool last = ((passes - 1 - p) & 1) == 0;  // the last pass lands in ci_w, wt_w
+    int32_t *c1 = last ? g->ci_w : tmp_ci, *w1 = last ? g->wt_w : tmp_wt;
+    ++g->launches;
+    k_wsort<<<g->num_sms * 8, 32 * kWSortWarps, 0, g->stream>>>(g->rp, g->n, c0, w0, c1, w1, 8 * p);
+    c0 = c1;
+    w0 = w1;
+  }
   GC_CUDA(cudaGetLastError());
+  return GC_OK;
+}
+
+int wsearch_occupancy(const gc_graph *g, int *blocks_per_sm) {
+  const int form = wform(g);
+  const size_t smem = form == 2 ? 0 : wfar_smem(g->n);
+  for (int mode : {kWRelabel, kWGain, kWFarness}) {  // the result is the farness searches'
+    if (smem)  // (the limit is the process's, not the graph's: the largest any graph needs)
+      GC_CUDA(cudaFuncSetAttribute(wsearch_fn(mode, form), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                   (int)wfar_smem(kWFarSmemN)));
+    GC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, wsearch_fn(mode, form), wthreads(mode, form),
+                                                          smem));
+  }
   return GC_OK;
 }
 
@@ -241,25 +466,6 @@ int launch_wcheck(gc_graph *g, bool mirror, int32_t *bad, int32_t *max_w) {
   ++g->launches;
   k_wcheck<<<g->num_sms * 8, 256, 0, g->stream>>>(g->rp, g->ci, g->wt, g->n, mirror ? 1 : 0, bad, max_w);
   GC_CUDA(cudaGetLastError());
-  return GC_OK;
-}
-
-__global__ void k_w_iota(int32_t *p, int32_t n) {
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) p[i] = i;
-}
-
-int launch_iota(gc_graph *g, int32_t *p, int32_t n) {
-  ++g->launches;
-  k_w_iota<<<g->num_sms * 4, 256, 0, g->stream>>>(p, n);
-  GC_CUDA(cudaGetLastError());
-  return GC_OK;
-}
-
-int wsssp_occupancy(int *blocks_per_sm) {
-  int a = 0, b = 0;
-  GC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, k_wsssp<kWFarness>, kWThreads, 0));
-  GC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_wsssp<kWGain>, kWThreads, 0));
-  *blocks_per_sm = std::min(a, b);
   return GC_OK;
 }
 
