@@ -810,17 +810,20 @@ int gc_greedy_bits(gc_graph *g, int32_t k, const gc_opts *opts_in, int32_t *out_
   auto t0 = std::chrono::steady_clock::now();
   const int64_t launches0 = g->launches;
   const int32_t n = g->n;
+  const bool small = n <= kBitsCtaN;  // words in shared memory: the sums and the control block borrow the handle's
   const int W = std::min(32, (n + 63) / 64);  // 64 W targets per chunk
   const size_t bytes_B = 2 * (size_t)n * W * sizeof(unsigned long long) + 2 * (size_t)n;  // words, row flags
   const size_t bytes = ws_align(bytes_B) + ws_align((size_t)n * sizeof(long long)) + ws_align(sizeof(BitsCtl));
   unsigned char *mem = nullptr;
-  if (cudaMalloc((void **)&mem, bytes) != cudaSuccess) {
+  if (!small && cudaMalloc((void **)&mem, bytes) != cudaSuccess) {
     cudaGetLastError();
     return fail(GC_ENOMEM, "gc_greedy_bits: device allocation failed");
   }
   unsigned long long *B = (unsigned long long *)mem;
-  long long *out = (long long *)(mem + ws_align(bytes_B));
-  BitsCtl *ctl = (BitsCtl *)(mem + ws_align(bytes_B) + ws_align((size_t)n * sizeof(long long)));
+  static_assert(sizeof(BitsCtl) <= sizeof(BfsCtl), "the BFS control block serves as the sweep's");
+  long long *out = small ? g->ub : (long long *)(mem + ws_align(bytes_B));
+  BitsCtl *ctl = small ? (BitsCtl *)g->bctl
+                       : (BitsCtl *)(mem + ws_align(bytes_B) + ws_align((size_t)n * sizeof(long long)));
   BitsCtl h;
   auto done = [&](int rc) {
     cudaStreamSynchronize(g->stream);
@@ -836,6 +839,43 @@ int gc_greedy_bits(gc_graph *g, int32_t k, const gc_opts *opts_in, int32_t *out_
     return GC_OK;
   };
   int64_t levels = 0;
+  auto finish = [&](int64_t f) {
+    *out_farness = f;
+    if (!stats) return;
+    memset(stats, 0, sizeof(*stats));
+    stats->rounds = k;
+    stats->levels = levels;
+    stats->evals = (int64_t)n * k;
+    stats->kernel_launches = g->launches - launches0;
+    stats->ms_total = std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count();
+  };
+  if (small) {  // every round on the device, the picks read back at the end
+    std::vector<int32_t> pk(k);
+    std::vector<long long> pg(k), pd(k);
+    auto rounds = [&]() -> int {
+      GC_TRY(launch_bits_small(g, k, out, ctl));
+      GC_CUDA(cudaMemcpyAsync(&h, ctl, sizeof(BitsCtl), cudaMemcpyDeviceToHost, g->stream));
+      GC_CUDA(cudaMemcpyAsync(pk.data(), g->picks, (size_t)k * sizeof(int32_t), cudaMemcpyDeviceToHost, g->stream));
+      GC_CUDA(cudaMemcpyAsync(pg.data(), g->pgain, (size_t)k * sizeof(long long), cudaMemcpyDeviceToHost, g->stream));
+      GC_CUDA(cudaMemcpyAsync(pd.data(), g->pdec, (size_t)k * sizeof(long long), cudaMemcpyDeviceToHost, g->stream));
+      GC_TRY(sync(g));
+      if (h.err) return fail(h.err, h.err == GC_EDISCONNECTED ? "graph is disconnected" : "bit-vector sweep failed");
+      return GC_OK;
+    };
+    int rc = rounds();
+    if (rc != GC_OK) return done(rc);
+    levels = (int64_t)h.levels;
+    int64_t f = pg[0];
+    for (int32_t r = 0; r < k; ++r) {
+      if (pg[r] != pd[r])
+        return done(fail(GC_EINTERNAL, "gc_greedy_bits: gain of the pick disagrees with the d_S update (round " +
+                                           std::to_string(r) + ")"));
+      if (r > 0) f -= pg[r];
+      out_group[r] = pk[r];
+    }
+    finish(f);
+    return done(GC_OK);
+  }
   int rc = sweep(0);  // round 0: s0 = argmin (farness, id)
   if (rc != GC_OK) return done(rc);
   levels += (int64_t)h.levels;
@@ -863,15 +903,7 @@ int gc_greedy_bits(gc_graph *g, int32_t k, const gc_opts *opts_in, int32_t *out_
     f -= gain;
     out_group[r] = pick;
   }
-  *out_farness = f;
-  if (stats) {
-    memset(stats, 0, sizeof(*stats));
-    stats->rounds = k;
-    stats->levels = levels;
-    stats->evals = (int64_t)n * k;
-    stats->kernel_launches = g->launches - launches0;
-    stats->ms_total = std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count();
-  }
+  finish(f);
   return done(GC_OK);
 }
 

@@ -24,7 +24,18 @@
 // the sweep for target t is a BFS from t cut at depth d_S[t] - 1, the pruned
 // SSSP of Sec. 4.1 seen from the other end.
 //
-// One cooperative launch per round; every level ends with a grid barrier.
+// Up to kBitsCtaN vertices (k_bits_cta): a CTA takes 32 targets, and the words
+// of all vertices (two buffers of n 32-bit words) and the sums fit its shared
+// memory.  The sweep of a CTA's targets needs no other CTA, so a level ends with
+// a CTA barrier and its neighbour words are shared-memory reads; k_bits_pick, one
+// CTA, then takes the best vertex and updates d_S, so the rounds follow one
+// another on the stream without a host round trip.  Bound by the latency of a
+// level (row pointers, columns, words, one barrier).  Measured in ms, k = 50
+// (the last: k = 20), against the chunks below: road-like 64 x 64 34.0 -> 7.0; BA
+// 2000, m = 5, 7.4 -> 2.3; R-MAT scale 12 30.7 -> 5.6, scale 14 89.6 -> 11.7.
+//
+// Above that (k_bits_round): chunks of 64 W targets in global memory, one
+// cooperative launch per round, every level ends with a grid barrier.
 #include <limits.h>
 #include <string.h>
 
@@ -41,6 +52,213 @@ namespace gc {
 typedef unsigned long long u64;
 
 constexpr int kBitsThreads = 256;
+
+// 32 targets per CTA: targets [32 b, 32 b + 32).  MODE and sums as in
+// k_bits_round below; out starts at zero.
+constexpr int kBitsCtaThreads = 1024;
+
+template <int MODE>
+__global__ void __launch_bounds__(kBitsCtaThreads) k_bits_cta(const int32_t *__restrict__ rp,
+                                                              const int32_t *__restrict__ ci, int32_t n,
+                                                              const int32_t *__restrict__ dS, long long *out,
+                                                              BitsCtl *ctl) {
+  extern __shared__ uint32_t s_bits[];  // two word buffers and the sums, n each
+  const int tid = threadIdx.x, lane = tid & 31, T = kBitsCtaThreads;
+  uint32_t *cur = s_bits, *nxt = s_bits + n;
+  int32_t *sum = reinterpret_cast<int32_t *>(s_bits + 2 * (size_t)n);
+  const int base = 32 * blockIdx.x, cs = min(32, n - base);
+  // every warp keeps the targets' d_S, one per lane (farness: never reached)
+  const int dt = lane < cs ? (MODE == 0 ? INT_MAX : __ldg(dS + base + lane)) : 0;
+  for (int u = tid; u < n; u += T) {
+    const bool own = u >= base && u < base + cs;
+    const bool in = own && (MODE == 0 || __ldg(dS + u) > 0);
+    cur[u] = in ? 1u << (u - base) : 0u;
+    sum[u] = MODE == 0 ? cs - (own ? 1 : 0) : (in ? 1 : 0);  // level 0
+  }
+  cta_sync();
+  int i = 1;
+  for (; i <= n; ++i) {
+    const uint32_t mask = __ballot_sync(0xffffffffu, dt > i);  // the targets still counted at level i
+    if (mask == 0u) break;  // (the same in every warp)
+    bool chg = false;
+    // a thread per row of at most 32 entries, the warp together for longer ones
+    for (int w0 = tid & ~31; w0 < n; w0 += T) {
+      const int u = w0 + lane;
+      uint32_t own = 0u, x = 0u;
+      int r0 = 0, r1 = 0;
+      if (u < n) {
+        own = x = cur[u];
+        if ((own & mask) != mask) {  // (else every counted target is in already)
+          r0 = __ldg(rp + u);
+          r1 = __ldg(rp + u + 1);
+        }
+      }
+      const bool lng = r1 - r0 > 32;
+      if (!lng) {
+        for (int e = r0; e < r1; e += 4) {
+          int v[4];
+#pragma unroll
+          for (int k = 0; k < 4; ++k) v[k] = e + k < r1 ? __ldg(ci + e + k) : u;
+#pragma unroll
+          for (int k = 0; k < 4; ++k) x |= cur[v[k]];
+        }
+      }
+      for (unsigned m = __ballot_sync(0xffffffffu, lng); m; m &= m - 1) {
+        const int q = __ffs(m) - 1;
+        const int a = __shfl_sync(0xffffffffu, r0, q), b = __shfl_sync(0xffffffffu, r1, q);
+        uint32_t y = 0u;
+        for (int e = a + lane; e < b; e += 32) y |= cur[__ldg(ci + e)];
+        y = __reduce_or_sync(0xffffffffu, y);
+        if (lane == q) x |= y;
+      }
+      if (u < n) {
+        x &= mask;
+        nxt[u] = x;
+        const int pc = __popc(x);
+        sum[u] += MODE == 1 ? pc : cs - pc;
+        chg |= x != (own & mask);
+      }
+    }
+    uint32_t *t = cur;
+    cur = nxt;
+    nxt = t;
+    // farness: once no word changed, every later level adds nothing
+    __syncwarp();
+    const int any = __syncthreads_or(chg ? 1 : 0);
+    if (MODE == 0 && !any) break;
+  }
+  for (int u = tid; u < n; u += T)
+    if (sum[u]) atomicAdd(reinterpret_cast<u64 *>(&out[u]), (u64)(long long)sum[u]);
+  if (tid == 0) atomicAdd(&ctl->levels, (u64)i);
+}
+
+// One CTA: the round's pick from the sums (MODE 0 the smallest farness, MODE 1
+// the largest gain among u with d_S[u] > 0; ties: smaller id) to picks[r] and
+// pgain[r], the sums back to zero, and d_S updated by the pruned relabel BFS from
+// the pick (Sec. 4.1; MODE 0: a fresh BFS), its decrease (MODE 0: the farness) to
+// pdec[r].  A vertex that round 0 does not reach: *err.
+template <int MODE>
+__global__ void __launch_bounds__(kBitsCtaThreads) k_bits_pick(const int32_t *__restrict__ rp,
+                                                               const int32_t *__restrict__ ci, int32_t n, int32_t *dS,
+                                                               long long *out, int32_t r, int32_t *picks,
+                                                               long long *pgain, long long *pdec, int32_t *err) {
+  extern __shared__ uint32_t s_bits[];  // the BFS queue: every relabelled vertex in BFS order
+  __shared__ long long s_v[32];
+  __shared__ int s_id[32];
+  __shared__ int s_n;
+  int32_t *q = reinterpret_cast<int32_t *>(s_bits);
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, T = kBitsCtaThreads;
+  long long bv = LLONG_MIN;
+  int bid = -1;
+  for (int u = tid; u < n; u += T) {
+    const long long v = MODE == 0 ? -out[u] : (dS[u] > 0 ? out[u] : LLONG_MIN);
+    out[u] = 0;
+    if (v != LLONG_MIN && better_max(v, u, bv, bid)) {
+      bv = v;
+      bid = u;
+    }
+    if (MODE == 0) dS[u] = kInf;
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const long long ov = __shfl_xor_sync(0xffffffffu, bv, o);
+    const int oid = __shfl_xor_sync(0xffffffffu, bid, o);
+    if (better_max(ov, oid, bv, bid)) {
+      bv = ov;
+      bid = oid;
+    }
+  }
+  if (lane == 0) {
+    s_v[wid] = bv;
+    s_id[wid] = bid;
+  }
+  cta_sync();
+  bv = s_v[0];
+  bid = s_id[0];
+  for (int w = 1; w < T / 32; ++w)
+    if (better_max(s_v[w], s_id[w], bv, bid)) {
+      bv = s_v[w];
+      bid = s_id[w];
+    }
+  cta_sync();  // (s_v is the reduction scratch below)
+  if (bid < 0) {  // no vertex left: k <= n rules it out
+    if (tid == 0) atomicExch(err, GC_EINTERNAL);
+    return;
+  }
+  long long dec = 0;
+  if (tid == 0) {
+    picks[r] = bid;
+    pgain[r] = MODE == 0 ? -bv : bv;
+    if (MODE == 1) dec = dS[bid];
+    dS[bid] = 0;
+    q[0] = bid;
+    s_n = 1;
+  }
+  cta_sync();
+  int a = 0, b = 1;
+  for (int nd = 1; a < b; ++nd) {  // the vertices at distance nd - 1 are q[a..b)
+    auto claim = [&](int w) {
+      if (nd >= *(volatile int32_t *)&dS[w]) return;
+      const int old = atomicMin(&dS[w], nd);
+      if (old <= nd) return;
+      dec += MODE == 0 ? (long long)nd : (long long)(old - nd);
+      q[atomicAdd(&s_n, 1)] = w;
+    };
+    for (int i0 = a + (tid & ~31); i0 < b; i0 += T) {
+      const int i = i0 + lane;
+      int r0 = 0, r1 = 0;
+      if (i < b) {
+        r0 = __ldg(rp + q[i]);
+        r1 = __ldg(rp + q[i] + 1);
+      }
+      const bool lng = r1 - r0 > 32;
+      if (!lng)
+        for (int e = r0; e < r1; ++e) claim(__ldg(ci + e));
+      for (unsigned m = __ballot_sync(0xffffffffu, lng); m; m &= m - 1) {
+        const int t = __ffs(m) - 1;
+        const int x = __shfl_sync(0xffffffffu, r0, t), y = __shfl_sync(0xffffffffu, r1, t);
+        for (int e = x + lane; e < y; e += 32) claim(__ldg(ci + e));
+      }
+    }
+    cta_sync();
+    a = b;
+    b = s_n;
+    cta_sync();
+  }
+  dec = block_sum(dec, s_v);
+  if (tid == 0) {
+    pdec[r] = dec;
+    if (MODE == 0 && b != n) atomicExch(err, GC_EDISCONNECTED);
+  }
+}
+
+// k rounds of bitGreedy++ on a graph of at most kBitsCtaN vertices, enqueued on
+// the handle's stream: picks, gains (round 0: the farness) and d_S decreases to
+// g->picks, g->pgain, g->pdec; out (n sums) and ctl are zeroed here.
+int launch_bits_small(gc_graph *g, int32_t k, long long *out, BitsCtl *ctl) {
+  const int n = g->n, grid = (n + 31) / 32;
+  const size_t smem = (size_t)n * 12, smem_q = (size_t)n * 4;
+  GC_CUDA(cudaMemsetAsync(ctl, 0, sizeof(BitsCtl), g->stream));
+  GC_CUDA(cudaMemsetAsync(out, 0, (size_t)n * sizeof(long long), g->stream));
+  for (const void *f : {(const void *)k_bits_cta<0>, (const void *)k_bits_cta<1>})
+    GC_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, kBitsCtaN * 12));
+  for (const void *f : {(const void *)k_bits_pick<0>, (const void *)k_bits_pick<1>})
+    GC_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, kBitsCtaN * 4));
+  g->launches += 2 * k;
+  for (int32_t r = 0; r < k; ++r) {
+    if (r == 0) {
+      k_bits_cta<0><<<grid, kBitsCtaThreads, smem, g->stream>>>(g->rp, g->ci, n, g->dS, out, ctl);
+      k_bits_pick<0><<<1, kBitsCtaThreads, smem_q, g->stream>>>(g->rp, g->ci, n, g->dS, out, r, g->picks, g->pgain,
+                                                                g->pdec, &ctl->err);
+    } else {
+      k_bits_cta<1><<<grid, kBitsCtaThreads, smem, g->stream>>>(g->rp, g->ci, n, g->dS, out, ctl);
+      k_bits_pick<1><<<1, kBitsCtaThreads, smem_q, g->stream>>>(g->rp, g->ci, n, g->dS, out, r, g->picks, g->pgain,
+                                                                g->pdec, &ctl->err);
+    }
+  }
+  GC_CUDA(cudaGetLastError());
+  return GC_OK;
+}
 
 // MODE 0: out[u] += sum_i (cs - |b^i_u|) over the chunk (farness, S empty).
 // MODE 1: out[u] += sum_i |b^i_u AND NOT b^i_S| over the chunk (gains).

@@ -157,6 +157,7 @@ struct BitsCtl {
   unsigned long long best;    // packed arg-best of the round
   unsigned long long levels;  // levels swept, summed over the target chunks
 };
+constexpr int32_t kBitsCtaN = 16000;  // up to here a CTA holds the words and sums of 32 targets (12 bytes per vertex)
 constexpr int32_t kBitsMaxN = 65536;  // bit-vector variant: packed 32-bit values (farness < 2^31)
 
 // One entry of the claim log of the persistent lazy kernel: at BFS level
@@ -483,6 +484,7 @@ int launch_wcheck(gc_graph *g, bool mirror, int32_t *bad, int32_t *max_w);
 // gets the packed arg-best (see k_bits_argbest)
 int launch_bits_round(gc_graph *g, int mode, unsigned long long *B, long long *out, BitsCtl *ctl, int W,
                       int64_t tns);
+int launch_bits_small(gc_graph *g, int32_t k, long long *out, BitsCtl *ctl);
 int launch_gather_f0(gc_graph *g);
 int launch_round_begin(gc_graph *g);
 int launch_round_end(gc_graph *g);
