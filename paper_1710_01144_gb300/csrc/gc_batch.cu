@@ -1011,7 +1011,8 @@ static __device__ bool team_lazy(const BatchArgs &a, int g, TeamCtl *tc, Team tm
     const u64 l0 = *(volatile u64 *)&lc->best_seg0, l1 = *(volatile u64 *)&lc->best_seg1;
     if (!wide && blane >= 0 && blane < kLanes && l0 <= l1 && l1 <= clog_cap) {
       const u64 bit = 1ull << blane;
-      u64 dec_sum = 0;
+      u64 dec_sum = 0, rel = 0;
+      log_update_row(a.rpf, a.cif, a.dS, pick, dec_sum, rel, tm);
       for (u64 i = l0 + (u64)b * blockDim.x + tid; i < l1; i += (u64)tm.G * blockDim.x) {
         const int4 e = *reinterpret_cast<const int4 *>(clog + i);
         if (!(((u64)(unsigned)e.z | ((u64)(unsigned)e.w << 32)) & bit)) continue;

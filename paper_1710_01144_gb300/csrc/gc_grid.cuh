@@ -76,7 +76,8 @@ static __device__ __forceinline__ int warp_find_start(const int32_t *start, int 
 // kBatchRest then runs the rest in every CTA, after a grid barrier the caller
 // placed between the two.  kBatchAll does both with a barrier of its own.
 // With `log` (gain mode), every claim that wins lanes at level L >= 1 appends
-// {w, L, lanes won} at *log_n (one warp-aggregated slot per claim round); slots
+// {w, L, lanes won}, except the neighbours of a candidate at d_S = 2 (see below:
+// a pick's row holds them, log_update_row), at *log_n (one warp-aggregated slot per claim round); slots
 // at or past log_cap are counted in *log_n but not written.
 // With `acc`, each thread adds its work counts (scalar and union adjacency
 // entries, frontier entries, pushes) to *acc instead of the batch summing them
@@ -108,6 +109,7 @@ static __device__ __forceinline__ bool grid_gain_batch(const int32_t *__restrict
   __shared__ int s_go[T + 1];  // staged entries: start of each entry's range in the level's edge space
   __shared__ int s_rs[T];
   __shared__ u64 s_sm[T];
+  __shared__ int s_c3[MODE == kModeGain ? T : 1];  // level 0: entries of the row whose d_S was >= 3 at the build
   __shared__ int s_x0;
   __shared__ u64 s_red[32];
   // farness mode: running per-lane distance sums and counts, and the level's sums
@@ -253,6 +255,7 @@ static __device__ __forceinline__ bool grid_gain_batch(const int32_t *__restrict
           s_go[tid] = qstart[xi];
           s_sm[tid] = m;
           s_rs[tid] = __ldg(rp + u);
+          if (MODE == kModeGain) s_c3[tid] = (L == 0 && c3) ? __ldg(c3 + u) : INT_MAX;
           if (s_go[tid] >= es && s_go[tid] < ee) {  // counted once: by the CTA holding the entry's first edge
             const int deg = (c3 && L > 0) ? __ldg(c3 + u) : __ldg(rp + u + 1) - s_rs[tid];
             c_union += (u64)deg;
@@ -266,11 +269,13 @@ static __device__ __forceinline__ bool grid_gain_batch(const int32_t *__restrict
         for (long long e0 = a0 + (long long)(tid & ~31) * kGridIlp; e0 < a1; e0 += (long long)T * kGridIlp) {
           // kGridIlp entries per thread: loads of all are issued before any claim
           int w[kGridIlp], sl[kGridIlp];
+          bool two[kGridIlp];  // d_S[w] <= 2 by its place in the row
 #pragma unroll
           for (int k = 0; k < kGridIlp; ++k) {
             const long long e = e0 + k * 32 + lane;
             w[k] = -1;
             sl[k] = 0;
+            two[k] = false;
             if (e < a1) {
               int l = 0, h = cntx - 1;  // staged entry holding e (every entry's range is non-empty)
               while (l < h) {
@@ -280,6 +285,7 @@ static __device__ __forceinline__ bool grid_gain_batch(const int32_t *__restrict
               }
               sl[k] = l;
               w[k] = __ldg(ci + s_rs[l] + (int)(e - s_go[l]));
+              if (MODE == kModeGain) two[k] = (int)(e - s_go[l]) >= s_c3[l];
             }
           }
           // everything indexed by the neighbour is loaded at once: d_S, the
@@ -293,8 +299,8 @@ static __device__ __forceinline__ bool grid_gain_batch(const int32_t *__restrict
             const bool ok = w[k] >= 0;
             dw[k] = (MODE == kModeGain && ok) ? dS[w[k]] : 0;
             mxw[k] = (MODE == kModeGain && mx && ok) ? __ldg(mx + w[k]) : INT_MAX;
-            lw[k] = ok ? row_len(rp, c3, w[k], nlev) : 0;
-            vp[k] = ok ? __ldcg(&ws.vis[w[k] - voff]) : 0ull;
+            lw[k] = ok && !two[k] ? row_len(rp, c3, w[k], nlev) : 0;
+            vp[k] = ok && !two[k] ? __ldcg(&ws.vis[w[k] - voff]) : 0ull;
           }
           u64 nb[kGridIlp];
 #pragma unroll
@@ -310,22 +316,31 @@ static __device__ __forceinline__ bool grid_gain_batch(const int32_t *__restrict
           // lane that reaches w at this level (won here or by a concurrent
           // claim), and the thread that finds the word empty queues w.  w is
           // expanded at level nlev only if some neighbour may still be claimed.
+          // A neighbour at d_S = 2 of a candidate (level 0) gains 1 and that is
+          // all: no later level can claim it (that takes d_S > 2), and the row
+          // holds it once.  So it is neither marked visited nor logged; the d_S
+          // update takes such vertices from the pick's own row.  They are most of
+          // a batch's claims, each otherwise two atomics on a random 32-byte
+          // record and a log entry: lazy rounds of R-MAT scale 24 (283 MB of
+          // records, beyond L2) 20.6 -> 15.4 ms, of scale 20 7.40 -> 6.56 ms.
           u64 ov[kGridIlp], on[kGridIlp];
 #pragma unroll
           for (int k = 0; k < kGridIlp; ++k) {
-            ov[k] = nb[k] ? atomicOr(&ws.vis[w[k] - voff], nb[k]) : ~0ull;
+            two[k] = MODE == kModeGain && L == 0 && dw[k] == 2;
+            ov[k] = !nb[k] ? ~0ull : two[k] ? 0ull : atomicOr(&ws.vis[w[k] - voff], nb[k]);
             on[k] = (nb[k] && mxw[k] > nlev + 1) ? atomicOr(&nxt[w[k] - voff], nb[k]) : ~0ull;
           }
 #pragma unroll
           for (int k = 0; k < kGridIlp; ++k) {
             u64 won = nb[k] & ~ov[k];
-            const bool fresh = won && ov[k] == 0;
+            const bool fresh = won && ov[k] == 0 && !two[k];
             const bool q = on[k] == 0ull;
+            if (MODE == kModeGain && q && two[k]) lw[k] = row_len(rp, c3, w[k], nlev);
             // the warp's appends -- next frontier (slot and range start),
             // touched list, claim log -- take their slots by atomics that lane
             // 0 issues together, so that their round trips overlap
             const unsigned qm = __ballot_sync(0xffffffffu, q), fm = __ballot_sync(0xffffffffu, fresh);
-            const unsigned lm = (MODE == kModeGain && log) ? __ballot_sync(0xffffffffu, won != 0ull) : 0u;
+            const unsigned lm = (MODE == kModeGain && log) ? __ballot_sync(0xffffffffu, won != 0ull && !two[k]) : 0u;
             const int deg = q ? lw[k] : 0;
             int incl = deg;  // inclusive prefix of the degrees over the queueing lanes
             if (qm) {
@@ -359,7 +374,7 @@ static __device__ __forceinline__ bool grid_gain_batch(const int32_t *__restrict
             }
             if (lm) {
               bl = __shfl_sync(0xffffffffu, bl, 0) + (unsigned long long)__popc(lm & below);
-              if (won && bl < log_cap)
+              if (won && !two[k] && bl < log_cap)
                 *reinterpret_cast<int4 *>(log + bl) =
                     make_int4(w[k], nlev, (int)(unsigned)won, (int)(unsigned)(won >> 32));
             }
@@ -505,6 +520,23 @@ static __device__ __forceinline__ bool grid_gain_batch(const int32_t *__restrict
   }
   if (!ok2 && b == 0 && tid == 0) atomicExch(&gctl->err, GC_ETIMEOUT);
   return ok2;
+}
+
+// The part of a d_S update from the claim log that the log leaves out: the
+// neighbours of the pick at d_S = 2 drop to 1.  Adds to this thread's decrease
+// and relabel counts.  Every CTA of the team, the last one first: short rows
+// fall to CTAs that the log's entries leave idle.
+static __device__ __forceinline__ void log_update_row(const int32_t *__restrict__ rp, const int32_t *__restrict__ ci,
+                                                      int32_t *dS, int pick, u64 &dec, u64 &rel, Team tm) {
+  const int r0 = __ldg(rp + pick), r1 = __ldg(rp + pick + 1);
+  for (int e = r0 + (tm.G - 1 - tm.b) * (int)blockDim.x + (int)threadIdx.x; e < r1; e += tm.G * (int)blockDim.x) {
+    const int w = __ldg(ci + e);
+    if (dS[w] != 2) continue;
+    if (atomicMin(&dS[w], 1) == 2) {
+      ++dec;
+      ++rel;
+    }
+  }
 }
 
 // Relabel BFS over the whole grid: dist[w] <- min(dist[w], level) from the

@@ -214,6 +214,7 @@ __global__ void __launch_bounds__(kGridGainThreads, 1)
       // from the claim log: the pick's lane, in the entries of its batch
       const u64 bit = 1ull << blane;
       u64 dec = 0, rel = 0;
+      log_update_row(rp, ci, dS, *(volatile int32_t *)&lc->best_id, dec, rel, whole_grid());
       for (unsigned long long i = s0 + (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x; i < s1;
            i += (unsigned long long)gridDim.x * blockDim.x) {
         const int4 e = *reinterpret_cast<const int4 *>(clog + i);
