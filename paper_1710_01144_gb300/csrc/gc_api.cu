@@ -147,11 +147,14 @@ static int device_errors(gc_graph *g) {
 // d_S <- BFS from the device array seeds[0..n_seeds); checks connectivity.
 static int distances_from(gc_graph *g, const int32_t *seeds_dev, int32_t n_seeds, int64_t tns,
                           int64_t *farness) {
-  GC_TRY(launch_fill_i32(g, g->dS, kInf, g->n));
-  GC_TRY(launch_bfs_relabel(g, g->dS, seeds_dev, n_seeds, tns));
-  GC_TRY(launch_sum_dist(g, g->dS));
-  GC_TRY(read_ctl(g));
-  if (g->h_bctl->err) return device_errors(g);
+  GC_TRY(launch_bfs(g, g->dS, seeds_dev, n_seeds, tns, true));
+  GC_CUDA(cudaMemcpyAsync(g->h_sctl, g->sctl, sizeof(SelCtl), cudaMemcpyDeviceToHost, g->stream));
+  GC_CUDA(cudaMemcpyAsync(g->h_bctl, g->bctl, sizeof(BfsCtl), cudaMemcpyDeviceToHost, g->stream));
+  GC_TRY(sync(g));
+  if (g->h_bctl->err) {
+    GC_TRY(read_ctl(g));
+    return device_errors(g);
+  }
   if (g->h_sctl->count != 0)
     return fail(GC_EDISCONNECTED, "graph is disconnected: the BFS from " + std::to_string(n_seeds) +
                                       " seed(s) left " + std::to_string(g->h_sctl->count) + " of " +
@@ -355,7 +358,6 @@ int gc_group_farness(gc_graph *g, const int32_t *S, int32_t s_len, int64_t *out_
     return fail(GC_EINVAL, "bad argument to gc_group_farness");
   GC_TRY(check_ids(g, S, s_len, "S"));
   GC_CUDA(cudaMemcpyAsync(g->io_a, S, (size_t)s_len * sizeof(int32_t), cudaMemcpyHostToDevice, g->stream));
-  GC_CUDA(cudaMemsetAsync(g->bctl, 0, sizeof(BfsCtl), g->stream));
   return distances_from(g, g->io_a, s_len, timeout_ns(nullptr), out_farness);
 }
 
@@ -366,8 +368,7 @@ static int gains_core(gc_graph *g, const int32_t *S_dev, int32_t s_len, const in
   if (check) {
     GC_TRY(distances_from(g, S_dev, s_len, timeout_ns(nullptr), nullptr));
   } else {
-    GC_TRY(launch_fill_i32(g, g->dS, kInf, g->n));
-    GC_TRY(launch_bfs_relabel(g, g->dS, S_dev, s_len, timeout_ns(nullptr)));
+    GC_TRY(launch_bfs(g, g->dS, S_dev, s_len, timeout_ns(nullptr), true));
   }
   // How deep the graph is is known on the device only: two launches, one of
   // which does the work (the other ends at once).  Distances to a group of more
@@ -894,7 +895,7 @@ int gc_greedy_bits(gc_graph *g, int32_t k, const gc_opts *opts_in, int32_t *out_
     const long long gain = (long long)(h.best >> 32);
     // d_S <- min(d_S, d(pick, .)) by the pruned relabel BFS; its decrease is the gain
     GC_CUDA(cudaMemcpyAsync(g->io_a, &pick, sizeof(int32_t), cudaMemcpyHostToDevice, g->stream));
-    if ((rc = launch_bfs_relabel(g, g->dS, g->io_a, 1, tns)) != GC_OK) return done(rc);
+    if ((rc = launch_bfs(g, g->dS, g->io_a, 1, tns, false)) != GC_OK) return done(rc);
     if ((rc = read_ctl(g)) != GC_OK) return done(rc);
     if (g->h_bctl->err) return done(device_errors(g));
     if ((long long)g->h_bctl->decrease != gain)
@@ -1357,8 +1358,7 @@ int gc_greedy(gc_graph *g, int32_t k, const gc_opts *opts_in, int32_t *out_group
     const int32_t pick = g->h_sctl->best_id;
     gains_picked[r] = g->h_sctl->best_gain;
     GC_TRY(launch_round_end(g));
-    GC_CUDA(cudaMemsetAsync(g->bctl, 0, sizeof(BfsCtl), g->stream));
-    GC_TRY(launch_bfs_relabel(g, g->dS, &g->sctl->best_id, 1, tns, pruned));
+    GC_TRY(launch_bfs(g, g->dS, &g->sctl->best_id, 1, tns, false, pruned));
     GC_CUDA(cudaMemcpyAsync(&g->h_bctl->decrease, &g->bctl->decrease, 2 * sizeof(unsigned long long),
                             cudaMemcpyDeviceToHost, g->stream));
     GC_TRY(sync(g));

@@ -99,7 +99,11 @@ struct BfsCtl {
   int32_t levels;       // levels completed
   unsigned long long decrease;  // sum over relabelled vertices of (old - new), old finite
   unsigned long long relabelled;
-  int32_t blk_tot[kMaxGridCtas];  // per-CTA adjacency totals of the level
+  unsigned long long local_pk;  // the frontier that local levels ended with
+  unsigned long long list;  // a frontier collected after bottom-up levels (counts as in pk)
+  long long seen, esum, sum;  // after local levels: vertices, adjacency entries and distances so far
+  int32_t lev;          // and the level reached
+  int32_t pad;
 };
 
 // Gain-kernel control block.  batch_next is zeroed before every launch; err,
@@ -391,13 +395,14 @@ int cuda_fail(cudaError_t e, const char *what);
   } while (0)
 
 // ------------------------------------------------------------ launches -----
-// Grid-wide relabel BFS: dist[w] <- min(dist[w], level) from the seeds,
-// expanding only where the label decreased.  dist must already hold either
-// kInf (fresh BFS) or the current d_S (pruned update, Sec. 4.1).
+// Grid-wide BFS from the device array seeds[0..n_seeds).  fresh: dist <- the
+// distances, sctl->sum and sctl->count their sum and the unreached vertices (if
+// g->sctl).  Otherwise dist holds d_S and becomes min(d_S, d(seeds, .)) (pruned
+// update, Sec. 4.1).
 // pruned: use the pruned adjacency (g->rpf, g->cif, g->c3; valid only for
 // d_S updates after it was built from an earlier d_S) instead of the full CSR.
-int launch_bfs_relabel(gc_graph *g, int32_t *dist, const int32_t *seeds, int32_t n_seeds,
-                       int64_t timeout_ns, bool pruned = false);
+int launch_bfs(gc_graph *g, int32_t *dist, const int32_t *seeds, int32_t n_seeds, int64_t timeout_ns, bool fresh,
+               bool pruned = false);
 int launch_fill_i32(gc_graph *g, int32_t *p, int32_t v, int64_t count);
 int launch_fill_i64(gc_graph *g, long long *p, long long v, int64_t count);
 // sum of dist and count of unreached -> sctl->sum, sctl->count
@@ -417,7 +422,7 @@ enum GainMode { kModeGain = 0, kModeFarness = 1 };
 // n_cand_dev (optional) overrides n_cand with a count held in device memory.
 // lanes: candidates per batch (1..64); fewer lanes spread one step's work
 // over more CTAs.
-// pruned (gain mode only): the pruned adjacency, as for launch_bfs_relabel.
+// pruned (gain mode only): the pruned adjacency, as for launch_bfs.
 // fresh_ctl: *gctl has just been zeroed (so batch_next need not be).
 // shallow_only: does nothing if the BFS that filled d_S had more than
 // kWideLevels levels (launch_solo beside it does the work).

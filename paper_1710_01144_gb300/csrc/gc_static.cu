@@ -160,8 +160,7 @@ extern "C" int gc_marginal_gains_static(int32_t n, const int32_t *row_ptr, const
     set_error("cudaMemsetAsync on the static scratch failed");
     return GC_ECUDA;
   }
-  if ((rc = launch_fill_i32(&g, g.dS, kInf, n)) != GC_OK) return rc;
-  if ((rc = launch_bfs_relabel(&g, g.dS, S, s_len, 10000000000LL)) != GC_OK) return rc;
+  if ((rc = launch_bfs(&g, g.dS, S, s_len, 10000000000LL, true)) != GC_OK) return rc;
   if ((rc = launch_gains(&g, kModeGain, cand, n_cand, nullptr, (long long *)out_gain, 0)) != GC_OK) return rc;
   if (n_cand > 0) {
     const int blocks = (n_cand + 255) / 256 < 4 * g.num_sms ? (n_cand + 255) / 256 : 4 * g.num_sms;
