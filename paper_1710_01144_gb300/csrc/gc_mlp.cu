@@ -1,8 +1,7 @@
 // Kernels and C ABI of the candidate-proposal network (gc_mlp.cuh):
-// features, forward, backward (activations + weight-gradient reductions),
-// Adam, and a minibatch training loop -- all hand-written float32 kernels on
-// CUDA cores (the network is 4801 parameters; there is no dense contraction
-// large enough for tensor cores to matter).
+// features, forward, gradient, Adam, and a minibatch training loop -- all
+// float32 kernels on CUDA cores (the tensor cores hold no float32 product, and
+// the proposal's training is specified in float32).
 #include <limits.h>
 #include <math.h>
 #include <string.h>
@@ -18,14 +17,13 @@
 struct gc_mlp {
   int32_t max_batch = 0;
   cudaStream_t stream = nullptr;
-  float *params = nullptr;  // [kMlpParams]
-  float *grad = nullptr;    // [kMlpParams]
+  int slots = 0;                     // CTAs of the tile kernels that are resident at once
+  float *params = nullptr;           // [kMlpParams]
+  float *grad = nullptr;             // [kMlpGradLen]: the gradient, then the loss
   float *adam_m = nullptr, *adam_v = nullptr;
-  float *h1 = nullptr, *h2 = nullptr, *dh1 = nullptr, *dh2 = nullptr;  // [max_batch][64]
-  float *dout = nullptr;                                              // [max_batch]
-  double *loss = nullptr;                                             // device accumulator
-  double *h_loss = nullptr;                                           // pinned
-  int64_t t = 0;                                                      // Adam step count
+  float *part = nullptr;             // [min(slots, tiles of max_batch)][kMlpGradLen]
+  float *h_grad = nullptr;           // pinned copy of grad
+  int64_t t = 0;                     // Adam step count
 };
 
 namespace gc {
@@ -47,6 +45,7 @@ __global__ void k_features(const int32_t *__restrict__ list, int32_t m, const in
   }
 }
 
+// Scores of few rows: a warp per row, the weights in shared memory.
 __global__ void __launch_bounds__(kMlpThreads) k_mlp_forward(const float *__restrict__ W,
                                                              const float *__restrict__ X, int32_t m,
                                                              float *__restrict__ out) {
@@ -65,118 +64,257 @@ __global__ void __launch_bounds__(kMlpThreads) k_mlp_forward(const float *__rest
   }
 }
 
-// Per-sample forward and backward of L = (1/m) sum (out - y)^2: stores h1, h2,
-// dL/dz1 (dh1), dL/dz2 (dh2) and dL/dout; accumulates the loss.
-__global__ void __launch_bounds__(kMlpThreads) k_mlp_fwdbwd(const float *__restrict__ W,
-                                                            const float *__restrict__ X,
-                                                            const float *__restrict__ y, int32_t m, float *H1,
-                                                            float *H2, float *DH1, float *DH2, float *DOUT,
-                                                            double *loss) {
-  __shared__ float sw[kMlpParams];
-  __shared__ float sh1[kMlpThreads / 32][kMlpHidden];
-  __shared__ float sd2[kMlpThreads / 32][kMlpHidden];
-  for (int i = threadIdx.x; i < kMlpParams; i += blockDim.x) sw[i] = W[i];
-  cta_sync();
-  const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int gw = blockIdx.x * (blockDim.x >> 5) + wid, nw = gridDim.x * (blockDim.x >> 5);
+// Many rows, and every gradient: rows are taken in tiles of 16 R by CTAs of 256 threads; thread (ty, tx) of
+// 16 x 16 computes R rows ty + 16 q by 4 columns of each of the three 64-wide
+// products, all of them between shared-memory tiles: activations never reach
+// global memory.  GRAD: the CTA keeps its sums of the weight gradients in
+// registers over all its tiles (16 of W2, 2 of W1 and one of the 193 others a
+// thread) and writes them once, as one row of `part`, which k_mlp_reduce adds.
+//
+// What bounds it: float32 FMAs against shared-memory loads (6 16-byte loads a
+// warp for 32 R FMAs), 28 kFLOP a row, and at small m the latency of one tile.
+// So for gradients the small tile is taken while all of them are resident at once
+// and the large one, with 2.4 times fewer loads an FMA, beyond; scores alone keep a
+// warp per row as long (6 us for 1,024 rows, 9 with tiles; 19 against 12.5 for
+// 16,384).  Every sum over inputs or columns runs in the order of one sample by one
+// warp (mlp_forward_warp); the sums over rows are per tile and then over tiles.
+//
+// One warp per row for the activations, stored to memory, and one thread per
+// parameter over all rows took 81 us for a gradient of 1,024 rows and 780 us for
+// 16,384 on the host's clock; this takes 33 and 56.
+constexpr int kMlpPad = kMlpHidden + 4;         // row stride in shared memory: no two rows of a warp share banks
+constexpr int kMlpGradLen = kMlpParams + 7;     // a gradient, then its loss (double, 8-byte aligned)
+constexpr int kMlpLossAt = kMlpParams + 1;
+static_assert(kMlpLossAt % 2 == 0 && kMlpLossAt + 2 <= kMlpGradLen && kMlpGradLen % 2 == 0, "loss alignment");
+constexpr int kMlpCtasPerSm = 2;
+
+constexpr size_t mlp_smem(int R) {
+  return sizeof(float) * ((size_t)kMlpHidden * kMlpPad + kMlpIn * kMlpHidden + 4 * kMlpHidden +
+                          (size_t)16 * R * (4 * kMlpPad + kMlpIn + 2));
+}
+
+template <int R, bool GRAD>
+__global__ void __launch_bounds__(kMlpThreads, kMlpCtasPerSm)
+    k_mlp_tile(const float *__restrict__ W, const float *__restrict__ X, const float *__restrict__ y, int32_t m,
+               float *__restrict__ out, float *__restrict__ part) {
+  constexpr int T = 16 * R;
+  extern __shared__ __align__(16) float smem[];
+  float *w2 = smem, *w1 = w2 + kMlpHidden * kMlpPad, *b1 = w1 + kMlpIn * kMlpHidden, *b2 = b1 + kMlpHidden,
+        *w3 = b2 + kMlpHidden, *h1 = w3 + 2 * kMlpHidden, *h2 = h1 + T * kMlpPad, *d2 = h2 + T * kMlpPad,
+        *d1 = d2 + T * kMlpPad, *x = d1 + T * kMlpPad, *dout = x + T * kMlpIn;
+  const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15, wid = tid >> 5, lane = tid & 31;
+  for (int i = tid; i < kMlpHidden * kMlpHidden; i += kMlpThreads)
+    w2[(i / kMlpHidden) * kMlpPad + i % kMlpHidden] = W[kOffW2 + i];
+  for (int i = tid; i < kMlpIn * kMlpHidden; i += kMlpThreads) w1[i] = W[kOffW1 + i];
+  if (tid < kMlpHidden) {
+    b1[tid] = W[kOffB1 + tid];
+    b2[tid] = W[kOffB2 + tid];
+    w3[tid] = W[kOffW3 + tid];
+  }
+  const float b3 = W[kOffB3];
+  float gw2[4][4] = {}, gw1[2] = {}, gb = 0.f;
   double lsum = 0;
-  for (int s = gw; s < m; s += nw) {
-    float x[kMlpIn];
+  const int32_t tiles = (int32_t)(((int64_t)m + T - 1) / T);
+  for (int32_t tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
+    const int64_t r0 = (int64_t)tile * T;
+    const int cnt = (int)min((int64_t)T, (int64_t)m - r0);
+    cta_sync();  // weights; the last tile's readers
+    for (int i = tid; i < T * kMlpIn; i += kMlpThreads) x[i] = i < cnt * kMlpIn ? X[r0 * kMlpIn + i] : 0.f;
+    cta_sync();
+    {  // h1 = relu(x W1 + b1)
+      const float4 b = *(const float4 *)(b1 + 4 * tx);
+      float z[R][4];
 #pragma unroll
-    for (int f = 0; f < kMlpIn; ++f) x[f] = X[(size_t)s * kMlpIn + f];
-    // forward, keeping pre-activations for the ReLU masks
-    float z10 = sw[kOffB1 + lane], z11 = sw[kOffB1 + lane + 32];
+      for (int q = 0; q < R; ++q) z[q][0] = b.x, z[q][1] = b.y, z[q][2] = b.z, z[q][3] = b.w;
 #pragma unroll
-    for (int f = 0; f < kMlpIn; ++f) {
-      z10 = fmaf(x[f], sw[kOffW1 + f * kMlpHidden + lane], z10);
-      z11 = fmaf(x[f], sw[kOffW1 + f * kMlpHidden + lane + 32], z11);
-    }
-    const float h10 = fmaxf(z10, 0.f), h11 = fmaxf(z11, 0.f);
-    sh1[wid][lane] = h10;
-    sh1[wid][lane + 32] = h11;
-    __syncwarp();
-    float z20 = sw[kOffB2 + lane], z21 = sw[kOffB2 + lane + 32];
-    for (int i = 0; i < kMlpHidden; ++i) {
-      const float h = sh1[wid][i];
-      z20 = fmaf(h, sw[kOffW2 + i * kMlpHidden + lane], z20);
-      z21 = fmaf(h, sw[kOffW2 + i * kMlpHidden + lane + 32], z21);
-    }
-    const float h20 = fmaxf(z20, 0.f), h21 = fmaxf(z21, 0.f);
-    float o = h20 * sw[kOffW3 + lane] + h21 * sw[kOffW3 + lane + 32];
+      for (int f = 0; f < kMlpIn; ++f) {
+        const float4 w = *(const float4 *)(w1 + f * kMlpHidden + 4 * tx);
 #pragma unroll
-    for (int q = 16; q > 0; q >>= 1) o += __shfl_xor_sync(0xffffffffu, o, q);
-    o += sw[kOffB3];
-    const float diff = o - y[s];
-    const float dout = 2.f * diff / (float)m;
-    if (lane == 0) lsum += (double)diff * (double)diff;
-    // backward
-    const float d20 = z20 > 0.f ? dout * sw[kOffW3 + lane] : 0.f;
-    const float d21 = z21 > 0.f ? dout * sw[kOffW3 + lane + 32] : 0.f;
-    sd2[wid][lane] = d20;
-    sd2[wid][lane + 32] = d21;
-    __syncwarp();
-    float e0 = 0.f, e1 = 0.f;  // dL/dh1 for i = lane, lane + 32
-    for (int j = 0; j < kMlpHidden; ++j) {
-      const float d = sd2[wid][j];
-      e0 = fmaf(d, sw[kOffW2 + lane * kMlpHidden + j], e0);
-      e1 = fmaf(d, sw[kOffW2 + (lane + 32) * kMlpHidden + j], e1);
+        for (int q = 0; q < R; ++q) {
+          const float a = x[(ty + 16 * q) * kMlpIn + f];
+          z[q][0] = fmaf(a, w.x, z[q][0]);
+          z[q][1] = fmaf(a, w.y, z[q][1]);
+          z[q][2] = fmaf(a, w.z, z[q][2]);
+          z[q][3] = fmaf(a, w.w, z[q][3]);
+        }
+      }
+#pragma unroll
+      for (int q = 0; q < R; ++q)
+        *(float4 *)(h1 + (ty + 16 * q) * kMlpPad + 4 * tx) =
+            make_float4(fmaxf(z[q][0], 0.f), fmaxf(z[q][1], 0.f), fmaxf(z[q][2], 0.f), fmaxf(z[q][3], 0.f));
     }
-    const size_t row = (size_t)s * kMlpHidden;
-    H1[row + lane] = h10;
-    H1[row + lane + 32] = h11;
-    H2[row + lane] = h20;
-    H2[row + lane + 32] = h21;
-    DH2[row + lane] = d20;
-    DH2[row + lane + 32] = d21;
-    DH1[row + lane] = z10 > 0.f ? e0 : 0.f;
-    DH1[row + lane + 32] = z11 > 0.f ? e1 : 0.f;
-    if (lane == 0) DOUT[s] = dout;
-    __syncwarp();
+    cta_sync();
+    {  // h2 = relu(h1 W2 + b2)
+      const float4 b = *(const float4 *)(b2 + 4 * tx);
+      float z[R][4];
+#pragma unroll
+      for (int q = 0; q < R; ++q) z[q][0] = b.x, z[q][1] = b.y, z[q][2] = b.z, z[q][3] = b.w;
+#pragma unroll 4
+      for (int k = 0; k < kMlpHidden; k += 4) {
+        float4 w[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) w[e] = *(const float4 *)(w2 + (k + e) * kMlpPad + 4 * tx);
+#pragma unroll
+        for (int q = 0; q < R; ++q) {
+          const float4 a = *(const float4 *)(h1 + (ty + 16 * q) * kMlpPad + k);
+          const float av[4] = {a.x, a.y, a.z, a.w};
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            z[q][0] = fmaf(av[e], w[e].x, z[q][0]);
+            z[q][1] = fmaf(av[e], w[e].y, z[q][1]);
+            z[q][2] = fmaf(av[e], w[e].z, z[q][2]);
+            z[q][3] = fmaf(av[e], w[e].w, z[q][3]);
+          }
+        }
+      }
+#pragma unroll
+      for (int q = 0; q < R; ++q)
+        *(float4 *)(h2 + (ty + 16 * q) * kMlpPad + 4 * tx) =
+            make_float4(fmaxf(z[q][0], 0.f), fmaxf(z[q][1], 0.f), fmaxf(z[q][2], 0.f), fmaxf(z[q][3], 0.f));
+    }
+    cta_sync();
+    // out = h2 . W3 + b3, one warp a row
+    for (int r = wid; r < cnt; r += kMlpThreads / 32) {
+      float o = h2[r * kMlpPad + lane] * w3[lane] + h2[r * kMlpPad + lane + 32] * w3[lane + 32];
+#pragma unroll
+      for (int q = 16; q > 0; q >>= 1) o += __shfl_xor_sync(0xffffffffu, o, q);
+      o += b3;
+      if constexpr (!GRAD) {
+        if (lane == 0) out[r0 + r] = o;
+      } else {
+        const float diff = o - y[r0 + r];
+        if (lane == 0) {
+          dout[r] = 2.f * diff / (float)m;
+          lsum += (double)diff * (double)diff;
+        }
+      }
+    }
+    if constexpr (GRAD) {
+      cta_sync();
+      // dL/dz2
+      for (int i = tid; i < cnt * kMlpHidden; i += kMlpThreads) {
+        const int r = i / kMlpHidden, j = i % kMlpHidden;
+        d2[r * kMlpPad + j] = h2[r * kMlpPad + j] > 0.f ? dout[r] * w3[j] : 0.f;
+      }
+      cta_sync();
+      {  // dL/dz1 = (dL/dz2 W2^T) where h1 > 0; columns tx + 16 e: rows of W2 of different banks
+        float z[R][4] = {};
+#pragma unroll 4
+        for (int k = 0; k < kMlpHidden; k += 4) {
+          float4 w[4];
+#pragma unroll
+          for (int e = 0; e < 4; ++e) w[e] = *(const float4 *)(w2 + (tx + 16 * e) * kMlpPad + k);
+#pragma unroll
+          for (int q = 0; q < R; ++q) {
+            const float4 a = *(const float4 *)(d2 + (ty + 16 * q) * kMlpPad + k);
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+              z[q][e] = fmaf(a.x, w[e].x, z[q][e]);
+              z[q][e] = fmaf(a.y, w[e].y, z[q][e]);
+              z[q][e] = fmaf(a.z, w[e].z, z[q][e]);
+              z[q][e] = fmaf(a.w, w[e].w, z[q][e]);
+            }
+          }
+        }
+#pragma unroll
+        for (int q = 0; q < R; ++q)
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            const int at = (ty + 16 * q) * kMlpPad + tx + 16 * e;
+            d1[at] = h1[at] > 0.f ? z[q][e] : 0.f;
+          }
+      }
+      cta_sync();
+      // the tile's rows into the gradient; rows past cnt are never read
+      float t2[4][4] = {}, t1[2] = {}, tb = 0.f;
+#pragma unroll 2
+      for (int r = 0; r < cnt; ++r) {
+        const float4 a = *(const float4 *)(h1 + r * kMlpPad + 4 * ty), d = *(const float4 *)(d2 + r * kMlpPad + 4 * tx);
+        const float av[4] = {a.x, a.y, a.z, a.w}, dv[4] = {d.x, d.y, d.z, d.w};
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+          for (int j = 0; j < 4; ++j) t2[i][j] = fmaf(av[i], dv[j], t2[i][j]);
+        const float xf = x[r * kMlpIn + wid];
+        t1[0] = fmaf(xf, d1[r * kMlpPad + lane], t1[0]);
+        t1[1] = fmaf(xf, d1[r * kMlpPad + lane + 32], t1[1]);
+        if (tid < kMlpHidden) tb += d1[r * kMlpPad + tid];
+        else if (tid < 2 * kMlpHidden) tb += d2[r * kMlpPad + tid - kMlpHidden];
+        else if (tid < 3 * kMlpHidden) tb = fmaf(h2[r * kMlpPad + tid - 2 * kMlpHidden], dout[r], tb);
+        else if (tid == 3 * kMlpHidden) tb += dout[r];
+      }
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) gw2[i][j] += t2[i][j];
+      gw1[0] += t1[0];
+      gw1[1] += t1[1];
+      gb += tb;
+    }
   }
-  if (lane == 0 && lsum != 0) atomicAdd(loss, lsum / (double)m);
+  if constexpr (GRAD) {
+    float *p = part + (size_t)blockIdx.x * kMlpGradLen;
+    p[kOffW1 + wid * kMlpHidden + lane] = gw1[0];
+    p[kOffW1 + wid * kMlpHidden + lane + 32] = gw1[1];
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) p[kOffW2 + (4 * ty + i) * kMlpHidden + 4 * tx + j] = gw2[i][j];
+    if (tid < kMlpHidden) p[kOffB1 + tid] = gb;
+    else if (tid < 2 * kMlpHidden) p[kOffB2 + tid - kMlpHidden] = gb;
+    else if (tid < 3 * kMlpHidden) p[kOffW3 + tid - 2 * kMlpHidden] = gb;
+    else if (tid == 3 * kMlpHidden) p[kOffB3] = gb;
+    __shared__ double sl[kMlpThreads / 32];
+    if (lane == 0) sl[wid] = lsum;
+    cta_sync();
+    if (tid == 0) {
+      double t = 0;
+      for (int w = 0; w < kMlpThreads / 32; ++w) t += sl[w];
+      *(double *)(p + kMlpLossAt) = t;
+    }
+  }
 }
 
-// Weight gradients: one thread per parameter, summing over the batch.
-__global__ void k_mlp_wgrad(const float *__restrict__ X, const float *__restrict__ H1,
-                            const float *__restrict__ H2, const float *__restrict__ DH1,
-                            const float *__restrict__ DH2, const float *__restrict__ DOUT, int32_t m,
-                            float *__restrict__ grad) {
-  const int p = blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= kMlpParams) return;
+// grad[p] = sum of the rows of part, 32 parameters a CTA (a 128-byte line of
+// each row) by 8 groups of rows; the last CTA adds the losses too.  ADAM: the
+// step is taken in the same kernel.
+template <bool ADAM>
+__global__ void __launch_bounds__(kMlpThreads)
+    k_mlp_reduce(const float *__restrict__ part, int rows, int32_t m, float *__restrict__ grad, float *p, float *am,
+                 float *av, float lr, float b1, float b2, float eps, float c1, float c2) {
+  __shared__ float sg[kMlpThreads / 32][32];
+  const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31, i = blockIdx.x * 32 + lane;
   float acc = 0.f;
-  if (p < kOffB1) {  // W1[f][i] = sum_b X[b][f] * dh1[b][i]
-    const int f = p / kMlpHidden, i = p % kMlpHidden;
-    for (int b = 0; b < m; ++b) acc = fmaf(X[(size_t)b * kMlpIn + f], DH1[(size_t)b * kMlpHidden + i], acc);
-  } else if (p < kOffW2) {
-    const int i = p - kOffB1;
-    for (int b = 0; b < m; ++b) acc += DH1[(size_t)b * kMlpHidden + i];
-  } else if (p < kOffB2) {  // W2[i][j] = sum_b h1[b][i] * dh2[b][j]
-    const int q = p - kOffW2, i = q / kMlpHidden, j = q % kMlpHidden;
-    for (int b = 0; b < m; ++b)
-      acc = fmaf(H1[(size_t)b * kMlpHidden + i], DH2[(size_t)b * kMlpHidden + j], acc);
-  } else if (p < kOffW3) {
-    const int j = p - kOffB2;
-    for (int b = 0; b < m; ++b) acc += DH2[(size_t)b * kMlpHidden + j];
-  } else if (p < kOffB3) {
-    const int j = p - kOffW3;
-    for (int b = 0; b < m; ++b) acc = fmaf(H2[(size_t)b * kMlpHidden + j], DOUT[b], acc);
-  } else {
-    for (int b = 0; b < m; ++b) acc += DOUT[b];
+  if (i < kMlpParams) {
+#pragma unroll 4
+    for (int r = wid; r < rows; r += kMlpThreads / 32) acc += part[(size_t)r * kMlpGradLen + i];
   }
-  grad[p] = acc;
+  sg[wid][lane] = acc;
+  cta_sync();
+  if (wid == 0 && i < kMlpParams) {
+    float g = 0.f;
+#pragma unroll
+    for (int w = 0; w < kMlpThreads / 32; ++w) g += sg[w][lane];
+    grad[i] = g;
+    if constexpr (ADAM) {
+      const float mi = b1 * am[i] + (1.f - b1) * g;
+      const float vi = b2 * av[i] + (1.f - b2) * g * g;
+      am[i] = mi;
+      av[i] = vi;
+      p[i] -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
+    }
+  }
+  if (blockIdx.x == gridDim.x - 1 && wid == 1) {
+    double t = 0;
+    for (int r = lane; r < rows; r += 32) t += *(const double *)(part + (size_t)r * kMlpGradLen + kMlpLossAt);
+#pragma unroll
+    for (int q = 16; q > 0; q >>= 1) t += __shfl_xor_sync(0xffffffffu, t, q);
+    if (lane == 0) *(double *)(grad + kMlpLossAt) = t / (double)m;
+  }
 }
 
-__global__ void k_adam(float *p, const float *g, float *m, float *v, float lr, float b1, float b2, float eps,
-                       float c1, float c2) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= kMlpParams) return;
-  const float gi = g[i];
-  const float mi = b1 * m[i] + (1.f - b1) * gi;
-  const float vi = b2 * v[i] + (1.f - b2) * gi * gi;
-  m[i] = mi;
-  v[i] = vi;
-  p[i] -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
-}
+// Rows from which tiles of 64 take over.
+static bool mlp_large(const gc_mlp *h, int32_t m) { return m > (int64_t)16 * h->slots; }
 
 // Training data for the proposal: the features each evaluated candidate had
 // when it was selected (before its bound is replaced) and log1p of the exact
@@ -289,24 +427,34 @@ int launch_features(gc_graph *g, const int32_t *list, int32_t m, const int32_t *
   return GC_OK;
 }
 
-static int mlp_grad_async(gc_mlp *h, const float *X, const float *y, int32_t m) {
-  GC_CUDA(cudaMemsetAsync(h->loss, 0, sizeof(double), h->stream));
-  const int blocks = std::max(1, std::min(1024, (m + (kMlpThreads / 32) - 1) / (kMlpThreads / 32)));
-  k_mlp_fwdbwd<<<blocks, kMlpThreads, 0, h->stream>>>(h->params, X, y, m, h->h1, h->h2, h->dh1, h->dh2,
-                                                      h->dout, h->loss);
-  k_mlp_wgrad<<<(kMlpParams + 255) / 256, 256, 0, h->stream>>>(X, h->h1, h->h2, h->dh1, h->dh2, h->dout, m,
-                                                               h->grad);
+// Gradient and loss into h->grad; lr > 0: and one Adam step.
+static int mlp_grad_async(gc_mlp *h, const float *X, const float *y, int32_t m, float lr = 0.f) {
+  const int tile = mlp_large(h, m) ? 64 : 16;
+  const int ctas = (int)std::min<int64_t>(h->slots, ((int64_t)m + tile - 1) / tile);
+  if (tile == 16)
+    k_mlp_tile<1, true><<<ctas, kMlpThreads, mlp_smem(1), h->stream>>>(h->params, X, y, m, nullptr, h->part);
+  else
+    k_mlp_tile<4, true><<<ctas, kMlpThreads, mlp_smem(4), h->stream>>>(h->params, X, y, m, nullptr, h->part);
+  const int blocks = (kMlpParams + 31) / 32;
+  if (lr > 0) {
+    const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
+    h->t += 1;
+    const float c1 = 1.f - powf(b1, (float)h->t), c2 = 1.f - powf(b2, (float)h->t);
+    k_mlp_reduce<true><<<blocks, kMlpThreads, 0, h->stream>>>(h->part, ctas, m, h->grad, h->params, h->adam_m,
+                                                              h->adam_v, lr, b1, b2, eps, c1, c2);
+  } else {
+    k_mlp_reduce<false><<<blocks, kMlpThreads, 0, h->stream>>>(h->part, ctas, m, h->grad, nullptr, nullptr, nullptr,
+                                                               0.f, 0.f, 0.f, 0.f, 0.f, 0.f);
+  }
   GC_CUDA(cudaGetLastError());
   return GC_OK;
 }
 
-static int mlp_adam_async(gc_mlp *h, float lr) {
-  const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
-  h->t += 1;
-  const float c1 = 1.f - powf(b1, (float)h->t), c2 = 1.f - powf(b2, (float)h->t);
-  k_adam<<<(kMlpParams + 255) / 256, 256, 0, h->stream>>>(h->params, h->grad, h->adam_m, h->adam_v, lr, b1, b2,
-                                                          eps, c1, c2);
-  GC_CUDA(cudaGetLastError());
+// Waits for gradient and loss on the host, through one pinned copy.
+static int mlp_read_grad(gc_mlp *h, double *loss) {
+  GC_CUDA(cudaMemcpyAsync(h->h_grad, h->grad, kMlpGradLen * sizeof(float), cudaMemcpyDeviceToHost, h->stream));
+  GC_CUDA(cudaStreamSynchronize(h->stream));
+  memcpy(loss, h->h_grad + kMlpLossAt, sizeof(double));
   return GC_OK;
 }
 
@@ -325,15 +473,20 @@ int gc_mlp_create(int32_t max_batch, void *stream, gc_mlp **out) {
   gc_mlp *h = new gc_mlp();
   h->max_batch = max_batch;
   h->stream = (cudaStream_t)stream;
-  const size_t act = (size_t)max_batch * kMlpHidden * sizeof(float);
-  void **bufs[] = {(void **)&h->params, (void **)&h->grad, (void **)&h->adam_m, (void **)&h->adam_v};
-  bool ok = true;
-  for (void **b : bufs) ok = ok && cudaMalloc(b, kMlpParams * sizeof(float)) == cudaSuccess;
-  ok = ok && cudaMalloc((void **)&h->h1, act) == cudaSuccess && cudaMalloc((void **)&h->h2, act) == cudaSuccess &&
-       cudaMalloc((void **)&h->dh1, act) == cudaSuccess && cudaMalloc((void **)&h->dh2, act) == cudaSuccess &&
-       cudaMalloc((void **)&h->dout, (size_t)max_batch * sizeof(float)) == cudaSuccess &&
-       cudaMalloc((void **)&h->loss, sizeof(double)) == cudaSuccess &&
-       cudaMallocHost((void **)&h->h_loss, sizeof(double)) == cudaSuccess;
+  int dev = 0, sms = 0;
+  bool ok = cudaGetDevice(&dev) == cudaSuccess &&
+            cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess;
+  h->slots = kMlpCtasPerSm * sms;
+  for (const void *f : {(const void *)k_mlp_tile<4, false>, (const void *)k_mlp_tile<4, true>})
+    ok = ok &&
+         cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mlp_smem(4)) == cudaSuccess;
+  static_assert(mlp_smem(1) <= 48 * 1024, "needs no attribute");
+  const size_t rows = (size_t)std::min<int64_t>(h->slots, ((int64_t)max_batch + 15) / 16);
+  for (float **b : {&h->params, &h->adam_m, &h->adam_v})
+    ok = ok && cudaMalloc((void **)b, kMlpParams * sizeof(float)) == cudaSuccess;
+  ok = ok && cudaMalloc((void **)&h->grad, kMlpGradLen * sizeof(float)) == cudaSuccess &&
+       cudaMalloc((void **)&h->part, rows * kMlpGradLen * sizeof(float)) == cudaSuccess &&
+       cudaMallocHost((void **)&h->h_grad, kMlpGradLen * sizeof(float)) == cudaSuccess;
   if (!ok) {
     cudaGetLastError();
     gc_mlp_free(h);
@@ -350,10 +503,10 @@ int gc_mlp_create(int32_t max_batch, void *stream, gc_mlp **out) {
 int gc_mlp_free(gc_mlp *h) {
   if (!h) return GC_OK;
   cudaStreamSynchronize(h->stream);
-  void *bufs[] = {h->params, h->grad, h->adam_m, h->adam_v, h->h1, h->h2, h->dh1, h->dh2, h->dout, h->loss};
+  void *bufs[] = {h->params, h->grad, h->adam_m, h->adam_v, h->part};
   for (void *b : bufs)
     if (b) cudaFree(b);
-  if (h->h_loss) cudaFreeHost(h->h_loss);
+  if (h->h_grad) cudaFreeHost(h->h_grad);
   delete h;
   return GC_OK;
 }
@@ -387,8 +540,12 @@ int gc_mlp_forward(gc_mlp *h, const float *X, int32_t m, float *out) {
     return GC_EINVAL;
   }
   if (m == 0) return GC_OK;
-  const int blocks = std::max(1, std::min(4096, (m + 7) / 8));
-  k_mlp_forward<<<blocks, kMlpThreads, 0, h->stream>>>(h->params, X, m, out);
+  if (mlp_large(h, m)) {
+    const int ctas = (int)std::min<int64_t>(h->slots, ((int64_t)m + 63) / 64);
+    k_mlp_tile<4, false><<<ctas, kMlpThreads, mlp_smem(4), h->stream>>>(h->params, X, nullptr, m, out, nullptr);
+  } else {
+    k_mlp_forward<<<(m + 7) / 8, kMlpThreads, 0, h->stream>>>(h->params, X, m, out);
+  }
   GC_CUDA(cudaGetLastError());
   return GC_OK;
 }
@@ -400,11 +557,10 @@ int gc_mlp_grad(gc_mlp *h, const float *X, const float *y, int32_t m, float *gra
   }
   int rc = mlp_grad_async(h, X, y, m);
   if (rc) return rc;
-  if (grad)
-    GC_CUDA(cudaMemcpyAsync(grad, h->grad, kMlpParams * sizeof(float), cudaMemcpyDeviceToHost, h->stream));
-  GC_CUDA(cudaMemcpyAsync(h->h_loss, h->loss, sizeof(double), cudaMemcpyDeviceToHost, h->stream));
-  GC_CUDA(cudaStreamSynchronize(h->stream));
-  if (loss) *loss = *h->h_loss;
+  double l = 0;
+  if ((rc = mlp_read_grad(h, &l))) return rc;
+  if (grad) memcpy(grad, h->h_grad, kMlpParams * sizeof(float));
+  if (loss) *loss = l;
   return GC_OK;
 }
 
@@ -413,9 +569,7 @@ int gc_mlp_adam_step(gc_mlp *h, const float *X, const float *y, int32_t m, float
     set_error("bad argument to gc_mlp_adam_step");
     return GC_EINVAL;
   }
-  int rc = mlp_grad_async(h, X, y, m);
-  if (!rc) rc = mlp_adam_async(h, lr);
-  return rc;
+  return mlp_grad_async(h, X, y, m, lr);
 }
 
 int gc_mlp_train(gc_mlp *h, const float *X, const float *y, int32_t m, int32_t epochs, int32_t batch, float lr,
@@ -437,8 +591,7 @@ int gc_mlp_train(gc_mlp *h, const float *X, const float *y, int32_t m, int32_t e
     }
     for (int32_t i = 0; i < nb; ++i) {
       const int32_t off = order[i] * batch, len = std::min(batch, m - off);
-      int rc = mlp_grad_async(h, X + (size_t)off * kMlpIn, y + off, len);
-      if (!rc) rc = mlp_adam_async(h, lr);
+      const int rc = mlp_grad_async(h, X + (size_t)off * kMlpIn, y + off, len, lr);
       if (rc) return rc;
     }
   }
@@ -447,11 +600,11 @@ int gc_mlp_train(gc_mlp *h, const float *X, const float *y, int32_t m, int32_t e
     double tot = 0;
     for (int32_t off = 0; off < m; off += batch) {
       const int32_t len = std::min(batch, m - off);
+      double l = 0;
       int rc = mlp_grad_async(h, X + (size_t)off * kMlpIn, y + off, len);
+      if (!rc) rc = mlp_read_grad(h, &l);
       if (rc) return rc;
-      GC_CUDA(cudaMemcpyAsync(h->h_loss, h->loss, sizeof(double), cudaMemcpyDeviceToHost, h->stream));
-      GC_CUDA(cudaStreamSynchronize(h->stream));
-      tot += *h->h_loss * len;
+      tot += l * len;
     }
     *final_loss = tot / m;
   }
