@@ -514,8 +514,24 @@ int gc_top_closeness(gc_graph *g, int32_t k, const gc_opts *opts_in, int32_t *ou
   const int32_t n_probe = std::min<int32_t>(g->h_sctl->n_sel, (k + kLanes - 1) / kLanes * kLanes);
   if (n_probe < k) return fail(GC_EINTERNAL, "top-k closeness: fewer probes than k");
   GC_TRY(launch_clamp_nsel(g, n_probe));
+  const auto wide_lanes = [&](int32_t m) {
+    const int want = opts.round0_lanes > 0 ? opts.round0_lanes : (m > 128 ? 256 : m > 64 ? 128 : 64);
+    return want >= 512 ? 8 : want >= 256 ? 4 : want >= 128 ? 2 : 1;
+  };
+  // Shallow graphs: searches to the end spend nearly everything on two or three
+  // levels that hold nearly all edges; from the unreached side each of these is
+  // one pass over the edges for all lanes (R-MAT scale 18, k 100:
+  // both launches of 64 lanes 2.5 ms, the call 3.6 -> 1.2)
+  bool wide_probes = false;
+  if (opts.round0_lanes >= 0 && ecc <= kShallowLevels && opts.max_ctas == 0) {
+    const int rc = launch_round0_wide(g, g->list, n_probe, g->lgain, wide_lanes(n_probe), 0, false, tns, 0);
+    if (rc != GC_OK && rc != GC_ENOMEM) return rc;
+    wide_probes = rc == GC_OK;  // no room for its lane words: the 64-lane batches below
+  }
   if (deep) {
     GC_TRY(launch_solo(g, kModeFarness, g->list, n_probe, nullptr, g->lgain, nullptr, 0, true, false));
+  } else if (wide_probes) {
+    // launched above
   } else if (n_probe <= kRound0GridMax) {
     for (int32_t off = 0; off < n_probe; off += kLanes)
       GC_TRY(launch_gains_grid(g, kModeFarness, g->list + off, std::min<int32_t>(kLanes, n_probe - off), nullptr,
@@ -547,8 +563,7 @@ int gc_top_closeness(gc_graph *g, int32_t k, const gc_opts *opts_in, int32_t *ou
   }
   int r0_w = 0;
   if (n_surv > 0 && opts.round0_lanes >= 0 && ecc <= kShallowLevels) {
-    const int want = opts.round0_lanes > 0 ? opts.round0_lanes : (n_surv > 128 ? 256 : n_surv > 64 ? 128 : 64);
-    r0_w = want >= 512 ? 8 : want >= 256 ? 4 : want >= 128 ? 2 : 1;
+    r0_w = wide_lanes(n_surv);
     if (opts.round0_lanes == 0) {  // the same choice as round 0 of gc_greedy
       GC_TRY(launch_sum_two_hop(g, (unsigned long long *)g->g3));
       unsigned long long two_hop_sum = 0;
