@@ -456,6 +456,7 @@ int gc_gain_upper_bounds(gc_graph *g, const int32_t *S, int32_t s_len, int64_t *
   // pruned rows from the distances of S[0] alone: every group containing S[0]
   // has d_S <= d(S[0], .), so the rows keep every neighbour it can still use
   GC_TRY(distances_from(g, g->io_b, 1, timeout_ns(nullptr), nullptr));
+  GC_TRY(launch_row_stats(g));
   GC_TRY(launch_prune_csr(g));
   if (s_len == 1) {
     GC_TRY(launch_round1_bound(g));
@@ -1126,13 +1127,13 @@ int gc_greedy(gc_graph *g, int32_t k, const gc_opts *opts_in, int32_t *out_group
     GC_TRY(distances_from(g, &g->sctl->arg_id, 1, tns, &f));
     if (f != f_s0) return fail(GC_EINTERNAL, "farness of s0 disagrees between round 0 and the BFS");
   }
+  const bool expand_bound = !(opts.flags & GC_OPT_NO_EXPAND_BOUND);
+  const bool prune = !(opts.flags & GC_OPT_FULL_ADJACENCY) && !deep;
+  if (expand_bound || prune) GC_TRY(launch_row_stats(g));
   // neighbour bound for the pruning of useless expansions in every later round
-  if (!(opts.flags & GC_OPT_NO_EXPAND_BOUND)) {
-    GC_TRY(launch_max_nbr(g));
-    g->mx = g->mx_buf;
-  }
+  if (expand_bound) g->mx = g->mx_buf;
   // pruned adjacency: drop the entries no later round can use (d_S[w] <= 1)
-  if (!(opts.flags & GC_OPT_FULL_ADJACENCY) && !deep) {
+  if (prune) {
     GC_TRY(launch_prune_csr(g));
     pruned = true;
   }

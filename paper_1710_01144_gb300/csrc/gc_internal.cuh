@@ -500,11 +500,13 @@ int launch_record(gc_graph *g, int32_t round, long long prev_gain);
 // round 1 with the proposal: of the candidates in g->list (n_sel of them, the
 // largest bounds, at most 1024), keep the 64 with the largest predicted gain
 int launch_round1_propose(gc_graph *g, long long prev_gain);
-// mx[u] = max_{w in N(u)} d_S[w] into g->mx_buf (an upper bound for every later d_S)
-int launch_max_nbr(gc_graph *g);
+// from the d_S now in g->dS: mx[u] = max_{w in N(u)} d_S[w] into g->mx_buf (an
+// upper bound for every later d_S), the pruned rows' sizes (g->io_a, g->c3), the
+// terms of the round-1 bounds (g->c3s) and d_S as classes (g->bq0)
+int launch_row_stats(gc_graph *g);
 // the list of long rows used by the row-wise kernels' CTA-per-row companions
 int launch_heavy_rows(gc_graph *g);
-// pruned adjacency (g->rpf, g->cif, g->c3) from the d_S now in g->dS
+// pruned adjacency (g->rpf, g->cif, g->c3), directly after launch_row_stats
 int launch_prune_csr(gc_graph *g);
 int launch_round1_bound(gc_graph *g);
 // the same bound for the group whose distances are in d_S, over the pruned rows
