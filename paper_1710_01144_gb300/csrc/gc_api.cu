@@ -30,7 +30,7 @@ static int fail(int code, const std::string &msg) {
   return code;
 }
 
-constexpr int32_t kRound0GridMax = 256;  // round-0 survivors handled by grid-wide batches
+constexpr int32_t kRound0GridMax = 256;  // round-0 survivors (round-1 candidates) handled by grid-wide batches
 constexpr int kRound0Pivots = 8;         // round 0: at most this many pivot bounds
 constexpr int kSoloStages = 12;          // deep graphs: at most this many sampled stages per round
 constexpr int kSoloRegion = 96;          // deep graphs: persistent rounds once n <= this times the round
@@ -1333,9 +1333,17 @@ int gc_greedy(gc_graph *g, int32_t k, const gc_opts *opts_in, int32_t *out_group
           GC_TRY(grid_timed(kModeGain, g->list, 0, &g->sctl->n_sel, g->lgain));
         } else {
           // every unevaluated candidate whose bound reaches the best exact
-          // gain so far, in 64-lane batches, one CTA each
+          // gain so far, in 64-lane batches: one CTA each, or over the whole
+          // grid while a few batches would leave most CTAs idle (R-MAT scale
+          // 24, one candidate: 3.2 ms on a CTA, 0.3 over the grid)
           GC_TRY(launch_select(g, kSelLazy, r, 0, kTauHost, g->h_sctl->best_gain));
-          GC_TRY(gains_timed(kModeGain, g->list, 0, &g->sctl->n_sel, kLanes));
+          GC_CUDA(cudaMemcpyAsync(g->h_sctl, g->sctl, sizeof(SelCtl), cudaMemcpyDeviceToHost, g->stream));
+          GC_TRY(sync(g));
+          const int32_t m1 = g->h_sctl->n_sel;
+          if (m1 > kRound0GridMax) GC_TRY(gains_timed(kModeGain, g->list, m1, nullptr, kLanes));
+          for (int32_t off = 0; off < m1 && m1 <= kRound0GridMax; off += kLanes)
+            GC_TRY(grid_timed(kModeGain, g->list + off, std::min<int32_t>(kLanes, m1 - off), nullptr,
+                              g->lgain + off));
         }
       } else if (r == 1) {  // no bounds: all of V \ S
         if (heavy > 0) {
