@@ -109,6 +109,19 @@ __device__ __forceinline__ void cta_gain_batch(const int32_t *__restrict__ rp, c
   if (tid == 0) s_qn = 0;
   cta_sync();
 
+  u64 sum_a = 0, sum_b = 0;  // this warp's claims of lanes `lane` and `lane` + 32
+  unsigned cnt_a = 0, cnt_b = 0;
+  auto flush_sums = [&]() {
+    u64 *const s_sum = MODE == kModeGain ? s_gain : s_deg;
+    if (sum_a) atomicAdd(&s_sum[lane], sum_a);
+    if (sum_b) atomicAdd(&s_sum[lane + 32], sum_b);
+    if (MODE == kModeFarness) {
+      if (cnt_a) atomicAdd(&s_cnt[lane], (int)cnt_a);
+      if (cnt_b) atomicAdd(&s_cnt[lane + 32], (int)cnt_b);
+      cnt_a = cnt_b = 0;
+    }
+    sum_a = sum_b = 0;
+  };
   int L = 0;
   for (; F > 0; ++L) {
     const int nlev = L + 1;
@@ -210,34 +223,17 @@ __device__ __forceinline__ void cta_gain_batch(const int32_t *__restrict__ rp, c
             qnxt_v[bq + __popc(qm & below)] = w[k];
             ++cnt.push;
           }
-          // per-lane sums: a claim of one lane (the common case: a row's
-          // entries carry the lane of the vertex being expanded) is summed over
-          // the warp's threads that won the same lane, one thread adds the sum
-          // (farness: deg - 1 of the claimed vertex; the distances follow from
-          // the counts, level by level)
-          const u64 wt = MODE == kModeGain ? (u64)(dw[k] - nlev) : (u64)(dw[k] - 1);
-          u64 *const s_sum = MODE == kModeGain ? s_gain : s_deg;
-          const bool one = won != 0ull && (won & (won - 1ull)) == 0ull;
-          const int j1 = one ? __ffsll((long long)won) - 1 : -1;  // (the -1 group adds nothing here)
-          const unsigned grp = __match_any_sync(0xffffffffu, j1);
-          if (one) {
-            // wt < 2^31: two 16-bit halves keep the 32-lane sums exact
-            const unsigned lo = __reduce_add_sync(grp, (unsigned)(wt & 0xffffu));
-            const unsigned hi = __reduce_add_sync(grp, (unsigned)(wt >> 16));
-            if (lane == __ffs(grp) - 1) {
-              atomicAdd(&s_sum[j1], (u64)lo + ((u64)hi << 16));
-              if (MODE == kModeFarness) atomicAdd(&s_cnt[j1], __popc(grp));
-            }
-          } else if (won) {
-            do {
-              const int j = __ffsll((long long)won) - 1;
-              won &= won - 1;
-              atomicAdd(&s_sum[j], wt);
-              if (MODE == kModeFarness) atomicAdd(&s_cnt[j], 1);
-            } while (won);
-          }
+          // per-lane sums, kept by the threads of the warp (farness: deg - 1 of
+          // the claimed vertex; the distances follow from the counts, level by
+          // level)
+          warp_lane_sums<MODE == kModeFarness>(won, (unsigned)(MODE == kModeGain ? dw[k] - nlev : dw[k] - 1), sum_a,
+                                               sum_b, cnt_a, cnt_b);
         }
       }
+      cta_sync();
+    }
+    if (MODE == kModeFarness) {
+      flush_sums();
       cta_sync();
     }
     const int Fn = s_qn;
@@ -269,6 +265,10 @@ __device__ __forceinline__ void cta_gain_batch(const int32_t *__restrict__ rp, c
       for (int i = tid; i < F; i += T) nxt[qcur_v[i] - voff] = 0;
       break;
     }
+  }
+  if (MODE == kModeGain) {
+    flush_sums();
+    cta_sync();
   }
   cnt.levels += (u64)L;
   ++cnt.batches;

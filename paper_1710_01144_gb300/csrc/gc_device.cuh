@@ -114,6 +114,61 @@ __device__ __forceinline__ T block_sum(T v, T *sh) {
   return r;
 }
 
+// Sums of the claims of one warp by batch lane: thread t won the lanes in `won`,
+// each worth wt.  Thread j gets the sums of lanes j and j + 32 added to a and b, and
+// with COUNT their numbers to ca and cb.  The 32 x 64 bits are transposed (10
+// shuffles), so that thread j holds the threads that won lane j, and the weights are
+// taken by bit planes (a gain is 1 or 2 nearly always): a fixed cost, where an
+// atomic a lane and claim on 64 shared words serialises a warp whose claims hold
+// many lanes, as on every level but the first few of a batch.  Lazy rounds in ms,
+// before and now: BA n = 50,000, m = 1 20.2, 15.5; n = 200,000, m = 8 4.6, 3.7; R-MAT
+// scale 20 6.3, 5.9; 64-lane batches of one CTA on BA n = 50,000 12.8, 8.1.
+template <bool COUNT>
+__device__ __forceinline__ void warp_lane_sums(unsigned long long won, unsigned wt, unsigned long long &a,
+                                               unsigned long long &b, unsigned &ca, unsigned &cb) {
+  const int lane = threadIdx.x & 31;
+  unsigned x = (unsigned)won, y = (unsigned)(won >> 32);
+  const unsigned ox = __reduce_or_sync(0xffffffffu, x), oy = __reduce_or_sync(0xffffffffu, y);
+  if (!(ox | oy)) return;
+  if (won == 0) wt = 0;
+  if (__popc(ox) + __popc(oy) == 1) {  // one lane alone: a long row at level 0
+    const unsigned n1 = COUNT ? __popc(__ballot_sync(0xffffffffu, won != 0)) : 0u;
+    const unsigned long long s = (unsigned long long)__reduce_add_sync(0xffffffffu, wt & 0xffffu) +
+                                 ((unsigned long long)__reduce_add_sync(0xffffffffu, wt >> 16) << 16);
+    if (lane == __ffs(ox | oy) - 1) {
+      if (ox) {
+        a += s;
+        if (COUNT) ca += n1;
+      } else {
+        b += s;
+        if (COUNT) cb += n1;
+      }
+    }
+    return;
+  }
+  unsigned low = 0x0000ffffu;  // bit positions without bit j
+#pragma unroll
+  for (int j = 16; j > 0; j >>= 1, low ^= low << j) {
+    const unsigned p = __shfl_xor_sync(0xffffffffu, x, j), q = __shfl_xor_sync(0xffffffffu, y, j);
+    if (lane & j) {
+      x = (x & ~low) | ((p & ~low) >> j);
+      y = (y & ~low) | ((q & ~low) >> j);
+    } else {
+      x = (x & low) | ((p & low) << j);
+      y = (y & low) | ((q & low) << j);
+    }
+  }
+  if (COUNT) {
+    ca += __popc(x);
+    cb += __popc(y);
+  }
+  for (unsigned m = __reduce_or_sync(0xffffffffu, wt), i = 0; m; m >>= 1, ++i) {
+    const unsigned plane = __ballot_sync(0xffffffffu, (wt >> i) & 1u);
+    a += (unsigned long long)__popc(x & plane) << i;
+    b += (unsigned long long)__popc(y & plane) << i;
+  }
+}
+
 // Block-wide exclusive scan of int32 (blockDim.x <= 1024); returns the
 // exclusive prefix, *total gets the block total.  `sh` needs 33 entries.
 __device__ __forceinline__ int block_excl_scan(int v, int *sh, int *total) {

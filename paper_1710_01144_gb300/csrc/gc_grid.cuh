@@ -269,6 +269,18 @@ static __device__ __forceinline__ bool grid_gain_batch(const int32_t *__restrict
     __syncwarp();
   };
 
+  u64 sum_a = 0, sum_b = 0;  // this warp's claims of lanes `lane` and `lane` + 32
+  unsigned cnt_a = 0, cnt_b = 0;
+  auto flush_sums = [&]() {
+    if (sum_a) atomicAdd(&s_gain[lane], sum_a);
+    if (sum_b) atomicAdd(&s_gain[lane + 32], sum_b);
+    if (MODE == kModeFarness) {
+      if (cnt_a) atomicAdd(&s_cnt[lane], cnt_a);
+      if (cnt_b) atomicAdd(&s_cnt[lane + 32], cnt_b);
+      cnt_a = cnt_b = 0;
+    }
+    sum_a = sum_b = 0;
+  };
   int L = 0, F_prev = 0;
   for (; ok; ++L) {
     const unsigned long long pk = *(volatile unsigned long long *)&ctl->pk[L % 3];
@@ -404,32 +416,11 @@ static __device__ __forceinline__ bool grid_gain_batch(const int32_t *__restrict
               __syncwarp();
               if (pend >= 32) append(32, nlev);
             }
-            // per-lane sums: claims that won one lane (the common case: a
-            // row's entries all carry the lane of the vertex being expanded)
-            // are summed over the threads of the warp that won the same lane,
-            // and one thread adds the sum; claims of several lanes add each
-            // (farness: deg - 1 of the claimed vertex; the distances follow from
-            // the counts, level by level)
-            const u64 wt = MODE == kModeGain ? (u64)(dw[k] - nlev) : (u64)(lw[k] - 1);
-            const bool one = won != 0ull && (won & (won - 1ull)) == 0ull;
-            const int j1 = one ? __ffsll((long long)won) - 1 : -1;  // (the -1 group adds nothing here)
-            const unsigned grp = __match_any_sync(0xffffffffu, j1);
-            if (one) {
-              // wt < 2^31: two 16-bit halves keep the 32-lane sums exact
-              const unsigned lo = __reduce_add_sync(grp, (unsigned)(wt & 0xffffu));
-              const unsigned hi = __reduce_add_sync(grp, (unsigned)(wt >> 16));
-              if (lane == __ffs(grp) - 1) {
-                atomicAdd(&s_gain[j1], (u64)lo + ((u64)hi << 16));
-                if (MODE == kModeFarness) atomicAdd(&s_cnt[j1], (unsigned)__popc(grp));
-              }
-            } else if (won) {
-              do {
-                const int j = __ffsll((long long)won) - 1;
-                won &= won - 1;
-                atomicAdd(&s_gain[j], wt);
-                if (MODE == kModeFarness) atomicAdd(&s_cnt[j], 1u);
-              } while (won);
-            }
+            // per-lane sums, kept by the threads of the warp (farness: deg - 1 of
+            // the claimed vertex; the distances follow from the counts, level by
+            // level)
+            warp_lane_sums<MODE == kModeFarness>(won, (unsigned)(MODE == kModeGain ? dw[k] - nlev : lw[k] - 1), sum_a,
+                                                 sum_b, cnt_a, cnt_b);
           }
         }
         const int done_end = s_go[cntx];
@@ -440,6 +431,7 @@ static __device__ __forceinline__ bool grid_gain_batch(const int32_t *__restrict
       if (pend) append(pend, nlev);
     }
     if (MODE == kModeFarness) {
+      flush_sums();
       cta_sync();
       if (tid < kLanes) {  // the vertices claimed at distance L + 1
         if (s_gain[tid]) atomicAdd(&ctl->dgain[(L + 1) % 3][tid], s_gain[tid]);
@@ -490,6 +482,7 @@ static __device__ __forceinline__ bool grid_gain_batch(const int32_t *__restrict
   // L = levels expanded
   // ---- results ----
   if (MODE == kModeGain) {
+    flush_sums();
     cta_sync();
     if (tid < kLanes && s_gain[tid]) atomicAdd(&ctl->gain[tid], s_gain[tid]);
   }
