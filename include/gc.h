@@ -374,6 +374,7 @@ int gc_top_closeness(gc_graph *g, int32_t k, const gc_opts *opts, int32_t *out_i
  *           (flags & GC_DEVICE_PTRS, copied); every weight >= 1 and the same
  *           in both rows of an edge.
  * flags   : GC_DEVICE_PTRS | GC_VALIDATE (also check the two rows agree).
+ * The handle also keeps its rows in the order of their weights (8 nnz bytes more).
  * Errors  : GC_EINVAL (a weight below 1, or rows that disagree under
  *           GC_VALIDATE), GC_ERANGE ((n - 1) x max weight >= 2^30: path
  *           lengths could overflow the int32 distances), GC_ENOMEM, GC_ECUDA. */
@@ -381,8 +382,8 @@ int gc_set_weights(gc_graph *g, const int32_t *weights, uint32_t flags);
 
 /* gc_greedy_weighted -- Greedy on the weighted graph: Algorithm 2 with weighted
  * distances, the pruned searches of Sec. 4.1 (valid for positive weights) and
- * the lazy bounds of Sec. 4.2; s0 = argmin f({v}) by a full search from every
- * vertex; ties to the smallest id.  Farness = sum of weighted distances (int64).
+ * the lazy bounds of Sec. 4.2; s0 = argmin f({v}) by a search from every vertex,
+ * cut once it cannot win any more; ties to the smallest id.  Farness = sum of weighted distances (int64).
  * Requires gc_set_weights.  k, opts, out_group, out_farness, stats: as
  * gc_greedy (stats: rounds, steps, evals, round0_evals, ms_total, launches).
  * Errors   : GC_EINVAL (no weights, bad k), GC_EDISCONNECTED, GC_ENOMEM,
@@ -396,7 +397,8 @@ int gc_greedy_weighted(gc_graph *g, int32_t k, const gc_opts *opts, int32_t *out
  * neighbours, the gain of u being sum_i |b^i_u AND NOT b^i_S| and, in round 0,
  * the farness of u being sum_i (n - |b^i_u|).  The vectors are held for 64 W
  * target vertices at a time (W <= 32 words per vertex, two buffers of n x W
- * words: the memory limit), and a target's bit is dropped once d_S of the
+ * words: the memory limit; for n <= 16,000, 32 targets per CTA in shared memory
+ * instead), and a target's bit is dropped once d_S of the
  * target is reached (pruning).  No lazy bounds: every round is a full sweep.
  * For small graphs: n <= 65536.
  * k, opts, out_group, out_farness, stats: as gc_greedy (stats: rounds, levels
@@ -420,7 +422,7 @@ int gc_greedy_bits(gc_graph *g, int32_t k, const gc_opts *opts, int32_t *out_gro
 #define GC_MLP_HIDDEN 64
 #define GC_MLP_PARAMS 4801
 
-typedef struct gc_mlp gc_mlp; /* opaque: parameters, Adam state, activation scratch */
+typedef struct gc_mlp gc_mlp; /* opaque: parameters, Adam state, partial gradients */
 
 /* gc_mlp_create -- a network with zero parameters; max_batch bounds the
  * minibatch of gc_mlp_grad / gc_mlp_adam_step / gc_mlp_train.  stream as in

@@ -151,7 +151,7 @@ constexpr int kBatchSweepMin = 1024;
 
 static __device__ __forceinline__ bool bsync(const BatchArgs &a) { return grid_sync(&a.ctl->bar, &a.ctl->err, a.tns); }
 
-// The pruned adjacency of the single-graph path (k_prune_count in gc_bfs.cu)
+// The pruned adjacency of the single-graph path (k_row_stats in gc_rows.cu)
 // over the union CSR, built inside the solve once d_S = d(s0, .) is known:
 // rows keep the neighbours with d_S >= 2, those with d_S >= 3 first (c3 of
 // them).  Count per vertex into a.q0 (free here), scan across CTAs (each
@@ -407,7 +407,7 @@ static __device__ void cta_build_list(const BatchArgs &a, int g) {
 }
 
 // Two-hop upper bound of Delta(v|S) for the group whose distances are d (the
-// inequality and its derivation are those of k_round1_bound in gc_bfs.cu):
+// inequality and its derivation are those of the round-1 bounds in gc_rows.cu):
 // d[v] + sum over the pruned row of v of ((d[w] - 1)^+ + c3[w]), plus the
 // graph's G3 = sum_u (d[u] - 3)^+ added by the caller.  One warp per v.
 static __device__ __forceinline__ long long warp_two_hop(const BatchArgs &a, const int32_t *d, const int32_t *c3,

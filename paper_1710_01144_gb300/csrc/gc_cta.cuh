@@ -25,7 +25,7 @@ struct GainCounters {
 // lanes of that word, which the expanding thread reads and clears; so no
 // separate commit pass is needed between levels.
 //
-// With c3 (the pruned adjacency, see k_prune_count), rp/ci are the pruned
+// With c3 (the pruned adjacency, see k_row_stats), rp/ci are the pruned
 // rows: level 0 scans a whole row, later levels only its first c3[u] entries.
 //
 // RO_GRAPH / RO_DS: read rp, ci, c3, mx / dS through the read-only data path.

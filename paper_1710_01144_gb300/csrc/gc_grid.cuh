@@ -1,6 +1,6 @@
 // Device-side bodies of the grid-wide kernels (cooperative launches): the
 // 64-lane pruned multi-source BFS for one batch (see gc_gain_grid.cu) and the
-// relabel BFS that maintains d_S (see gc_bfs.cu).  Both synchronise through a
+// relabel BFS that maintains d_S (k_bfs in gc_bfs.cu is its form as one launch).  Both synchronise through a
 // caller-supplied bounded grid barrier, so they can run as phases of a larger
 // persistent kernel (gc_lazy.cu).
 // The adjacency (rp, ci, c3) and the neighbour bound mx are read through the
@@ -66,7 +66,7 @@ static __device__ __forceinline__ int warp_find_start(const int32_t *start, int 
 // warp-wide search, stages the entries covering its slice in shared memory
 // and expands them edge by edge.  A vertex with nothing left to claim (gain
 // mode: every neighbour's d_S <= its level + 1) is counted but never queued.
-// With c3 (pruned adjacency, see k_prune_count) rp/ci are the pruned rows and
+// With c3 (pruned adjacency, see k_row_stats) rp/ci are the pruned rows and
 // levels >= 1 scan only their first c3[u] entries.  With voff/ws_n (one graph
 // of a block-diagonal union) the vertices are [voff, voff + ws_n): workspace 0
 // and gx are laid out for ws_n vertices and indexed by w - voff.
