@@ -327,7 +327,9 @@ int gc_load_csr(int32_t n, const int32_t *row_ptr, const int32_t *col_idx, uint3
   // graphs only (roads, grids, trees)
   if (nnz <= (int64_t)kSoloDegree * n) {
     if ((rc = solo_plan(n, g->num_sms, std::min<size_t>(free_b / 16, (size_t)1 << 30), &g->solo_ctas))) return bail(rc);
-    if (g->solo_ctas > 0 && (rc = dalloc(&g->solo_q, (size_t)g->solo_ctas * N))) return bail(rc);
+    if (g->solo_ctas > 0 && dalloc(&g->solo_q, (size_t)g->solo_ctas * N) != GC_OK) {
+      g->solo_ctas = 0;  // no room: deep graphs take the 64-lane batches
+    }
   }
   if (cudaMemsetAsync(g->ws, 0, (size_t)want * g->ws_stride, st) != cudaSuccess ||
       cudaMemsetAsync(g->hist, 0, kHistBins * sizeof(unsigned int), st) != cudaSuccess ||
