@@ -9,10 +9,10 @@
 #include <vector>
 
 #include "../../include/gc.h"
+#include "gc_rules.h"
 
 namespace gc {
 
-constexpr int32_t kInf = 0x3fffffff;  // "unreached" distance (d + 1 cannot overflow)
 constexpr int kLanes = 64;            // candidates per bit-parallel batch (one uint64 word)
 constexpr int kGainThreads = 512;     // threads per CTA of the gain kernel
 constexpr int kCta0SelectMax = 4096;  // lazy selection by CTA 0 up to this list length, grid-wide above

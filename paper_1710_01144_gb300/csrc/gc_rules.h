@@ -1,0 +1,27 @@
+// Rules that need neither a device nor the CUDA runtime: plain functions of
+// numbers, the same in kernels, host code and host-only programs.
+#pragma once
+
+#include <stdint.h>
+
+#ifdef __CUDACC__
+#define GC_HD __host__ __device__ __forceinline__
+#else
+#define GC_HD inline
+#endif
+
+namespace gc {
+
+constexpr int32_t kInf = 0x3fffffff;  // "unreached" distance (d + 1 cannot overflow)
+
+// Buckets of the weighted searches (gc_weighted.cu).  A bucket takes the entries
+// that lead to less than its end T; T = kInf - 1 is the last one and takes every
+// entry.  The end of the bucket after the nearest pending entry mn, `delta` wide:
+GC_HD int32_t w_bucket_end(int32_t mn, int32_t delta) { return mn > kInf - 1 - delta ? kInf - 1 : mn + delta; }
+// An entry that leads to distance x is in the bucket that ends at T.  The nearest
+// pending entry always is in the next bucket, so every bucket makes progress: an
+// entry may lead to exactly kInf - 1 (n vertices, weights of (2^30 - 2) / (n - 1)),
+// which x < T alone would leave pending for ever.
+GC_HD bool w_in_bucket(int32_t x, int32_t T) { return T == kInf - 1 || x < T; }
+
+}  // namespace gc

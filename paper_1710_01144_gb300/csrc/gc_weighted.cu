@@ -236,7 +236,7 @@ __global__ void __launch_bounds__(TH)
             du = dist(u);
             const int e1 = rp[u + 1];
             e0 = again ? ptr[u] : rp[u];
-            // (one bucket: the whole row)
+            // (the last bucket: the whole row)
             int lo = T == kInf - 1 ? e1 : e0, step = 4;  // galloping: the prefixes are short
             while (lo + step <= e1 && du + wt[lo + step - 1] < T) {
               lo += step;
@@ -327,10 +327,10 @@ __global__ void __launch_bounds__(TH)
         break;
       }
       // ---- the next bucket: rows with an entry below the new T go on ----
-      T = mn > kInf - 1 - delta ? kInf - 1 : mn + delta;
+      T = w_bucket_end(mn, delta);
       for (int q = tid; q < left; q += TH) {
         const int u = pend[q];
-        if (dist(u) + wt[ptr[u]] < T) cur[atomicAdd(&s_F, 1)] = ~u;
+        if (w_in_bucket(dist(u) + wt[ptr[u]], T)) cur[atomicAdd(&s_F, 1)] = ~u;
       }
     }
     cta_sync();
