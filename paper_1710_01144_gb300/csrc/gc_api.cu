@@ -677,7 +677,9 @@ int gc_set_weights(gc_graph *g, const int32_t *weights, uint32_t flags) {
   // the rows ordered by weight, for round 0 of gc_greedy_weighted
   g->w_max = h[1];
   int rc = GC_OK;
-  if (!g->ci_w && ((rc = dalloc(&g->ci_w, (size_t)g->nnz)) || (rc = dalloc(&g->wt_w, (size_t)g->nnz)))) return rc;
+  if (!alloc_missing([&](auto *&p) { return (rc = dalloc(&p, (size_t)g->nnz)) == GC_OK; }, [](void *p) { cudaFree(p); },
+                     g->ci_w, g->wt_w))
+    return rc;
   int32_t *tmp = nullptr;  // cif (scratch here) holds the ids of a middle pass, tmp its weights
   if (g->w_max > 255 && (rc = dalloc(&tmp, (size_t)g->nnz))) return rc;
   rc = launch_wsort(g, g->cif, tmp);

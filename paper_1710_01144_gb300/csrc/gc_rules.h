@@ -1,5 +1,5 @@
-// Rules that need neither a device nor the CUDA runtime: plain functions of
-// numbers, the same in kernels, host code and host-only programs.
+// Rules that need neither a device nor the CUDA runtime: plain functions, the same
+// in kernels, host code and host-only programs.
 #pragma once
 
 #include <stdint.h>
@@ -23,5 +23,25 @@ GC_HD int32_t w_bucket_end(int32_t mn, int32_t delta) { return mn > kInf - 1 - d
 // entry may lead to exactly kInf - 1 (n vertices, weights of (2^30 - 2) / (n - 1)),
 // which x < T alone would leave pending for ever.
 GC_HD bool w_in_bucket(int32_t x, int32_t T) { return T == kInf - 1 || x < T; }
+
+// Buffers that are only of use together: alloc(p) for each that is null, which sets
+// p and returns true, or returns false.  After a failure those that this call made
+// are given back by release(p) and null again, so that a later call starts over and
+// none is used while another is missing.
+template <class Alloc, class Release, class... T>
+bool alloc_missing(Alloc alloc, Release release, T *&...p) {
+  const bool had[] = {p != nullptr...};
+  bool ok = true;
+  ((ok = ok && (p || alloc(p))), ...);
+  if (ok) return true;
+  int i = 0;
+  auto back = [&](auto *&q, bool keep) {
+    if (keep) return;
+    if (q) release(q);
+    q = nullptr;
+  };
+  (back(p, had[i++]), ...);
+  return false;
+}
 
 }  // namespace gc

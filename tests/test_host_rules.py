@@ -15,6 +15,29 @@ using namespace gc;
 extern "C" {
 int32_t bucket_end(int32_t mn, int32_t delta) { return w_bucket_end(mn, delta); }
 int in_bucket(int32_t x, int32_t T) { return w_in_bucket(x, T); }
+
+// a stand-in for a device allocator: the allocation of index `fail` fails
+static int g_live, g_made, g_fail;
+static int g_cells[64];
+static bool fake_alloc(int *&p) {
+  if (g_made++ == g_fail) return false;
+  ++g_live;
+  p = &g_cells[g_made];
+  return true;
+}
+// three buffers, of which the bits of `had` are there already; returns the bits of
+// those that are there after the call, with bit 8 set if it succeeded
+static int *g_p[3];
+int buffers(int had, int fail) {
+  g_live = g_made = 0;
+  g_fail = fail;
+  for (int i = 0; i < 3; ++i) g_p[i] = (had >> i) & 1 ? &g_cells[40 + i] : nullptr;
+  const bool ok = alloc_missing(fake_alloc, [](int *) { --g_live; }, g_p[0], g_p[1], g_p[2]);
+  int there = 0;
+  for (int i = 0; i < 3; ++i) there |= (g_p[i] != nullptr) << i;
+  return there | (ok ? 256 : 0);
+}
+int live() { return g_live; }
 }
 """
 
@@ -37,3 +60,13 @@ def test_next_bucket_takes_the_nearest_entry(rules, mn, delta):
     assert T <= INF - 1 and (T == INF - 1 or T == mn + delta)
     if T < INF - 1:  # and nothing past its end
         assert not rules.in_bucket(T, T) and rules.in_bucket(T - 1, T)
+
+
+@pytest.mark.parametrize("had", range(8))
+def test_buffers_of_a_group_come_and_go_together(rules, had):
+    missing = 3 - bin(had).count("1")
+    for fail in range(missing):  # none stays behind without the others, none is lost
+        assert rules.buffers(had, fail) == had
+        assert rules.live() == 0
+    assert rules.buffers(had, missing) == 256 | 7
+    assert rules.live() == missing
