@@ -1463,11 +1463,11 @@ struct gc_batch {
   LazyCtl *lc = nullptr;
   int32_t *act = nullptr, *act_n = nullptr, *kk = nullptr, *bstart = nullptr;
   int32_t A = 0, act_cap = 0;
-  int32_t kcap = 0;
+  int32_t kcap = 0, h_kcap = 0;  // picks a graph that the device buffers, the pinned copy hold
   int32_t *picks = nullptr;
   long long *pgain = nullptr;
   int32_t *seeds = nullptr;
-  int32_t seeds_cap = 0;
+  int64_t seeds_cap = 0;
   int32_t *slist = nullptr, *scount = nullptr, *tstart = nullptr;
   BatchCtl *ctl = nullptr, *h_ctl = nullptr;
   GainCtl *gctl = nullptr, *h_gctl = nullptr;
@@ -1722,59 +1722,31 @@ int gc_batch_greedy(gc_batch *b, const int32_t *ks, const gc_opts *opts_in, int3
   const bool capture = (opts.flags & GC_OPT_CAPTURE) != 0;
   auto t0 = std::chrono::steady_clock::now();
   cudaStream_t st = b->stream;
-  // (re)size per-call buffers; a resize invalidates a captured sequence
-  bool resized = false;
-  if (kmax > b->kcap) {
-    cudaFree(b->picks);
-    cudaFree(b->pgain);
-    b->picks = nullptr;
-    b->pgain = nullptr;
-    if (!balloc(&b->picks, (size_t)b->count * kmax) || !balloc(&b->pgain, (size_t)b->count * kmax)) {
-      set_error("gc_batch_greedy: allocation failed");
-      return GC_ENOMEM;
-    }
-    b->kcap = kmax;
-    resized = true;
-    if (b->h_picks_pinned) cudaFreeHost(b->h_picks_pinned);
-    if (cudaMallocHost((void **)&b->h_picks_pinned, (size_t)b->count * kmax * sizeof(int32_t)) != cudaSuccess) {
-      set_error("gc_batch_greedy: pinned allocation failed");
-      return GC_ENOMEM;
-    }
-  }
-  if (!b->h_far_pinned && cudaMallocHost((void **)&b->h_far_pinned, (size_t)b->count * sizeof(long long)) != cudaSuccess) {
-    set_error("gc_batch_greedy: pinned allocation failed");
+  // (re)size per-call buffers; a resize, or a failed one, invalidates a captured sequence
+  const int64_t need_seeds = std::max<int64_t>(b->count, ksum);
+  if (kmax > b->kcap || need_seeds > b->seeds_cap || A > b->act_cap) b->cap_k.clear();
+  const auto dev = [](size_t count) { return [count](auto *&p) { return balloc(&p, count); }; };
+  const auto dev_free = [](void *p) { cudaFree(p); };
+  const auto pin = [](size_t count) {
+    return [count](auto *&p) { return cudaMallocHost((void **)&p, count * sizeof(*p)) == cudaSuccess; };
+  };
+  const auto pin_free = [](void *p) { cudaFreeHost(p); };
+  const size_t graphs = (size_t)b->count;
+  if (!grow_buffers(b->kcap, kmax, dev(graphs * kmax), dev_free, b->picks, b->pgain) ||
+      !grow_buffers(b->seeds_cap, need_seeds, dev((size_t)need_seeds), dev_free, b->seeds) ||
+      !grow_buffers(b->act_cap, A, dev(graphs * A), dev_free, b->act)) {
+    set_error("gc_batch_greedy: allocation failed");
     return GC_ENOMEM;
   }
-  const int64_t need_seeds = std::max<int64_t>(b->count, ksum);
-  if (need_seeds > b->seeds_cap) {
-    cudaFree(b->seeds);
-    if (!balloc(&b->seeds, (size_t)need_seeds)) {
-      set_error("gc_batch_greedy: allocation failed");
-      return GC_ENOMEM;
-    }
-    b->seeds_cap = (int32_t)need_seeds;
-    resized = true;
-  }
-  if (A > b->act_cap) {
-    cudaFree(b->act);
-    if (!balloc(&b->act, (size_t)b->count * A)) {
-      set_error("gc_batch_greedy: allocation failed");
-      return GC_ENOMEM;
-    }
-    b->act_cap = A;
-    resized = true;
-  }
-  if (!b->h_k_pinned && (cudaMallocHost((void **)&b->h_k_pinned, (size_t)b->count * sizeof(int32_t)) != cudaSuccess ||
-                         cudaMallocHost((void **)&b->h_bstart_pinned, ((size_t)b->count + 1) * sizeof(int32_t)) !=
-                             cudaSuccess ||
-                         cudaMallocHost((void **)&b->h_order_pinned, (size_t)b->count * sizeof(int32_t)) !=
-                             cudaSuccess)) {
+  if (!grow_buffers(b->h_kcap, kmax, pin(graphs * kmax), pin_free, b->h_picks_pinned) ||
+      !alloc_missing(pin(graphs + 1), pin_free, b->h_far_pinned, b->h_k_pinned, b->h_bstart_pinned, b->h_order_pinned)) {
+    cudaGetLastError();
     set_error("gc_batch_greedy: pinned allocation failed");
     return GC_ENOMEM;
   }
   std::vector<int32_t> bstart(b->count + 1, 0);
   for (int32_t g = 0; g < b->count; ++g) bstart[g + 1] = bstart[g] + (b->h_n[g] + lanes1 - 1) / lanes1;
-  const bool same = b->exec && !resized && b->cap_k == std::vector<int32_t>(ks, ks + b->count) && b->cap_A == A && b->cap_grid_min_n == opts.batch_grid_min_n && b->cap_flags == opts.flags &&
+  const bool same = b->exec && b->cap_k == std::vector<int32_t>(ks, ks + b->count) && b->cap_A == A && b->cap_grid_min_n == opts.batch_grid_min_n && b->cap_flags == opts.flags &&
                     b->cap_lanes == lanes1 && b->cap_lazy_ctas == opts.lazy_ctas;
   BatchArgs a;
   a.rp = b->rp;

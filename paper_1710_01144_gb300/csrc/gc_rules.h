@@ -44,4 +44,20 @@ bool alloc_missing(Alloc alloc, Release release, T *&...p) {
   return false;
 }
 
+// Buffers that grow together: cap follows what is there, also when a growth fails
+// (0 then, with every pointer null).  False on a failure.
+template <class Cap, class Alloc, class Release, class... T>
+bool grow_buffers(Cap &cap, Cap want, Alloc alloc, Release release, T *&...p) {
+  if (want <= cap) return true;
+  auto drop = [&](auto *&q) {
+    if (q) release(q);
+    q = nullptr;
+  };
+  (drop(p), ...);
+  cap = 0;
+  if (!alloc_missing(alloc, release, p...)) return false;
+  cap = want;
+  return true;
+}
+
 }  // namespace gc

@@ -38,6 +38,18 @@ int buffers(int had, int fail) {
   return there | (ok ? 256 : 0);
 }
 int live() { return g_live; }
+
+// two buffers of one capacity: bit 0 and 1 for those that are there, bit 8 for
+// success, and the capacity from bit 9 on
+static int *g_q[2];
+static int g_cap;
+void grow_start() { g_q[0] = g_q[1] = nullptr; g_cap = g_live = 0; }
+int grow(int want, int fail) {
+  g_made = 0;
+  g_fail = fail;
+  const bool ok = grow_buffers(g_cap, want, fake_alloc, [](int *) { --g_live; }, g_q[0], g_q[1]);
+  return (g_q[0] != nullptr) | (g_q[1] != nullptr) << 1 | (ok ? 256 : 0) | g_cap << 9;
+}
 }
 """
 
@@ -70,3 +82,13 @@ def test_buffers_of_a_group_come_and_go_together(rules, had):
         assert rules.live() == 0
     assert rules.buffers(had, missing) == 256 | 7
     assert rules.live() == missing
+
+
+def test_capacity_follows_the_buffers(rules):
+    rules.grow_start()
+    assert rules.grow(5, 9) == 3 | 256 | 5 << 9
+    assert rules.grow(4, 0) == 3 | 256 | 5 << 9  # large enough: nothing is allocated
+    for fail in (0, 1):
+        assert rules.grow(8, fail) == 0 and rules.live() == 0  # no buffer, and no capacity either
+        assert rules.grow(4, fail) == 0  # so a smaller want is not taken for granted
+        assert rules.grow(4, 9) == 3 | 256 | 4 << 9 and rules.live() == 2
