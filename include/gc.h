@@ -20,7 +20,9 @@
  *
  * Graph format: int32 CSR.  row_ptr[n+1] with row_ptr[0] = 0 and
  * non-decreasing entries; col_idx[row_ptr[n]] neighbour ids in [0, n); each
- * undirected edge is stored in both rows.  nnz = row_ptr[n] < 2^31.
+ * undirected edge is stored in both rows.  nnz = row_ptr[n] < 2^31.  Rows that
+ * are not strictly increasing, or that repeat an entry or hold their own vertex,
+ * give the same results (GC_VALIDATE refuses them), a little slower.
  *
  * Streams: every call is ordered on the stream given to gc_load_csr (a
  * cudaStream_t passed as void*, NULL = legacy default stream).  Calls that

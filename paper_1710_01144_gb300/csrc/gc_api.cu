@@ -349,6 +349,9 @@ int gc_load_csr(int32_t n, const int32_t *row_ptr, const int32_t *col_idx, uint3
     cudaFree(g->dec);
     g->dec = nullptr;
     if (rc) return bail(rc);
+    g->simple = 1;  // checked
+  } else if ((rc = simple_rows(g->rp, g->ci, n, nnz, g->num_sms, st, g->g3, &g->simple))) {
+    return bail(rc);
   }
   if (cudaStreamSynchronize(st) != cudaSuccess) return bail(fail(GC_ECUDA, "load failed"));
   *out = g;

@@ -134,6 +134,7 @@ struct BatchArgs {
   int32_t team_size;
   int32_t list_cap;   // entries of a shared-memory list (a power of two, at most kCta0SelectMax)
   int32_t grid_min_n; // graphs with at least this many vertices run their lazy rounds grid-wide
+  int32_t simple;     // no row holds an entry twice or its own vertex
   int32_t bounded;    // round 1 with two-hop bounds (batch_round1_bounded) and the refresh after it
   long long *g3;      // [2 * count]: sum of (d - 3)^+ per graph for round 1, then for the refresh
   unsigned long long tns;
@@ -496,7 +497,7 @@ static __device__ __noinline__ bool team_batch(const BatchArgs &a, int g, const 
   return grid_gain_batch<MODE>(gain ? a.rpf : a.rp, gain ? a.cif : a.ci, a.N, gain ? a.dS1 : a.dS, cand, nl, nullptr,
                                s_out, ws0, gx, a.goff, &tc->gg, a.gctl, &tc->bar, &a.ctl->err, a.tns,
                                gain ? a.mx : nullptr, gain ? a.c3 : nullptr, o, a.max_n, kBatchAll, nullptr, nullptr,
-                               0, nullptr, tm, gx_n, gain ? nullptr : &tc->best, a.ng[g]);
+                               0, nullptr, tm, gx_n, gain ? nullptr : &tc->best, a.ng[g], a.simple != 0);
 }
 
 // The tasks of the lists in slist (scount entries per graph) that tstart counts,
@@ -943,7 +944,7 @@ static __device__ bool team_lazy(const BatchArgs &a, int g, TeamCtl *tc, Team tm
         if (d == 0)
           grid_gain_batch<kModeGain>(a.rpf, a.cif, a.N, a.dS, s_st.sel, 0, &s_st.nsel, s_st.gout, ws0, gx, a.goff,
                                      &tc->gg, a.gctl, &tc->bar, &a.ctl->err, a.tns, a.mx, a.c3, o, a.max_n,
-                                     kBatchLevel0, clog, &lc->log_n, clog_cap, nullptr, tm, ng);
+                                     kBatchLevel0, clog, &lc->log_n, clog_cap, nullptr, tm, ng);  // (the candidates alone)
       }
     } else if (wide) {
       if (b == 0)
@@ -996,7 +997,8 @@ static __device__ bool team_lazy(const BatchArgs &a, int g, TeamCtl *tc, Team tm
         if (!grid_gain_batch<kModeGain>(a.rpf, a.cif, a.N, a.dS, st0 ? s_st.sel : lc->sel, 0,
                                         st0 ? &s_st.nsel : &lc->n_sel, st0 ? s_st.gout : lc->gsel, ws0, gx, a.goff,
                                         &tc->gg, a.gctl, &tc->bar, &a.ctl->err, a.tns, a.mx, a.c3, o, a.max_n,
-                                        lean ? kBatchRest : kBatchAll, clog, &lc->log_n, clog_cap, &gcnt, tm, ng))
+                                        lean ? kBatchRest : kBatchAll, clog, &lc->log_n, clog_cap, &gcnt, tm, ng,
+                                        nullptr, 0, a.simple != 0))
           return false;
         if (!lean && !sync()) return false;  // a team-wide fold reads the gains CTA 0 wrote
         if (lead && *(volatile int32_t *)&tc->gg.err) atomicExch(&a.ctl->err, *(volatile int32_t *)&tc->gg.err);
@@ -1459,6 +1461,7 @@ struct gc_batch {
   size_t ws_stride = 0;
   unsigned long long *packed = nullptr;
   unsigned long long *cls = nullptr;
+  int32_t simple = 0;
   long long *fa = nullptr, *farness = nullptr, *bestf = nullptr, *g3 = nullptr;
   LazyCtl *lc = nullptr;
   int32_t *act = nullptr, *act_n = nullptr, *kk = nullptr, *bstart = nullptr;
@@ -1668,7 +1671,8 @@ static int batch_load_impl(int32_t count, const int32_t *const *row_ptrs, const 
   if (cp) {
     k_union_fix<<<b->num_sms * 8, 256, 0, st>>>(b->rp, b->ci, b->gid, b->off, d_eoff, count, (int32_t)N, E);
     k_iota<<<b->num_sms * 8, 256, 0, st>>>(b->iota, (int32_t)N);
-    cp = cudaGetLastError() == cudaSuccess && cudaStreamSynchronize(st) == cudaSuccess;
+    cp = cudaGetLastError() == cudaSuccess && simple_rows(b->rp, b->ci, (int32_t)N, E, b->num_sms, st,
+                                                          reinterpret_cast<unsigned long long *>(b->g3), &b->simple) == GC_OK;
   }
   cudaFree(d_eoff);
   if (!cp) {
@@ -1783,6 +1787,7 @@ int gc_batch_greedy(gc_batch *b, const int32_t *ks, const gc_opts *opts_in, int3
   a.cls = b->cls;
   a.bounded = (opts.flags & GC_OPT_NO_ROUND1_BOUND) ? 0 : 1;
   a.g3 = b->g3;
+  a.simple = b->simple;
   a.grid_min_n = opts.batch_grid_min_n == 0 ? kBatchGridMinN
                  : (opts.batch_grid_min_n < 0 ? INT32_MAX : opts.batch_grid_min_n);
   // the lazy rounds' plan: the graphs left to teams, longest first, and the

@@ -30,9 +30,11 @@ __global__ void __launch_bounds__(kGridGainThreads, 2)
                  const int32_t *__restrict__ dS, const int32_t *__restrict__ cand, int32_t nl_arg,
                  const int32_t *__restrict__ nl_dev, long long *__restrict__ out, unsigned char *ws_base,
                  int32_t *gx, int32_t *__restrict__ goff, GridGainCtl *ctl, GainCtl *gctl,
-                 unsigned long long timeout_ns, const int32_t *__restrict__ mx, const int32_t *__restrict__ c3) {
+                 unsigned long long timeout_ns, const int32_t *__restrict__ mx, const int32_t *__restrict__ c3,
+                 int32_t simple) {
   grid_gain_batch<MODE>(rp, ci, n, dS, cand, nl_arg, nl_dev, out, ws_base, gx, goff, ctl, gctl, &ctl->bar,
-                        &ctl->err, timeout_ns, mx, c3);
+                        &ctl->err, timeout_ns, mx, c3, 0, -1, kBatchAll, nullptr, nullptr, 0, nullptr, whole_grid(), -1,
+                        nullptr, 0, simple != 0);
 }
 
 int grid_gain_occupancy(int *blocks_per_sm) {
@@ -51,7 +53,7 @@ int launch_gains_grid(gc_graph *g, int mode, const int32_t *cand, int32_t nl, co
   const bool pr = pruned && mode == kModeGain;
   const int32_t *rp = pr ? g->rpf : g->rp, *ci = pr ? g->cif : g->ci, *dS = g->dS;
   const int32_t *c3 = pr ? g->c3 : nullptr;
-  int32_t n = g->n;
+  int32_t n = g->n, simple = g->simple;
   unsigned char *ws = g->ws;
   int32_t *gx = g->gx;
   int32_t *goff = g->goff;
@@ -61,7 +63,7 @@ int launch_gains_grid(gc_graph *g, int mode, const int32_t *cand, int32_t nl, co
   const int32_t *mx = mode == kModeGain ? g->mx : nullptr;
   void *args[] = {(void *)&rp,  (void *)&ci,   (void *)&n,   (void *)&dS,  (void *)&cand,
                   (void *)&nl,  (void *)&nl_dev, (void *)&out, (void *)&ws, (void *)&gx, (void *)&goff,
-                  (void *)&ctl, (void *)&gctl, (void *)&tns, (void *)&mx, (void *)&c3};
+                  (void *)&ctl, (void *)&gctl, (void *)&tns, (void *)&mx, (void *)&c3, (void *)&simple};
   ++g->launches;
   if (mode == kModeGain)
     GC_CUDA(cudaLaunchCooperativeKernel((const void *)k_gains_grid<kModeGain>, dim3(g->grid_ctas),

@@ -79,6 +79,8 @@ static __device__ __forceinline__ int warp_find_start(const int32_t *start, int 
 // {w, L, lanes won}, except the neighbours of a candidate at d_S = 2 (see below:
 // a pick's row holds them, log_update_row), at *log_n (one warp-aggregated slot per claim round); slots
 // at or past log_cap are counted in *log_n but not written.
+// simple: no row holds an entry twice or its own vertex (needed by that exception;
+// otherwise these neighbours are claimed and logged like all others).
 // With `acc`, each thread adds its work counts (scalar and union adjacency
 // entries, frontier entries, pushes) to *acc instead of the batch summing them
 // over the CTA and into gctl (a persistent caller sums them once at its end).
@@ -102,7 +104,7 @@ static __device__ __forceinline__ bool grid_gain_batch(const int32_t *__restrict
                                 int phase = kBatchAll, ClaimRec *log = nullptr,
                                 unsigned long long *log_n = nullptr, unsigned long long log_cap = 0,
                                 GridCounts *acc = nullptr, Team tm = whole_grid(), int gx_n = -1,
-                                const long long *best_of = nullptr, int n_graph = 0) {
+                                const long long *best_of = nullptr, int n_graph = 0, bool simple = false) {
   constexpr int T = kGridGainThreads;
   __shared__ u64 s_gain[kLanes];
   __shared__ unsigned int s_cnt[kLanes];
@@ -124,6 +126,7 @@ static __device__ __forceinline__ bool grid_gain_batch(const int32_t *__restrict
   const int nl = nl_dev ? min(kLanes, *(volatile const int32_t *)nl_dev) : nl_arg;
   if (ws_n < 0) ws_n = n;
   if (gx_n < 0) gx_n = ws_n;
+  const int count2 = simple ? 2 : 0;  // the d_S that a level-0 neighbour is counted at without a claim
   const long long n_all = best_of ? n_graph : n;  // farness mode: the vertices a search must reach
   const GainWs ws = gain_ws(ws_base, 0, ws_n, 0);
   // frontier lists by level mod 3 and range starts by level parity (selected,
@@ -324,7 +327,7 @@ static __device__ __forceinline__ bool grid_gain_batch(const int32_t *__restrict
           s_go[tid] = qstart[xi];
           s_sm[tid] = m;
           s_rs[tid] = __ldg(rp + u);
-          if (MODE == kModeGain) s_c3[tid] = (L == 0 && c3) ? __ldg(c3 + u) : INT_MAX;
+          if (MODE == kModeGain) s_c3[tid] = (L == 0 && c3 && count2) ? __ldg(c3 + u) : INT_MAX;
           if (s_go[tid] >= es && s_go[tid] < ee) {  // counted once: by the CTA holding the entry's first edge
             const int deg = (c3 && L > 0) ? __ldg(c3 + u) : __ldg(rp + u + 1) - s_rs[tid];
             c_union += (u64)deg;
@@ -387,7 +390,7 @@ static __device__ __forceinline__ bool grid_gain_batch(const int32_t *__restrict
           // expanded at level nlev only if some neighbour may still be claimed.
           // A neighbour at d_S = 2 of a candidate (level 0) gains 1 and that is
           // all: no later level can claim it (that takes d_S > 2), and the row
-          // holds it once.  So it is neither marked visited nor logged; the d_S
+          // holds it once (simple rows).  So it is neither marked visited nor logged; the d_S
           // update takes such vertices from the pick's own row.  They are most of
           // a batch's claims, each otherwise two atomics on a random 32-byte
           // record and a log entry: lazy rounds of R-MAT scale 24 (283 MB of
@@ -395,7 +398,7 @@ static __device__ __forceinline__ bool grid_gain_batch(const int32_t *__restrict
           u64 ov[kGridIlp], on[kGridIlp];
 #pragma unroll
           for (int k = 0; k < kGridIlp; ++k) {
-            two[k] = MODE == kModeGain && L == 0 && dw[k] == 2;
+            two[k] = MODE == kModeGain && L == 0 && dw[k] == count2;
             ov[k] = !nb[k] ? ~0ull : two[k] ? 0ull : atomicOr(&ws.vis[w[k] - voff], nb[k]);
             on[k] = (nb[k] && mxw[k] > nlev + 1) ? atomicOr(&nxt[w[k] - voff], nb[k]) : ~0ull;
           }

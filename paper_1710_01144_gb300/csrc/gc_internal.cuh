@@ -297,6 +297,7 @@ struct gc_graph {
   int w_ctas = 0;
   unsigned int *w_task = nullptr;
   int32_t w_max = 0;               // largest weight
+  int32_t simple = 0;              // no row holds an entry twice or its own vertex (simple_rows)
   int32_t *ci_w = nullptr, *wt_w = nullptr;  // the rows ordered by weight (built by gc_set_weights)
   // candidates per batch of the CTA-batched gain kernel (gc_set_gain_lanes):
   // 64, or 128 / 256 for the wide kernel (gc_gain_wide.cu), whose per-CTA
@@ -504,6 +505,10 @@ int launch_round1_propose(gc_graph *g, long long prev_gain);
 // upper bound for every later d_S), the pruned rows' sizes (g->io_a, g->c3), the
 // terms of the round-1 bounds (g->c3s) and d_S as classes (g->bq0)
 int launch_row_stats(gc_graph *g);
+// *simple <- 1 if every row is strictly increasing and none holds its own vertex
+// (waits for the stream; bad: scratch, one word)
+int simple_rows(const int32_t *rp, const int32_t *ci, int32_t n, int64_t nnz, int num_sms, cudaStream_t stream,
+                unsigned long long *bad, int32_t *simple);
 // the list of long rows used by the row-wise kernels' CTA-per-row companions
 int launch_heavy_rows(gc_graph *g);
 // pruned adjacency (g->rpf, g->cif, g->c3), directly after launch_row_stats

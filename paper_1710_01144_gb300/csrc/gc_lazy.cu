@@ -42,7 +42,7 @@ __global__ void __launch_bounds__(kGridGainThreads, 1)
                   int32_t wide, long long local_max, long long *akey, int32_t *ast,
                   int32_t *gx, int32_t *wsel, long long *wgain, int32_t *wpos, int32_t wcap,
                   const int32_t *__restrict__ rp_full, const int32_t *__restrict__ c3, GridSelScratch *gsel,
-                  ClaimRec *clog, unsigned long long clog_cap) {
+                  ClaimRec *clog, unsigned long long clog_cap, int32_t simple) {
   __shared__ unsigned long long s_red[32];
   extern __shared__ __align__(16) unsigned char s_list[];  // kLazyListSmem bytes
   const int m = *m_dev;
@@ -141,7 +141,7 @@ __global__ void __launch_bounds__(kGridGainThreads, 1)
           if (d == 0) {
             grid_gain_batch<kModeGain>(rp, ci, n, dS, s_st.sel, 0, &s_st.nsel, s_st.gout, ws, gx, goff, gg, gctl,
                                        &lc->bar, &lc->err, tns, mx, c3, 0, -1, kBatchLevel0, clog, &lc->log_n,
-                                       clog_cap);
+                                       clog_cap);  // (level 0: the candidates alone)
           } else if (d == 1 && threadIdx.x == 0) {
             picks[r] = s_st.bid;
             pgain[r] = s_st.bgain;
@@ -181,7 +181,7 @@ __global__ void __launch_bounds__(kGridGainThreads, 1)
       } else {
         ok = grid_gain_batch<kModeGain>(rp, ci, n, dS, bsel, 0, bnsel, bout, ws, gx, goff, gg, gctl, &lc->bar,
                                         &lc->err, tns, mx, c3, 0, -1, lean ? kBatchRest : kBatchAll, clog,
-                                        &lc->log_n, clog_cap, &gcnt);
+                                        &lc->log_n, clog_cap, &gcnt, whole_grid(), -1, nullptr, 0, simple != 0);
         // the gains are in lc->gsel, written by CTA 0: only a grid-wide fold
         // needs them published
         if (!lean) ok = ok && grid_sync(&lc->bar, &lc->err, tns);
@@ -343,7 +343,7 @@ int launch_lazy_rounds(gc_graph *g, int32_t k, int64_t timeout_ns, const float *
   const int32_t *rp = pruned ? g->rpf : g->rp, *ci = pruned ? g->cif : g->ci;
   const int32_t *rp_full = g->rp, *c3 = pruned ? g->c3 : nullptr;
   GridSelScratch *gsel = g->gsel;
-  int32_t n = g->n;
+  int32_t n = g->n, simple = g->simple;
   int32_t *dS = g->dS;
   long long *ub = g->ub;
   int32_t *stamp = g->stamp;
@@ -375,7 +375,8 @@ int launch_lazy_rounds(gc_graph *g, int32_t k, int64_t timeout_ns, const float *
                   (void *)&mx,    (void *)&prop,  (void *)&fill, (void *)&two_hop, (void *)&score,
                   (void *)&ws_stride, (void *)&wide, (void *)&local_max, (void *)&akey,
                   (void *)&ast, (void *)&gx, (void *)&wsel, (void *)&wgain, (void *)&wpos, (void *)&wcap,
-                  (void *)&rp_full, (void *)&c3, (void *)&gsel, (void *)&clog, (void *)&clog_cap};
+                  (void *)&rp_full, (void *)&c3, (void *)&gsel, (void *)&clog, (void *)&clog_cap,
+                  (void *)&simple};
   ++g->launches;
   GC_CUDA(cudaLaunchCooperativeKernel((const void *)k_lazy_rounds, dim3(grid), dim3(kGridGainThreads), args,
                                       kLazyListSmem, g->stream));
