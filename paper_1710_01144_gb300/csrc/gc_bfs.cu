@@ -42,6 +42,9 @@ __global__ void k_fill_i64(long long *p, long long v, int64_t count) {
 //   level after level until it grows past that, while the others wait at one grid
 //   barrier.  A level then costs a CTA's dependent loads (2 us) without the grid
 //   barrier and the list's trip through L2: deep graphs have nothing but such levels.
+//   After kBfsLocalLevels of them all CTAs meet, so that no wait grows with the depth
+//   of the graph (the time limit is each wait's, and a path of millions of vertices
+//   takes seconds).
 // - bottom-up (fresh only): when the frontier holds more entries than an eighth of
 //   those left, every unreached vertex looks in its own row for a neighbour at the
 //   frontier's distance and stops at the first: on R-MAT graphs the frontier at
@@ -55,6 +58,7 @@ __global__ void k_fill_i64(long long *p, long long v, int64_t count) {
 // with short distances, where a larger kBfsLocal (4096) lost (64 x 64, 100 seeds:
 // 243 against 171 us, 216 before).
 constexpr int kBfsLocal = 768;   // adjacency entries (three per thread)
+constexpr int kBfsLocalLevels = 256;  // half a millisecond
 constexpr int kBfsStage = 256;    // frontier entries staged at a time (= threads)
 
 __global__ void __launch_bounds__(kBfsThreads) k_bfs(const int32_t *__restrict__ rp, const int32_t *__restrict__ ci,
@@ -216,7 +220,7 @@ __global__ void __launch_bounds__(kBfsThreads) k_bfs(const int32_t *__restrict__
           ++l;
           F = (int)(pk >> 32);
           E = (long long)(pk & 0xffffffffull);
-          if (F == 0 || E > kBfsLocal) break;
+          if (F == 0 || E > kBfsLocal || l - L >= kBfsLocalLevels) break;
         }
         if (tid == 0) {
           ctl->local_pk = pk;
