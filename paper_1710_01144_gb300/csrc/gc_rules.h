@@ -24,6 +24,21 @@ GC_HD int32_t w_bucket_end(int32_t mn, int32_t delta) { return mn > kInf - 1 - d
 // which x < T alone would leave pending for ever.
 GC_HD bool w_in_bucket(int32_t x, int32_t T) { return T == kInf - 1 || x < T; }
 
+// Whether vertex v, entry i of a list of m, is in the list's sample of about `want`:
+// spread by a hash of its id and `salt`.  The first entry always is, so that no
+// sample is empty (one of few CTAs' worth often would be: want = 1 in 37 of 100
+// lists) and a lazy step always has a candidate to search.
+GC_HD bool sample_takes(int32_t i, int32_t v, int32_t m, int32_t want, uint32_t salt) {
+  const uint64_t lim = m > want ? ((uint64_t)want << 32) / (uint64_t)m : ~0ull;
+  uint32_t h = ((uint32_t)v + 1u + salt * 0x10001u) * 0x9E3779B1u;  // multiplicative hashing (2^32 over the golden ratio)
+  h ^= h >> 16;
+  h *= 0x9E3779B1u;
+  h ^= h >> 13;
+  h *= 0x9E3779B1u;
+  h ^= h >> 16;
+  return i == 0 || (uint64_t)h < lim;
+}
+
 // Buffers that are only of use together: alloc(p) for each that is null, which sets
 // p and returns true, or returns false.  After a failure those that this call made
 // are given back by release(p) and null again, so that a later call starts over and

@@ -334,23 +334,16 @@ int launch_relax(gc_graph *g, bool farness, const int32_t *region, int32_t hops,
   return GC_OK;
 }
 
-// About `want` of the m listed vertices, spread by a hash of their id and
-// `salt`, into `sample`; *count (zeroed by the caller) gets how many, at most m.
+// About `want` of the m listed vertices (sample_takes) into `sample`; *count (zeroed
+// by the caller) gets how many, 1 to m.
 __global__ void k_sample(const int32_t *__restrict__ list, const int32_t *m_dev, int32_t want, uint32_t salt,
                          int32_t *sample, int32_t *count) {
   const int m = *m_dev;
-  const u64 lim = m > want ? ((u64)want << 32) / (u64)m : ~0ull;
   const int lane = threadIdx.x & 31;
   for (int base = (blockIdx.x * blockDim.x + threadIdx.x) & ~31; base < m; base += gridDim.x * blockDim.x) {
     const int i = base + lane;
     const int v = i < m ? list[i] : 0;
-    uint32_t h = ((uint32_t)v + 1u + salt * 0x10001u) * 0x9E3779B1u;  // multiplicative hashing (2^32 over the golden ratio)
-    h ^= h >> 16;
-    h *= 0x9E3779B1u;
-    h ^= h >> 13;
-    h *= 0x9E3779B1u;
-    h ^= h >> 16;
-    const bool take = i < m && (u64)h < lim;
+    const bool take = i < m && sample_takes(i, v, m, want, salt);
     const unsigned tm = __ballot_sync(0xffffffffu, take);
     int at = 0;
     if (lane == 0 && tm) at = atomicAdd(count, __popc(tm));

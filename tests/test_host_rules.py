@@ -4,6 +4,7 @@ import ctypes
 import os
 import subprocess
 
+import numpy as np
 import pytest
 
 CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_1710_01144_gb300", "csrc")
@@ -15,6 +16,12 @@ using namespace gc;
 extern "C" {
 int32_t bucket_end(int32_t mn, int32_t delta) { return w_bucket_end(mn, delta); }
 int in_bucket(int32_t x, int32_t T) { return w_in_bucket(x, T); }
+
+int sample(const int32_t *list, int m, int want, uint32_t salt) {
+  int c = 0;
+  for (int i = 0; i < m; ++i) c += sample_takes(i, list[i], m, want, salt);
+  return c;
+}
 
 // a stand-in for a device allocator: the allocation of index `fail` fails
 static int g_live, g_made, g_fail;
@@ -92,3 +99,19 @@ def test_capacity_follows_the_buffers(rules):
         assert rules.grow(8, fail) == 0 and rules.live() == 0  # no buffer, and no capacity either
         assert rules.grow(4, fail) == 0  # so a smaller want is not taken for granted
         assert rules.grow(4, 9) == 3 | 256 | 4 << 9 and rules.live() == 2
+
+
+@pytest.mark.parametrize("want", [1, 2, 5, 64, 2432])
+def test_samples_are_never_empty(rules, want):
+    rng = np.random.default_rng(want)
+    sizes = []
+    for salt in range(60):
+        for m in (1, want, 2 * want + 1, 40 * want):
+            v = np.sort(rng.choice(100 * want + 50, m, replace=False)).astype(np.int32)
+            c = rules.sample(v.ctypes.data_as(ctypes.c_void_p), m, want, salt)
+            assert 1 <= c <= m
+            if m <= want:
+                assert c == m
+            elif m == 40 * want:
+                sizes.append(c)
+    assert abs(np.mean(sizes) - want) <= 1 + 4 * np.sqrt(want / len(sizes))  # the mean of binomial counts, and the first entry
