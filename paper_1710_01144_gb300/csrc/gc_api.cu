@@ -79,7 +79,7 @@ static void release(gc_graph *g) {
                  g->ws, g->dec, g->ggctl, g->goff, g->lctl, g->picks, g->pgain, g->pdec, g->mx_buf,
                  g->two_hop, g->score, g->rec_count, g->akey, g->ast, g->gx, g->wsel, g->wpos, g->wgain,
                  g->lev_cnt, g->lev_C, g->lev_M, g->lev_max, g->rpf, g->cif, g->c3, g->gsel, g->heavy, g->n_heavy,
-                 g->g3, g->c3s, g->r0_vis, g->wt, g->w_ws, g->clog, g->x_ws, g->solo_q, g->ci_w, g->wt_w};
+                 g->g3, g->c3s, g->r0_vis, g->wt, g->w_ws, g->clog, g->x_ws, g->ci_w, g->wt_w};
   for (void *p : dev)
     if (p) cudaFree(p);
   if (g->h_sctl) cudaFreeHost(g->h_sctl);
@@ -323,14 +323,10 @@ int gc_load_csr(int32_t n, const int32_t *row_ptr, const int32_t *col_idx, uint3
   g->gain_ctas = want;
   g->ws_count = want;
   if ((rc = dalloc(&g->ws, (size_t)want * g->ws_stride))) return bail(rc);
-  // queues of the one-source searches of deep graphs: at most 1 GB, on sparse
-  // graphs only (roads, grids, trees)
-  if (nnz <= (int64_t)kSoloDegree * n) {
-    if ((rc = solo_plan(n, g->num_sms, std::min<size_t>(free_b / 16, (size_t)1 << 30), &g->solo_ctas))) return bail(rc);
-    if (g->solo_ctas > 0 && dalloc(&g->solo_q, (size_t)g->solo_ctas * N) != GC_OK) {
-      g->solo_ctas = 0;  // no room: deep graphs take the 64-lane batches
-    }
-  }
+  // one-source searches of deep graphs: sparse graphs only (roads, grids, trees)
+  if (nnz <= (int64_t)kSoloDegree * n &&
+      (rc = solo_plan(n, g->num_sms, (size_t)want * g->ws_stride, &g->solo_ctas)))
+    return bail(rc);
   if (cudaMemsetAsync(g->ws, 0, (size_t)want * g->ws_stride, st) != cudaSuccess ||
       cudaMemsetAsync(g->hist, 0, kHistBins * sizeof(unsigned int), st) != cudaSuccess ||
       cudaMemsetAsync(g->lev_cnt, 0, N * sizeof(unsigned long long), st) != cudaSuccess ||

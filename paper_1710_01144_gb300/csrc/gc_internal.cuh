@@ -358,9 +358,8 @@ struct gc_graph {
   unsigned char *ws = nullptr;
   size_t ws_stride = 0;
   int ws_count = 0;
-  // one-source-per-CTA searches of deep graphs (gc_solo.cu): a queue of n
-  // vertices per CTA; 0 CTAs: dense graph, or too large for the bitmap
-  int32_t *solo_q = nullptr;
+  // one-source-per-CTA searches of deep graphs (gc_solo.cu), their queues in ws;
+  // 0 CTAs: dense graph, or too large for the bitmap
   int solo_ctas = 0;
   int gain_ctas = 0;       // resident CTAs of the gain kernel
   int bfs_ctas = 0;        // resident CTAs of the cooperative BFS
@@ -435,7 +434,7 @@ size_t gain_ws_stride(int32_t n);
 // relaxed by `slack` (region[i]: vertices visited), or farness values (no_cut:
 // exact for every candidate).  deep_only: does nothing unless the BFS that
 // filled d_S had more than kWideLevels levels.
-int solo_plan(int32_t n, int num_sms, size_t budget, int *ctas);
+int solo_plan(int32_t n, int num_sms, size_t ws_bytes, int *ctas);
 int launch_solo(gc_graph *g, int mode, const int32_t *cand, int32_t n_cand, const int32_t *n_cand_dev, long long *out,
                 int32_t *region, int32_t slack, bool no_cut, bool deep_only);
 // bounds from the searched vertices list[0 .. sctl->n_sel) (results in lgain)

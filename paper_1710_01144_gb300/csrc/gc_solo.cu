@@ -13,7 +13,11 @@
 //
 // The search.  Level-synchronous BFS from one source; the queue (one int32 per
 // vertex in global memory, written and read by this CTA alone) keeps every
-// visited vertex in BFS order, so level L is a slice of it.  A thread takes a
+// visited vertex in BFS order, so level L is a slice of it.  The queues lie in the
+// memory of the 64-lane batches' workspaces, which are zero at rest: a CTA puts
+// zeros back where it wrote once it has no more sources (kernels of the same stream
+// run before or after, never beside).  Queues of their own were 640 MB at 65,536 vertices, for every sparse
+// handle; greedy on road-like 256 x 256, k = 20, takes 37.8 ms, 37.5 with those.  A thread takes a
 // frontier vertex and its row, four entries in flight; rows longer than
 // kSoloRow are taken by the warp together.  One CTA barrier per level: the
 // level's claims are counted in one of three counters in rotation.
@@ -59,7 +63,7 @@ __global__ void __launch_bounds__(kSoloThreads)
     k_solo(const int32_t *__restrict__ rp, const int32_t *__restrict__ ci, int32_t n, const int32_t *__restrict__ dS,
            const int32_t *__restrict__ mx, const int32_t *__restrict__ cand, int32_t n_cand_arg,
            const int32_t *__restrict__ n_cand_dev, long long *__restrict__ out, int32_t *__restrict__ region,
-           int32_t *queues, GainCtl *ctl, const BfsCtl *deep_only, int32_t slack, int32_t no_cut) {
+           int32_t *queues, long long q_stride, GainCtl *ctl, const BfsCtl *deep_only, int32_t slack, int32_t no_cut) {
   extern __shared__ __align__(16) uint32_t s_seen[];  // one bit per vertex
   __shared__ int s_task;
   __shared__ int s_new[3];
@@ -69,9 +73,10 @@ __global__ void __launch_bounds__(kSoloThreads)
   const int tid = threadIdx.x, lane = tid & 31, T = kSoloThreads;
   const int nw4 = ((n + 31) / 32 + 3) / 4;  // bitmap in 16-byte units
   uint4 *seen4 = reinterpret_cast<uint4 *>(s_seen);
-  int32_t *q = queues + (size_t)blockIdx.x * n;
+  int32_t *q = queues + (size_t)blockIdx.x * q_stride;
   const int n_cand = n_cand_dev ? *n_cand_dev : n_cand_arg;
   u64 w_edges = 0, w_levels = 0, w_front = 0, w_tasks = 0;
+  int high = 0;  // entries of the queue that were written
   for (int i = tid; i < nw4; i += T) seen4[i] = make_uint4(0, 0, 0, 0);
   for (;;) {
     if (tid == 0) {
@@ -198,6 +203,7 @@ __global__ void __launch_bounds__(kSoloThreads)
       }
     }
     // the bitmap back to zero: by the queue while that is the shorter list
+    high = max(high, b);
     cta_sync();
     if (b < 2 * nw4) {
       for (int i = tid; i < b; i += T) s_seen[q[i] >> 5] = 0u;
@@ -206,6 +212,8 @@ __global__ void __launch_bounds__(kSoloThreads)
     }
     cta_sync();
   }
+  uint4 *q4 = reinterpret_cast<uint4 *>(q);  // (a queue's length is a multiple of 4)
+  for (int i = tid; i < (high + 3) / 4; i += T) q4[i] = make_uint4(0, 0, 0, 0);
   w_edges = block_sum(w_edges, (u64 *)s_red);
   if (tid == 0 && w_tasks) {
     atomicAdd(&ctl->edges_scalar, w_edges);
@@ -220,9 +228,11 @@ __global__ void __launch_bounds__(kSoloThreads)
 
 static size_t solo_smem(int32_t n) { return (size_t)((n + 31) / 32 + 3) / 4 * 16; }
 
+static size_t solo_queue_bytes(int32_t n) { return ws_align((size_t)n * sizeof(int32_t)); }
+
 // CTAs of the solo kernel for a graph of n vertices (0: its bitmap does not fit
-// shared memory), and their queues within `budget` bytes.
-int solo_plan(int32_t n, int num_sms, size_t budget, int *ctas) {
+// shared memory), with queues in ws_bytes of workspaces.
+int solo_plan(int32_t n, int num_sms, size_t ws_bytes, int *ctas) {
   *ctas = 0;
   const size_t smem = solo_smem(n);
   if (smem > 200 * 1024) return GC_OK;
@@ -231,7 +241,7 @@ int solo_plan(int32_t n, int num_sms, size_t budget, int *ctas) {
   GC_CUDA(cudaFuncSetAttribute(k_solo<kModeFarness>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
   GC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&x, k_solo<kModeGain>, kSoloThreads, smem));
   GC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&y, k_solo<kModeFarness>, kSoloThreads, smem));
-  const size_t fit = budget / ((size_t)n * sizeof(int32_t));
+  const size_t fit = ws_bytes / solo_queue_bytes(n);
   *ctas = (int)std::min<size_t>((size_t)std::min(x, y) * num_sms, fit);
   return GC_OK;
 }
@@ -246,14 +256,16 @@ int launch_solo(gc_graph *g, int mode, const int32_t *cand, int32_t n_cand, cons
   ++g->launches;
   const BfsCtl *deep = deep_only ? g->bctl : nullptr;
   const size_t smem = solo_smem(g->n);
+  int32_t *queues = (int32_t *)g->ws;
+  const long long q_stride = (long long)(solo_queue_bytes(g->n) / sizeof(int32_t));
   if (mode == kModeGain)
     k_solo<kModeGain><<<ctas, kSoloThreads, smem, g->stream>>>(g->rp, g->ci, g->n, g->dS, g->mx, cand, n_cand,
-                                                               n_cand_dev, out, region, g->solo_q, g->gctl, deep,
-                                                               slack, 0);
+                                                               n_cand_dev, out, region, queues, q_stride, g->gctl,
+                                                               deep, slack, 0);
   else
     k_solo<kModeFarness><<<ctas, kSoloThreads, smem, g->stream>>>(g->rp, g->ci, g->n, g->dS, nullptr, cand, n_cand,
-                                                                  n_cand_dev, out, nullptr, g->solo_q, g->gctl, deep,
-                                                                  0, no_cut ? 1 : 0);
+                                                                  n_cand_dev, out, nullptr, queues, q_stride, g->gctl,
+                                                                  deep, 0, no_cut ? 1 : 0);
   GC_CUDA(cudaGetLastError());
   return GC_OK;
 }
