@@ -291,27 +291,89 @@ __global__ void k_relax_seed(const int32_t *__restrict__ list, const int32_t *m_
 }
 
 // One hop: val1[v] <- min(val0[v], min over neighbours w of val0[w] + slope[w]),
-// the slope following the value taken.  slope0 == nullptr: the constant `step`.
-__global__ void __launch_bounds__(256) k_relax(const int32_t *__restrict__ rp, const int32_t *__restrict__ ci,
-                                               int32_t n, const long long *__restrict__ val0,
-                                               const int32_t *__restrict__ slope0, long long *__restrict__ val1,
-                                               int32_t *__restrict__ slope1, long long step) {
-  for (int v = blockIdx.x * blockDim.x + threadIdx.x; v < n; v += gridDim.x * blockDim.x) {
-    long long best = val0[v];
-    int sl = slope0 ? slope0[v] : 0;
-    for (int e = rp[v]; e < rp[v + 1]; ++e) {
+// the slope following the value taken.  slope0 == nullptr: the constant `step`.  A
+// thread per row of at most kSoloRow entries, the warp together for longer ones, the
+// CTA for those of the list of long rows: deep graphs may have hubs (a broom of
+// 100,000 leaves, k = 5, on this path: 1,240 ms with a thread per row, 68 so; road-like
+// 120 x 120 with a vertex of 50,000 leaves, k = 10: 816, 88).
+constexpr int kRelaxThreads = 256;
+
+__global__ void __launch_bounds__(kRelaxThreads)
+    k_relax(const int32_t *__restrict__ rp, const int32_t *__restrict__ ci, int32_t n,
+            const long long *__restrict__ val0, const int32_t *__restrict__ slope0, long long *__restrict__ val1,
+            int32_t *__restrict__ slope1, long long step, const int32_t *__restrict__ heavy,
+            const int32_t *__restrict__ nh) {
+  __shared__ long long s_v[kRelaxThreads / 32];
+  __shared__ int s_sl[kRelaxThreads / 32];
+  const int tid = threadIdx.x, lane = tid & 31;
+  long long best;
+  int sl;
+  auto start = [&](int v) {
+    best = val0[v];
+    sl = slope0 ? slope0[v] : 0;
+  };
+  auto take = [&](long long y, int s) {
+    if (y < best) {
+      best = y;
+      sl = s;
+    }
+  };
+  auto scan = [&](int e0, int e1, int by) {
+    for (int e = e0; e < e1; e += by) {
       const int w = ci[e];
       const long long x = val0[w];
       if (x == LLONG_MAX) continue;
       const int s = slope0 ? slope0[w] : 0;
-      const long long y = x + (slope0 ? (long long)s : step);
-      if (y < best) {
+      take(x + (slope0 ? (long long)s : step), s);
+    }
+  };
+  auto fold_warp = [&]() {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      const long long y = __shfl_xor_sync(0xffffffffu, best, o);
+      const int s = __shfl_xor_sync(0xffffffffu, sl, o);
+      if (y < best || (y == best && s < sl)) {
         best = y;
         sl = s;
       }
     }
+  };
+  auto put = [&](int v) {
     val1[v] = best;
     if (slope1) slope1[v] = sl;
+  };
+  for (int base = (blockIdx.x * kRelaxThreads + tid) & ~31; base < n; base += gridDim.x * kRelaxThreads) {
+    const int v = base + lane;
+    const int r0 = v < n ? rp[v] : 0, r1 = v < n ? rp[v + 1] : 0, len = r1 - r0;
+    if (v < n && len <= kSoloRow) {
+      start(v);
+      scan(r0, r1, 1);
+      put(v);
+    }
+    for (unsigned m = __ballot_sync(0xffffffffu, len > kSoloRow && len <= kHeavyRow); m; m &= m - 1) {
+      const int t = __ffs(m) - 1;
+      const int x0 = __shfl_sync(0xffffffffu, r0, t), x1 = __shfl_sync(0xffffffffu, r1, t);
+      start(base + t);
+      scan(x0 + lane, x1, 32);
+      fold_warp();
+      if (lane == 0) put(base + t);
+    }
+  }
+  for (int i = blockIdx.x; i < *nh; i += gridDim.x) {
+    const int v = heavy[i];
+    start(v);
+    scan(rp[v] + tid, rp[v + 1], kRelaxThreads);
+    fold_warp();
+    cta_sync();  // the last row's readers
+    if (lane == 0) {
+      s_v[tid >> 5] = best;
+      s_sl[tid >> 5] = sl;
+    }
+    cta_sync();
+    if (tid == 0) {
+      for (int w = 1; w < kRelaxThreads / 32; ++w) take(s_v[w], s_sl[w]);
+      put(v);
+    }
   }
 }
 
@@ -336,7 +398,8 @@ int launch_relax(gc_graph *g, bool farness, const int32_t *region, int32_t hops,
   k_relax_seed<<<g->red_blocks, 256, 0, g->stream>>>(g->list, &g->sctl->n_sel, g->lgain, region, farness ? 1 : 0, v0,
                                                      s0);
   for (int h = 0; h < hops; ++h) {
-    k_relax<<<blocks, 256, 0, g->stream>>>(g->rp, g->ci, g->n, v0, s0, v1, s1, (long long)g->n - 2);
+    k_relax<<<blocks, kRelaxThreads, 0, g->stream>>>(g->rp, g->ci, g->n, v0, s0, v1, s1, (long long)g->n - 2, g->heavy,
+                                                     g->n_heavy);
     std::swap(v0, v1);
     std::swap(s0, s1);
   }
