@@ -500,10 +500,12 @@ int gc_top_closeness(gc_graph *g, int32_t k, const gc_opts *opts_in, int32_t *ou
   GC_TRY(launch_fill_i64(g, g->f0, -1, g->n));
   GC_TRY(launch_round0_keys(g));
   GC_TRY(launch_argmin_lb(g));
-  GC_TRY(distances_from(g, &g->sctl->arg_id, 1, tns, nullptr));
+  int64_t f_a = 0;
+  GC_TRY(distances_from(g, &g->sctl->arg_id, 1, tns, &f_a));
   const int32_t ecc = g->h_bctl->levels;
   if (ecc > kShallowLevels) GC_TRY(launch_pivot_bound(g));
-  const bool deep = ecc > kShallowLevels && g->solo_ctas > 0 && opts.round0_lanes == 0 && opts.max_ctas == 0;
+  const bool deep = ecc > kShallowLevels && far_apart(f_a, g->n) && g->solo_ctas > 0 && opts.round0_lanes == 0 &&
+                    opts.max_ctas == 0;
   // 2. probes, searched with no cut (threshold +infinity, kept fixed)
   struct {
     long long best_f;
@@ -984,7 +986,8 @@ int gc_greedy(gc_graph *g, int32_t k, const gc_opts *opts_in, int32_t *out_group
   GC_TRY(launch_fill_i64(g, g->f0, -1, g->n));
   GC_TRY(launch_round0_keys(g));
   GC_TRY(launch_argmin_lb(g));
-  GC_TRY(distances_from(g, &g->sctl->arg_id, 1, tns, nullptr));
+  int64_t f_a = 0;
+  GC_TRY(distances_from(g, &g->sctl->arg_id, 1, tns, &f_a));
   int32_t ds_src = g->h_sctl->arg_id;  // the vertex whose BFS distances are in d_S
   GC_TRY(launch_round0_seed(g));
   GC_TRY(launch_select(g, kSelKey, 0, 0, kTauDevice, 0));
@@ -1033,7 +1036,8 @@ int gc_greedy(gc_graph *g, int32_t k, const gc_opts *opts_in, int32_t *out_group
   const bool auto_steps = opts.step_mode == 0 && opts.step_form == 0 && opts.eval_per_step == 0 &&
                           opts.step_lanes == 0 && opts.max_ctas == 0 && opts.active_target == 0 &&
                           opts.lazy_ctas == 0 && opts.round1_heavy == 0 && opts.local_update_max_gain == 0;
-  const bool deep = ecc_a > kShallowLevels && g->solo_ctas > 0 && opts.round0_lanes == 0 && auto_steps &&
+  const bool deep = ecc_a > kShallowLevels && far_apart(f_a, g->n) && g->solo_ctas > 0 && opts.round0_lanes == 0 &&
+                    auto_steps &&
                     !opts.use_proposal && !(g->rec_X && g->rec_cap > 0) && g->gain_lanes == kLanes &&
                     !(opts.flags & (GC_OPT_NO_ROUND1_BOUND | GC_OPT_NO_EXPAND_BOUND | GC_OPT_FULL_ADJACENCY));
   int64_t solo_upd = 0;  // deep graphs: labels lowered by the d_S updates of rounds >= 2

@@ -24,6 +24,22 @@ GC_HD int32_t w_bucket_end(int32_t mn, int32_t delta) { return mn > kInf - 1 - d
 // which x < T alone would leave pending for ever.
 GC_HD bool w_in_bucket(int32_t x, int32_t T) { return T == kInf - 1 || x < T; }
 
+// Whether the mean distance `sum` / n of a search is long for n vertices: on roads,
+// grids and lattices its square is a share of n (a quarter on a square grid), on
+// graphs that a search fills in a few levels it is not, whatever tail of a few
+// vertices makes them deep.  On the latter one-source searches lose to the 64-lane
+// batches, which share rows among sources that reach them at one level, and to the
+// degree and two-hop bounds.  Measured, greedy k = 5 (one-source, 64-lane, ms; mean^2
+// / n): attachment graph of 100,000 vertices with a path of 40 at one of them 285, 8
+// (0.0001); broom of 30,000 leaves 40, 12 (0.0002); recursive tree n = 5,000 5.8, 2.2
+// (0.003); 6 attachment graphs of 5,000 in a row 14.0, 13.9 (0.003); tree of 5,000 with
+// such a path 2.0, 3.9 (0.006); ring of 30,000 with 2,500 chords 9.5, 18.8 (0.009);
+// road-like 40 x 40 1.6, 4.4 (0.25), 200 x 200 14, 138.
+GC_HD bool far_apart(int64_t sum, int64_t n) {
+  const double mean = (double)sum / (double)n;
+  return mean * mean * 200.0 >= (double)n;
+}
+
 // Whether vertex v, entry i of a list of m, is in the list's sample of about `want`:
 // spread by a hash of its id and `salt`.  The first entry always is, so that no
 // sample is empty (one of few CTAs' worth often would be: want = 1 in 37 of 100

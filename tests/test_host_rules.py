@@ -16,6 +16,7 @@ using namespace gc;
 extern "C" {
 int32_t bucket_end(int32_t mn, int32_t delta) { return w_bucket_end(mn, delta); }
 int in_bucket(int32_t x, int32_t T) { return w_in_bucket(x, T); }
+int far(int64_t sum, int64_t n) { return far_apart(sum, n); }
 
 int sample(const int32_t *list, int m, int want, uint32_t salt) {
   int c = 0;
@@ -115,3 +116,15 @@ def test_samples_are_never_empty(rules, want):
             elif m == 40 * want:
                 sizes.append(c)
     assert abs(np.mean(sizes) - want) <= 1 + 4 * np.sqrt(want / len(sizes))  # the mean of binomial counts, and the first entry
+
+
+def test_far_apart(rules):
+    far = lambda s, n: bool(rules.far(ctypes.c_int64(s), ctypes.c_int64(n)))
+    for n in (1, 2, 100, 10**6, 2**31 - 1):
+        assert far(n * n // 4 + 1, n)                       # a path
+        assert far(int(n * 0.5 * n**0.5) + 1, n)            # a square grid
+        assert far(2**62, n)                                # (no overflow)
+    for n in (10**3, 10**5, 2**31 - 1):
+        assert not far(2 * n, n) and not far(0, n)          # a star
+    assert far(10000 * 1000, 10000) and not far(10000 * 7, 10000)
+    assert far(10**6 * 71, 10**6) and not far(10**6 * 70, 10**6)  # mean^2 = n / 200 between the two
