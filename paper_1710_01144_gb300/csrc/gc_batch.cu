@@ -53,7 +53,7 @@ struct BatchCtl {
   int32_t err;
   int32_t remaining;  // graphs that still need lazy rounds
   int32_t nseeds;     // seeds of the next relabel BFS
-  int32_t task;       // dynamic task counter of P4
+  int32_t task, task2;  // dynamic task counters (P2, P4): the teams', the single CTAs'
   int32_t pad0;
   unsigned long long pk[3];  // relabel BFS frontiers (see BfsCtl)
   int32_t pad;
@@ -115,7 +115,7 @@ struct BatchArgs {
   long long *pgain;
   int32_t *seeds;  // [max(count, sum k)]
   int32_t *slist;  // round-0 survivors, graph-aligned [N]
-  int32_t *scount, *tstart;  // per-graph survivor counts, task prefix [count+1]
+  int32_t *scount, *tstart;  // per-graph survivor counts, task prefixes [2 (count+1)]
   BatchCtl *ctl;
   GainCtl *gctl;
   // lazy rounds (k_batch_lazy): teams of team_size CTAs, each with its control
@@ -134,6 +134,7 @@ struct BatchArgs {
   int32_t team_size;
   int32_t list_cap;   // entries of a shared-memory list (a power of two, at most kCta0SelectMax)
   int32_t grid_min_n; // graphs with at least this many vertices run their lazy rounds grid-wide
+  int32_t team_entries, far;  // entries from which a graph's short lists go to teams; 1: round 0 takes the far counts
   int32_t simple;     // no row holds an entry twice or its own vertex
   int32_t bounded;    // round 1 with two-hop bounds (batch_round1_bounded) and the refresh after it
   long long *g3;      // [2 * count]: sum of (d - 3)^+ per graph for round 1, then for the refresh
@@ -443,29 +444,54 @@ static __device__ void seg_sum_excess3(const BatchArgs &a, const int32_t *d, lon
   }
 }
 
-// Graphs with at most this many listed vertices run their tasks by teams.
+// Graphs with at most this many listed vertices and at least kTeamEntries adjacency
+// entries run their tasks by teams: a CTA alone finishes a small graph's batch before
+// a team has met at its barriers.  Rounds 0 and 1 in ms by teams and by CTAs: 180
+// graphs of 63 to 300 vertices 1.23, 0.46; 8 R-MAT graphs of 59,000 entries 0.48, 0.36;
+// one attachment graph of 80,000 entries 0.43, 0.57, of 480,000 0.67, 1.22.
 constexpr int kTeamListMax = 4 * kLanes;
+constexpr int32_t kTeamEntries = 1 << 16;
+// Batches whose largest graph is smaller go without the far counts: their searches
+// cost less than the pass and its two barriers (60 vertices: round 0 0.12, 0.10 ms).
+constexpr int32_t kFarMinN = 4096;
 
-// tstart[g] = tasks (64 listed vertices each) of the graphs before g, of the
-// graphs with short lists or of the others; the task counter starts again.
-// One thread.
-static __device__ void task_prefix(const BatchArgs &a, bool short_lists) {
-  int acc = 0;
-  for (int g = 0; g < a.count; ++g) {
-    a.tstart[g] = acc;
-    const int m = a.scount[g];
-    if ((m <= kTeamListMax) == short_lists) acc += (m + kLanes - 1) / kLanes;
+// tstart[g] = tasks (64 listed vertices each) of the graphs before g that go to
+// teams, tstart[count + 1 + g] = of those that go to single CTAs; both task counters
+// start again.  One CTA.
+static __device__ void task_prefix(const BatchArgs &a) {
+  __shared__ int s_scan[33];
+  const int tid = threadIdx.x, T = blockDim.x;
+  int32_t *const solo = a.tstart + a.count + 1;
+  int teams = 0, ctas = 0;
+  for (int base = 0; base < a.count; base += T) {
+    const int g = base + tid;
+    int t = 0, c = 0;
+    if (g < a.count) {
+      const int m = a.scount[g], o = a.off[g];
+      (m <= kTeamListMax && a.rp[o + a.ng[g]] - a.rp[o] >= a.team_entries ? t : c) = (m + kLanes - 1) / kLanes;
+    }
+    int all_t, all_c;
+    const int x = block_excl_scan(t, s_scan, &all_t), y = block_excl_scan(c, s_scan, &all_c);
+    if (g < a.count) {
+      a.tstart[g] = teams + x;
+      solo[g] = ctas + y;
+    }
+    teams += all_t;
+    ctas += all_c;
   }
-  a.tstart[a.count] = acc;
-  a.ctl->task = 0;
+  if (tid == 0) {
+    a.tstart[a.count] = teams;
+    solo[a.count] = ctas;
+    a.ctl->task = a.ctl->task2 = 0;
+  }
 }
 
-// the graph with tstart[g] <= task < tstart[g + 1]
-static __device__ int task_graph(const BatchArgs &a, int task) {
+// the graph with start[g] <= task < start[g + 1]
+static __device__ int task_graph(const BatchArgs &a, const int32_t *start, int task) {
   int lo = 0, hi = a.count - 1;
   while (lo < hi) {
     const int mid = (lo + hi + 1) >> 1;
-    if (a.tstart[mid] <= task) lo = mid;
+    if (start[mid] <= task) lo = mid;
     else hi = mid - 1;
   }
   return lo;
@@ -500,18 +526,18 @@ static __device__ __noinline__ bool team_batch(const BatchArgs &a, int g, const 
                                0, nullptr, tm, gx_n, gain ? nullptr : &tc->best, a.ng[g], a.simple != 0);
 }
 
-// The tasks of the lists in slist (scount entries per graph) that tstart counts,
-// by teams of S CTAs:
+// The tasks of the lists in slist (scount entries per graph) that start counts, from
+// the counter *task_next, by teams of S CTAs:
 // kModeFarness  f0[v] <- f({v}) or -1, cut by the graph's best (round 0);
 // kModeGain     ub[v] <- Delta(v | {s0}), stamp[v] <- 1, bestf[g] <- the best gain.
 // Ends without a grid barrier.
 template <int MODE>
 static __device__ bool run_tasks(const BatchArgs &a, const GainWs &myws, GainCounters &cnt, long long *s_out,
-                                 const int S) {
+                                 const int32_t *start, int32_t *task_next, const int S) {
   __shared__ int s_task;
   __shared__ long long s_ll[32];
   const int tid = threadIdx.x;
-  const int n_tasks = a.tstart[a.count];
+  const int n_tasks = start[a.count];
   const int t = blockIdx.x / S;
   const Team tm{(int)blockIdx.x - t * S, S};
   if ((t + 1) * S > (int)gridDim.x) return true;  // a remainder of fewer than S CTAs
@@ -519,19 +545,19 @@ static __device__ bool run_tasks(const BatchArgs &a, const GainWs &myws, GainCou
   const LaneGraphs lg = MODE == kModeFarness ? LaneGraphs{a.gid, a.ng, a.bestf} : LaneGraphs();
   for (;;) {
     if (S == 1) {
-      if (tid == 0) s_task = atomicAdd(&a.ctl->task, 1);
+      if (tid == 0) s_task = atomicAdd(task_next, 1);
       cta_sync();
     } else {
       if (tm.b == 0) {  // the next task and a fresh control block for its batch
         unsigned int *w = reinterpret_cast<unsigned int *>(&tc->gg);
         for (int i = tid; i < (int)(sizeof(GridGainCtl) / 4); i += blockDim.x) w[i] = 0;
         if (tid == 0) {
-          const int next = atomicAdd(&a.ctl->task, 1);
+          const int next = atomicAdd(task_next, 1);
           tc->g = next;
           // one threshold for the whole team: other teams may lower the graph's
           // best while this batch runs, and every CTA must cut the same lanes
           if (MODE == kModeFarness && next < n_tasks)
-            tc->best = *(volatile long long *)&a.bestf[task_graph(a, next)];
+            tc->best = *(volatile long long *)&a.bestf[task_graph(a, start, next)];
         }
       }
       if (!grid_sync(&tc->bar, &a.ctl->err, a.tns, tm)) return false;
@@ -541,7 +567,7 @@ static __device__ bool run_tasks(const BatchArgs &a, const GainWs &myws, GainCou
     const int task = s_task;
     cta_sync();
     if (task >= n_tasks) return true;
-    const int g = task_graph(a, task), o = a.off[g], first = (task - a.tstart[g]) * kLanes;
+    const int g = task_graph(a, start, task), o = a.off[g], first = (task - start[g]) * kLanes;
     const int nl = min(kLanes, a.scount[g] - first);
     const int32_t *cand = a.slist + o + first;
     int levels = 0;
@@ -578,18 +604,19 @@ static __device__ bool run_tasks(const BatchArgs &a, const GainWs &myws, GainCou
   }
 }
 
-// Every task of the lists: short lists by teams, then long ones by CTAs.  Called
-// after a grid barrier (the lists are complete), ends with one.
+// Every task of the lists: the teams' first, then the single CTAs'; who is done with
+// one kind goes on to the other.  Called after a grid barrier (the lists are
+// complete), ends with one.
 template <int MODE>
 static __device__ bool batch_tasks(const BatchArgs &a, const GainWs &myws, GainCounters &cnt, long long *s_out) {
-  for (int pass = 0; pass < 2; ++pass) {
-    if (blockIdx.x == 0 && threadIdx.x == 0) task_prefix(a, pass == 0);
-    if (!bsync(a)) return false;
-    const int n_tasks = a.tstart[a.count];
-    if (n_tasks && !run_tasks<MODE>(a, myws, cnt, s_out, pass == 0 ? task_team(n_tasks, gridDim.x) : 1)) return false;
-    if (!bsync(a)) return false;
-  }
-  return true;
+  if (blockIdx.x == 0) task_prefix(a);
+  if (!bsync(a)) return false;
+  const int32_t *solo = a.tstart + a.count + 1;
+  const int n_team = a.tstart[a.count], n_solo = solo[a.count];
+  if (n_team && !run_tasks<MODE>(a, myws, cnt, s_out, a.tstart, &a.ctl->task, task_team(n_team, gridDim.x)))
+    return false;
+  if (n_solo && !run_tasks<MODE>(a, myws, cnt, s_out, solo, &a.ctl->task2, 1)) return false;
+  return bsync(a);
 }
 
 // Round 0: the far counts of the single-graph path (k_far_counts, k_far_bound in
@@ -1119,7 +1146,7 @@ __global__ void __launch_bounds__(kBatchThreads, 2) k_batch_solve(const BatchArg
   if (b == 0 && tid == 0) a.ctl->pk[0] = a.ctl->pk[1] = a.ctl->pk[2] = 0;
   if (!bsync(a)) return;
   // ---- P2: round-0 survivors (every v with LB(v) <= f_a) ----
-  if (!batch_far_bounds(a)) return;
+  if (a.far && !batch_far_bounds(a)) return;
   // P2a, one CTA per graph: compact the graph's survivors into its own region
   // of slist (graph-aligned, so batches never mix graphs)
   for (int g = b; g < a.count; g += G) {
@@ -1320,8 +1347,11 @@ __global__ void __launch_bounds__(kBatchThreads, 2) k_batch_solve(const BatchArg
 // grid in turn; the others go to teams of team_size consecutive CTAs, each team
 // taking the next graph of `order` (longest first) and running it to
 // completion, so that no graph waits for another graph's step.  One CTA per SM
-// (128 registers), as in the single-graph kernel.
-__global__ void __launch_bounds__(kBatchThreads, 1) k_batch_lazy(const BatchArgs a) {
+// (128 registers), as in the single-graph kernel; two (64 registers) where more small
+// graphs than SMs go to single CTAs (200 attachment graphs of 1,000 vertices, k = 40,
+// lazy rounds: 1.77 ms against 2.58; of 300, 1.46 against 2.11).
+template <int PER_SM>
+__global__ void __launch_bounds__(kBatchThreads, PER_SM) k_batch_lazy(const BatchArgs a) {
   extern __shared__ __align__(16) unsigned char s_list[];  // list_cap * 21 bytes
   __shared__ u64 s_red[32];
   if (*(volatile int32_t *)&a.ctl->stage != 1) return;  // an earlier phase failed
@@ -1522,7 +1552,7 @@ static bool balloc(T **p, size_t count) {
 }
 
 // The lazy rounds' plan: sorts the graphs by estimated time (longest first)
-// and returns the CTAs of a team: the power of two with the shortest list
+// and returns the CTAs of a team: the power of two with about the shortest list
 // schedule.  `ctas` > 0 asks for that size.  The estimate of a round in
 // microseconds is fitted to team sizes 1 to 76: a step's barriers, selection and
 // dependent loads do not shrink with the team, its edges and the bound refreshes
@@ -1540,25 +1570,26 @@ static int plan_teams(const gc_batch *b, const int32_t *ks, std::vector<int32_t>
   });
   const int G = b->lazy_ctas;
   if (ctas > 0) return std::min<int>(ctas, G);
-  int best = 1;
-  double best_t = 0;
+  std::vector<double> end;  // of the whole schedule, for teams of 1, 2, 4, ...
   for (int s = 1; s <= G; s *= 2) {
     // list scheduling in that order: the next graph goes to the team that is free first
     std::priority_queue<double, std::vector<double>, std::greater<double>> load(
         std::greater<double>(), std::vector<double>((size_t)(G / s), 0.0));
     double t = 0;
     for (int32_t g : order) {
-      const double end = load.top() + est(g, s);
+      const double e = load.top() + est(g, s);
       load.pop();
-      load.push(end);
-      t = std::max(t, end);
+      load.push(e);
+      t = std::max(t, e);
     }
-    if (s == 1 || t < best_t) {
-      best = s;
-      best_t = t;
-    }
+    end.push_back(t);
   }
-  return best;
+  // the smallest team within 5% of the best: a larger one's barriers cost more than the
+  // estimate knows (one graph of 60 vertices, k = 20: 0.46 ms on one CTA, 0.55 on 128)
+  const double limit = 1.05 * *std::min_element(end.begin(), end.end());
+  int s = 0;
+  while (end[s] > limit) ++s;
+  return 1 << s;
 }
 
 // The union CSR of `count` graphs.  Host arrays (nnzs == nullptr: the entry
@@ -1613,15 +1644,19 @@ static int batch_load_impl(int32_t count, const int32_t *const *row_ptrs, const 
     return GC_ECUDA;
   }
   b->ctas = std::min(kMaxGridCtas, occ * b->num_sms);
-  if (cudaFuncSetAttribute(k_batch_lazy, cudaFuncAttributeMaxDynamicSharedMemorySize, kLazyListSmem) != cudaSuccess ||
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_batch_lazy, kBatchThreads, kLazyListSmem) != cudaSuccess ||
+  if (cudaFuncSetAttribute(k_batch_lazy<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kLazyListSmem) !=
+          cudaSuccess ||
+      cudaFuncSetAttribute(k_batch_lazy<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, kLazyListSmem) !=
+          cudaSuccess ||
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_batch_lazy<1>, kBatchThreads, kLazyListSmem) !=
+          cudaSuccess ||
       occ < 1 ||
       cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_batch_check, kBatchThreads, 0) != cudaSuccess || occ < 1) {
     batch_release(b);
     set_error("gc_batch_load: the batch kernels cannot be resident");
     return GC_ECUDA;
   }
-  b->lazy_ctas = std::min(b->ctas, std::min(kMaxGridCtas, b->num_sms));
+  b->lazy_ctas = std::min(b->ctas, b->num_sms);
   const size_t Nn = (size_t)N;
   bool ok = balloc(&b->rp, Nn + 1) && balloc(&b->ci, (size_t)E) && balloc(&b->gid, Nn) &&
             balloc(&b->off, (size_t)count + 1) && balloc(&b->ng, (size_t)count) && balloc(&b->iota, Nn) &&
@@ -1631,12 +1666,12 @@ static int batch_load_impl(int32_t count, const int32_t *const *row_ptrs, const 
             balloc(&b->farness, (size_t)count) && balloc(&b->bestf, (size_t)count) &&
             balloc(&b->lc, (size_t)count) && balloc(&b->act_n, (size_t)count) &&
             balloc(&b->kk, (size_t)count) && balloc(&b->bstart, (size_t)count + 1) && balloc(&b->ctl, 1) &&
-            balloc(&b->slist, Nn) && balloc(&b->scount, (size_t)count) && balloc(&b->tstart, (size_t)count + 1) &&
+            balloc(&b->slist, Nn) && balloc(&b->scount, (size_t)count) && balloc(&b->tstart, 2 * ((size_t)count + 1)) &&
             balloc(&b->rpf, Nn + 1) && balloc(&b->cif, std::max<size_t>(1, (size_t)E)) && balloc(&b->c3, Nn) &&
             balloc(&b->dS1, Nn) && balloc(&b->g3, 2 * (size_t)count) &&
             balloc(&b->gx, 3 * Nn) && balloc(&b->clog, 2 * Nn) && balloc(&b->teams, (size_t)b->ctas + 1) &&
-            balloc(&b->gsel, (size_t)b->lazy_ctas + 1) && balloc(&b->wsel, (size_t)b->lazy_ctas * kLanes) &&
-            balloc(&b->wgain, (size_t)b->lazy_ctas * kLanes) && balloc(&b->depth, (size_t)count) &&
+            balloc(&b->gsel, (size_t)b->ctas + 1) && balloc(&b->wsel, (size_t)b->ctas * kLanes) &&
+            balloc(&b->wgain, (size_t)b->ctas * kLanes) && balloc(&b->depth, (size_t)count) &&
             balloc(&b->order, (size_t)count) && balloc(&b->cls, 2 * (size_t)count) &&
             balloc(&b->gctl, 1) && cudaMallocHost((void **)&b->h_ctl, sizeof(BatchCtl)) == cudaSuccess &&
             cudaMallocHost((void **)&b->h_gctl, sizeof(GainCtl)) == cudaSuccess;
@@ -1788,6 +1823,8 @@ int gc_batch_greedy(gc_batch *b, const int32_t *ks, const gc_opts *opts_in, int3
   a.bounded = (opts.flags & GC_OPT_NO_ROUND1_BOUND) ? 0 : 1;
   a.g3 = b->g3;
   a.simple = b->simple;
+  a.team_entries = kTeamEntries;
+  a.far = b->max_n >= kFarMinN;
   a.grid_min_n = opts.batch_grid_min_n == 0 ? kBatchGridMinN
                  : (opts.batch_grid_min_n < 0 ? INT32_MAX : opts.batch_grid_min_n);
   // the lazy rounds' plan: the graphs left to teams, longest first, and the
@@ -1799,6 +1836,19 @@ int gc_batch_greedy(gc_batch *b, const int32_t *ks, const gc_opts *opts_in, int3
   a.team_size = plan_teams(b, ks, order, opts.lazy_ctas);
   a.list_cap = kLanes;
   while (a.list_cap < A && a.list_cap < kCta0SelectMax) a.list_cap *= 2;
+  const size_t list_smem = (size_t)a.list_cap * 21;
+  // two CTAs per SM for many small graphs (all of them: big ones need the registers)
+  int lazy_ctas = b->lazy_ctas;
+  const void *lazy_fn = (const void *)k_batch_lazy<1>;
+  if (a.team_size == 1 && a.order_n > lazy_ctas && a.order_n == b->count &&
+      *std::max_element(b->h_nnz.begin(), b->h_nnz.end()) < kTeamEntries) {
+    int occ = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_batch_lazy<2>, kBatchThreads, list_smem) ==
+            cudaSuccess && occ >= 2) {
+      lazy_ctas = std::min(b->ctas, 2 * b->num_sms);
+      lazy_fn = (const void *)k_batch_lazy<2>;
+    }
+  }
   a.ub = b->ub;
   a.key = b->key;
   a.f0 = b->f0;
@@ -1840,7 +1890,7 @@ int gc_batch_greedy(gc_batch *b, const int32_t *ks, const gc_opts *opts_in, int3
                              st)))
       return e;
     if ((e = cudaMemsetAsync(b->teams, 0, (1 + (size_t)b->ctas) * sizeof(TeamCtl), st))) return e;
-    if ((e = cudaMemsetAsync(b->gsel, 0, (1 + (size_t)(b->lazy_ctas / a.team_size)) * sizeof(GridSelScratch), st)))
+    if ((e = cudaMemsetAsync(b->gsel, 0, (1 + (size_t)(lazy_ctas / a.team_size)) * sizeof(GridSelScratch), st)))
       return e;
     if ((e = cudaMemsetAsync(b->cls, 0, 2 * (size_t)b->count * sizeof(unsigned long long), st))) return e;
     if ((e = cudaMemsetAsync(b->depth, 0, (size_t)b->count * sizeof(int32_t), st))) return e;
@@ -1849,8 +1899,7 @@ int gc_batch_greedy(gc_batch *b, const int32_t *ks, const gc_opts *opts_in, int3
                                          st)))
       return e;
     if (kmax > 2 &&
-        (e = cudaLaunchCooperativeKernel((const void *)k_batch_lazy, dim3(b->lazy_ctas), dim3(kBatchThreads), args,
-                                         (size_t)a.list_cap * 21, st)))
+        (e = cudaLaunchCooperativeKernel(lazy_fn, dim3(lazy_ctas), dim3(kBatchThreads), args, list_smem, st)))
       return e;
     if ((e = cudaLaunchCooperativeKernel((const void *)k_batch_check, dim3(b->ctas), dim3(kBatchThreads), args, 0,
                                          st)))
