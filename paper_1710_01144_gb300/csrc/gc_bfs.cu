@@ -631,8 +631,8 @@ int launch_bfs(gc_graph *g, int32_t *dist, const int32_t *seeds, int32_t n_seeds
   void *args[] = {(void *)&rp, (void *)&ci,  (void *)&n,   (void *)&dist, (void *)&seeds, (void *)&n_seeds, (void *)&q0,
                   (void *)&q1, (void *)&st0, (void *)&st1, (void *)&ctl,  (void *)&sctl,  (void *)&tns,     (void *)&c3,
                   (void *)&fr};
-  // few CTAs on small graphs: cheaper barriers
-  const int grid = std::min(std::min(g->bfs_ctas, kMaxGridCtas), std::max(1, (n + 2 * kBfsThreads - 1) / (2 * kBfsThreads)));
+  static_assert(kBfsThreads == 256, "bfs_grid counts CTAs of 256 threads");
+  const int grid = (int)std::min<int64_t>(std::min(g->bfs_ctas, kMaxGridCtas), bfs_grid(n, g->nnz));
   ++g->launches;
   GC_CUDA(cudaLaunchCooperativeKernel((const void *)k_bfs, dim3(grid), dim3(kBfsThreads), args, 0, g->stream));
   return GC_OK;

@@ -40,6 +40,16 @@ GC_HD bool far_apart(int64_t sum, int64_t n) {
   return mean * mean * 200.0 >= (double)n;
 }
 
+// CTAs of 256 threads for a BFS over a whole graph: few on small graphs, for cheaper
+// barriers, but enough for the entries of the level that holds nearly all of them.  By
+// the vertices alone, two a thread, a random graph of 4,000 vertices and 1.6M entries
+// had 8 CTAs: farness from one vertex 115 us, 87 with every CTA, 53 with 97 (64
+// entries a thread); top-1 closeness there 488, 423, 412 us.
+GC_HD int64_t bfs_grid(int64_t n, int64_t nnz) {
+  const int64_t v = (n + 511) / 512, e = nnz / 16384;
+  return v > e ? (v > 1 ? v : 1) : e;
+}
+
 // Whether vertex v, entry i of a list of m, is in the list's sample of about `want`:
 // spread by a hash of its id and `salt`.  The first entry always is, so that no
 // sample is empty (one of few CTAs' worth often would be: want = 1 in 37 of 100

@@ -17,6 +17,7 @@ extern "C" {
 int32_t bucket_end(int32_t mn, int32_t delta) { return w_bucket_end(mn, delta); }
 int in_bucket(int32_t x, int32_t T) { return w_in_bucket(x, T); }
 int far(int64_t sum, int64_t n) { return far_apart(sum, n); }
+int64_t grid_of_bfs(int64_t n, int64_t nnz) { return bfs_grid(n, nnz); }
 
 int sample(const int32_t *list, int m, int want, uint32_t salt) {
   int c = 0;
@@ -128,3 +129,10 @@ def test_far_apart(rules):
         assert not far(2 * n, n) and not far(0, n)          # a star
     assert far(10000 * 1000, 10000) and not far(10000 * 7, 10000)
     assert far(10**6 * 71, 10**6) and not far(10**6 * 70, 10**6)  # mean^2 = n / 200 between the two
+
+
+@pytest.mark.parametrize("n,nnz,ctas", [(1, 0, 1), (512, 511, 1), (513, 2000, 2), (2000, 20000, 4), (4000, 1600000, 97),
+                                        (600, 359400, 21), (10**6, 4 * 10**6, 1954), (2**31 - 1, 2**31 - 1, 2**22)])
+def test_bfs_grid_has_ctas_for_the_entries(rules, n, nnz, ctas):
+    rules.grid_of_bfs.restype = ctypes.c_int64
+    assert rules.grid_of_bfs(ctypes.c_int64(n), ctypes.c_int64(nnz)) == ctas
