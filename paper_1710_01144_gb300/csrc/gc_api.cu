@@ -34,7 +34,6 @@ constexpr int32_t kRound0GridMax = 256;  // round-0 survivors (round-1 candidate
 constexpr int kRound0Pivots = 8;         // round 0: at most this many pivot bounds
 constexpr int kSoloStages = 12;          // deep graphs: at most this many sampled stages per round
 constexpr int kSoloRegion = 96;          // deep graphs: persistent rounds once n <= this times the round
-constexpr int32_t kWholeSearchMax = 1024;  // weighted round 0: full searches up to this many vertices (one wave)
 constexpr int kSoloDegree = 8;           // graphs up to this average degree may take the one-source searches
 constexpr int32_t kShallowLevels = 32;   // round 0: wide bottom-up batches up to this BFS depth
 // gc_greedy, lists that cannot certify a pick: from this many candidates whose
@@ -732,7 +731,7 @@ int gc_greedy_weighted(gc_graph *g, int32_t k, const gc_opts *opts_in, int32_t *
   // searched first, in full; their best farness cuts the other searches ----
   GC_TRY(launch_fill_i64(g, g->f0, -1, n));
   GC_TRY(launch_fill_i64(g, &g->gctl->best_f, LLONG_MAX, 1));
-  const bool whole = n <= kWholeSearchMax;
+  const bool whole = w_whole_search(n, g->nnz);
   if (!whole) {
     GC_TRY(launch_fill_i64(g, g->ub, 0, n));
     GC_TRY(launch_degree_keys(g));

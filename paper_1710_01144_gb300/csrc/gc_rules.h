@@ -24,6 +24,16 @@ GC_HD int32_t w_bucket_end(int32_t mn, int32_t delta) { return mn > kInf - 1 - d
 // which x < T alone would leave pending for ever.
 GC_HD bool w_in_bucket(int32_t x, int32_t T) { return T == kInf - 1 || x < T; }
 
+// Whether round 0 of the weighted greedy searches every vertex in full, in one bucket
+// and one wave of CTAs, instead of in buckets with a cut.  Dense rows hold mostly
+// entries that no shortest path takes, which buckets never read.  Measured, k = 6, ms
+// (in full, in buckets), weights up to 1 and 1000: complete n = 1,000 3.4 and 12.1, 1.3
+// and 5.4; n = 300 0.85 and 1.70, 0.78 and 1.42; n = 150 0.69 and 0.99, 0.75 and 0.96;
+// random n = 1,000, rows of 182 1.78 and 3.93, 1.35 and 2.22, of 22 1.06 and 1.37, 1.08
+// and 1.34; ring n = 1,000, rows of 32 1.47 and 4.0, 1.90 and 2.9; random n = 500, rows
+// of 21 0.72 and 0.99, 0.80 and 1.10.
+GC_HD bool w_whole_search(int64_t n, int64_t nnz) { return n <= 1024 && (n < 256 || nnz <= 64 * n); }
+
 // Whether the mean distance `sum` / n of a search is long for n vertices: on roads,
 // grids and lattices its square is a share of n (a quarter on a square grid), on
 // graphs that a search fills in a few levels it is not, whatever tail of a few

@@ -94,6 +94,13 @@ __global__ void __launch_bounds__(32 * kWSortWarps) k_wsort(const int32_t *__res
 // global memory are written and read in order.  Larger graphs keep them in the
 // workspace.
 constexpr int kWFarSmemN = 48000;  // 199 KB, and 13 KB of static arrays at 1024 threads
+// Steps of at most 32 queued vertices belong to warp 0: their rows by a scan over its
+// lanes, and up to this many entries relaxed without a CTA barrier; more go to the CTA
+// (five barriers a step instead of nine).  Paths and strips have little but such steps.
+// k = 6, ms, with one warp a row and no buckets, with every step by the CTA, now: path
+// n = 2,000, weights up to 1000, 17.0, 27.7, 16.4; grid strip 5 x 1,000, unit weights
+// 21.8, 27.2, 20.0; road-like 100 x 100, up to 16, 78.8, 23.8, 20.6.
+constexpr int kWWarpEntries = 128;
 constexpr unsigned kWNear = 1u, kWBucket = 2u;  // queued; listed in a bucket (settled at its end)
 
 // per CTA: near queues, pending and bucket lists, ptr, and without SM the
@@ -133,13 +140,13 @@ __global__ void k_wfar_init(unsigned char *base, size_t stride, int32_t n) {
 // kWGain     out[i]: the gain (0 for a member of S).
 // kWRelabel  out[0]: the decrease of d_S over labels with a finite old value.
 template <int MODE, int TH, bool SM>
-__global__ void __launch_bounds__(TH)
+__global__ void __launch_bounds__(TH, TH == 512 ? 4 : 1)
     k_wsearch(const int32_t *__restrict__ rp, const int32_t *__restrict__ ci, const int32_t *__restrict__ wt,
               int32_t n, int32_t *dS, const int32_t *list, const int32_t *m_dev, int32_t m_arg, long long *out,
               unsigned char *ws_base, size_t ws_stride, unsigned int *task, long long *best, int32_t w_max,
               int32_t delta_arg, int32_t *err) {
   extern __shared__ __align__(16) int32_t s_dist[];  // SM: distances, then the two flag bitmaps
-  __shared__ int s_i, s_F, s_nt, s_np, s_nb, s_min;
+  __shared__ int s_i, s_F, s_nt, s_np, s_nb, s_min, s_state, s_rows, s_total;
   __shared__ int s_off[TH], s_e0[TH], s_du[TH];
   __shared__ int s_scan[33];
   __shared__ long long s_bst;
@@ -163,6 +170,68 @@ __global__ void __launch_bounds__(TH)
   auto unqueue = [&](int v) {
     if (SM) atomicAnd(&s_near[v >> 5], ~(1u << (v & 31)));
     else atomicAnd(&fl[v], ~kWNear);
+  };
+  int T = 0;
+  // the part of a queued vertex's row up to T, entries [e0, lo): from the start,
+  // or, for a settled vertex taken up again (queued as ~u), from where the last
+  // bucket stopped; its distance is one value for the whole row (if it is lowered
+  // meanwhile the vertex is queued again)
+  auto row_part = [&](int x, int &du, int &e0, int &lo) -> int {
+    const int u = x < 0 ? ~x : x;
+    du = dist(u);
+    const int e1 = rp[u + 1];
+    e0 = x < 0 ? ptr[u] : rp[u];
+    // (the last bucket: the whole row)
+    lo = T == kInf - 1 ? e1 : e0;
+    int step = 4;  // galloping: the prefixes are short
+    while (lo + step <= e1 && du + wt[lo + step - 1] < T) {
+      lo += step;
+      step *= 2;
+    }
+    int hi = min(e1, lo + step);
+    while (lo < hi) {
+      const int mid = (lo + hi) >> 1;
+      if (du + wt[mid] < T) lo = mid + 1;
+      else hi = mid;
+    }
+    return u;
+  };
+  auto take = [&](int x, int u, int lo) {
+    if (x >= 0) {
+      unqueue(u);
+      if (flag(u, kWBucket)) bucket[atomicAdd(&s_nb, 1)] = u;
+    }
+    ptr[u] = lo;
+  };
+  // entry e of `total` in the parts of `rows` rows: row j is the largest with
+  // s_off[j] <= e.  A thread's entries ascend, so j starts at the last one's: with
+  // long parts the next row is a step or two away (galloping), with short ones it
+  // is searched for.  A search over all TH rows for every entry was half of the time
+  // on dense graphs (random n = 4,000, rows of 400, weights up to 16: 10.9 -> 7.9 ms
+  // a call).
+  auto relax = [&](int e, int rows, int total, int &j, int32_t *nxt) {
+    int hi = rows - 1;
+    if (total >= 32 * rows) {
+      int step = 1;
+      while (j + step <= hi && s_off[j + step] <= e) {
+        j += step;
+        step *= 2;
+      }
+      hi = min(hi, j + step - 1);
+    }
+    while (j < hi) {
+      const int mid = (j + hi + 1) >> 1;
+      if (s_off[mid] <= e) j = mid;
+      else hi = mid - 1;
+    }
+    const int x = s_e0[j] + (e - s_off[j]);
+    const int w = ci[x], nd = s_du[j] + wt[x];
+    if (MODE != kWFarness && nd >= dS[w]) return;  // pruned (Sec. 4.1)
+    if (nd >= dist(w)) return;
+    const int old = lower(w, nd);
+    if (nd >= old) return;
+    if (!SM && old == kInf) touched[atomicAdd(&s_nt, 1)] = w;
+    if (flag(w, kWNear)) nxt[atomicAdd(&s_F, 1)] = w;
   };
   const int m = m_dev ? *m_dev : m_arg;
   for (;;) {
@@ -204,7 +273,7 @@ __global__ void __launch_bounds__(TH)
       s_F = 1;
       s_np = 0;
     }
-    int T = min(delta, kInf - 1);
+    T = min(delta, kInf - 1);
     long long sum = 0, cnt = 0;  // settled: farness, gain or decrease, and vertices (the same in every thread)
     bool cut = false;
     int32_t *cur = q0, *nxt = q1;
@@ -214,43 +283,82 @@ __global__ void __launch_bounds__(TH)
       // ---- one bucket: label-correcting below T ----
       for (;;) {
         cta_sync();
-        const int F = s_F;
+        int F = s_F;
         cta_sync();
         if (F == 0) break;
-        if (tid == 0) s_F = 0;
-        for (int base = 0; base < F; base += TH) {
-          // a thread per queued vertex: its distance (one value for the whole
-          // row; if it is lowered meanwhile the vertex is queued again) and the
-          // part of its row up to T: from the start, or, for a settled vertex
-          // taken up again (queued as ~u), from where the last bucket stopped
-          const int q = base + tid;
-          int du = 0, e0 = 0, len = 0;
-          if (q < F) {
-            const int x = cur[q];
-            const bool again = x < 0;
-            const int u = again ? ~x : x;
-            if (!again) {
-              unqueue(u);
-              if (flag(u, kWBucket)) bucket[atomicAdd(&s_nb, 1)] = u;
+        if (F <= 32) {
+          // few queued vertices: warp 0 alone, step after step, while they stay few;
+          // the entries of a step by the whole CTA if they are many, and back here
+          if (tid < 32) {
+            int32_t *c = cur, *x = nxt;
+            int state = 0, total = 0;  // bit 0: the queues have changed places, bit 1: entries for the CTA
+            for (int f = F; f > 0 && f <= 32; state ^= 1) {
+              int q = 0, u = 0, du = 0, e0 = 0, lo = 0;
+              if (lane < f) {
+                q = c[lane];
+                u = row_part(q, du, e0, lo);
+                take(q, u, lo);
+              }
+              int incl = lo - e0;
+#pragma unroll
+              for (int o = 1; o < 32; o <<= 1) {
+                const int y = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o) incl += y;
+              }
+              total = __shfl_sync(0xffffffffu, incl, 31);
+              s_off[lane] = incl - (lo - e0);
+              s_e0[lane] = e0;
+              s_du[lane] = du;
+              if (lane == 0) s_F = 0;
+              if (total > kWWarpEntries) {
+                state |= 2;
+                if (lane == 0) s_rows = f;
+                break;
+              }
+              __syncwarp();
+              int j = 0;
+              for (int e = lane; e < total; e += 32) relax(e, f, total, j, x);
+              __syncwarp();
+              int32_t *t = c;
+              c = x;
+              x = t;
+              f = *(volatile int *)&s_F;
+              __syncwarp();
             }
-            du = dist(u);
-            const int e1 = rp[u + 1];
-            e0 = again ? ptr[u] : rp[u];
-            // (the last bucket: the whole row)
-            int lo = T == kInf - 1 ? e1 : e0, step = 4;  // galloping: the prefixes are short
-            while (lo + step <= e1 && du + wt[lo + step - 1] < T) {
-              lo += step;
-              step *= 2;
+            if (lane == 0) {
+              s_state = state;
+              s_total = total;
             }
-            int hi = min(e1, lo + step);
-            while (lo < hi) {
-              const int mid = (lo + hi) >> 1;
-              if (du + wt[mid] < T) lo = mid + 1;
-              else hi = mid;
-            }
-            ptr[u] = lo;
-            len = lo - e0;
           }
+          cta_sync();
+          const int state = s_state;
+          F = s_F;
+          if (state & 1) {
+            int32_t *t = cur;
+            cur = nxt;
+            nxt = t;
+          }
+          cta_sync();
+          if (state & 2) {
+            const int rows = s_rows, total = s_total;
+            int j = 0;
+            for (int e = tid; e < total; e += TH) relax(e, rows, total, j, nxt);
+            int32_t *t = cur;
+            cur = nxt;
+            nxt = t;
+            continue;
+          }
+          if (F == 0) break;
+        }
+        if (tid == 0) s_F = 0;
+        for (int base = 0; base < F; base += TH) {  // a thread per queued vertex
+          const int q = base + tid;
+          int u = -1, du = 0, e0 = 0, lo = 0;
+          if (q < F) {
+            u = row_part(cur[q], du, e0, lo);
+            take(cur[q], u, lo);
+          }
+          const int len = lo - e0;
           int total;
           const int off = block_excl_scan(len, s_scan, &total);
           s_off[tid] = off;
@@ -258,22 +366,9 @@ __global__ void __launch_bounds__(TH)
           s_du[tid] = du;
           cta_sync();
           // the chunk's entries, spread over the threads
-          for (int e = tid; e < total; e += TH) {
-            int lo = 0, hi = TH - 1;  // largest j with s_off[j] <= e (its row is non-empty)
-            while (lo < hi) {
-              const int mid = (lo + hi + 1) >> 1;
-              if (s_off[mid] <= e) lo = mid;
-              else hi = mid - 1;
-            }
-            const int x = s_e0[lo] + (e - s_off[lo]);
-            const int w = ci[x], nd = s_du[lo] + wt[x];
-            if (MODE != kWFarness && nd >= dS[w]) continue;  // pruned (Sec. 4.1)
-            if (nd >= dist(w)) continue;
-            const int old = lower(w, nd);
-            if (nd >= old) continue;
-            if (!SM && old == kInf) touched[atomicAdd(&s_nt, 1)] = w;
-            if (flag(w, kWNear)) nxt[atomicAdd(&s_F, 1)] = w;
-          }
+          const int rows = min(TH, F - base);
+          int j = 0;
+          for (int e = tid; e < total; e += TH) relax(e, rows, total, j, nxt);
           cta_sync();
         }
         int32_t *t = cur;

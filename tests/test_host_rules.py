@@ -17,6 +17,7 @@ extern "C" {
 int32_t bucket_end(int32_t mn, int32_t delta) { return w_bucket_end(mn, delta); }
 int in_bucket(int32_t x, int32_t T) { return w_in_bucket(x, T); }
 int far(int64_t sum, int64_t n) { return far_apart(sum, n); }
+int whole_search(int64_t n, int64_t nnz) { return w_whole_search(n, nnz); }
 int64_t grid_of_bfs(int64_t n, int64_t nnz) { return bfs_grid(n, nnz); }
 
 int sample(const int32_t *list, int m, int want, uint32_t salt) {
@@ -136,3 +137,9 @@ def test_far_apart(rules):
 def test_bfs_grid_has_ctas_for_the_entries(rules, n, nnz, ctas):
     rules.grid_of_bfs.restype = ctypes.c_int64
     assert rules.grid_of_bfs(ctypes.c_int64(n), ctypes.c_int64(nnz)) == ctas
+
+
+@pytest.mark.parametrize("n,nnz,whole", [(1, 0, 1), (255, 255 * 254, 1), (256, 256 * 64, 1), (256, 256 * 64 + 1, 0),
+                                         (1024, 65536, 1), (1024, 65538, 0), (1025, 2050, 0), (2**30, 2**31 - 1, 0)])
+def test_whole_weighted_searches(rules, n, nnz, whole):
+    assert rules.whole_search(ctypes.c_int64(n), ctypes.c_int64(nnz)) == whole
