@@ -31,8 +31,8 @@
 // CTA, then takes the best vertex and updates d_S, so the rounds follow one
 // another on the stream without a host round trip.  Bound by the latency of a
 // level (row pointers, columns, words, one barrier).  Measured in ms, k = 50
-// (the last: k = 20), against the chunks below: road-like 64 x 64 34.0 -> 7.0; BA
-// 2000, m = 5, 7.4 -> 2.3; R-MAT scale 12 30.7 -> 5.6, scale 14 89.6 -> 11.7.
+// (the last: k = 20), against the chunks below: road-like 64 x 64 33.9 -> 6.3; BA
+// 2000, m = 5, 7.4 -> 2.2; R-MAT scale 12 30.7 -> 4.0, scale 14 89.6 -> 5.4.
 //
 // Above that (k_bits_round): chunks of 64 W targets in global memory, one
 // cooperative launch per round, every level ends with a grid barrier.
@@ -56,8 +56,17 @@ constexpr int kBitsThreads = 256;
 // 32 targets per CTA: targets [32 b, 32 b + 32).  MODE and sums as in
 // k_bits_round below; out starts at zero.
 constexpr int kBitsCtaThreads = 1024;
+// Two forms.  Sparse (ROW = 32): rows of up to 32 entries go to a thread each.  Dense
+// (ROW = kBitsRow), where rows average more than kBitsDense entries: threads of a warp
+// read different lines, so such rows exceed L1, and rows of 17 to 32 entries go to the
+// warp, four at a time; and level 1 is taken from the targets' rows.  20 rounds in ms,
+// chunks, sparse form, dense form: random n = 15,900, rows of 18 15.4, 13.7, 10.6, of 34
+// 15.7, 27.9, 17.1, of 129 16.1, 30.2, 9.7; n = 4,000, rows of 482 5.9, 8.1, 5.0; ring n
+// = 8,000, rows of 32 98, 207, 69, of 128 59, 38.4, 37.5; R-MAT scale 14 90, 11.6, 5.4.
+constexpr int kBitsRow = 16;
+constexpr int kBitsDense = 8;
 
-template <int MODE>
+template <int MODE, int ROW>
 __global__ void __launch_bounds__(kBitsCtaThreads) k_bits_cta(const int32_t *__restrict__ rp,
                                                               const int32_t *__restrict__ ci, int32_t n,
                                                               const int32_t *__restrict__ dS, long long *out,
@@ -82,42 +91,83 @@ __global__ void __launch_bounds__(kBitsCtaThreads) k_bits_cta(const int32_t *__r
     const uint32_t mask = __ballot_sync(0xffffffffu, dt > i);  // the targets still counted at level i
     if (mask == 0u) break;  // (the same in every warp)
     bool chg = false;
-    // a thread per row of at most 32 entries, the warp together for longer ones
-    for (int w0 = tid & ~31; w0 < n; w0 += T) {
-      const int u = w0 + lane;
-      uint32_t own = 0u, x = 0u;
-      int r0 = 0, r1 = 0;
-      if (u < n) {
-        own = x = cur[u];
-        if ((own & mask) != mask) {  // (else every counted target is in already)
-          r0 = __ldg(rp + u);
-          r1 = __ldg(rp + u + 1);
+    auto finish = [&](int u, uint32_t own, uint32_t x) {
+      const int pc = __popc(x);
+      sum[u] += MODE == 1 ? pc : cs - pc;
+      chg |= x != (own & mask);
+    };
+    if (ROW < 32 && i == 1) {
+      // level 1: the neighbours of each target, a warp a target (rows hold both
+      // directions), instead of every row of the graph.  With two or three levels
+      // this is half of a round: random n = 15,900, rows of 256, 43.5 -> 8.6 ms for
+      // 20 rounds (17.4 by the chunks)
+      for (int u = tid; u < n; u += T) nxt[u] = cur[u] & mask;
+      cta_sync();
+      static_assert(kBitsCtaThreads / 32 == 32, "a warp a target");
+      const int t = tid >> 5;
+      if ((mask >> t) & 1u) {
+        const int r1 = __ldg(rp + base + t + 1);
+#pragma unroll 4
+        for (int e = __ldg(rp + base + t) + lane; e < r1; e += 32) atomicOr(&nxt[__ldg(ci + e)], 1u << t);
+      }
+      cta_sync();
+      for (int u = tid; u < n; u += T) finish(u, cur[u], nxt[u]);
+    } else {
+      // a thread per row of at most ROW entries, the warp together for longer ones
+      for (int w0 = tid & ~31; w0 < n; w0 += T) {
+        const int u = w0 + lane;
+        uint32_t own = 0u, x = 0u;
+        int r0 = 0, r1 = 0;
+        if (u < n) {
+          own = x = cur[u];
+          if ((own & mask) != mask) {  // (else every counted target is in already)
+            r0 = __ldg(rp + u);
+            r1 = __ldg(rp + u + 1);
+          }
         }
-      }
-      const bool lng = r1 - r0 > 32;
-      if (!lng) {
-        for (int e = r0; e < r1; e += 4) {
-          int v[4];
+        const int len = r1 - r0;
+        if (len <= ROW) {
+          for (int e = r0; e < r1; e += 4) {
+            int v[4];
 #pragma unroll
-          for (int k = 0; k < 4; ++k) v[k] = e + k < r1 ? __ldg(ci + e + k) : u;
+            for (int k = 0; k < 4; ++k) v[k] = e + k < r1 ? __ldg(ci + e + k) : u;
 #pragma unroll
-          for (int k = 0; k < 4; ++k) x |= cur[v[k]];
+            for (int k = 0; k < 4; ++k) x |= cur[v[k]];
+          }
         }
-      }
-      for (unsigned m = __ballot_sync(0xffffffffu, lng); m; m &= m - 1) {
-        const int q = __ffs(m) - 1;
-        const int a = __shfl_sync(0xffffffffu, r0, q), b = __shfl_sync(0xffffffffu, r1, q);
-        uint32_t y = 0u;
-        for (int e = a + lane; e < b; e += 32) y |= cur[__ldg(ci + e)];
-        y = __reduce_or_sync(0xffffffffu, y);
-        if (lane == q) x |= y;
-      }
-      if (u < n) {
-        x &= mask;
-        nxt[u] = x;
-        const int pc = __popc(x);
-        sum[u] += MODE == 1 ? pc : cs - pc;
-        chg |= x != (own & mask);
+        unsigned lng = __ballot_sync(0xffffffffu, len > ROW);
+        if (ROW < 32 && lng) {
+          const unsigned more = __ballot_sync(0xffffffffu, len > 32);
+          for (unsigned m = lng & ~more; m;) {  // four rows in flight
+            int q[4], w[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+              q[k] = m ? __ffs(m) - 1 : 32;
+              m &= m - 1;
+              const int a = __shfl_sync(0xffffffffu, r0, q[k] & 31), l = __shfl_sync(0xffffffffu, len, q[k] & 31);
+              w[k] = q[k] < 32 && lane < l ? __ldg(ci + a + lane) : -1;
+            }
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+              const uint32_t y = __reduce_or_sync(0xffffffffu, w[k] >= 0 ? cur[w[k]] : 0u);
+              if (lane == q[k]) x |= y;
+            }
+          }
+          lng = more;
+        }
+        for (; lng; lng &= lng - 1) {
+          const int q = __ffs(lng) - 1;
+          const int a = __shfl_sync(0xffffffffu, r0, q), b = __shfl_sync(0xffffffffu, r1, q);
+          uint32_t y = 0u;
+          for (int e = a + lane; e < b; e += 32) y |= cur[__ldg(ci + e)];
+          y = __reduce_or_sync(0xffffffffu, y);
+          if (lane == q) x |= y;
+        }
+        if (u < n) {
+          x &= mask;
+          nxt[u] = x;
+          finish(u, own, x);
+        }
       }
     }
     uint32_t *t = cur;
@@ -245,18 +295,21 @@ int launch_bits_small(gc_graph *g, int32_t k, long long *out, BitsCtl *ctl) {
   const size_t smem = (size_t)n * 12, smem_q = (size_t)n * 4;
   GC_CUDA(cudaMemsetAsync(ctl, 0, sizeof(BitsCtl), g->stream));
   GC_CUDA(cudaMemsetAsync(out, 0, (size_t)n * sizeof(long long), g->stream));
-  for (const void *f : {(const void *)k_bits_cta<0>, (const void *)k_bits_cta<1>})
+  const bool dense = g->nnz > (int64_t)kBitsDense * n;
+  const auto far = dense ? k_bits_cta<0, kBitsRow> : k_bits_cta<0, 32>;
+  const auto gain = dense ? k_bits_cta<1, kBitsRow> : k_bits_cta<1, 32>;
+  for (const void *f : {(const void *)far, (const void *)gain})
     GC_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, kBitsCtaN * 12));
   for (const void *f : {(const void *)k_bits_pick<0>, (const void *)k_bits_pick<1>})
     GC_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, kBitsCtaN * 4));
   g->launches += 2 * k;
   for (int32_t r = 0; r < k; ++r) {
     if (r == 0) {
-      k_bits_cta<0><<<grid, kBitsCtaThreads, smem, g->stream>>>(g->rp, g->ci, n, g->dS, out, ctl);
+      far<<<grid, kBitsCtaThreads, smem, g->stream>>>(g->rp, g->ci, n, g->dS, out, ctl);
       k_bits_pick<0><<<1, kBitsCtaThreads, smem_q, g->stream>>>(g->rp, g->ci, n, g->dS, out, r, g->picks, g->pgain,
                                                                 g->pdec, &ctl->err);
     } else {
-      k_bits_cta<1><<<grid, kBitsCtaThreads, smem, g->stream>>>(g->rp, g->ci, n, g->dS, out, ctl);
+      gain<<<grid, kBitsCtaThreads, smem, g->stream>>>(g->rp, g->ci, n, g->dS, out, ctl);
       k_bits_pick<1><<<1, kBitsCtaThreads, smem_q, g->stream>>>(g->rp, g->ci, n, g->dS, out, r, g->picks, g->pgain,
                                                                 g->pdec, &ctl->err);
     }
