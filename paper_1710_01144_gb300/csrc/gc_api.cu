@@ -371,10 +371,12 @@ static int gains_core(gc_graph *g, const int32_t *S_dev, int32_t s_len, const in
     GC_TRY(launch_bfs(g, g->dS, S_dev, s_len, timeout_ns(nullptr), true));
   }
   // How deep the graph is is known on the device only: two launches, one of
-  // which does the work (the other ends at once).  Distances to a group of more
-  // than one vertex in 32 are short on any graph.
+  // which does the work (the other ends at once).  A group of more than one vertex in
+  // 32 is taken to be spread out, with no distances above kWideLevels, and spared the
+  // idle launch; a group at one end of a path is deep all the same and takes the
+  // 64-lane batches.
   const bool solo = g->solo_ctas > 0 && g->gain_lanes == kLanes && (int64_t)s_len * 32 <= g->n;
-  if (solo) GC_TRY(launch_solo(g, kModeGain, cand_dev, n_cand, nullptr, out_dev, nullptr, 0, false, true));
+  if (solo) GC_TRY(launch_deep_gains(g, cand_dev, n_cand, out_dev, true));
   return launch_gains(g, kModeGain, cand_dev, n_cand, nullptr, out_dev, 0, kLanes, false, true, solo);
 }
 
@@ -401,7 +403,7 @@ int gc_marginal_gains(gc_graph *g, const int32_t *S, int32_t s_len, const int32_
     GC_TRY(gain_event(g, 0, &e0));
     GC_TRY(gain_event(g, 1, &e1));
     GC_CUDA(cudaEventRecord(e0, g->stream));
-    if (solo) GC_TRY(launch_solo(g, kModeGain, g->list, len, nullptr, g->lgain, nullptr, 0, false, false));
+    if (solo) GC_TRY(launch_deep_gains(g, g->list, len, g->lgain, false));
     else GC_TRY(launch_gains(g, kModeGain, g->list, len, nullptr, g->lgain, 0));
     GC_CUDA(cudaEventRecord(e1, g->stream));
     GC_CUDA(cudaMemcpyAsync(out_gain + off, g->lgain, (size_t)len * sizeof(long long),

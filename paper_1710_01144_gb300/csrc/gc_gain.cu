@@ -36,7 +36,7 @@ namespace gc {
 
 size_t gain_ws_stride(int32_t n) { return gain_ws_bytes(n); }
 
-template <int MODE>
+template <int MODE, bool REST = false>
 __global__ void __launch_bounds__(kGainThreads, 2)
     k_gains64(const int32_t *__restrict__ rp, const int32_t *__restrict__ ci, int32_t n,
               const int32_t *__restrict__ dS, const int32_t *__restrict__ cand, int32_t n_cand_arg,
@@ -49,7 +49,14 @@ __global__ void __launch_bounds__(kGainThreads, 2)
   if (shallow_only && *(volatile const int32_t *)&shallow_only->levels > kWideLevels) return;
   const int tid = threadIdx.x;
   const GainWs ws = gain_ws(ws_base, ws_stride, n, blockIdx.x);
-  const int n_cand = n_cand_dev ? *n_cand_dev : n_cand_arg;
+  int n_cand = n_cand_dev ? *n_cand_dev : n_cand_arg;
+  if (REST) {
+    const int first = *(volatile const int32_t *)&ctl->rest_first;
+    if (first >= n_cand) return;  // (batch_next stays zero)
+    cand += first;
+    out += first;
+    n_cand -= first;
+  }
   const int n_batches = (n_cand + lanes - 1) / lanes;
   GainCounters cnt;
   for (;;) {
@@ -93,7 +100,7 @@ int gain_kernel_occupancy(int *blocks_per_sm) {
 
 int launch_gains(gc_graph *g, int mode, const int32_t *cand, int32_t n_cand,
                  const int32_t *n_cand_dev, long long *out, int max_ctas, int lanes, bool pruned,
-                 bool fresh_ctl, bool shallow_only) {
+                 bool fresh_ctl, bool shallow_only, bool rest_only) {
   if (!n_cand_dev && n_cand <= 0) return GC_OK;
   if (lanes < 1 || lanes > kLanes) lanes = kLanes;
   // full batches of gains at the handle's width above 64: the wide kernel
@@ -109,7 +116,11 @@ int launch_gains(gc_graph *g, int mode, const int32_t *cand, int32_t n_cand,
   ++g->launches;
   const bool pr = pruned && mode == kModeGain;
   const int32_t *rp = pr ? g->rpf : g->rp, *ci = pr ? g->cif : g->ci, *c3 = pr ? g->c3 : nullptr;
-  if (mode == kModeGain)
+  if (mode == kModeGain && rest_only)
+    k_gains64<kModeGain, true><<<ctas, kGainThreads, 0, g->stream>>>(
+        rp, ci, g->n, g->dS, cand, n_cand, n_cand_dev, out, g->ws, g->ws_stride, g->gctl, lanes, g->mx,
+        LaneGraphs(), c3, nullptr);
+  else if (mode == kModeGain)
     k_gains64<kModeGain><<<ctas, kGainThreads, 0, g->stream>>>(
         rp, ci, g->n, g->dS, cand, n_cand, n_cand_dev, out, g->ws, g->ws_stride, g->gctl, lanes, g->mx,
         LaneGraphs(), c3, shallow_only ? g->bctl : nullptr);

@@ -127,6 +127,10 @@ struct GainCtl {
   // farness mode: nonzero keeps best_f fixed (top-k closeness cuts at the
   // k-th best, not at the best farness a search completes with)
   int32_t fixed_best;
+  // gains of many candidates on deep graphs: 0 undecided, 1 one-source searches take
+  // all, 2 the 64-lane batches take those from rest_first on
+  int32_t lanes_rest;
+  int32_t rest_first;
   int32_t pad;
 };
 
@@ -425,18 +429,24 @@ enum GainMode { kModeGain = 0, kModeFarness = 1 };
 // pruned (gain mode only): the pruned adjacency, as for launch_bfs.
 // fresh_ctl: *gctl has just been zeroed (so batch_next need not be).
 // shallow_only: does nothing if the BFS that filled d_S had more than
-// kWideLevels levels (launch_solo beside it does the work).
+// kWideLevels levels (launch_solo beside it does the work).  rest_only: only the
+// candidates from gctl->rest_first on.
 int launch_gains(gc_graph *g, int mode, const int32_t *cand, int32_t n_cand,
                  const int32_t *n_cand_dev, long long *out, int max_ctas, int lanes = kLanes,
-                 bool pruned = false, bool fresh_ctl = false, bool shallow_only = false);
+                 bool pruned = false, bool fresh_ctl = false, bool shallow_only = false, bool rest_only = false);
 size_t gain_ws_stride(int32_t n);
 // One candidate per CTA (deep graphs, gc_solo.cu): gains with the pruning
 // relaxed by `slack` (region[i]: vertices visited), or farness values (no_cut:
 // exact for every candidate).  deep_only: does nothing unless the BFS that
-// filled d_S had more than kWideLevels levels.
+// filled d_S had more than kWideLevels levels.  head > 0 (gains): the first searches
+// decide whether the 64-lane batches take the rest (lanes_take_rest).
 int solo_plan(int32_t n, int num_sms, size_t ws_bytes, int *ctas);
 int launch_solo(gc_graph *g, int mode, const int32_t *cand, int32_t n_cand, const int32_t *n_cand_dev, long long *out,
-                int32_t *region, int32_t slack, bool no_cut, bool deep_only);
+                int32_t *region, int32_t slack, bool no_cut, bool deep_only, int32_t head = 0);
+// The gains of cand[0 .. n_cand) on a deep graph, d_S from the last launch_bfs: by
+// one-source searches, the rest of many candidates by whichever form the first searches
+// show to be the better (lanes_take_rest).  deep_only as in launch_solo.
+int launch_deep_gains(gc_graph *g, const int32_t *cand, int32_t n_cand, long long *out, bool deep_only);
 // bounds from the searched vertices list[0 .. sctl->n_sel) (results in lgain)
 // to the vertices within `hops` of them: key (farness) or ub of candidates not
 // evaluated in `round`

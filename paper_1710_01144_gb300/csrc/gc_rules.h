@@ -60,6 +60,21 @@ GC_HD int64_t bfs_grid(int64_t n, int64_t nnz) {
   return v > e ? (v > 1 ? v : 1) : e;
 }
 
+// Gains of many candidates on a large deep graph, after the first of them by one-source
+// searches, `lanes` searches of `edges` adjacency entries: whether the 64-lane batches
+// take the rest.  Searches that reach much of a graph whose distances are short share
+// their rows; with many of them the batches win.  Measured on graphs of short distances
+// with a path of 20 or 40, all vertices as candidates (share of the entries a search
+// scans; one-source, 64-lane, ms): attachment graph n = 100,000, m = 3, groups of 1, 2,
+// 4, 8 (0.32; 195, 130), (0.22; 133, 100), (0.15; 89, 77), (0.03; 21, 28); n = 300,000
+// (0.14; 777, 619), (0.20; 1142, 803), (0.12; 663, 558), (0.03; 149, 202); random n =
+// 100,000 (0.34; 232, 159), (0.17; 113, 101), (0.11; 76, 79); n = 50,000 (0.44; 35, 42).
+// 40,000 candidates on the first 79, 66, 20,000 of them 41, 43.
+constexpr int32_t kLanesHead = 8192, kLanesFrom = 32768, kLanesMinN = 65536;
+GC_HD bool lanes_take_rest(uint64_t edges, uint64_t lanes, int64_t nnz, int64_t sum, int64_t n) {
+  return !far_apart(sum, n) && (double)edges * 9.0 >= (double)lanes * (double)nnz;
+}
+
 // Whether vertex v, entry i of a list of m, is in the list's sample of about `want`:
 // spread by a hash of its id and `salt`.  The first entry always is, so that no
 // sample is empty (one of few CTAs' worth often would be: want = 1 in 37 of 100

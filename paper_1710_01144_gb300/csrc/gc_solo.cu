@@ -57,13 +57,15 @@ constexpr int kSoloRow = 32;  // longer rows are shared by the warp
 
 // With `deep_only`, the kernel runs only if the BFS that filled d_S went deeper
 // than kWideLevels (bctl->levels); otherwise the 64-lane kernel launched beside
-// it does the work.
-template <int MODE>
-__global__ void __launch_bounds__(kSoloThreads)
+// it does the work.  With MANY, the first `head` searches count what they scan, and the
+// first CTA to come for a later one decides whether the 64-lane batches take the rest.
+template <int MODE, bool MANY = false>
+__global__ void __launch_bounds__(kSoloThreads, 16)
     k_solo(const int32_t *__restrict__ rp, const int32_t *__restrict__ ci, int32_t n, const int32_t *__restrict__ dS,
            const int32_t *__restrict__ mx, const int32_t *__restrict__ cand, int32_t n_cand_arg,
            const int32_t *__restrict__ n_cand_dev, long long *__restrict__ out, int32_t *__restrict__ region,
-           int32_t *queues, long long q_stride, GainCtl *ctl, const BfsCtl *deep_only, int32_t slack, int32_t no_cut) {
+           int32_t *queues, long long q_stride, GainCtl *ctl, const BfsCtl *deep_only, int32_t slack, int32_t no_cut,
+           int32_t head, const SelCtl *sctl) {
   extern __shared__ __align__(16) uint32_t s_seen[];  // one bit per vertex
   __shared__ int s_task;
   __shared__ int s_new[3];
@@ -76,11 +78,21 @@ __global__ void __launch_bounds__(kSoloThreads)
   int32_t *q = queues + (size_t)blockIdx.x * q_stride;
   const int n_cand = n_cand_dev ? *n_cand_dev : n_cand_arg;
   u64 w_edges = 0, w_levels = 0, w_front = 0, w_tasks = 0;
+  unsigned w_head = 0;  // searches whose counts are in *ctl already
+  bool stop = false;    // thread 0
   int high = 0;  // entries of the queue that were written
   for (int i = tid; i < nw4; i += T) seen4[i] = make_uint4(0, 0, 0, 0);
   for (;;) {
     if (tid == 0) {
-      s_task = (int)atomicAdd(&ctl->batch_next, 1u);
+      const int rest = MANY ? *(volatile int32_t *)&ctl->lanes_rest : 0;
+      s_task = MANY && stop ? n_cand : (int)atomicAdd(&ctl->batch_next, 1u);
+      stop = rest == 2;  // (after the one just taken)
+      if (MANY && rest == 0 && s_task >= head)  // the first searches are through, or nearly
+        atomicCAS(&ctl->lanes_rest, 0,
+                  lanes_take_rest(*(volatile u64 *)&ctl->edges_scalar, *(volatile u64 *)&ctl->lanes, __ldg(rp + n),
+                                  (int64_t) * (volatile unsigned long long *)&sctl->sum, n)
+                      ? 2
+                      : 1);
       s_new[0] = s_new[1] = s_new[2] = 0;
       if (MODE == kModeFarness) s_best = no_cut ? LLONG_MAX : *(volatile long long *)&ctl->best_f;
     }
@@ -186,6 +198,16 @@ __global__ void __launch_bounds__(kSoloThreads)
     w_levels += (u64)L;
     ++w_tasks;
     if (MODE == kModeGain) acc = block_sum(acc, s_red);
+    if (MANY && task < head) {
+      w_edges = block_sum(w_edges, (u64 *)s_red);
+      if (tid == 0) {
+        atomicAdd(&ctl->edges_scalar, w_edges);
+        atomicAdd(&ctl->edges_union, w_edges);
+        atomicAdd(&ctl->lanes, 1ull);
+      }
+      w_edges = 0;
+      ++w_head;
+    }
     if (tid == 0) {
       if (MODE == kModeGain) {
         out[task] = (long long)dc + acc;
@@ -222,7 +244,7 @@ __global__ void __launch_bounds__(kSoloThreads)
     atomicAdd(&ctl->batches, w_tasks);
     atomicAdd(&ctl->frontier, w_front);
     atomicAdd(&ctl->pushes, w_front);
-    atomicAdd(&ctl->lanes, w_tasks);
+    atomicAdd(&ctl->lanes, w_tasks - w_head);
   }
 }
 
@@ -238,6 +260,7 @@ int solo_plan(int32_t n, int num_sms, size_t ws_bytes, int *ctas) {
   if (smem > 200 * 1024) return GC_OK;
   int x = 0, y = 0;
   GC_CUDA(cudaFuncSetAttribute(k_solo<kModeGain>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
+  GC_CUDA(cudaFuncSetAttribute(k_solo<kModeGain, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
   GC_CUDA(cudaFuncSetAttribute(k_solo<kModeFarness>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
   GC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&x, k_solo<kModeGain>, kSoloThreads, smem));
   GC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&y, k_solo<kModeFarness>, kSoloThreads, smem));
@@ -247,7 +270,7 @@ int solo_plan(int32_t n, int num_sms, size_t ws_bytes, int *ctas) {
 }
 
 int launch_solo(gc_graph *g, int mode, const int32_t *cand, int32_t n_cand, const int32_t *n_cand_dev, long long *out,
-                int32_t *region, int32_t slack, bool no_cut, bool deep_only) {
+                int32_t *region, int32_t slack, bool no_cut, bool deep_only, int32_t head) {
   if (!n_cand_dev && n_cand <= 0) return GC_OK;
   // (with deep_only the caller has just zeroed *gctl)
   if (!deep_only) GC_CUDA(cudaMemsetAsync(&g->gctl->batch_next, 0, sizeof(unsigned int), g->stream));
@@ -258,16 +281,38 @@ int launch_solo(gc_graph *g, int mode, const int32_t *cand, int32_t n_cand, cons
   const size_t smem = solo_smem(g->n);
   int32_t *queues = (int32_t *)g->ws;
   const long long q_stride = (long long)(solo_queue_bytes(g->n) / sizeof(int32_t));
-  if (mode == kModeGain)
+  if (mode == kModeGain && head > 0)
+    k_solo<kModeGain, true><<<ctas, kSoloThreads, smem, g->stream>>>(g->rp, g->ci, g->n, g->dS, g->mx, cand, n_cand,
+                                                                     n_cand_dev, out, region, queues, q_stride,
+                                                                     g->gctl, deep, slack, 0, head, g->sctl);
+  else if (mode == kModeGain)
     k_solo<kModeGain><<<ctas, kSoloThreads, smem, g->stream>>>(g->rp, g->ci, g->n, g->dS, g->mx, cand, n_cand,
                                                                n_cand_dev, out, region, queues, q_stride, g->gctl,
-                                                               deep, slack, 0);
+                                                               deep, slack, 0, 0, nullptr);
   else
     k_solo<kModeFarness><<<ctas, kSoloThreads, smem, g->stream>>>(g->rp, g->ci, g->n, g->dS, nullptr, cand, n_cand,
                                                                   n_cand_dev, out, nullptr, queues, q_stride, g->gctl,
-                                                                  deep, 0, no_cut ? 1 : 0);
+                                                                  deep, 0, no_cut ? 1 : 0, 0, nullptr);
   GC_CUDA(cudaGetLastError());
   return GC_OK;
+}
+
+// What the one-source searches left to the 64-lane batches (all in stream order, so that
+// the call needs no host read and can be captured).
+__global__ void k_lanes_rest(GainCtl *ctl, int32_t n_cand) {
+  ctl->rest_first = ctl->lanes_rest == 2 ? (int32_t)min(ctl->batch_next, (unsigned)n_cand) : n_cand;
+  ctl->batch_next = 0;
+}
+
+int launch_deep_gains(gc_graph *g, const int32_t *cand, int32_t n_cand, long long *out, bool deep_only) {
+  const bool many = n_cand > kLanesFrom && g->n >= kLanesMinN;
+  const int rc = launch_solo(g, kModeGain, cand, n_cand, nullptr, out, nullptr, 0, false, deep_only,
+                             many ? kLanesHead : 0);
+  if (rc != GC_OK || !many) return rc;
+  ++g->launches;
+  k_lanes_rest<<<1, 1, 0, g->stream>>>(g->gctl, n_cand);
+  GC_CUDA(cudaGetLastError());
+  return launch_gains(g, kModeGain, cand, n_cand, nullptr, out, 0, kLanes, false, true, false, true);
 }
 
 // ---- bounds for the neighbourhoods of searched vertices ----

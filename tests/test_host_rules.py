@@ -17,6 +17,9 @@ extern "C" {
 int32_t bucket_end(int32_t mn, int32_t delta) { return w_bucket_end(mn, delta); }
 int in_bucket(int32_t x, int32_t T) { return w_in_bucket(x, T); }
 int far(int64_t sum, int64_t n) { return far_apart(sum, n); }
+int lanes_rest(uint64_t edges, uint64_t lanes, int64_t nnz, int64_t sum, int64_t n) {
+  return lanes_take_rest(edges, lanes, nnz, sum, n);
+}
 int whole_search(int64_t n, int64_t nnz) { return w_whole_search(n, nnz); }
 int64_t grid_of_bfs(int64_t n, int64_t nnz) { return bfs_grid(n, nnz); }
 
@@ -143,3 +146,13 @@ def test_bfs_grid_has_ctas_for_the_entries(rules, n, nnz, ctas):
                                          (1024, 65536, 1), (1024, 65538, 0), (1025, 2050, 0), (2**30, 2**31 - 1, 0)])
 def test_whole_weighted_searches(rules, n, nnz, whole):
     assert rules.whole_search(ctypes.c_int64(n), ctypes.c_int64(nnz)) == whole
+
+
+def test_lanes_take_the_rest(rules):
+    def rest(share, mean, n=100000, nnz=600000, lanes=8192):
+        return bool(rules.lanes_rest(ctypes.c_uint64(int(share * lanes * nnz)), ctypes.c_uint64(lanes), ctypes.c_int64(nnz),
+                                     ctypes.c_int64(int(mean * n)), ctypes.c_int64(n)))
+
+    assert rest(0.3, 5.2) and rest(0.112, 5.2) and not rest(0.110, 5.2)
+    assert not rest(0.5, 200.0)                      # a road network
+    assert rest(1.0, 5.0, 2**31 - 1, 2**31 - 1, 2**31 - 1)  # (no overflow)
