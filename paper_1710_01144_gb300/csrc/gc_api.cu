@@ -682,12 +682,8 @@ int gc_set_weights(gc_graph *g, const int32_t *weights, uint32_t flags) {
   if (!alloc_missing([&](auto *&p) { return (rc = dalloc(&p, (size_t)g->nnz)) == GC_OK; }, [](void *p) { cudaFree(p); },
                      g->ci_w, g->wt_w))
     return rc;
-  int32_t *tmp = nullptr;  // cif (scratch here) holds the ids of a middle pass, tmp its weights
-  if (g->w_max > 255 && (rc = dalloc(&tmp, (size_t)g->nnz))) return rc;
-  rc = launch_wsort(g, g->cif, tmp);
-  if (rc == GC_OK) rc = sync(g);
-  cudaFree(tmp);
-  GC_TRY(rc);
+  GC_TRY(launch_wsort(g, g->cif));  // (cif: scratch until round 1 of gc_greedy)
+  GC_TRY(sync(g));
   g->w_ok = true;
   return GC_OK;
 }

@@ -489,7 +489,7 @@ enum WMode { kWFarness = 0, kWGain = 1, kWRelabel = 2 };
 size_t wws_stride(int32_t n);
 int wsearch_occupancy(const gc_graph *g, int *blocks_per_sm);
 int launch_wfar_init(gc_graph *g);
-int launch_wsort(gc_graph *g, int32_t *tmp_ci, int32_t *tmp_wt);
+int launch_wsort(gc_graph *g, int32_t *tmp);
 int launch_wsearch(gc_graph *g, int mode, const int32_t *list, const int32_t *m_dev, int32_t m, long long *out,
                    long long *best, int32_t delta);
 int launch_wcheck(gc_graph *g, bool mirror, int32_t *bad, int32_t *max_w);
