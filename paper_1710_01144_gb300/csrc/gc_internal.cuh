@@ -139,15 +139,12 @@ struct GridGainCtl {
   GridBar bar;
   int32_t err;
   int32_t levels;     // levels the last batch expanded
-  int32_t qn[2];      // (unused)
   int32_t touched;    // vertices with a non-zero visited word
   int32_t pad;
   // frontier of level L, by L mod 3: entries (high 32 bits) and adjacency
   // entries (low 32 bits), both taken by one atomicAdd per push
   unsigned long long pk[3];
   unsigned long long gain[kLanes];  // gain mode: per-lane gain
-  unsigned long long cnt[kLanes];   // (unused in farness mode, see dgain/dcnt)
-  int32_t blk_tot[kMaxGridCtas];    // per-CTA adjacency totals of the level
   // farness mode: per-lane sums of deg - 1 and counts of the vertices claimed at
   // distance d, in dgain/dcnt[d mod 3] (written during one level, read by every
   // CTA after its barrier, cleared two levels later)

@@ -537,7 +537,6 @@ static __device__ void lazy_cta0_step(const int32_t *act, int32_t m, long long *
   // a fresh grid-batch control block for the evaluation (grid form only)
   if (gg && tid < kLanes) {
     gg->gain[tid] = 0;
-    gg->cnt[tid] = 0;
   }
   if (tid == 0) {
     lc->n_sel = taken < kLanes ? taken : kLanes;
@@ -651,7 +650,6 @@ static __device__ void lean_step(const int32_t *act, long long *ub, int32_t *sta
   else dec = 0;
   if (dec == 0 && tid < kLanes) {  // a fresh grid-batch control block
     gg->gain[tid] = 0;
-    gg->cnt[tid] = 0;
   }
   if (tid == 0) {
     st.dec = dec;
@@ -946,7 +944,6 @@ static __device__ bool grid_lazy_step(const int32_t *act, int32_t m, long long *
   }
   if (b == 0 && gg && tid < kLanes) {
     gg->gain[tid] = 0;
-    gg->cnt[tid] = 0;
   }
   return true;
 }
