@@ -113,7 +113,11 @@ typedef struct gc_opts {
                               64 largest bounds, certification and d_S update on
                               the device) */
   int32_t active_target;   /* step_mode 3: initial size of its candidate list
-                              (grown x4 when the list cannot certify a pick);
+                              (when the list cannot certify a pick: rebuilt at
+                              the same size up to six times, grown x4 beyond;
+                              wide steps: grown x4 at once; not grown when a
+                              sweep has evaluated every bound that still reaches
+                              the best gain);
                               0 = 2048 for grid-wide steps, max(4096, two wide
                               steps) for wide ones */
   int32_t round1_heavy;    /* round 1: this many highest-degree candidates are
@@ -490,6 +494,9 @@ typedef struct gc_batch gc_batch; /* opaque: union CSR + per-graph state */
 
 /* gc_batch_load -- count graphs given by host CSR arrays row_ptrs[g],
  * col_idxs[g] with ns[g] vertices (each connected, format as for gc_load_csr).
+ * Device memory: about 130 bytes per vertex and 8 per adjacency entry of the
+ * union, and workspaces of 44 bytes per vertex of the largest graph for each CTA
+ * that fits.
  * flags: reserved (0).  Errors: GC_EINVAL, GC_ERANGE (union beyond int32 CSR),
  * GC_ENOMEM, GC_ECUDA. */
 int gc_batch_load(int32_t count, const int32_t *const *row_ptrs, const int32_t *const *col_idxs, const int32_t *ns,

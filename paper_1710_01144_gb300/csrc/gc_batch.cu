@@ -15,9 +15,10 @@
 //   P2  every v with LB(v) <= f_a evaluated by the 64-lane BFS in farness
 //       mode with per-graph cuts (graph-aligned batches, by teams of CTAs on
 //       graphs with few survivors), after the far counts have raised the
-//       bounds; per graph s0 = argmin (f, id).  Measured with round 1's
-//       batches by teams too: rounds 0 and 1 of 24 mixed graphs 45 + 32 -> 17
-//       + 12 ms, of 256 graphs 623 + 190 -> 493 + 167 ms
+//       bounds; per graph s0 = argmin (f, id).  With round 1's batches by
+//       teams too, rounds 0 and 1 of 24 mixed graphs went from 45 + 32 to 17 + 12
+//       ms, of 256 graphs from 623 + 190 to 493 + 167 (other kernels as they were
+//       then)
 //   P3  BFS from all s0 (d_S), per-graph farness, neighbour bound mx
 //   P4  round 1: every candidate of every graph, graph-aligned 64-lane batches
 //       from a dynamic task counter; per-graph argmax; picks; BFS from picks
@@ -28,7 +29,8 @@
 //       so no graph waits for another.  A team's steps are those of the
 //       single-graph persistent kernel.  One CTA per graph, as before, left
 //       most of the GPU idle behind the slowest graph: 24 mixed graphs 717 ms
-//       (lazy rounds 634), with teams and sweeps 102 ms; 256 graphs 1468 -> 976 ms.
+//       (lazy rounds 634), 256 graphs 1468; by teams, with the sweeps and all later
+//       steps, 34 to 37 and 377.
 //   P7  check: one BFS from every graph's whole group; each graph's farness
 //       must equal f(s0) minus the sum of its accepted gains.
 #include <limits.h>
@@ -147,8 +149,8 @@ constexpr int kBatchThreads = kGainThreads;
 constexpr int32_t kBatchGridMinN = 1 << 21;
 
 // lazy rounds: a list that cannot certify a pick starts a sweep when more than
-// this many bounds reach the best gain (16 steps of 64): 24 mixed graphs 207 ->
-// 102 ms, 256 graphs 1109 -> 976 ms
+// this many bounds reach the best gain (16 steps of 64): when they came, 24 mixed
+// graphs 207 -> 102 ms, 256 graphs 1109 -> 976 (34 to 37 and 377 with all later steps)
 constexpr int kBatchSweepMin = 1024;
 
 static __device__ __forceinline__ bool bsync(const BatchArgs &a) { return grid_sync(&a.ctl->bar, &a.ctl->err, a.tns); }

@@ -374,8 +374,9 @@ __global__ void __launch_bounds__(kRedThreads) k_heavy_rows(const int32_t *__res
 // atomics on the count array (71 MB at scale 24, it stays in L2).  Measured:
 // R-MAT scale 24, k = 50: round 0 166.5 -> 14.7 ms, the call 215.6 -> 64.2 ms;
 // top-100 closeness at scale 18: 17.4 -> 3.60 ms (12,848 survivors -> 57); one
-// survivor batch at scale 20: 9.88 -> 9.84 ms, so the counts run whenever any
-// vertex survives on a shallow graph.
+// survivor batch at scale 20: 9.88 -> 9.84 ms.  They run on shallow graphs with more
+// than 64 survivors: up to 64 are one batch, which costs no more than the counts.
+
 // cnt[w] += the classes of w's neighbours of degree 1 .. kFarDeg (low half
 // {1, 2}, high half the rest), one thread per such neighbour's row;
 // total[0..1] = members per class.  cnt and total start at zero.

@@ -65,11 +65,13 @@ GC_HD int64_t bfs_grid(int64_t n, int64_t nnz) {
 // take the rest.  Searches that reach much of a graph whose distances are short share
 // their rows; with many of them the batches win.  Measured on graphs of short distances
 // with a path of 20 or 40, all vertices as candidates (share of the entries a search
-// scans; one-source, 64-lane, ms): attachment graph n = 100,000, m = 3, groups of 1, 2,
-// 4, 8 (0.32; 195, 130), (0.22; 133, 100), (0.15; 89, 77), (0.03; 21, 28); n = 300,000
-// (0.14; 777, 619), (0.20; 1142, 803), (0.12; 663, 558), (0.03; 149, 202); random n =
-// 100,000 (0.34; 232, 159), (0.17; 113, 101), (0.11; 76, 79); n = 50,000 (0.44; 35, 42).
-// 40,000 candidates on the first 79, 66, 20,000 of them 41, 43.
+// scans; all by one-source searches, by this rule, ms): attachment graph n = 100,000, m
+// = 3, groups of 1, 2, 4, 8 (0.32; 195, 86), (0.22; 133, 70), (0.15; 89, 56), (0.03; 21,
+// 21); n = 300,000 (0.14; 777, 412), (0.20; 1142, 489), (0.12; 663, 387), (0.03, but
+// more for the first ids; 149, 170); random n = 100,000 (0.34; 232, 102), (0.17; 113,
+// 67), (0.11; 76, 54), (0.05; 36, 35).  40,000 candidates on the first 79, 44.  50,000
+// vertices, all of them: 42 by the 64-lane batches as they were before the one-source
+// searches, 35 by these (130 and 195 at 100,000).
 constexpr int32_t kLanesHead = 8192, kLanesFrom = 32768, kLanesMinN = 65536;
 GC_HD bool lanes_take_rest(uint64_t edges, uint64_t lanes, int64_t nnz, int64_t sum, int64_t n) {
   return !far_apart(sum, n) && (double)edges * 9.0 >= (double)lanes * (double)nnz;

@@ -145,8 +145,8 @@ __global__ void __launch_bounds__(32 * kWSortLong) k_wsort_long(const int32_t *_
 // A search's random accesses are its distances and two flags per vertex.  For
 // 300 to 1,200 searches at a time they do not fit L2 (round 0 at scale 14: 26 ms
 // with them in the workspace, bound by DRAM sectors), so up to kWFarSmemN
-// vertices they live in shared memory (SM: 13 ms; four CTAs of 512 threads per SM
-// at scale 14, one of 1024 beyond 24,000 vertices); the queues and lists in
+// vertices they live in shared memory (SM: 13 ms; four CTAs of 512 threads per SM up
+// to about 11,000 vertices, three at scale 14, one of 1024 beyond 24,000); the queues and lists in
 // global memory are written and read in order.  Larger graphs keep them in the
 // workspace.
 constexpr int kWFarSmemN = 48000;  // 199 KB, and 13 KB of static arrays at 1024 threads
