@@ -24,10 +24,10 @@ namespace gc {
 // bits of the weights each, least significant first.  A middle pass moves entry numbers
 // alone, the last one the ids and weights.  A warp takes a segment of a row, 32 entries
 // at a time, and ranks the equal digits of a tile by match-any: a row is one segment,
-// rows of more than kHeavyRow entries are kWSortLong, by a CTA.  The whole call, ms, a
+// rows of more than kHeavyRow entries are kWSortWarps, by a CTA.  The whole call, ms, a
 // warp a row and scratch weights allocated, now: star of 16,000, weights up to 1000,
-// 0.59, 0.26; of 1,000,000 33, 12; R-MAT scale 18 1.52, 0.65; complete n = 600 0.23, 0.08.
-constexpr int kWSortWarps = 8, kWSortLong = 32;
+// 0.54, 0.21; of 1,000,000 33, 12; R-MAT scale 18 1.50, 0.64; complete n = 600 0.21, 0.10.
+constexpr int kWSortWarps = 32;
 
 struct WSort {
   const int32_t *ci, *wt;   // the rows as they are
@@ -70,13 +70,40 @@ __device__ __forceinline__ void wsort_move(const WSort &w, int e0, int e1, int *
   }
 }
 
-__global__ void __launch_bounds__(32 * kWSortWarps) k_wsort(const int32_t *__restrict__ rp, int32_t n, const WSort w) {
+// Long rows first, a CTA each, then the others, a warp each.
+__global__ void __launch_bounds__(32 * kWSortWarps) k_wsort(const int32_t *__restrict__ rp, int32_t n,
+                                                            const int32_t *__restrict__ heavy,
+                                                            const int32_t *__restrict__ nh, const WSort w) {
   __shared__ int s_at[kWSortWarps][256];
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  __shared__ int s_scan[33];
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   int *at = s_at[wid];
+  for (int i = blockIdx.x; i < *nh; i += gridDim.x) {
+    const int e0 = rp[heavy[i]], len = rp[heavy[i] + 1] - e0;
+    // warp k: entries [len k / 32, len (k + 1) / 32)
+    const int a = e0 + (int)((long long)len * wid / kWSortWarps);
+    const int b = e0 + (int)((long long)len * (wid + 1) / kWSortWarps);
+    wsort_count(w, a, b, at);
+    cta_sync();
+    // counts -> first slots: digits in order, a digit's segments in order
+    int sum = 0;
+    if (tid < 256)
+      for (int k = 0; k < kWSortWarps; ++k) sum += s_at[k][tid];
+    int total;
+    int first = e0 + block_excl_scan(sum, s_scan, &total);
+    if (tid < 256)
+      for (int k = 0; k < kWSortWarps; ++k) {
+        const int c = s_at[k][tid];
+        s_at[k][tid] = first;
+        first += c;
+      }
+    cta_sync();
+    wsort_move(w, a, b, at);
+    cta_sync();  // s_at is reused
+  }
   for (int v = blockIdx.x * kWSortWarps + wid; v < n; v += gridDim.x * kWSortWarps) {
     const int e0 = rp[v], e1 = rp[v + 1];
-    if (e1 - e0 > kHeavyRow) continue;  // k_wsort_long
+    if (e1 - e0 > kHeavyRow) continue;
     wsort_count(w, e0, e1, at);
     int carry = e0;  // counts -> first slots
     for (int base = 0; base < 256; base += 32) {
@@ -92,36 +119,6 @@ __global__ void __launch_bounds__(32 * kWSortWarps) k_wsort(const int32_t *__res
     }
     __syncwarp();
     wsort_move(w, e0, e1, at);
-  }
-}
-
-__global__ void __launch_bounds__(32 * kWSortLong) k_wsort_long(const int32_t *__restrict__ rp,
-                                                               const int32_t *__restrict__ heavy,
-                                                               const int32_t *__restrict__ nh, const WSort w) {
-  __shared__ int s_at[kWSortLong][256];
-  __shared__ int s_scan[33];
-  const int tid = threadIdx.x, wid = tid >> 5;
-  for (int i = blockIdx.x; i < *nh; i += gridDim.x) {
-    const int e0 = rp[heavy[i]], len = rp[heavy[i] + 1] - e0;
-    // warp k: entries [len k / 32, len (k + 1) / 32)
-    const int a = e0 + (int)((long long)len * wid / kWSortLong), b = e0 + (int)((long long)len * (wid + 1) / kWSortLong);
-    wsort_count(w, a, b, s_at[wid]);
-    cta_sync();
-    // counts -> first slots: digits in order, a digit's segments in order
-    int sum = 0;
-    if (tid < 256)
-      for (int k = 0; k < kWSortLong; ++k) sum += s_at[k][tid];
-    int total;
-    int at = e0 + block_excl_scan(sum, s_scan, &total);
-    if (tid < 256)
-      for (int k = 0; k < kWSortLong; ++k) {
-        const int c = s_at[k][tid];
-        s_at[k][tid] = at;
-        at += c;
-      }
-    cta_sync();
-    wsort_move(w, a, b, s_at[wid]);
-    cta_sync();  // s_at is reused
   }
 }
 
@@ -587,14 +584,14 @@ int launch_wsearch(gc_graph *g, int mode, const int32_t *list, const int32_t *m_
 int launch_wsort(gc_graph *g, int32_t *tmp) {
   int passes = 1;
   while (passes < 4 && (g->w_max >> (8 * passes)) > 0) ++passes;
+  const int grid = std::min(g->num_sms * 2, (g->n + kWSortWarps - 1) / kWSortWarps);
   WSort w{g->ci, g->wt, nullptr, nullptr, g->ci_w, g->wt_w, 0};
   for (int p = 0; p < passes; ++p) {
     const int left = passes - 1 - p;
     w.to = left == 0 ? nullptr : (left & 1) ? tmp : g->ci_w;
     w.shift = 8 * p;
-    g->launches += 2;
-    k_wsort<<<g->num_sms * 8, 32 * kWSortWarps, 0, g->stream>>>(g->rp, g->n, w);
-    k_wsort_long<<<g->num_sms * 2, 32 * kWSortLong, 0, g->stream>>>(g->rp, g->heavy, g->n_heavy, w);
+    ++g->launches;
+    k_wsort<<<grid, 32 * kWSortWarps, 0, g->stream>>>(g->rp, g->n, g->heavy, g->n_heavy, w);
     w.from = w.to;
   }
   GC_CUDA(cudaGetLastError());
